@@ -1,7 +1,8 @@
 // kp_mlp.cu -- the learned proposal's network: inference and training
-// kernels and the kp_mlp_* entry points of include/kp.h.  Inference runs
-// 32-row tiles on mma.sync (the same tile code the planner's loop uses);
-// every training GEMM of the backward pass runs on the tcgen05 tensor cores
+// kernels and the kp_mlp_* entry points of include/kp.h.  Inference is one
+// kernel on the tcgen05 tensor cores (kp_mlp_tc.cuh); training's forward pass
+// runs 32-row tiles on mma.sync (the same tile code the planner's loop uses)
+// and every training GEMM of the backward pass runs on the tcgen05 tensor cores
 // (kp_tc.cuh: TMA-staged BF16 operands, FP32 accumulation in tensor memory);
 // FP32 master weights and Adam moments.
 // Like the planner, the network context allocates no device memory: it
@@ -14,6 +15,7 @@
 
 #include "../../include/kp.h"
 #include "kp_mlp.cuh"
+#include "kp_mlp_tc.cuh"
 #include "kp_tc.cuh"
 
 namespace kp {
@@ -34,7 +36,7 @@ constexpr int N_WEIGHTS_BF16 = MLP_H * MLP_IN + MLP_H * MLP_H + MLP_OUT * MLP_H;
 // the raw outputs, and when given the BF16 inputs and hidden activations
 // (training) or the heads (inference: mean, log_std per row).
 __global__ void __launch_bounds__(256) kp_mlp_forward_kernel(MlpWeights w, const float* x, int M,
-                                                             float* raw, float* heads,
+                                                             float* raw,
                                                              bf16* xb, bf16* h1, bf16* h2,
                                                              bf16* xbt, int ldt) {
   __shared__ __align__(16) bf16 sX[MLP_TILE * MLP_XS];
@@ -50,15 +52,6 @@ __global__ void __launch_bounds__(256) kp_mlp_forward_kernel(MlpWeights w, const
   }
   __syncthreads();
   mlp_tile_forward<MLP_TILE / 16>(w, sX, sH, raw, row0, rows, h1, h2);
-  if (heads && threadIdx.x < rows) {
-    const int r = row0 + threadIdx.x;
-    float mean[MLP_NQ], ls[MLP_NQ];
-    mlp_heads(raw + (size_t)r * MLP_OUT, mean, ls);
-    for (int i = 0; i < MLP_NQ; ++i) {
-      heads[(size_t)r * MLP_OUT + i] = mean[i];
-      heads[(size_t)r * MLP_OUT + MLP_NQ + i] = ls[i];
-    }
-  }
 }
 
 // ---------------------------------------------------------------------------
@@ -198,16 +191,19 @@ __global__ void kp_mlp_transpose_kernel(const bf16* a, int M, int cols, bf16* at
 
 // Parameter i rounded to BF16 into the row-major weight copy (training
 // kernels) and into the fragment-order copy (the planner's loop kernel).
-__device__ __forceinline__ void store_weight(int i, float pi, bf16* wb, bf16* wf, bf16* w2t) {
+__device__ __forceinline__ void store_weight(int i, float pi, bf16* wb, bf16* wf, bf16* w2t,
+                                             bf16* wt) {
   const bf16 b = __float2bfloat16_rn(pi);
   if (i < OFF_B1) {
     wb[i] = b;
+    wt[tc::wt_index_w1(i / MLP_IN, i % MLP_IN)] = b;
     wf[frag_index_hidden(i / MLP_IN, i % MLP_IN, MLP_IN)] = b;
   } else if (i >= OFF_W2 && i < OFF_B2) {
     const int j = i - OFF_W2;
     wb[MLP_H * MLP_IN + j] = b;
     wf[MLP_H * MLP_IN + frag_index_hidden(j / MLP_H, j % MLP_H, MLP_H)] = b;
     w2t[(j % MLP_H) * MLP_H + j / MLP_H] = b;
+    wt[tc::wt_index_w2(j / MLP_H, j % MLP_H)] = b;
   } else if (i >= OFF_W3 && i < OFF_B3) {
     const int j = i - OFF_W3;
     wb[MLP_H * MLP_IN + MLP_H * MLP_H + j] = b;
@@ -217,7 +213,8 @@ __device__ __forceinline__ void store_weight(int i, float pi, bf16* wb, bf16* wf
 
 __device__ __forceinline__ void adam_update(int i, float* p, const float* g, float* m, float* v,
                                             float lr, float beta1, float beta2, float eps,
-                                            float c1, float c2, bf16* wb, bf16* wf, bf16* w2t) {
+                                            float c1, float c2, bf16* wb, bf16* wf, bf16* w2t,
+                                            bf16* wt) {
   const float gi = g[i];
   const float mi = beta1 * m[i] + (1.0f - beta1) * gi;
   const float vi = beta2 * v[i] + (1.0f - beta2) * gi * gi;
@@ -225,15 +222,15 @@ __device__ __forceinline__ void adam_update(int i, float* p, const float* g, flo
   v[i] = vi;
   const float pi = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
   p[i] = pi;
-  store_weight(i, pi, wb, wf, w2t);
+  store_weight(i, pi, wb, wf, w2t, wt);
 }
 
 __global__ void kp_mlp_adam_kernel(float* p, const float* g, float* m, float* v, int n, float lr,
                                    float beta1, float beta2, float eps, float c1, float c2,
-                                   bf16* wb, bf16* wf, bf16* w2t) {
+                                   bf16* wb, bf16* wf, bf16* w2t, bf16* wt) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  adam_update(i, p, g, m, v, lr, beta1, beta2, eps, c1, c2, wb, wf, w2t);
+  adam_update(i, p, g, m, v, lr, beta1, beta2, eps, c1, c2, wb, wf, w2t, wt);
 }
 
 // ---- device-driven epoch (one CUDA graph launch per mini-batch) -------------
@@ -264,13 +261,13 @@ __global__ void kp_mlp_gather_kernel(const EpochCtl* ec, int B, float* xg, float
 
 // Adam with the step count and learning rate read from the epoch control.
 __global__ void kp_mlp_adam_dev_kernel(float* p, const float* g, float* m, float* v, int n,
-                                       const EpochCtl* ec, bf16* wb, bf16* wf, bf16* w2t) {
+                                       const EpochCtl* ec, bf16* wb, bf16* wf, bf16* w2t, bf16* wt) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const float beta1 = 0.9f, beta2 = 0.999f;
   const float step = (float)(ec->step + 1);
   const float c1 = 1.0f - powf(beta1, step), c2 = 1.0f - powf(beta2, step);
-  adam_update(i, p, g, m, v, ec->lr, beta1, beta2, 1e-8f, c1, c2, wb, wf, w2t);
+  adam_update(i, p, g, m, v, ec->lr, beta1, beta2, 1e-8f, c1, c2, wb, wf, w2t, wt);
 }
 
 __global__ void kp_mlp_epoch_tail_kernel(EpochCtl* ec, const float* loss) {
@@ -279,10 +276,10 @@ __global__ void kp_mlp_epoch_tail_kernel(EpochCtl* ec, const float* loss) {
   ec->batch += 1;
 }
 
-__global__ void kp_mlp_round_kernel(const float* p, bf16* wb, bf16* wf, bf16* w2t) {
+__global__ void kp_mlp_round_kernel(const float* p, bf16* wb, bf16* wf, bf16* w2t, bf16* wt) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N_PARAMS) return;
-  store_weight(i, p[i], wb, wf, w2t);
+  store_weight(i, p[i], wb, wf, w2t, wt);
 }
 
 }  // namespace kp
@@ -303,6 +300,8 @@ struct kp_mlp {
   bf16* wb;  // W1 | W2 | W3 in BF16, row-major
   bf16* wf;  // the same in fragment order (planner loop)
   bf16* w2t; // W2 transposed ([in][out], tensor-core backward)
+  bf16* wt;  // W2 and W1 in tensor-core operand order (inference)
+  int num_sms;
   bf16 *dh2t, *h1t, *h2t, *dh1t;  // [256][ldt] transposed activations
   bf16 *xbt, *drawt;               // [32][ldt], [8][ldt]
   int ldt;
@@ -320,7 +319,7 @@ struct kp_mlp {
 namespace {
 
 struct MlpLayout {
-  size_t p, m, v, g, wb, wf, w2t, dh2t, h1t, h2t, dh1t, xbt, drawt, err, xg, tg, ec, loss, raw, d_raw, xb, h1, h2, d_raw_b, dh2, dh1, total;
+  size_t p, m, v, g, wb, wf, w2t, wt, dh2t, h1t, h2t, dh1t, xbt, drawt, err, xg, tg, ec, loss, raw, d_raw, xb, h1, h2, d_raw_b, dh2, dh1, total;
 };
 
 size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -343,6 +342,7 @@ MlpLayout mlp_layout(int B) {
   L.wb = take((size_t)N_WEIGHTS_BF16 * 2);
   L.wf = take((size_t)N_WEIGHTS_BF16 * 2);
   L.w2t = take((size_t)MLP_H * MLP_H * 2);
+  L.wt = take((size_t)tc::WT_ELEMS * 2);
   L.dh2t = take((size_t)MLP_H * ld_t(B) * 2);
   L.h1t = take((size_t)MLP_H * ld_t(B) * 2);
   L.h2t = take((size_t)MLP_H * ld_t(B) * 2);
@@ -459,6 +459,8 @@ kp_status tc_configure() {
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_BYTES));
     MLP_CUDA(cudaFuncSetAttribute(tc::tc_gemm_kernel<tc::EPI_BIAS_RELU_BF16>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_BYTES));
+    MLP_CUDA(cudaFuncSetAttribute(tc::kp_mlp_forward_tc_kernel,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize, tc::FT_SMEM));
     done = true;
   }
   return KP_OK;
@@ -479,7 +481,7 @@ kp_status forward_backward(kp_mlp* n, const float* x, const float* t, int M) {
   MLP_CUDA(cudaMemsetAsync(n->g, 0, (size_t)N_PARAMS * 4, n->stream));
   MLP_CUDA(cudaMemsetAsync(n->loss, 0, 4, n->stream));
   kp_mlp_forward_kernel<<<(M + MLP_TILE - 1) / MLP_TILE, 256, 0, n->stream>>>(
-      w, x, M, n->raw, nullptr, n->xb, n->h1, n->h2, n->xbt, n->ldt);
+      w, x, M, n->raw, n->xb, n->h1, n->h2, n->xbt, n->ldt);
   MLP_CUDA(cudaGetLastError());
   kp_mlp_head_loss_kernel<<<(M + 255) / 256, 256, 0, n->stream>>>(
       n->raw, t, M, n->d_raw, n->d_raw_b, n->loss, n->drawt, n->ldt, n->g + OFF_B3);
@@ -568,6 +570,7 @@ kp_status kp_mlp_create(void* dev_arena, size_t arena_bytes, int32_t max_batch,
   n->wb = reinterpret_cast<bf16*>(A + L.wb);
   n->wf = reinterpret_cast<bf16*>(A + L.wf);
   n->w2t = reinterpret_cast<bf16*>(A + L.w2t);
+  n->wt = reinterpret_cast<bf16*>(A + L.wt);
   n->dh2t = reinterpret_cast<bf16*>(A + L.dh2t);
   n->h1t = reinterpret_cast<bf16*>(A + L.h1t);
   n->h2t = reinterpret_cast<bf16*>(A + L.h2t);
@@ -588,7 +591,15 @@ kp_status kp_mlp_create(void* dev_arena, size_t arena_bytes, int32_t max_batch,
   n->d_raw_b = reinterpret_cast<bf16*>(A + L.d_raw_b);
   n->dh2 = reinterpret_cast<bf16*>(A + L.dh2);
   n->dh1 = reinterpret_cast<bf16*>(A + L.dh1);
-  kp_status s = kp_mlp_set_params(n, host_params);
+  int dev = 0;
+  kp_status s = KP_OK;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&n->num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    cudaGetLastError();
+    s = KP_ERR_CUDA;
+  }
+  if (s == KP_OK) s = tc_configure();
+  if (s == KP_OK) s = kp_mlp_set_params(n, host_params);
   if (s != KP_OK) {
     delete n;
     return s;
@@ -606,7 +617,7 @@ kp_status kp_mlp_set_params(kp_mlp* n, const float* host_params) {
   MLP_CUDA(cudaMemsetAsync(n->m, 0, (size_t)N_PARAMS * 4, n->stream));
   MLP_CUDA(cudaMemsetAsync(n->v, 0, (size_t)N_PARAMS * 4, n->stream));
   MLP_CUDA(cudaMemsetAsync(n->err, 0, 16, n->stream));
-  kp_mlp_round_kernel<<<(N_PARAMS + 255) / 256, 256, 0, n->stream>>>(n->p, n->wb, n->wf, n->w2t);
+  kp_mlp_round_kernel<<<(N_PARAMS + 255) / 256, 256, 0, n->stream>>>(n->p, n->wb, n->wf, n->w2t, n->wt);
   MLP_CUDA(cudaGetLastError());
   MLP_CUDA(cudaStreamSynchronize(n->stream));
   n->step = 0;
@@ -626,8 +637,22 @@ int32_t kp_mlp_num_params(void) { return N_PARAMS; }
 kp_status kp_mlp_forward(kp_mlp* n, const float* dev_x, int32_t M, float* dev_out) {
   if (!n || !dev_x || !dev_out || M < 0 || M > n->max_batch) return KP_ERR_ARG;
   if (M == 0) return KP_OK;
-  kp_mlp_forward_kernel<<<(M + MLP_TILE - 1) / MLP_TILE, 256, 0, n->stream>>>(
-      weights_of(n), dev_x, M, n->raw, dev_out, nullptr, nullptr, nullptr, nullptr, 0);
+  const MlpWeights w = weights_of(n);
+  tc::FtArgs a{};
+  a.wt = n->wt;
+  a.W3 = w.W3;
+  a.b1 = w.b1;
+  a.b2 = w.b2;
+  a.b3 = w.b3;
+  a.x = dev_x;
+  a.out = dev_out;
+  a.M = M;
+  a.vec = ((uintptr_t)dev_x & 15u) == 0 && ((uintptr_t)dev_out & 7u) == 0;
+  a.err = n->err;
+  a.wait_ns = 2000000000ull;
+  const int tiles = (M + tc::FT_ROWS - 1) / tc::FT_ROWS;
+  tc::kp_mlp_forward_tc_kernel<<<tiles < n->num_sms ? tiles : n->num_sms, tc::FT_THREADS,
+                                 tc::FT_SMEM, n->stream>>>(a);
   MLP_CUDA(cudaGetLastError());
   return KP_OK;
 }
@@ -657,7 +682,7 @@ kp_status kp_mlp_train_step(kp_mlp* n, const float* dev_x, const float* dev_t, i
   kp_mlp_adam_kernel<<<(N_PARAMS + 255) / 256, 256, 0, n->stream>>>(n->p, n->g, n->m, n->v,
                                                                     N_PARAMS, lr, b1, b2, 1e-8f,
                                                                     c1, c2, n->wb, n->wf,
-                                                                    n->w2t);
+                                                                    n->w2t, n->wt);
   MLP_CUDA(cudaGetLastError());
   if (host_loss) {
     MLP_CUDA(cudaMemcpyAsync(host_loss, n->loss, 4, cudaMemcpyDeviceToHost, n->stream));
@@ -699,7 +724,7 @@ kp_status kp_mlp_train_epoch(kp_mlp* n, const float* dev_x, const float* dev_t,
                                                                                    n->tg);
     s = forward_backward(n, n->xg, n->tg, B);
     kp_mlp_adam_dev_kernel<<<(N_PARAMS + 255) / 256, 256, 0, n->stream>>>(
-        n->p, n->g, n->m, n->v, N_PARAMS, n->ec, n->wb, n->wf, n->w2t);
+        n->p, n->g, n->m, n->v, N_PARAMS, n->ec, n->wb, n->wf, n->w2t, n->wt);
     kp_mlp_epoch_tail_kernel<<<1, 1, 0, n->stream>>>(n->ec, n->loss);
     cudaGraph_t g = nullptr;
     const cudaError_t e = cudaStreamEndCapture(n->stream, &g);

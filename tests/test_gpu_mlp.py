@@ -61,6 +61,40 @@ def test_forward_matches_oracle(M, n):
     np.testing.assert_allclose(out[:, 4:], ref[:, 4:], atol=2e-2)
 
 
+@pytest.mark.parametrize("n", [1, 127, 128, 129, 152 * 128, 152 * 128 + 1, 3 * 152 * 128 + 77])
+def test_forward_tile_edges(M, n):
+    """The tensor-core inference kernel at the edges of its 128-row tiles and
+    of its one-tile-per-SM grid (one CTA walking several tiles), and through
+    unaligned device pointers, against the same arithmetic in plain torch:
+    BF16 operands, FP32 sums.  A sum in another order can round a hidden
+    value to the neighbouring BF16 number (2^-8 of it): the output moves by
+    one such step times an output weight (at most 0.1 sqrt(6 / 256)) times
+    the hidden value (below 8 here), so 2e-3 bounds a few of them."""
+    import torch
+    mlp, planner = M
+    net = mlp.Mlp(mlp.init_params(3), max_batch=n)
+    x = torch.from_numpy(_data(n, n)[0]).cuda()
+    out = net.forward(x)
+
+    def rnd(v):
+        return v.to(torch.bfloat16).double()
+
+    W1, b1, W2, b2, W3, b3 = [torch.from_numpy(v.copy()).cuda() for v in
+                              mlp.split(mlp.init_params(3))]
+    h = rnd((rnd(x) @ rnd(W1).T + b1.double()).clamp(min=0))
+    h = rnd((h @ rnd(W2).T + b2.double()).clamp(min=0))
+    o = h @ rnd(W3).T + b3.double()
+    ref = torch.cat([torch.tanh(o[:, :4]), o[:, 4:].clamp(-4, 1)], 1)
+    assert float((out.double() - ref).abs().max()) <= 2e-3
+    # 4-byte aligned input and output
+    xb = torch.zeros(n * 32 + 1, device="cuda")
+    ob = torch.zeros(n * 8 + 1, device="cuda")
+    xb[1:] = x.reshape(-1)
+    assert planner.lib().kp_mlp_forward(net._ctx, xb.data_ptr() + 4, n, ob.data_ptr() + 4) == 0
+    torch.cuda.synchronize()
+    assert torch.equal(ob[1:].view(n, 8), out)
+
+
 def test_gradients_match_oracle(M):
     """Every parameter block's gradient against the FP64 oracle's
     backpropagation (relative L2 error, BF16 activations)."""
