@@ -308,7 +308,7 @@ static __device__ __noinline__ void phase_features(const KParams& P, const Team&
     }
     __syncthreads();
     if (P.mix_thr)
-      mlp_tile_forward<MLP_LOOP_TILE / 16, true>(w, sX, sH, P.net_raw, p0, rows, nullptr, nullptr);
+      mlp_tile_forward<MLP_LOOP_TILE / 16>(w, sX, sH, P.net_raw, p0, rows);
     __syncthreads();
   }
 }

@@ -1,6 +1,7 @@
 // kp_mlp.cuh -- the learned control proposal's network on the tensor cores:
-// BF16 operands, FP32 accumulation (mma.sync m16n8k16), shared by the
-// standalone inference/training kernels and the planner's loop kernel.
+// sizes, fragment helpers and the 32-row tile that the planner's loop kernel
+// evaluates (BF16 operands, FP32 accumulation, mma.sync m16n8k16).  Inference
+// and training of their own run on tcgen05 (kp_mlp_tc.cuh).
 //
 // Network: 32 inputs (24 node features, zero padded) -> 256 ReLU -> 256
 // ReLU -> 8 outputs; heads: mean = tanh(out[0..3]), log_std = clamp(out[4..7],
@@ -14,7 +15,6 @@
 namespace kp {
 
 constexpr int MLP_IN = 32, MLP_H = 256, MLP_OUT = 8, MLP_NQ = 4;
-constexpr int MLP_TILE = 32;           // rows per block tile (standalone kernels)
 constexpr int MLP_LOOP_TILE = 32;      // rows per block tile inside the planner loop
 constexpr int MLP_XS = MLP_IN + 8;     // padded smem row (bf16) of the input tile
 constexpr int MLP_HS = MLP_H + 8;      // padded smem row (bf16) of a hidden tile
@@ -22,7 +22,7 @@ constexpr float MLP_LOGSTD_MIN = -4.0f, MLP_LOGSTD_MAX = 1.0f;
 // shared memory of one loop tile: input rows + hidden rows (bf16)
 constexpr int MLP_LOOP_TILE_SMEM = MLP_LOOP_TILE * MLP_XS * 2 + MLP_LOOP_TILE * MLP_HS * 2;
 
-struct MlpWeights {
+struct MlpWeights {         // weights in fragment order
   const __nv_bfloat16* W1;  // [256][32]
   const float* b1;
   const __nv_bfloat16* W2;  // [256][256]
@@ -101,9 +101,9 @@ __device__ __forceinline__ void frag_b4_ordered(const __nv_bfloat16* Wf, int K, 
 
 // One dense ReLU layer on a tile of 16*MI rows: out = relu(in * W^T + b),
 // every warp producing 32 output columns.  'in' is a bf16 smem tile (row
-// stride ld_in, K columns).  Results stay in registers (acc) until the
+// stride ld_in, K columns), W in fragment order.  Results stay in registers (acc) until the
 // caller stores them.
-template <int K, int MI, bool ORDERED = false>
+template <int K, int MI>
 __device__ __forceinline__ void layer_relu(const __nv_bfloat16* in, int ld_in,
                                            const __nv_bfloat16* W, const float* bias,
                                            float acc[MI][4][4]) {
@@ -122,12 +122,7 @@ __device__ __forceinline__ void layer_relu(const __nv_bfloat16* in, int ld_in,
 #pragma unroll 4
   for (int k0 = 0; k0 < K; k0 += 16) {
     uint32_t a[MI][4], b[4][2];
-    if (ORDERED) {
-      frag_b4_ordered(W, K, k0 >> 4, b);
-    } else {
-#pragma unroll
-      for (int ni = 0; ni < 4; ++ni) frag_b(W, K, n_base + ni * 8, k0, b[ni]);
-    }
+    frag_b4_ordered(W, K, k0 >> 4, b);
 #pragma unroll
     for (int mi = 0; mi < MI; ++mi) frag_a(in, ld_in, mi * 16, k0, a[mi]);
 #pragma unroll
@@ -143,11 +138,9 @@ __device__ __forceinline__ void layer_relu(const __nv_bfloat16* in, int ld_in,
       for (int q = 0; q < 4; ++q) acc[mi][ni][q] = fmaxf(acc[mi][ni][q], 0.0f);
 }
 
-// Writes a layer's register results as bf16 into a smem tile (and, when
-// given, into global rows row0.. of a [rows][256] bf16 array).
+// Writes a layer's register results as bf16 into a smem tile.
 template <int MI>
-__device__ __forceinline__ void store_hidden(const float acc[MI][4][4], __nv_bfloat16* s,
-                                             __nv_bfloat16* g, int row0, int rows_valid) {
+__device__ __forceinline__ void store_hidden(const float acc[MI][4][4], __nv_bfloat16* s) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gi = lane >> 2, t = lane & 3;
 #pragma unroll
   for (int mi = 0; mi < MI; ++mi)
@@ -159,14 +152,12 @@ __device__ __forceinline__ void store_hidden(const float acc[MI][4][4], __nv_bfl
         const int c = warp * 32 + ni * 8 + 2 * t;
         const uint32_t v = pack_bf16(acc[mi][ni][2 * h], acc[mi][ni][2 * h + 1]);
         *reinterpret_cast<uint32_t*>(s + r * MLP_HS + c) = v;
-        if (g && r < rows_valid) *reinterpret_cast<uint32_t*>(g + (size_t)(row0 + r) * MLP_H + c) = v;
       }
 }
 
 // Forward pass of one tile of 16*MI rows.  sX holds the bf16 inputs (row
 // stride MLP_XS), sH is scratch (16*MI x MLP_HS bf16).  Writes the 8 raw
-// outputs of valid rows to raw[(row0 + r) * 8 ..] and, when g_h1/g_h2 are
-// given, the hidden activations (training).  Every thread of the block
+// outputs of valid rows to raw[(row0 + r) * 8 ..].  Every thread of the block
 // (256) must call it.
 //
 // The output layer (K = 256, 8 columns) is split over K: warp w multiplies
@@ -174,28 +165,24 @@ __device__ __forceinline__ void store_hidden(const float acc[MI][4][4], __nv_bfl
 // shared memory (over sH, once every warp has read h2); the partials are
 // then added in warp order.  Two dependent products per warp instead of
 // sixteen keep the tile's latency short.
-template <int MI, bool ORDERED = false>
+template <int MI>
 __device__ __forceinline__ void mlp_tile_forward(const MlpWeights& w, const __nv_bfloat16* sX,
                                                  __nv_bfloat16* sH, float* raw, int row0,
-                                                 int rows_valid, __nv_bfloat16* g_h1,
-                                                 __nv_bfloat16* g_h2) {
+                                                 int rows_valid) {
   float acc[MI][4][4];
-  layer_relu<MLP_IN, MI, ORDERED>(sX, MLP_XS, w.W1, w.b1, acc);
-  store_hidden<MI>(acc, sH, g_h1, row0, rows_valid);
+  layer_relu<MLP_IN, MI>(sX, MLP_XS, w.W1, w.b1, acc);
+  store_hidden<MI>(acc, sH);
   __syncthreads();
-  layer_relu<MLP_H, MI, ORDERED>(sH, MLP_HS, w.W2, w.b2, acc);
+  layer_relu<MLP_H, MI>(sH, MLP_HS, w.W2, w.b2, acc);
   __syncthreads();  // every warp has read h1
-  store_hidden<MI>(acc, sH, g_h2, row0, rows_valid);
+  store_hidden<MI>(acc, sH);
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gi = lane >> 2, t = lane & 3;
   float d[MI][4];
   uint32_t b[2][2];
-  if (ORDERED) {
+  {
     const uint4 u = __ldg(reinterpret_cast<const uint4*>(w.W3) + warp * 32 + lane);
     b[0][0] = u.x; b[0][1] = u.y; b[1][0] = u.z; b[1][1] = u.w;
-  } else {
-    frag_b(w.W3, MLP_H, 0, warp * 32, b[0]);
-    frag_b(w.W3, MLP_H, 0, warp * 32 + 16, b[1]);
   }
 #pragma unroll
   for (int mi = 0; mi < MI; ++mi) {

@@ -1,6 +1,6 @@
-// kp_mlp_tc.cuh -- the network's inference on the fifth-generation tensor
-// cores: all three layers of a 128-row tile in one kernel, weights and hidden
-// activations on chip.
+// kp_mlp_tc.cuh -- the network's inference and training on the fifth-generation
+// tensor cores: all layers of a 128-row tile in one kernel, forward and
+// backward, weights and hidden activations on chip.
 #pragma once
 
 #include "kp_mlp.cuh"
@@ -109,6 +109,17 @@ __device__ __forceinline__ void tmem_wait_ld(uint32_t* r) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int i = 0; i < N; ++i) asm volatile("" : "+r"(r[i]));
+}
+
+// 8 consecutive 32-bit columns of the calling thread's TMEM lane (waited for).
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7])
+      : "r"(taddr)
+      : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
 __device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) {
@@ -433,6 +444,496 @@ __global__ void __launch_bounds__(FT_THREADS, 1) kp_mlp_forward_tc_kernel(FtArgs
     tmem_dealloc(tmem, 512);
   }
   if (tid == 0 && s_fail) atomicExch(a.err, 200 + s_fail);
+}
+
+// ---------------------------------------------------------------------------
+// one training step's forward and backward pass
+// ---------------------------------------------------------------------------
+
+// Control of a device-driven epoch.
+struct EpochCtl {
+  const float* x;        // [rows][32] features
+  const float* t;        // [rows][4] targets
+  const int32_t* perm;   // row order of the epoch
+  int batch;             // index of the mini-batch in work
+  int step;              // Adam steps taken, the one in work included
+  float lr;
+  float loss_sum;        // sum of the mini-batch losses of the epoch
+};
+
+constexpr int ST_THREADS = 256;
+// shared memory: h1 (first the inputs and W1), h2 then dh2 (first two chunks
+// of W2), two chunks of W2 then dh1, the transposed inputs with a block of
+// ones, the transposed output gradient, W3 twice, the output gradient split
+// into three BF16 parts
+constexpr uint32_t ST_H1 = 0, ST_G = 65536, ST_W = 131072, ST_XT = 196608, ST_DT = ST_XT + 2 * 6144,
+                   ST_W3 = ST_DT + 2 * 2048, ST_DA = ST_W3 + 4 * 2048, ST_END = ST_DA + 8192;
+constexpr int ST_SMEM = (int)ST_END + 1024;
+constexpr uint32_t ST_X = ST_H1, ST_W1 = ST_H1 + 16384;  // before h1 is written
+constexpr uint32_t ST_B1 = ST_DA, ST_B2 = ST_DA + 1024;   // before the split gradient is
+
+struct StepArgs {
+  const __nv_bfloat16* wt;  // W2, W1 in operand order (wt_index_*)
+  const __nv_bfloat16* W3;  // row-major [8][256]
+  const float *b1, *b2, *b3;
+  const float *x, *t;       // [M][32], [M][4] (epoch null)
+  EpochCtl* epoch;          // rows perm[batch M ..] of epoch->x, epoch->t
+  int M;
+  float *g_W1, *g_b1, *g_W2, *g_b2, *g_W3, *g_b3, *loss;  // added to
+  int* err;
+  unsigned long long wait_ns;
+};
+
+// kind::f16 descriptor with the operands' majors (1: M or N contiguous).
+__host__ __device__ constexpr uint32_t idesc_majors(int M, int N, int a_mn, int b_mn) {
+  return idesc_bf16_f32(M, N) | ((uint32_t)a_mn << 15) | ((uint32_t)b_mn << 16);
+}
+
+// Descriptor of a 128-byte-swizzled operand whose M or N index is contiguous:
+// 64 of them in a 128-byte row, rows along K; 8-row groups 1024 bytes apart,
+// the next 64 of M or N 'next' bytes on.
+__device__ __forceinline__ uint64_t sdesc_mn128(uint32_t addr, uint32_t next) {
+  uint64_t d = (uint64_t)((addr >> 4) & 0x3FFFu);
+  d |= (uint64_t)(next >> 4) << 16;
+  d |= (uint64_t)(1024 >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)2 << 61;
+  return d;
+}
+
+__device__ __forceinline__ uint4 lds128(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "r"(addr)
+               : "memory");
+  return v;
+}
+
+__device__ __forceinline__ void sts16(uint32_t addr, __nv_bfloat16 v) {
+  asm volatile("st.shared.b16 [%0], %1;" ::"r"(addr), "h"(*reinterpret_cast<const uint16_t*>(&v))
+               : "memory");
+}
+
+__device__ __forceinline__ void red_add4(float* p, const uint32_t* r) {
+  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(__uint_as_float(r[0])),
+               "f"(__uint_as_float(r[1])), "f"(__uint_as_float(r[2])), "f"(__uint_as_float(r[3]))
+               : "memory");
+}
+
+// The two BF16 halves of v kept where those of h are not zero (h is the
+// output of a ReLU: positive or zero).
+__device__ __forceinline__ uint32_t keep_active(uint32_t v, uint32_t h) {
+  const uint32_t lo = (h & 0x00007fffu) ? 0x0000ffffu : 0u, hi = (h & 0x7fff0000u) ? 0xffff0000u : 0u;
+  return v & (lo | hi);
+}
+
+// Forward, loss and backward of one 128-row tile per CTA, every product on
+// the tensor cores, nothing of the tile in global memory but its inputs and
+// its gradient contributions.  The phases of a tile (X the inputs, D the
+// gradient of the eight outputs; thread = row 32 (w % 4) + lane and columns
+// 128 (w / 4) ..):
+//   h1 = relu(X W1' + b1), h2 = relu(h1 W2' + b2), raw = h2 W3' + b3; the
+//   loss and D (FP32);
+//   dW3 += D' h2;  dh2 = (D W3) where h2 > 0, D entering as three BF16 parts
+//   whose sum is the FP32 value (their products with W3 are exact);
+//   dh1 = (dh2 W2) where h1 > 0;  dW2 += dh2' h1;  dW1 += dh1' X; db2 and db1
+//   as products with a block of ones.
+// The transposed operands are the same shared-memory tiles read with their
+// other index contiguous, so nothing is transposed.  W2 is brought in twice,
+// half of it only once (its first half survives the forward pass).  Rows past
+// M have inputs 0, activations 0 and D 0.
+//
+// A mini-batch of 4096 is 32 tiles, so the pass is one tile's chain of twelve
+// products and epilogues, and the 32 x 75 K additions to the gradient; what it
+// replaces was 13 launches (row-major and transposed activations in global
+// memory, split-K products), 83 us a step with the optimiser's: now 33 us
+// (GB300, epochs of 16 steps of 4,096 rows: 1,336 -> 565 us with the parameter
+// read-back).
+__global__ void __launch_bounds__(ST_THREADS, 1) kp_mlp_step_kernel(StepArgs a) {
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ __align__(8) uint64_t b_w1, b_w2[4], b_mma, b_c[2], b_t0, b_r[2];
+  __shared__ uint32_t tmem_slot;
+  __shared__ int s_fail;
+  const uint32_t base = (saddr(smem_raw) + 1023u) & ~1023u;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int q = warp & 3, half = warp >> 2;
+  const int row0 = blockIdx.x * 128;
+  if (tid == 0) {
+    mbar_init(saddr(&b_w1), 1);
+    for (int c = 0; c < 4; ++c) mbar_init(saddr(&b_w2[c]), 1);
+    mbar_init(saddr(&b_mma), 1);
+    for (int c = 0; c < 2; ++c) {
+      mbar_init(saddr(&b_c[c]), 1);
+      mbar_init(saddr(&b_r[c]), 1);
+    }
+    mbar_init(saddr(&b_t0), 1);
+    s_fail = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    fence_async();
+    mbar_expect_tx(saddr(&b_w1), MLP_H * 64);
+    bulk_load(base + ST_W1, a.wt + WT_W1, MLP_H * 64, saddr(&b_w1));
+    for (int c = 0; c < 4; ++c) {
+      mbar_expect_tx(saddr(&b_w2[c]), MLP_H * 128);
+      bulk_load(base + (c < 2 ? ST_W + c * 32768 : ST_G + (c - 2) * 32768), a.wt + c * WT_CHUNK,
+                MLP_H * 128, saddr(&b_w2[c]));
+    }
+  }
+  if (warp == 0) {
+    __syncwarp();
+    tmem_alloc(saddr(&tmem_slot), 512);
+  }
+  // inputs: thread = row tid / 2 and 16 columns
+  const float *xs = a.x, *ts = a.t;
+  auto source_row = [&](int r) {  // row of x and t behind row r of the batch
+    return a.epoch ? (size_t)a.epoch->perm[(size_t)a.epoch->batch * a.M + r] : (size_t)r;
+  };
+  if (a.epoch) {
+    xs = a.epoch->x;
+    ts = a.epoch->t;
+  }
+  {
+    const int r = tid >> 1, part = tid & 1;
+    float v[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = 0.0f;
+    if (row0 + r < a.M) {
+      const float* src = xs + source_row(row0 + r) * MLP_IN + 16 * part;
+      if (((uintptr_t)src & 15u) == 0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float4 f = __ldg(reinterpret_cast<const float4*>(src) + i);
+          v[4 * i] = f.x; v[4 * i + 1] = f.y; v[4 * i + 2] = f.z; v[4 * i + 3] = f.w;
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = __ldg(src + i);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int c = 2 * part + i;
+      sts128(base + ST_X + (uint32_t)(r * 64 + ((c ^ ((r >> 1) & 3)) << 4)),
+             pack_bf16(v[8 * i], v[8 * i + 1]), pack_bf16(v[8 * i + 2], v[8 * i + 3]),
+             pack_bf16(v[8 * i + 4], v[8 * i + 5]), pack_bf16(v[8 * i + 6], v[8 * i + 7]));
+    }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const int n = 16 * part + i;
+      sts16(base + ST_XT + (uint32_t)((r >> 6) * 6144 + n * 128 + ((((r & 63) >> 3) ^ (n & 7)) << 4) +
+                                      (r & 7) * 2),
+            __float2bfloat16_rn(v[i]));
+    }
+  }
+  {
+    // ones (rows 32..47 of the transposed inputs), zeros (rows 8..15 of the
+    // transposed output gradient), W3 twice
+    const uint32_t one2 = 0x3F803F80u;
+    sts128(base + ST_XT + (uint32_t)((tid >> 7) * 6144 + 4096 + (tid & 127) * 16), one2, one2, one2, one2);
+    if (tid < 128)
+      sts128(base + ST_DT + (uint32_t)((tid >> 6) * 2048 + 1024 + (tid & 63) * 16), 0, 0, 0, 0);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int e = tid + 256 * i, c = e >> 7, copy = (e >> 6) & 1, n = (e >> 3) & 7, j = e & 7;
+      const uint4 w = *reinterpret_cast<const uint4*>(a.W3 + n * MLP_H + 64 * c + 8 * j);
+      sts128(base + ST_W3 + (uint32_t)(c * 2048 + copy * 1024 + n * 128 + ((j ^ n) << 4)), w.x, w.y, w.z,
+             w.w);
+    }
+    asm volatile("st.shared.f32 [%0], %1;" ::"r"(base + ST_B1 + 4 * tid), "f"(a.b1[tid]) : "memory");
+    asm volatile("st.shared.f32 [%0], %1;" ::"r"(base + ST_B2 + 4 * tid), "f"(a.b2[tid]) : "memory");
+  }
+  if (a.epoch && blockIdx.x == 0 && tid == 0) a.epoch->step += 1;  // read by the Adam launch
+  fence_async();
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tmem = tmem_slot;
+  const uint32_t tl = tmem + ((uint32_t)(32 * q) << 16);
+  const int r = 32 * q + lane;
+  const bool live = row0 + r < a.M;
+  // this row's piece 0 of a 128-byte-row tile (piece c at c ^ (r & 7))
+  const uint32_t hoff = (uint32_t)(r * 128 + ((r & 7) << 4));
+  uint32_t ph = 0;
+  auto wait = [&](uint64_t* bar, uint32_t parity, int site) {
+    mbar_wait_or(saddr(bar), parity, a.wait_ns, &s_fail, site);
+  };
+  auto wait_mma = [&](int site) {  // all threads: the products committed last are there
+    __syncwarp();
+    wait(&b_mma, ph, site);
+    ph ^= 1u;
+    __syncwarp();
+    fence_after();
+  };
+  auto publish = [&]() {  // shared-memory operands written, accumulators read
+    fence_async();
+    fence_before();
+    __syncthreads();
+    fence_after();
+  };
+  // bias, ReLU, BF16 of this thread's 128 columns of an accumulator into a tile
+  auto activate = [&](uint32_t acc, uint32_t tile, uint32_t bias) {
+#pragma unroll 1
+    for (int u = 0; u < 4; ++u) {
+      uint32_t v[32];
+      const int c0 = 128 * half + 32 * u;
+      tmem_ld32(acc + (uint32_t)c0, v);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint4 ba = lds128(base + bias + (uint32_t)(4 * (c0 + 8 * j)));
+        const uint4 bb = lds128(base + bias + (uint32_t)(4 * (c0 + 8 * j + 4)));
+        auto two = [](uint32_t x, uint32_t y) {
+          return make_float2(__uint_as_float(x), __uint_as_float(y));
+        };
+        const uint32_t* vv = v + 8 * j;
+        const uint32_t w0 = bias_relu_bf16(vv[0], vv[1], two(ba.x, ba.y)),
+                       w1 = bias_relu_bf16(vv[2], vv[3], two(ba.z, ba.w)),
+                       w2 = bias_relu_bf16(vv[4], vv[5], two(bb.x, bb.y)),
+                       w3 = bias_relu_bf16(vv[6], vv[7], two(bb.z, bb.w));
+        sts128(base + tile + (uint32_t)((c0 >> 6) * 16384) + (hoff ^ (uint32_t)((4 * (u & 1) + j) << 4)),
+               live ? w0 : 0u, live ? w1 : 0u, live ? w2 : 0u, live ? w3 : 0u);
+      }
+    }
+  };
+  // BF16 of this thread's 128 columns of an accumulator where the
+  // activations in tile 'act' are not zero, into 'tile' (which may be 'act')
+  auto mask = [&](uint32_t acc, uint32_t act, uint32_t tile) {
+#pragma unroll 1
+    for (int u = 0; u < 4; ++u) {
+      uint32_t v[32];
+      const int c0 = 128 * half + 32 * u;
+      tmem_ld32(acc + (uint32_t)c0, v);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint32_t off = (uint32_t)((c0 >> 6) * 16384) + (hoff ^ (uint32_t)((4 * (u & 1) + j) << 4));
+        const uint4 h = lds128(base + act + off);
+        const float* f = reinterpret_cast<const float*>(v + 8 * j);
+        sts128(base + tile + off, keep_active(pack_bf16(f[0], f[1]), h.x),
+               keep_active(pack_bf16(f[2], f[3]), h.y), keep_active(pack_bf16(f[4], f[5]), h.z),
+               keep_active(pack_bf16(f[6], f[7]), h.w));
+      }
+    }
+  };
+  // a 128 x 256 accumulator added to rows out0 .. of dW2 (blocks start at
+  // different columns, so that they meet on few addresses)
+  auto add_dw2 = [&](uint32_t acc, int out0) {
+    if (*((volatile int*)&s_fail) != 0) return;
+    float* dst = a.g_W2 + (size_t)(out0 + r) * MLP_H;
+#pragma unroll 1
+    for (int u = 0; u < 4; ++u) {
+      uint32_t v[32];
+      const int c0 = 128 * half + 32 * ((u + (int)blockIdx.x) & 3);
+      tmem_ld32(acc + (uint32_t)c0, v);
+#pragma unroll
+      for (int j = 0; j < 32; j += 4) red_add4(dst + c0 + j, v + j);
+    }
+  };
+  constexpr uint32_t ID_FWD = idesc_majors(128, 256, 0, 0), ID_RAW = idesc_majors(128, 16, 0, 0),
+                     ID_DW3 = idesc_majors(128, 16, 1, 0), ID_DH2 = idesc_majors(128, 256, 0, 1),
+                     ID_DH1 = idesc_majors(128, 64, 0, 1), ID_DW2 = idesc_majors(128, 256, 1, 1),
+                     ID_DW1 = idesc_majors(128, 48, 1, 0);
+  const uint32_t A0 = tmem, B0 = tmem + 256;  // the two halves of tensor memory
+
+  // ---- forward
+  if (tid == 0) {
+    wait(&b_w1, 0, 30);
+    fence_after();
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+      mma_bf16(A0, sdesc_sw64(base + ST_X + 32 * k), sdesc_sw64(base + ST_W1 + 32 * k), ID_FWD,
+               k != 0 ? 1u : 0u);
+    mma_commit(saddr(&b_mma));
+  }
+  wait_mma(31);
+  activate(tl, ST_H1, ST_B1);
+  publish();
+  if (tid == 0) {
+    for (int c = 0; c < 4; ++c) {
+      wait(&b_w2[c], 0, 32);
+      const uint32_t w = base + (c < 2 ? ST_W + c * 32768 : ST_G + (c - 2) * 32768);
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        mma_bf16(B0, sdesc_sw128(base + ST_H1 + c * 16384 + 32 * k), sdesc_sw128(w + 32 * k), ID_FWD,
+                 (c | k) != 0 ? 1u : 0u);
+    }
+    mma_commit(saddr(&b_mma));
+  }
+  wait_mma(33);
+  activate(tl + 256, ST_G, ST_B2);
+  publish();
+  if (tid == 0) {
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        mma_bf16(A0, sdesc_sw128(base + ST_G + c * 16384 + 32 * k),
+                 sdesc_sw128(base + ST_W3 + c * 2048 + 32 * k), ID_RAW, (c | k) != 0 ? 1u : 0u);
+    mma_commit(saddr(&b_mma));
+  }
+  float tv[MLP_NQ] = {0.0f, 0.0f, 0.0f, 0.0f};
+  if (half == 0 && live) {
+    const float* src = ts + source_row(row0 + r) * MLP_NQ;
+#pragma unroll
+    for (int i = 0; i < MLP_NQ; ++i) tv[i] = __ldg(src + i);
+  }
+  wait_mma(34);
+
+  // ---- loss and the outputs' gradient (one thread a row)
+  if (half == 0) {
+    uint32_t raw[8];
+    tmem_ld8(tl, raw);
+    const float inv_m = 1.0f / (float)a.M;
+    float l = 0.0f, d[MLP_OUT];
+#pragma unroll
+    for (int i = 0; i < MLP_NQ; ++i) {
+      const float mu = tanhf(__uint_as_float(raw[i]) + a.b3[i]);
+      const float lr = __uint_as_float(raw[MLP_NQ + i]) + a.b3[MLP_NQ + i];
+      const bool clamped = lr < MLP_LOGSTD_MIN || lr > MLP_LOGSTD_MAX;
+      const float ls = fminf(fmaxf(lr, MLP_LOGSTD_MIN), MLP_LOGSTD_MAX);
+      const float is = expf(-ls);
+      const float z = (tv[i] - mu) * is;
+      l += ls + 0.5f * z * z;
+      d[i] = live ? -z * is * (1.0f - mu * mu) * inv_m : 0.0f;
+      d[MLP_NQ + i] = live && !clamped ? (1.0f - z * z) * inv_m : 0.0f;
+    }
+    if (!live) l = 0.0f;
+    // three BF16 parts of each value: rounding, then what is left, twice
+    uint32_t part[3][4];
+    float rest[MLP_OUT];
+#pragma unroll
+    for (int n = 0; n < MLP_OUT; ++n) {
+      sts16(base + ST_DT + (uint32_t)((r >> 6) * 2048 + n * 128 + ((((r & 63) >> 3) ^ n) << 4) + (r & 7) * 2),
+            __float2bfloat16_rn(d[n]));
+      rest[n] = d[n];
+    }
+#pragma unroll
+    for (int p = 0; p < 3; ++p)
+#pragma unroll
+      for (int n = 0; n < MLP_OUT; n += 2) {
+        const __nv_bfloat162 b = __floats2bfloat162_rn(rest[n], rest[n + 1]);
+        part[p][n >> 1] = *reinterpret_cast<const uint32_t*>(&b);
+        rest[n] -= __bfloat162float(b.x);
+        rest[n + 1] -= __bfloat162float(b.y);
+      }
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+      sts128(base + ST_DA + (uint32_t)(r * 64 + ((p ^ ((r >> 1) & 3)) << 4)), p < 3 ? part[p < 3 ? p : 0][0] : 0u,
+             p < 3 ? part[p < 3 ? p : 0][1] : 0u, p < 3 ? part[p < 3 ? p : 0][2] : 0u,
+             p < 3 ? part[p < 3 ? p : 0][3] : 0u);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      l += __shfl_xor_sync(0xffffffffu, l, o);
+#pragma unroll
+      for (int n = 0; n < MLP_OUT; ++n) d[n] += __shfl_xor_sync(0xffffffffu, d[n], o);
+    }
+    if (lane == 0 && *((volatile int*)&s_fail) == 0) {
+      atomicAdd(a.loss, l / (float)a.M);
+#pragma unroll
+      for (int n = 0; n < MLP_OUT; ++n) atomicAdd(a.g_b3 + n, d[n]);
+    }
+  }
+  publish();
+
+  // ---- backward
+  if (tid == 0) {
+#pragma unroll
+    for (int m = 0; m < 2; ++m)
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        mma_bf16(A0 + 16 + 16 * m, sdesc_mn128(base + ST_G + m * 32768 + k * 2048, 16384),
+                 sdesc_sw128(base + ST_DT + (k >> 2) * 2048 + (k & 3) * 32), ID_DW3, k != 0 ? 1u : 0u);
+#pragma unroll
+    for (int k = 0; k < 2; ++k)  // both K groups of W3's tile hold W3: parts 0 and 1, then 2 and zeros
+      mma_bf16(B0, sdesc_sw64(base + ST_DA + 32 * k), sdesc_mn128(base + ST_W3, 2048), ID_DH2,
+               k != 0 ? 1u : 0u);
+    mma_commit(saddr(&b_mma));
+  }
+  wait_mma(35);
+  mask(tl + 256, ST_G, ST_G);
+  if (*((volatile int*)&s_fail) == 0) {
+    uint32_t v[8];
+    tmem_ld8(tl + 16 + 16 * half, v);
+#pragma unroll
+    for (int n = 0; n < MLP_OUT; ++n)
+      atomicAdd(a.g_W3 + n * MLP_H + 128 * half + r, __uint_as_float(v[n]));
+  }
+  publish();
+  if (tid == 0) {
+    auto dh1_chunk = [&](int c) {
+#pragma unroll
+      for (int k = 0; k < 16; ++k)
+        mma_bf16(A0 + 64 * c, sdesc_sw128(base + ST_G + (k >> 2) * 16384 + (k & 3) * 32),
+                 sdesc_mn128(base + ST_W + (c & 1) * 32768 + k * 2048, 0), ID_DH1, k != 0 ? 1u : 0u);
+    };
+    for (int c = 0; c < 2; ++c) {
+      dh1_chunk(c);
+      mma_commit(saddr(&b_c[c]));
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      mma_bf16(B0, sdesc_mn128(base + ST_G + k * 2048, 16384), sdesc_mn128(base + ST_H1 + k * 2048, 16384),
+               ID_DW2, k != 0 ? 1u : 0u);
+    mma_commit(saddr(&b_t0));
+    for (int c = 0; c < 2; ++c) {
+      wait(&b_c[c], 0, 36);
+      mbar_expect_tx(saddr(&b_r[c]), MLP_H * 128);
+      bulk_load(base + ST_W + c * 32768, a.wt + (2 + c) * WT_CHUNK, MLP_H * 128, saddr(&b_r[c]));
+    }
+    for (int c = 0; c < 2; ++c) {
+      wait(&b_r[c], 0, 37);
+      dh1_chunk(2 + c);
+    }
+    mma_commit(saddr(&b_mma));
+  }
+  __syncwarp();
+  wait(&b_t0, 0, 38);
+  __syncwarp();
+  fence_after();
+  add_dw2(tl + 256, 0);
+  wait_mma(39);
+  mask(tl, ST_H1, ST_W);
+  publish();
+  if (tid == 0) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      mma_bf16(A0, sdesc_mn128(base + ST_G + 32768 + k * 2048, 16384),
+               sdesc_mn128(base + ST_H1 + k * 2048, 16384), ID_DW2, k != 0 ? 1u : 0u);
+#pragma unroll
+    for (int m = 0; m < 2; ++m)
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const uint32_t xt = base + ST_XT + (k >> 2) * 6144 + (k & 3) * 32;
+        mma_bf16(B0 + 48 * m, sdesc_mn128(base + ST_W + m * 32768 + k * 2048, 16384), sdesc_sw128(xt), ID_DW1,
+                 k != 0 ? 1u : 0u);
+        mma_bf16(B0 + 96 + 16 * m, sdesc_mn128(base + ST_G + m * 32768 + k * 2048, 16384),
+                 sdesc_sw128(xt + 4096), ID_DW3, k != 0 ? 1u : 0u);
+      }
+    mma_commit(saddr(&b_mma));
+  }
+  wait_mma(40);
+  if (*((volatile int*)&s_fail) == 0) {
+    const int o = 128 * half + r;
+    uint32_t v[32], s[8];
+    tmem_ld32(tl + 256 + 48 * half, v);
+#pragma unroll
+    for (int j = 0; j < 32; j += 4) red_add4(a.g_W1 + (size_t)o * MLP_IN + j, v + j);
+    tmem_ld8(tl + 256 + 48 * half + 32, s);
+    atomicAdd(a.g_b1 + o, __uint_as_float(s[0]));
+    tmem_ld8(tl + 256 + 96 + 16 * half, s);
+    atomicAdd(a.g_b2 + o, __uint_as_float(s[0]));
+  }
+  add_dw2(tl, 128);
+  fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    fence_after();
+    tmem_dealloc(tmem, 512);
+  }
+  if (tid == 0 && s_fail) {
+    // a wait gave up: copies may be in flight, wait for them once more
+    mbar_wait(saddr(&b_w1), 0, a.wait_ns);
+    for (int c = 0; c < 4; ++c) mbar_wait(saddr(&b_w2[c]), 0, a.wait_ns);
+    for (int c = 0; c < 2; ++c) mbar_wait(saddr(&b_r[c]), 0, a.wait_ns);
+    atomicExch(a.err, 100 + s_fail);
+  }
 }
 
 }  // namespace tc

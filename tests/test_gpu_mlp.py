@@ -95,6 +95,44 @@ def test_forward_tile_edges(M, n):
     assert torch.equal(ob[1:].view(n, 8), out)
 
 
+@pytest.mark.parametrize("n", [1, 17, 127, 128, 129, 1000, 152 * 128 + 5])
+def test_gradients_tile_edges(M, n):
+    """The one-kernel forward and backward pass at the edges of its 128-row
+    tiles, against the same arithmetic in plain torch: BF16 operands and
+    activations, FP32 (here FP64) sums, the FP32 output gradient in the second
+    layer's gradient.  FP32 sums give 1e-6; where a sum in another order rounds
+    an activation to the neighbouring BF16 number (2^-8 of it, one of at least
+    256 in its row), a block moves by at most 2^-8 / sqrt(256) of itself per
+    row touched: 2.5e-4, and four of those bound the few that occur."""
+    import torch
+    mlp, _ = M
+    p = mlp.init_params(5)
+    net = mlp.Mlp(p, max_batch=n)
+    x, t = [torch.from_numpy(v).cuda() for v in _data(n, n)]
+    g, loss = net.gradients(x, t)
+
+    def rnd(v):
+        return v.to(torch.float32).to(torch.bfloat16).double()
+
+    W1, b1, W2, b2, W3, b3 = [torch.from_numpy(v.copy()).cuda() for v in mlp.split(p)]
+    W1, W2, W3, xb = rnd(W1), rnd(W2), rnd(W3), rnd(x)
+    h1 = rnd((xb @ W1.T + b1.double()).clamp(min=0))
+    h2 = rnd((h1 @ W2.T + b2.double()).clamp(min=0))
+    o = h2 @ W3.T + b3.double()
+    mu, raw = torch.tanh(o[:, :4]), o[:, 4:]
+    ls = raw.clamp(-4, 1)
+    z = (t.double() - mu) * torch.exp(-ls)
+    inside = ((raw >= -4) & (raw <= 1)).double()
+    d = torch.cat([-z * torch.exp(-ls) * (1 - mu * mu), (1 - z * z) * inside], 1) / n
+    d2 = rnd((d @ W3) * (h2 > 0))
+    d1 = rnd((d2 @ W2) * (h1 > 0))
+    ref = (d1.T @ xb, d1.sum(0), d2.T @ h1, d2.sum(0), rnd(d).T @ h2, d.sum(0))
+    assert abs(loss - float((ls + 0.5 * z * z).sum() / n)) <= 1e-5 * max(1.0, abs(loss))
+    for got, want in zip(mlp.split(g), ref):
+        want = want.cpu().numpy()
+        assert np.linalg.norm(got - want) <= 1e-3 * np.linalg.norm(want)
+
+
 def test_gradients_match_oracle(M):
     """Every parameter block's gradient against the FP64 oracle's
     backpropagation (relative L2 error, BF16 activations)."""
