@@ -46,32 +46,6 @@ KP_DECLARE_SYS(quad)
 // generic kernels
 // ---------------------------------------------------------------------------
 
-// Root-to-goal chain into P.traj rows (state 12, ctrl 4, steps), root first,
-// as a launch of its own after the no-allocation entry's loop launch (the
-// queries of a context do this inside their loop launch).
-__global__ void kp_extract_kernel(KParams P) {
-  if (blockIdx.x != 0 || threadIdx.x != 0) return;
-  KCtl* ctl = P.ctl;
-  const int g = ctl->goal_node;
-  if (g == KP_NO_GOAL || g < 0 || g >= P.t_e) {
-    ctl->n_edges = -1;
-    return;
-  }
-  int len = 0;
-  for (int v = g; v > 0 && len <= P.t_e; v = P.parent[v]) ++len;
-  ctl->n_edges = len;
-  if (len > KP_TRAJ_ROWS) return;
-  const int D = P.sys == KP_SYS_QUAD ? 12 : 6;
-  const int N = P.sys == KP_SYS_QUAD ? 4 : 3;
-  int row = len - 1;
-  for (int v = g; v > 0 && row >= 0; v = P.parent[v], --row) {
-    float* out = P.traj + (size_t)row * 17;
-    for (int i = 0; i < 12; ++i) out[i] = i < D ? P.st[(size_t)i * P.t_e + v] : 0.0f;
-    for (int i = 0; i < 4; ++i) out[12 + i] = i < N ? P.ctrl[(size_t)i * P.t_e + v] : 0.0f;
-    out[16] = (float)P.steps[v];
-  }
-}
-
 // Import fix-up: Cov from the visited flags, R_avail cleared.
 __global__ void kp_import_regions_kernel(KParams P) {
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < P.R; r += gridDim.x * blockDim.x) {
@@ -1586,86 +1560,151 @@ std::mutex g_static_mu;
 void* g_static_base[kStaticMaxDevices];  // device address of the scratch, per device
 
 // Raw {lo, hi} box rows -> the obstacle blob the loop kernel reads: padded
-// boxes, then a uniform broad-phase grid of g[0] g[1] g[2] cells (cell
-// starts, box ids of each cell in box order) and each cell's clearance, the
-// same structure the host builder makes for a context, built here by one
-// block of the device (the no-allocation path has no host staging).  A box
-// is listed in every cell of its range on each axis, the cell of a
-// coordinate v being the FP32 (v - lo) * scale clamped to [0, g - 1], as in
-// the hull test.  The clearance of a cell: the smallest over boxes of the
-// largest per-axis gap between the cell and the box in cell units, at most
-// KP_BP_CLEAR_CAP cells, less KP_BP_CLEAR_MARGIN, in sixteenths, rounded
-// down.  Shared memory: C + 1 ints of cell counts, then offsets.
-__global__ void __launch_bounds__(1024) kp_static_blob_kernel(
-    unsigned char* blob, const float* raw, int n, int pad, int gx, int gy, int gz, float sx,
-    float sy, float sz, float lx, float ly, float lz, int start_off, int ids_off, int clear_off) {
-  extern __shared__ int kcount[];
-  float* dst = reinterpret_cast<float*>(blob);
-  uint16_t* start = reinterpret_cast<uint16_t*>(blob + start_off);
-  uint16_t* ids = reinterpret_cast<uint16_t*>(blob + ids_off);
-  const int C = gx * gy * gz;
-  const int g3[3] = {gx, gy, gz};
-  const float s3[3] = {sx, sy, sz}, l3[3] = {lx, ly, lz};
-  for (int b = threadIdx.x; b < pad; b += blockDim.x) {
-    float* o = dst + (size_t)b * 8;
-    if (b < n) {
-      const float* in = raw + (size_t)b * 6;
-      o[0] = in[0] + 0.0f; o[1] = in[1] + 0.0f; o[2] = in[2] + 0.0f; o[3] = 0.0f;
-      o[4] = in[3] + 0.0f; o[5] = in[4] + 0.0f; o[6] = in[5] + 0.0f; o[7] = 0.0f;
-    } else {
-      o[0] = o[1] = o[2] = INFINITY;
-      o[4] = o[5] = o[6] = -INFINITY;
-      o[3] = o[7] = 0.0f;
-    }
+// boxes, then a uniform broad-phase grid of g^3 cells (cell starts, box ids of
+// each cell in box order) and each cell's clearance, the same structure the
+// host builder makes for a context, built here on the device (the
+// no-allocation path has no host staging).  A box is listed in every cell of
+// its range on each axis, the cell of a coordinate v being the FP32 (v - lo) *
+// scale clamped to [0, g - 1], as in the hull test.  The clearance of a cell:
+// the smallest over boxes of the largest per-axis gap between the cell and the
+// box in cell units, at most KP_BP_CLEAR_CAP cells, less KP_BP_CLEAR_MARGIN,
+// in sixteenths, rounded down.  The gaps are FP32: gaps up to the cap come
+// from coordinates of at most 16 + 4 cells, so they are off by less than 20 x
+// 3 roundings of 2^-24 (4e-6 cells), far below the margin of 1e-3.
+//
+// Eight lanes share a cell, each with an eighth of the boxes in order; 32
+// cells a block, so that 4096 cells fill 128 blocks.  Two launches: counts
+// and clearances, then the lists (every block adds up the counts before its
+// cells).  One block that did it all, with FP64 gaps (two a clock and SM) and
+// a one-thread prefix over the cells, took 550 us of a 940 us call with 16
+// boxes.
+struct StaticGrid {
+  unsigned char* blob;
+  const float* raw;  // [n][6]
+  uint32_t* count;   // [g^3] boxes of a cell
+  int n, pad, g;
+  float scale[3], lo[3];
+  int start_off, ids_off, clear_off;
+};
+
+constexpr int kCellLanes = 8, kCellsPerBlock = 256 / kCellLanes;
+
+// Box b as the blob holds it (no negative zeros).
+__device__ __forceinline__ void static_box(const StaticGrid& G, int b, float* lo, float* hi) {
+  const float* in = G.raw + (size_t)b * 6;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    lo[a] = in[a] + 0.0f;
+    hi[a] = in[3 + a] + 0.0f;
   }
-  __syncthreads();
-  auto in_range = [&](int b, const int* cc) {
-    for (int a = 0; a < 3; ++a) {
-      float f;
-      const float last = (float)(g3[a] - 1);
-      const int c0 = bp_cell_of(__fmul_rn(__fsub_rn(dst[b * 8 + a], l3[a]), s3[a]), last, &f);
-      const int c1 = bp_cell_of(__fmul_rn(__fsub_rn(dst[b * 8 + 4 + a], l3[a]), s3[a]), last, &f);
-      if (cc[a] < c0 || cc[a] > c1) return false;
+}
+
+// Whether the box is listed in cell cc; its gap to the cell in *gap.
+__device__ __forceinline__ bool static_listed(const StaticGrid& G, const float* lo, const float* hi,
+                                              const int* cc, float* gap) {
+  const float last = (float)(G.g - 1);
+  bool in = true;
+  float m = 0.0f;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const float tl = __fmul_rn(__fsub_rn(lo[a], G.lo[a]), G.scale[a]);
+    const float th = __fmul_rn(__fsub_rn(hi[a], G.lo[a]), G.scale[a]);
+    float f;
+    in = in && cc[a] >= bp_cell_of(tl, last, &f) && cc[a] <= bp_cell_of(th, last, &f);
+    m = fmaxf(m, fmaxf(tl - (float)(cc[a] + 1), (float)cc[a] - th));
+  }
+  *gap = m;
+  return in;
+}
+
+__device__ __forceinline__ void static_range(const StaticGrid& G, int* b0, int* b1) {
+  const int l = (int)(threadIdx.x % kCellLanes), per = (G.n + kCellLanes - 1) / kCellLanes;
+  *b0 = l * per < G.n ? l * per : G.n;
+  *b1 = *b0 + per < G.n ? *b0 + per : G.n;
+}
+
+__global__ void __launch_bounds__(256) kp_static_count_kernel(StaticGrid G) {
+  const int C = G.g * G.g * G.g;
+  const int c = (int)(blockIdx.x * kCellsPerBlock + threadIdx.x / kCellLanes);
+  for (int b = (int)(blockIdx.x * 256 + threadIdx.x); b < G.pad; b += (int)gridDim.x * 256) {
+    float4* o = reinterpret_cast<float4*>(G.blob) + 2 * b;
+    float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+    if (b < G.n) static_box(G, b, lo, hi);
+    o[0] = make_float4(lo[0], lo[1], lo[2], 0.0f);
+    o[1] = make_float4(hi[0], hi[1], hi[2], 0.0f);
+  }
+  const int cc[3] = {c % G.g, (c / G.g) % G.g, c / (G.g * G.g)};
+  int b0, b1, k = 0;
+  static_range(G, &b0, &b1);
+  float r = (float)KP_BP_CLEAR_CAP;
+  if (c < C)
+    for (int b = b0; b < b1; ++b) {
+      float lo[3], hi[3], gap;
+      static_box(G, b, lo, hi);
+      k += static_listed(G, lo, hi, cc, &gap) ? 1 : 0;
+      r = fminf(r, gap);
     }
-    return true;
+#pragma unroll
+  for (int o = kCellLanes / 2; o > 0; o >>= 1) {
+    k += __shfl_xor_sync(0xffffffffu, k, o);
+    r = fminf(r, __shfl_xor_sync(0xffffffffu, r, o));
+  }
+  if (c < C && threadIdx.x % kCellLanes == 0) {
+    G.count[c] = (uint32_t)k;
+    const float v = (r - (float)KP_BP_CLEAR_MARGIN) * 16.0f;
+    G.blob[G.clear_off + c] = v >= 1.0f ? (unsigned char)fminf(255.0f, floorf(v)) : (unsigned char)0;
+  }
+}
+
+__global__ void __launch_bounds__(256) kp_static_lists_kernel(StaticGrid G) {
+  __shared__ uint32_t red[8], own[kCellsPerBlock];
+  uint16_t* start = reinterpret_cast<uint16_t*>(G.blob + G.start_off);
+  uint16_t* ids = reinterpret_cast<uint16_t*>(G.blob + G.ids_off);
+  const int C = G.g * G.g * G.g, c0 = (int)blockIdx.x * kCellsPerBlock;
+  uint32_t s = 0;
+  for (int c = (int)threadIdx.x; c < c0; c += 256) s += G.count[c];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  if (threadIdx.x < kCellsPerBlock)
+    own[threadIdx.x] = c0 + (int)threadIdx.x < C ? G.count[c0 + threadIdx.x] : 0u;
+  __syncthreads();
+  const int i = (int)threadIdx.x / kCellLanes, c = c0 + i;
+  uint32_t pos = 0;
+  for (int w = 0; w < 8; ++w) pos += red[w];
+  for (int j = 0; j < i; ++j) pos += own[j];
+  const int cc[3] = {c % G.g, (c / G.g) % G.g, c / (G.g * G.g)};
+  int b0, b1;
+  static_range(G, &b0, &b1);
+  auto listed = [&](int b) {
+    float lo[3], hi[3], gap;
+    static_box(G, b, lo, hi);
+    return static_listed(G, lo, hi, cc, &gap);
   };
-  for (int c = threadIdx.x; c < C; c += blockDim.x) {
-    const int cc[3] = {c % gx, (c / gx) % gy, c / (gx * gy)};
-    int k = 0;
-    double r = (double)KP_BP_CLEAR_CAP;
-    for (int b = 0; b < n; ++b) {
-      k += in_range(b, cc) ? 1 : 0;
-      double gap = 0.0;
-      for (int a = 0; a < 3; ++a) {
-        const double bl = ((double)dst[b * 8 + a] - (double)l3[a]) * (double)s3[a];
-        const double bh = ((double)dst[b * 8 + 4 + a] - (double)l3[a]) * (double)s3[a];
-        gap = fmax(gap, fmax(bl - (double)(cc[a] + 1), (double)cc[a] - bh));
-      }
-      r = fmin(r, gap);
-    }
-    kcount[c] = k;
-    const double v = (r - KP_BP_CLEAR_MARGIN) * 16.0;
-    blob[clear_off + c] = v >= 1.0 ? (unsigned char)fmin(255.0, floor(v)) : (unsigned char)0;
+  uint32_t k = 0;
+  if (c < C)
+    for (int b = b0; b < b1; ++b) k += listed(b) ? 1u : 0u;
+  uint32_t before = k;  // listed boxes of the lanes before this one
+#pragma unroll
+  for (int o = 1; o < kCellLanes; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, before, o, kCellLanes);
+    if ((int)(threadIdx.x % kCellLanes) >= o) before += y;
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {  // cell starts: an exclusive prefix over the counts
-    int acc = 0;
-    for (int c = 0; c < C; ++c) {
-      start[c] = (uint16_t)acc;
-      acc += kcount[c];
-    }
-    start[C] = (uint16_t)acc;
+  before -= k;
+  if (c >= C) return;
+  if (threadIdx.x % kCellLanes == 0) {
+    start[c] = (uint16_t)pos;
+    if (c == C - 1) start[C] = (uint16_t)(pos + own[i]);
   }
-  __syncthreads();
-  // the ids, within the room the host counted for them (the same FP32 cell
+  // within the room the host counted for the lists (the same FP32 cell
   // arithmetic gives the same count; the bound only guards the blob)
-  const int room = (clear_off - ids_off) / 2;
-  for (int c = threadIdx.x; c < C; c += blockDim.x) {
-    const int cc[3] = {c % gx, (c / gx) % gy, c / (gx * gy)};
-    int pos = start[c];
-    for (int b = 0; b < n && pos < room; ++b)
-      if (in_range(b, cc)) ids[pos++] = (uint16_t)b;
-  }
+  const uint32_t room = (uint32_t)((G.clear_off - G.ids_off) / 2);
+  uint32_t at = pos + before;
+  for (int b = b0; b < b1; ++b)
+    if (listed(b)) {
+      if (at < room) ids[at] = (uint16_t)b;
+      ++at;
+    }
 }
 
 }  // namespace
@@ -1864,45 +1903,52 @@ extern "C" kp_status kp_plan_static(const kp_system* sys, const kp_workspace* ws
     if (e == cudaSuccess) e = r;
     return e == cudaSuccess;
   };
-  // obstacles: raw rows into the (not yet used) trajectory rows, padded on
-  // the device into the box slots
+  // obstacles: raw rows into the (not yet used) trajectory rows, the cells'
+  // counts behind them
   if (nb > 0)
     ok(cudaMemcpyAsync(A + lay.traj, obs->boxes, (size_t)nb * 24, cudaMemcpyHostToDevice, stream));
-  kp_static_blob_kernel<<<1, 1024, (size_t)(P.bp_g[0] * P.bp_g[1] * P.bp_g[2] + 1) * 4, stream>>>(
-      reinterpret_cast<unsigned char*>(A + lay.boxes), reinterpret_cast<const float*>(A + lay.traj),
-      nb, pad, P.bp_g[0], P.bp_g[1], P.bp_g[2], P.bp_scale[0], P.bp_scale[1], P.bp_scale[2],
-      ws->lo[0], ws->lo[1], ws->lo[2], P.bp_start_off, P.bp_ids_off, P.bp_clear_off);
-  ok(cudaGetLastError());
-  // everything that must start from zero (the scratch keeps old contents)
+  static_assert((size_t)KP_MAX_BOXES * 24 + (size_t)KP_BP_MAX_G * KP_BP_MAX_G * KP_BP_MAX_G * 4 <=
+                    (size_t)KP_TRAJ_ROWS * 17 * 4,
+                "boxes and counts fit the trajectory rows");
+  StaticGrid G{};
+  G.blob = reinterpret_cast<unsigned char*>(A + lay.boxes);
+  G.raw = reinterpret_cast<const float*>(A + lay.traj);
+  G.count = reinterpret_cast<uint32_t*>(A + lay.traj + (size_t)KP_MAX_BOXES * 24);
+  G.n = nb;
+  G.pad = pad;
+  G.g = P.bp_g[0];
+  for (int a = 0; a < 3; ++a) {
+    G.scale[a] = P.bp_scale[a];
+    G.lo[a] = ws->lo[a];
+  }
+  G.start_off = P.bp_start_off;
+  G.ids_off = P.bp_ids_off;
+  G.clear_off = P.bp_clear_off;
+  const int cell_blocks = (G.g * G.g * G.g + kCellsPerBlock - 1) / kCellsPerBlock;
+  // the control block starts from zero (the scratch keeps old contents, and a
+  // launch that timed out leaves its barrier word mid-phase)
   ok(cudaMemsetAsync(A + lay.ctl, 0, sizeof(KCtl), stream));
-  ok(cudaMemsetAsync(A + lay.visited, 0, d.n_sub, stream));
-  ok(cudaMemsetAsync(A + lay.claim, 0xff, d.n_sub * 4, stream));
-  ok(cudaMemsetAsync(A + lay.n_valid, 0, (size_t)d.R * 4, stream));
-  ok(cudaMemsetAsync(A + lay.n_invalid, 0, (size_t)d.R * 4, stream));
-  ok(cudaMemsetAsync(A + lay.cov, 0, (size_t)d.R * 4, stream));
-  ok(cudaMemsetAsync(A + lay.avail, 0, (size_t)d.R, stream));
+  if (e == cudaSuccess) {
+    kp_static_count_kernel<<<cell_blocks, 256, 0, stream>>>(G);
+    kp_static_lists_kernel<<<cell_blocks, 256, 0, stream>>>(G);
+    ok(cudaGetLastError());
+  }
   RootState root{};
   for (int i = 0; i < d.D; ++i) root.x[i] = x_init[i];
   const uint64_t max_ns = budget->max_ms > 0.0 ? (uint64_t)(budget->max_ms * 1e6) : 0ull;
+  // one launch, as kp_plan: initialisation, the passes, the chain
+  const int mode = KP_LOOP_RESET | KP_LOOP_EXTRACT;
   if (e == cudaSuccess) {
     switch (d.sys) {
       case KP_SYS_DI:
-        ok(launch_reset_di(P, root, stream));
-        ok(launch_loop_di(P, grid, smem, budget->max_iters, max_ns, false, stream, root, 0));
+        ok(launch_loop_di(P, grid, smem, budget->max_iters, max_ns, false, stream, root, mode));
         break;
       case KP_SYS_DUBINS:
-        ok(launch_reset_dubins(P, root, stream));
-        ok(launch_loop_dubins(P, grid, smem, budget->max_iters, max_ns, false, stream, root,
-                              0));
+        ok(launch_loop_dubins(P, grid, smem, budget->max_iters, max_ns, false, stream, root, mode));
         break;
       default:
-        ok(launch_reset_quad(P, root, stream));
-        ok(launch_loop_quad(P, grid, smem, budget->max_iters, max_ns, false, stream, root, 0));
+        ok(launch_loop_quad(P, grid, smem, budget->max_iters, max_ns, false, stream, root, mode));
     }
-  }
-  if (e == cudaSuccess) {
-    kp_extract_kernel<<<1, 32, 0, stream>>>(P);
-    ok(cudaGetLastError());
   }
   KCtl h{};
   ok(cudaMemcpyAsync(&h, A + lay.ctl, sizeof(KCtl), cudaMemcpyDeviceToHost, stream));
@@ -1918,19 +1964,20 @@ extern "C" kp_status kp_plan_static(const kp_system* sys, const kp_workspace* ws
   if (h.n_edges > traj->capacity || h.n_edges > KP_TRAJ_ROWS) return KP_ERR_ARG;
   const int n = h.n_edges;
   if (n > 0) {
-    const char* rows = A + lay.traj;
-    ok(cudaMemcpy2DAsync(traj->states, 12 * 4, rows, 17 * 4, 12 * 4, n, cudaMemcpyDeviceToHost,
-                         stream));
-    ok(cudaMemcpy2DAsync(traj->ctrls, 4 * 4, rows + 12 * 4, 17 * 4, 4 * 4, n,
+    // whole rows in pieces through the stack (strided copies into pageable
+    // memory are slower)
+    float piece[128 * 17];
+    for (int r0 = 0; r0 < n; r0 += 128) {
+      const int m = n - r0 < 128 ? n - r0 : 128;
+      ok(cudaMemcpyAsync(piece, A + lay.traj + (size_t)r0 * 17 * 4, (size_t)m * 17 * 4,
                          cudaMemcpyDeviceToHost, stream));
-    ok(cudaMemcpy2DAsync(traj->steps, 4, rows + 16 * 4, 17 * 4, 4, n, cudaMemcpyDeviceToHost,
-                         stream));
-    ok(cudaStreamSynchronize(stream));
-    if (e != cudaSuccess) return KP_ERR_CUDA;
-    for (int i = 0; i < n; ++i) {  // the rows carry the step count as a float
-      float f;
-      std::memcpy(&f, &traj->steps[i], 4);
-      traj->steps[i] = (int32_t)f;
+      ok(cudaStreamSynchronize(stream));
+      if (e != cudaSuccess) return KP_ERR_CUDA;
+      for (int i = 0; i < m; ++i) {
+        std::memcpy(traj->states + (size_t)(r0 + i) * 12, piece + i * 17, 12 * 4);
+        std::memcpy(traj->ctrls + (size_t)(r0 + i) * 4, piece + i * 17 + 12, 4 * 4);
+        traj->steps[r0 + i] = (int32_t)piece[i * 17 + 16];
+      }
     }
   }
   return KP_OK;

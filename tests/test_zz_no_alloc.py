@@ -120,3 +120,21 @@ def test_static_plan_takes_grid_regions_only(P):
     with the obstacles); the no-allocation entry point refuses it."""
     st, _ = static_plan(P, W.c1(0).with_(fso=True))
     assert st == P.ERR_ARG
+
+
+@pytest.mark.parametrize("n", [0, 1, 7, 8, 9, 65, 2000])
+def test_static_grid_at_box_counts(P, n):
+    """The device-built grid with box counts around its eight lanes a cell and
+    far above: the trajectory is kp_plan's bit for bit (every sample's verdict
+    is that of testing every box, whichever grid finds it)."""
+    side = (0.05, 0.15) if n < 100 else (0.005, 0.012)
+    w = W.c1(3)
+    boxes = W.random_boxes(3, n, side=side, keep_clear=[((0.1, 0.1, 0.1), 0.03),
+                                                        ((0.9, 0.9, 0.9), 0.06)]) \
+        if n else np.zeros((0, 6), np.float32)
+    w = w.with_(boxes=boxes)
+    st_ref, ref = P.Planner(w).plan(max_iters=60, capacity=1024)
+    st, got = static_plan(P, w, max_iters=60)
+    assert st == st_ref
+    for k in ("states", "ctrls", "steps"):
+        assert np.array_equal(got[k], ref[k])
