@@ -447,21 +447,129 @@ __global__ void __launch_bounds__(FT_THREADS, 1) kp_mlp_forward_tc_kernel(FtArgs
 }
 
 // ---------------------------------------------------------------------------
-// one training step's forward and backward pass
+// training: forward, backward and optimiser
 // ---------------------------------------------------------------------------
 
-// Control of a device-driven epoch.
-struct EpochCtl {
-  const float* x;        // [rows][32] features
-  const float* t;        // [rows][4] targets
-  const int32_t* perm;   // row order of the epoch
-  int batch;             // index of the mini-batch in work
-  int step;              // Adam steps taken, the one in work included
+// flat parameter vector (FP32), row-major: W1 b1 W2 b2 W3 b3
+constexpr int OFF_W1 = 0, OFF_B1 = OFF_W1 + MLP_H * MLP_IN, OFF_W2 = OFF_B1 + MLP_H,
+              OFF_B2 = OFF_W2 + MLP_H * MLP_H, OFF_W3 = OFF_B2 + MLP_H,
+              OFF_B3 = OFF_W3 + MLP_OUT * MLP_H, N_PARAMS = OFF_B3 + MLP_OUT;
+
+// A CTA's share of a mini-batch's gradient: groups of four parameters, then its
+// share of the loss.  At most ST_MAX_SLOTS CTAs work on tiles.  The groups of
+// dW1 and dW2 are in the order in which the warps hold them in tensor memory
+// (a lane a row, a warp's 32 lanes' groups together), so that a warp writes 512
+// contiguous bytes at a time: written in rows, where a warp's store touches 16
+// to 32 lines, the two halves of dW2 took 15,000 of a step's 57,000 clocks.
+constexpr int SLOT = N_PARAMS + 4, ST_MAX_SLOTS = 152;
+
+// Group of dW1 rows 32 (4 tile + q) + lane, columns 4 j ..
+__device__ __forceinline__ int slot_group_w1(int tile, int q, int j, int lane) {
+  return ((tile * 4 + q) * 8 + j) * 32 + lane;
+}
+
+// Group of dW2 rows 128 tile + 32 (warp % 4) + lane, columns 64 (warp / 4) +
+// 32 u + 4 j ..
+__device__ __forceinline__ int slot_group_w2(int tile, int warp, int u, int j, int lane) {
+  return OFF_W2 / 4 + (((tile * 16 + warp) * 2 + u) * 8 + j) * 32 + lane;
+}
+
+// First parameter of a slot's group.
+__device__ __forceinline__ int slot_param(int gr) {
+  if (gr < OFF_B1 / 4) return ((gr >> 8) * 32 + (gr & 31)) * MLP_IN + 4 * ((gr >> 5) & 7);
+  if (gr >= OFF_W2 / 4 && gr < OFF_B2 / 4) {
+    const int e = gr - OFF_W2 / 4, lane = e & 31, j = (e >> 5) & 7, u = (e >> 8) & 1,
+              warp = (e >> 9) & 15, tile = e >> 13;
+    return OFF_W2 + (128 * tile + 32 * (warp & 3) + lane) * MLP_H + 64 * (warp >> 2) + 32 * u + 4 * j;
+  }
+  return 4 * gr;
+}
+
+// Parameters i .. i + 3 (i a multiple of 4) rounded to BF16 into the copies
+// the kernels read: the hidden layers' weights in tensor-core operand order
+// (wt) and in the fragment order of the planner's loop kernel (wf); the output
+// layer's row-major (w3) and in fragment order.
+__device__ __forceinline__ void store_weights(int i, float4 p, __nv_bfloat16* w3, __nv_bfloat16* wf,
+                                              __nv_bfloat16* wt) {
+  const uint32_t lo = pack_bf16(p.x, p.y), hi = pack_bf16(p.z, p.w);
+  auto put = [&](__nv_bfloat16* row, __nv_bfloat16* f0, __nv_bfloat16* f2) {
+    *reinterpret_cast<uint2*>(row) = make_uint2(lo, hi);
+    *reinterpret_cast<uint32_t*>(f0) = lo;
+    *reinterpret_cast<uint32_t*>(f2) = hi;
+  };
+  if (i < OFF_B1) {
+    const int n = i / MLP_IN, k = i % MLP_IN;
+    put(wt + wt_index_w1(n, k), wf + frag_index_hidden(n, k, MLP_IN),
+        wf + frag_index_hidden(n, k + 2, MLP_IN));
+  } else if (i >= OFF_W2 && i < OFF_B2) {
+    const int n = (i - OFF_W2) / MLP_H, k = (i - OFF_W2) % MLP_H;
+    __nv_bfloat16* f = wf + MLP_H * MLP_IN;
+    put(wt + wt_index_w2(n, k), f + frag_index_hidden(n, k, MLP_H), f + frag_index_hidden(n, k + 2, MLP_H));
+  } else if (i >= OFF_W3 && i < OFF_B3) {
+    const int n = (i - OFF_W3) / MLP_H, k = (i - OFF_W3) % MLP_H;
+    __nv_bfloat16* f = wf + MLP_H * MLP_IN + MLP_H * MLP_H;
+    put(w3 + (i - OFF_W3), f + frag_index_out(n, k), f + frag_index_out(n, k + 2));
+  }
+}
+
+// Sum over the slots of a group, in slot order (read past L1: other SMs wrote
+// them).
+__device__ __forceinline__ float4 slot_sum(const float* slots, int n, int gr) {
+  const float4* g = reinterpret_cast<const float4*>(slots) + gr;
+  float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  for (int k0 = 0; k0 < n; k0 += 16) {  // sixteen loads in flight, the last ones too
+    float4 v[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k)
+      v[k] = k0 + k < n ? __ldcg(g + (size_t)(k0 + k) * (SLOT / 4)) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      s.x += v[k].x;
+      s.y += v[k].y;
+      s.z += v[k].z;
+      s.w += v[k].w;
+    }
+  }
+  return s;
+}
+
+struct AdamArgs {
+  float *p, *m, *v;
+  const float* slots;
+  int n_slots;
+  __nv_bfloat16 *w3, *wf, *wt;
   float lr;
-  float loss_sum;        // sum of the mini-batch losses of the epoch
 };
 
-constexpr int ST_THREADS = 256;
+// One Adam step (beta 0.9 / 0.999, eps 1e-8) on the parameters of a slot group;
+// c1, c2 = 1 - beta^step.
+__device__ __forceinline__ void adam_update(const AdamArgs& a, int gr, float c1, float c2) {
+  const int i = slot_param(gr);
+  const float beta1 = 0.9f, beta2 = 0.999f, eps = 1e-8f;
+  float4 p = *reinterpret_cast<const float4*>(a.p + i), m = *reinterpret_cast<const float4*>(a.m + i),
+         v = *reinterpret_cast<const float4*>(a.v + i);
+  const float4 g = slot_sum(a.slots, a.n_slots, gr);
+  auto one = [&](float& pi, float& mi, float& vi, float gi) {
+    mi = beta1 * mi + (1.0f - beta1) * gi;
+    vi = beta2 * vi + (1.0f - beta2) * gi * gi;
+    pi = pi - a.lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+  };
+  one(p.x, m.x, v.x, g.x);
+  one(p.y, m.y, v.y, g.y);
+  one(p.z, m.z, v.z, g.z);
+  one(p.w, m.w, v.w, g.w);
+  *reinterpret_cast<float4*>(a.p + i) = p;
+  *reinterpret_cast<float4*>(a.m + i) = m;
+  *reinterpret_cast<float4*>(a.v + i) = v;
+  store_weights(i, p, a.w3, a.wf, a.wt);
+}
+
+__device__ __forceinline__ void adam_corrections(int step, float* c1, float* c2) {
+  *c1 = 1.0f - powf(0.9f, (float)step);
+  *c2 = 1.0f - powf(0.999f, (float)step);
+}
+
+constexpr int ST_THREADS = 512;
 // shared memory: h1 (first the inputs and W1), h2 then dh2 (first two chunks
 // of W2), two chunks of W2 then dh1, the transposed inputs with a block of
 // ones, the transposed output gradient, W3 twice, the output gradient split
@@ -473,13 +581,16 @@ constexpr uint32_t ST_X = ST_H1, ST_W1 = ST_H1 + 16384;  // before h1 is written
 constexpr uint32_t ST_B1 = ST_DA, ST_B2 = ST_DA + 1024;   // before the split gradient is
 
 struct StepArgs {
-  const __nv_bfloat16* wt;  // W2, W1 in operand order (wt_index_*)
-  const __nv_bfloat16* W3;  // row-major [8][256]
-  const float *b1, *b2, *b3;
-  const float *x, *t;       // [M][32], [M][4] (epoch null)
-  EpochCtl* epoch;          // rows perm[batch M ..] of epoch->x, epoch->t
-  int M;
-  float *g_W1, *g_b1, *g_W2, *g_b2, *g_W3, *g_b3, *loss;  // added to
+  const float *x, *t;      // [rows][32], [rows][4]
+  const int32_t* perm;     // row behind each row of the batches (null: itself)
+  int M;                   // rows of a mini-batch
+  int64_t steps;           // mini-batches: rows s M .. of the order
+  int epoch;               // 1: an Adam step after each (cooperative launch)
+  int step0;               // Adam steps taken before
+  AdamArgs adam;           // parameters, BF16 copies, the slots
+  float* slots;            // each CTA's share of the gradient, written
+  float* loss_sum;         // epoch: sum over its mini-batches, 0 at launch
+  uint32_t* bar;           // epoch: grid barrier word, 0 at launch
   int* err;
   unsigned long long wait_ns;
 };
@@ -515,11 +626,19 @@ __device__ __forceinline__ void sts16(uint32_t addr, __nv_bfloat16 v) {
                : "memory");
 }
 
-__device__ __forceinline__ void red_add4(float* p, const uint32_t* r) {
-  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(__uint_as_float(r[0])),
-               "f"(__uint_as_float(r[1])), "f"(__uint_as_float(r[2])), "f"(__uint_as_float(r[3]))
-               : "memory");
+// 16 bytes of a slot: written by the CTA's first tile of a mini-batch, added to
+// by its later ones.
+__device__ __forceinline__ void slot_put4(float* p, const uint32_t* r, bool add) {
+  float4 v = make_float4(__uint_as_float(r[0]), __uint_as_float(r[1]), __uint_as_float(r[2]),
+                         __uint_as_float(r[3]));
+  if (add) {
+    const float4 o = *reinterpret_cast<const float4*>(p);
+    v = make_float4(o.x + v.x, o.y + v.y, o.z + v.z, o.w + v.w);
+  }
+  *reinterpret_cast<float4*>(p) = v;
 }
+
+__device__ __forceinline__ void slot_put(float* p, float v, bool add) { *p = add ? *p + v : v; }
 
 // The two BF16 halves of v kept where those of h are not zero (h is the
 // output of a ReLU: positive or zero).
@@ -528,11 +647,35 @@ __device__ __forceinline__ uint32_t keep_active(uint32_t v, uint32_t h) {
   return v & (lo | hi);
 }
 
-// Forward, loss and backward of one 128-row tile per CTA, every product on
-// the tensor cores, nothing of the tile in global memory but its inputs and
-// its gradient contributions.  The phases of a tile (X the inputs, D the
-// gradient of the eight outputs; thread = row 32 (w % 4) + lane and columns
-// 128 (w / 4) ..):
+// Waits (bounded, one thread) until all CTAs of the launch have arrived 'n'
+// times; false when the wait or another CTA gave up.  What the CTAs wrote
+// before their arrivals is visible to generic and bulk-copy reads after it.
+__device__ __forceinline__ bool grid_arrive_wait(uint32_t* bar, uint32_t n, const int* err,
+                                                 uint64_t limit_ns) {
+  __threadfence();
+  atomicAdd(bar, 1u);
+  uint64_t t0 = 0;
+  for (uint32_t i = 1;; ++i) {
+    uint32_t v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+    if ((int32_t)(v - n) >= 0) break;
+    if ((i & 63u) == 0) {
+      if (*((const volatile int*)err) != 0) return false;
+      if (t0 == 0) t0 = now_ns();
+      if (now_ns() - t0 > limit_ns) return false;
+    }
+  }
+  asm volatile("fence.proxy.async;" ::: "memory");
+  return true;
+}
+
+// Forward, loss and backward of 128-row tiles, every product on the tensor
+// cores, nothing of a tile in global memory but its inputs and its gradient
+// contributions; in an epoch (a cooperative launch of at most one CTA per SM)
+// every mini-batch ends with a grid barrier, each CTA's share of the Adam step
+// and another barrier, so the whole epoch is one launch.  The phases of a tile
+// (X the inputs, D the gradient of the eight outputs; thread = row 32 (w % 4) +
+// lane and columns 64 (w / 4) ..):
 //   h1 = relu(X W1' + b1), h2 = relu(h1 W2' + b2), raw = h2 W3' + b3; the
 //   loss and D (FP32);
 //   dW3 += D' h2;  dh2 = (D W3) where h2 > 0, D entering as three BF16 parts
@@ -544,119 +687,68 @@ __device__ __forceinline__ uint32_t keep_active(uint32_t v, uint32_t h) {
 // half of it only once (its first half survives the forward pass).  Rows past
 // M have inputs 0, activations 0 and D 0.
 //
-// A mini-batch of 4096 is 32 tiles, so the pass is one tile's chain of twelve
-// products and epilogues, and the 32 x 75 K additions to the gradient; what it
-// replaces was 13 launches (row-major and transposed activations in global
-// memory, split-K products), 83 us a step with the optimiser's: now 33 us
-// (GB300, epochs of 16 steps of 4,096 rows: 1,336 -> 565 us with the parameter
-// read-back).
-__global__ void __launch_bounds__(ST_THREADS, 1) kp_mlp_step_kernel(StepArgs a) {
+// Every CTA writes its share of the gradient to a slot of its own, and the
+// optimiser adds the slots up in slot order: additions in L2 by 32 CTAs took
+// 17,000 of a step's 57,000 clocks (L2 added 120 values a clock), and the
+// result now has the same bits every time.
+//
+// A mini-batch of 4096 is 32 tiles, so a step is one tile's chain of twelve
+// products and epilogues (21,000 clocks), 9,000 for the slot's 305 KB, 5,000
+// for the optimiser's share and 6,000 in the two barriers: 25 us (GB300).
+// Epochs of 16 steps of 4,096 rows: 1,333 us as 15 launches a step (row-major
+// and transposed activations in global memory, split-K products), 561 us as two
+// launches a step with this pass, 465 us now, with the parameter read-back (50
+// us).
+__global__ void __launch_bounds__(ST_THREADS, 1) kp_mlp_train_kernel(StepArgs a) {
   extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t b_w1, b_w2[4], b_mma, b_c[2], b_t0, b_r[2];
+  __shared__ __align__(8) uint64_t b_w1, b_w2[4], b_mma, b_c, b_t0, b_r;
+  __shared__ float s_red[4][MLP_NQ][3];  // sums over a warp's rows: loss, both gradients
+  __shared__ float s_b3[MLP_OUT];
   __shared__ uint32_t tmem_slot;
   __shared__ int s_fail;
   const uint32_t base = (saddr(smem_raw) + 1023u) & ~1023u;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int q = warp & 3, half = warp >> 2;
-  const int row0 = blockIdx.x * 128;
+  const int q = warp & 3, qt = warp >> 2;
   if (tid == 0) {
     mbar_init(saddr(&b_w1), 1);
     for (int c = 0; c < 4; ++c) mbar_init(saddr(&b_w2[c]), 1);
     mbar_init(saddr(&b_mma), 1);
-    for (int c = 0; c < 2; ++c) {
-      mbar_init(saddr(&b_c[c]), 1);
-      mbar_init(saddr(&b_r[c]), 1);
-    }
+    mbar_init(saddr(&b_c), 1);
+    mbar_init(saddr(&b_r), 1);
     mbar_init(saddr(&b_t0), 1);
     s_fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    fence_async();
-    mbar_expect_tx(saddr(&b_w1), MLP_H * 64);
-    bulk_load(base + ST_W1, a.wt + WT_W1, MLP_H * 64, saddr(&b_w1));
-    for (int c = 0; c < 4; ++c) {
-      mbar_expect_tx(saddr(&b_w2[c]), MLP_H * 128);
-      bulk_load(base + (c < 2 ? ST_W + c * 32768 : ST_G + (c - 2) * 32768), a.wt + c * WT_CHUNK,
-                MLP_H * 128, saddr(&b_w2[c]));
-    }
   }
   if (warp == 0) {
     __syncwarp();
     tmem_alloc(saddr(&tmem_slot), 512);
   }
-  // inputs: thread = row tid / 2 and 16 columns
-  const float *xs = a.x, *ts = a.t;
-  auto source_row = [&](int r) {  // row of x and t behind row r of the batch
-    return a.epoch ? (size_t)a.epoch->perm[(size_t)a.epoch->batch * a.M + r] : (size_t)r;
-  };
-  if (a.epoch) {
-    xs = a.epoch->x;
-    ts = a.epoch->t;
-  }
-  {
-    const int r = tid >> 1, part = tid & 1;
-    float v[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = 0.0f;
-    if (row0 + r < a.M) {
-      const float* src = xs + source_row(row0 + r) * MLP_IN + 16 * part;
-      if (((uintptr_t)src & 15u) == 0) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float4 f = __ldg(reinterpret_cast<const float4*>(src) + i);
-          v[4 * i] = f.x; v[4 * i + 1] = f.y; v[4 * i + 2] = f.z; v[4 * i + 3] = f.w;
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = __ldg(src + i);
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int c = 2 * part + i;
-      sts128(base + ST_X + (uint32_t)(r * 64 + ((c ^ ((r >> 1) & 3)) << 4)),
-             pack_bf16(v[8 * i], v[8 * i + 1]), pack_bf16(v[8 * i + 2], v[8 * i + 3]),
-             pack_bf16(v[8 * i + 4], v[8 * i + 5]), pack_bf16(v[8 * i + 6], v[8 * i + 7]));
-    }
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      const int n = 16 * part + i;
-      sts16(base + ST_XT + (uint32_t)((r >> 6) * 6144 + n * 128 + ((((r & 63) >> 3) ^ (n & 7)) << 4) +
-                                      (r & 7) * 2),
-            __float2bfloat16_rn(v[i]));
-    }
-  }
-  {
-    // ones (rows 32..47 of the transposed inputs), zeros (rows 8..15 of the
-    // transposed output gradient), W3 twice
+  // the parts of the operands that stay: ones (rows 32..47 of the transposed
+  // inputs), zeros (rows 8..15 of the transposed output gradient)
+  if (tid < 256) {
     const uint32_t one2 = 0x3F803F80u;
     sts128(base + ST_XT + (uint32_t)((tid >> 7) * 6144 + 4096 + (tid & 127) * 16), one2, one2, one2, one2);
-    if (tid < 128)
-      sts128(base + ST_DT + (uint32_t)((tid >> 6) * 2048 + 1024 + (tid & 63) * 16), 0, 0, 0, 0);
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int e = tid + 256 * i, c = e >> 7, copy = (e >> 6) & 1, n = (e >> 3) & 7, j = e & 7;
-      const uint4 w = *reinterpret_cast<const uint4*>(a.W3 + n * MLP_H + 64 * c + 8 * j);
-      sts128(base + ST_W3 + (uint32_t)(c * 2048 + copy * 1024 + n * 128 + ((j ^ n) << 4)), w.x, w.y, w.z,
-             w.w);
-    }
-    asm volatile("st.shared.f32 [%0], %1;" ::"r"(base + ST_B1 + 4 * tid), "f"(a.b1[tid]) : "memory");
-    asm volatile("st.shared.f32 [%0], %1;" ::"r"(base + ST_B2 + 4 * tid), "f"(a.b2[tid]) : "memory");
+  } else if (tid < 384) {
+    const int e = tid - 256;
+    sts128(base + ST_DT + (uint32_t)((e >> 6) * 2048 + 1024 + (e & 63) * 16), 0, 0, 0, 0);
   }
-  if (a.epoch && blockIdx.x == 0 && tid == 0) a.epoch->step += 1;  // read by the Adam launch
-  fence_async();
   fence_before();
   __syncthreads();
   fence_after();
   const uint32_t tmem = tmem_slot;
   const uint32_t tl = tmem + ((uint32_t)(32 * q) << 16);
   const int r = 32 * q + lane;
-  const bool live = row0 + r < a.M;
   // this row's piece 0 of a 128-byte-row tile (piece c at c ^ (r & 7))
-  const uint32_t hoff = (uint32_t)(r * 128 + ((r & 7) << 4));
-  uint32_t ph = 0;
+  const uint32_t hoff = (uint32_t)(r * 128 + ((r & 7) << 4) + qt * 16384);
+  const uint32_t A0 = tmem, B0 = tmem + 256;  // the two halves of tensor memory
+  const float* par = a.adam.p;
+  float* g = a.slots + (size_t)blockIdx.x * SLOT;
+  uint32_t ph = 0, ph_t = 0;  // parities: of b_mma, and of the once-a-tile barriers
   auto wait = [&](uint64_t* bar, uint32_t parity, int site) {
     mbar_wait_or(saddr(bar), parity, a.wait_ns, &s_fail, site);
   };
+  auto failed1 = [&]() { return *((volatile int*)&s_fail) != 0; };
+  auto failed = [&]() { return __any_sync(0xffffffffu, failed1()) != 0; };  // the warp agrees
   auto wait_mma = [&](int site) {  // all threads: the products committed last are there
     __syncwarp();
     wait(&b_mma, ph, site);
@@ -670,12 +762,12 @@ __global__ void __launch_bounds__(ST_THREADS, 1) kp_mlp_step_kernel(StepArgs a) 
     __syncthreads();
     fence_after();
   };
-  // bias, ReLU, BF16 of this thread's 128 columns of an accumulator into a tile
-  auto activate = [&](uint32_t acc, uint32_t tile, uint32_t bias) {
-#pragma unroll 1
-    for (int u = 0; u < 4; ++u) {
+  // bias, ReLU, BF16 of this thread's 64 columns of an accumulator into a tile
+  auto activate = [&](uint32_t acc, uint32_t tile, uint32_t bias, bool live) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
       uint32_t v[32];
-      const int c0 = 128 * half + 32 * u;
+      const int c0 = 64 * qt + 32 * u;
       tmem_ld32(acc + (uint32_t)c0, v);
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -689,22 +781,21 @@ __global__ void __launch_bounds__(ST_THREADS, 1) kp_mlp_step_kernel(StepArgs a) 
                        w1 = bias_relu_bf16(vv[2], vv[3], two(ba.z, ba.w)),
                        w2 = bias_relu_bf16(vv[4], vv[5], two(bb.x, bb.y)),
                        w3 = bias_relu_bf16(vv[6], vv[7], two(bb.z, bb.w));
-        sts128(base + tile + (uint32_t)((c0 >> 6) * 16384) + (hoff ^ (uint32_t)((4 * (u & 1) + j) << 4)),
-               live ? w0 : 0u, live ? w1 : 0u, live ? w2 : 0u, live ? w3 : 0u);
+        sts128(base + tile + (hoff ^ (uint32_t)((4 * u + j) << 4)), live ? w0 : 0u, live ? w1 : 0u,
+               live ? w2 : 0u, live ? w3 : 0u);
       }
     }
   };
-  // BF16 of this thread's 128 columns of an accumulator where the
-  // activations in tile 'act' are not zero, into 'tile' (which may be 'act')
+  // BF16 of this thread's 64 columns of an accumulator where the activations
+  // in tile 'act' are not zero, into 'tile' (which may be 'act')
   auto mask = [&](uint32_t acc, uint32_t act, uint32_t tile) {
-#pragma unroll 1
-    for (int u = 0; u < 4; ++u) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
       uint32_t v[32];
-      const int c0 = 128 * half + 32 * u;
-      tmem_ld32(acc + (uint32_t)c0, v);
+      tmem_ld32(acc + (uint32_t)(64 * qt + 32 * u), v);
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const uint32_t off = (uint32_t)((c0 >> 6) * 16384) + (hoff ^ (uint32_t)((4 * (u & 1) + j) << 4));
+        const uint32_t off = hoff ^ (uint32_t)((4 * u + j) << 4);
         const uint4 h = lds128(base + act + off);
         const float* f = reinterpret_cast<const float*>(v + 8 * j);
         sts128(base + tile + off, keep_active(pack_bf16(f[0], f[1]), h.x),
@@ -713,214 +804,310 @@ __global__ void __launch_bounds__(ST_THREADS, 1) kp_mlp_step_kernel(StepArgs a) 
       }
     }
   };
-  // a 128 x 256 accumulator added to rows out0 .. of dW2 (blocks start at
-  // different columns, so that they meet on few addresses)
-  auto add_dw2 = [&](uint32_t acc, int out0) {
-    if (*((volatile int*)&s_fail) != 0) return;
-    float* dst = a.g_W2 + (size_t)(out0 + r) * MLP_H;
-#pragma unroll 1
-    for (int u = 0; u < 4; ++u) {
-      uint32_t v[32];
-      const int c0 = 128 * half + 32 * ((u + (int)blockIdx.x) & 3);
-      tmem_ld32(acc + (uint32_t)c0, v);
+  // half 'tile' of dW2 (128 rows) from an accumulator into the slot
+  auto put_dw2 = [&](uint32_t acc, int tile, bool add) {
 #pragma unroll
-      for (int j = 0; j < 32; j += 4) red_add4(dst + c0 + j, v + j);
+    for (int u = 0; u < 2; ++u) {
+      uint32_t v[32];
+      tmem_ld32(acc + (uint32_t)(64 * qt + 32 * u), v);
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        slot_put4(g + 4 * slot_group_w2(tile, warp, u, j, lane), v + 4 * j, add);
     }
   };
   constexpr uint32_t ID_FWD = idesc_majors(128, 256, 0, 0), ID_RAW = idesc_majors(128, 16, 0, 0),
                      ID_DW3 = idesc_majors(128, 16, 1, 0), ID_DH2 = idesc_majors(128, 256, 0, 1),
-                     ID_DH1 = idesc_majors(128, 64, 0, 1), ID_DW2 = idesc_majors(128, 256, 1, 1),
+                     ID_DH1 = idesc_majors(128, 128, 0, 1), ID_DW2 = idesc_majors(128, 256, 1, 1),
                      ID_DW1 = idesc_majors(128, 48, 1, 0);
-  const uint32_t A0 = tmem, B0 = tmem + 256;  // the two halves of tensor memory
 
-  // ---- forward
-  if (tid == 0) {
-    wait(&b_w1, 0, 30);
-    fence_after();
-#pragma unroll
-    for (int k = 0; k < 2; ++k)
-      mma_bf16(A0, sdesc_sw64(base + ST_X + 32 * k), sdesc_sw64(base + ST_W1 + 32 * k), ID_FWD,
-               k != 0 ? 1u : 0u);
-    mma_commit(saddr(&b_mma));
-  }
-  wait_mma(31);
-  activate(tl, ST_H1, ST_B1);
-  publish();
-  if (tid == 0) {
-    for (int c = 0; c < 4; ++c) {
-      wait(&b_w2[c], 0, 32);
-      const uint32_t w = base + (c < 2 ? ST_W + c * 32768 : ST_G + (c - 2) * 32768);
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        mma_bf16(B0, sdesc_sw128(base + ST_H1 + c * 16384 + 32 * k), sdesc_sw128(w + 32 * k), ID_FWD,
-                 (c | k) != 0 ? 1u : 0u);
-    }
-    mma_commit(saddr(&b_mma));
-  }
-  wait_mma(33);
-  activate(tl + 256, ST_G, ST_B2);
-  publish();
-  if (tid == 0) {
-    for (int c = 0; c < 4; ++c)
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        mma_bf16(A0, sdesc_sw128(base + ST_G + c * 16384 + 32 * k),
-                 sdesc_sw128(base + ST_W3 + c * 2048 + 32 * k), ID_RAW, (c | k) != 0 ? 1u : 0u);
-    mma_commit(saddr(&b_mma));
-  }
-  float tv[MLP_NQ] = {0.0f, 0.0f, 0.0f, 0.0f};
-  if (half == 0 && live) {
-    const float* src = ts + source_row(row0 + r) * MLP_NQ;
-#pragma unroll
-    for (int i = 0; i < MLP_NQ; ++i) tv[i] = __ldg(src + i);
-  }
-  wait_mma(34);
-
-  // ---- loss and the outputs' gradient (one thread a row)
-  if (half == 0) {
-    uint32_t raw[8];
-    tmem_ld8(tl, raw);
-    const float inv_m = 1.0f / (float)a.M;
-    float l = 0.0f, d[MLP_OUT];
-#pragma unroll
-    for (int i = 0; i < MLP_NQ; ++i) {
-      const float mu = tanhf(__uint_as_float(raw[i]) + a.b3[i]);
-      const float lr = __uint_as_float(raw[MLP_NQ + i]) + a.b3[MLP_NQ + i];
-      const bool clamped = lr < MLP_LOGSTD_MIN || lr > MLP_LOGSTD_MAX;
-      const float ls = fminf(fmaxf(lr, MLP_LOGSTD_MIN), MLP_LOGSTD_MAX);
-      const float is = expf(-ls);
-      const float z = (tv[i] - mu) * is;
-      l += ls + 0.5f * z * z;
-      d[i] = live ? -z * is * (1.0f - mu * mu) * inv_m : 0.0f;
-      d[MLP_NQ + i] = live && !clamped ? (1.0f - z * z) * inv_m : 0.0f;
-    }
-    if (!live) l = 0.0f;
-    // three BF16 parts of each value: rounding, then what is left, twice
-    uint32_t part[3][4];
-    float rest[MLP_OUT];
-#pragma unroll
-    for (int n = 0; n < MLP_OUT; ++n) {
-      sts16(base + ST_DT + (uint32_t)((r >> 6) * 2048 + n * 128 + ((((r & 63) >> 3) ^ n) << 4) + (r & 7) * 2),
-            __float2bfloat16_rn(d[n]));
-      rest[n] = d[n];
-    }
-#pragma unroll
-    for (int p = 0; p < 3; ++p)
-#pragma unroll
-      for (int n = 0; n < MLP_OUT; n += 2) {
-        const __nv_bfloat162 b = __floats2bfloat162_rn(rest[n], rest[n + 1]);
-        part[p][n >> 1] = *reinterpret_cast<const uint32_t*>(&b);
-        rest[n] -= __bfloat162float(b.x);
-        rest[n + 1] -= __bfloat162float(b.y);
+  const int n_tiles = (a.M + 127) / 128;
+  uint32_t arrivals = 0;
+  for (int64_t s = 0; s < a.steps; ++s) {
+    for (int tile = blockIdx.x; tile < n_tiles; tile += (int)gridDim.x, ph_t ^= 1u) {
+      const int row0 = tile * 128;
+      const bool live = row0 + r < a.M, add = tile != (int)blockIdx.x;
+      auto source_row = [&](int row) {  // row of x and t behind row 'row' of the batch
+        const int64_t i = s * a.M + row;
+        return a.perm ? (size_t)a.perm[i] : (size_t)i;
+      };
+      if (tid == 0) {
+        // (the last tile's reads of these buffers are over; its generic
+        // writes to them come before the copies)
+        fence_async();
+        mbar_expect_tx(saddr(&b_w1), MLP_H * 64);
+        bulk_load(base + ST_W1, a.adam.wt + WT_W1, MLP_H * 64, saddr(&b_w1));
+        for (int c = 0; c < 4; ++c) {
+          mbar_expect_tx(saddr(&b_w2[c]), MLP_H * 128);
+          bulk_load(base + (c < 2 ? ST_W + c * 32768 : ST_G + (c - 2) * 32768),
+                    a.adam.wt + c * WT_CHUNK, MLP_H * 128, saddr(&b_w2[c]));
+        }
       }
+      {
+        // inputs: thread = row tid / 4 and 8 columns
+        const int xr = tid >> 2, part = tid & 3;
+        float v[8];
 #pragma unroll
-    for (int p = 0; p < 4; ++p)
-      sts128(base + ST_DA + (uint32_t)(r * 64 + ((p ^ ((r >> 1) & 3)) << 4)), p < 3 ? part[p < 3 ? p : 0][0] : 0u,
-             p < 3 ? part[p < 3 ? p : 0][1] : 0u, p < 3 ? part[p < 3 ? p : 0][2] : 0u,
-             p < 3 ? part[p < 3 ? p : 0][3] : 0u);
+        for (int i = 0; i < 8; ++i) v[i] = 0.0f;
+        if (row0 + xr < a.M) {
+          const float* src = a.x + source_row(row0 + xr) * MLP_IN + 8 * part;
+          if (((uintptr_t)src & 15u) == 0) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      l += __shfl_xor_sync(0xffffffffu, l, o);
+            for (int i = 0; i < 2; ++i) {
+              const float4 f = __ldg(reinterpret_cast<const float4*>(src) + i);
+              v[4 * i] = f.x; v[4 * i + 1] = f.y; v[4 * i + 2] = f.z; v[4 * i + 3] = f.w;
+            }
+          } else {
 #pragma unroll
-      for (int n = 0; n < MLP_OUT; ++n) d[n] += __shfl_xor_sync(0xffffffffu, d[n], o);
-    }
-    if (lane == 0 && *((volatile int*)&s_fail) == 0) {
-      atomicAdd(a.loss, l / (float)a.M);
+            for (int i = 0; i < 8; ++i) v[i] = __ldg(src + i);
+          }
+        }
+        sts128(base + ST_X + (uint32_t)(xr * 64 + ((part ^ ((xr >> 1) & 3)) << 4)), pack_bf16(v[0], v[1]),
+               pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
 #pragma unroll
-      for (int n = 0; n < MLP_OUT; ++n) atomicAdd(a.g_b3 + n, d[n]);
-    }
-  }
-  publish();
-
-  // ---- backward
-  if (tid == 0) {
-#pragma unroll
-    for (int m = 0; m < 2; ++m)
-#pragma unroll
-      for (int k = 0; k < 8; ++k)
-        mma_bf16(A0 + 16 + 16 * m, sdesc_mn128(base + ST_G + m * 32768 + k * 2048, 16384),
-                 sdesc_sw128(base + ST_DT + (k >> 2) * 2048 + (k & 3) * 32), ID_DW3, k != 0 ? 1u : 0u);
-#pragma unroll
-    for (int k = 0; k < 2; ++k)  // both K groups of W3's tile hold W3: parts 0 and 1, then 2 and zeros
-      mma_bf16(B0, sdesc_sw64(base + ST_DA + 32 * k), sdesc_mn128(base + ST_W3, 2048), ID_DH2,
-               k != 0 ? 1u : 0u);
-    mma_commit(saddr(&b_mma));
-  }
-  wait_mma(35);
-  mask(tl + 256, ST_G, ST_G);
-  if (*((volatile int*)&s_fail) == 0) {
-    uint32_t v[8];
-    tmem_ld8(tl + 16 + 16 * half, v);
-#pragma unroll
-    for (int n = 0; n < MLP_OUT; ++n)
-      atomicAdd(a.g_W3 + n * MLP_H + 128 * half + r, __uint_as_float(v[n]));
-  }
-  publish();
-  if (tid == 0) {
-    auto dh1_chunk = [&](int c) {
-#pragma unroll
-      for (int k = 0; k < 16; ++k)
-        mma_bf16(A0 + 64 * c, sdesc_sw128(base + ST_G + (k >> 2) * 16384 + (k & 3) * 32),
-                 sdesc_mn128(base + ST_W + (c & 1) * 32768 + k * 2048, 0), ID_DH1, k != 0 ? 1u : 0u);
-    };
-    for (int c = 0; c < 2; ++c) {
-      dh1_chunk(c);
-      mma_commit(saddr(&b_c[c]));
-    }
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-      mma_bf16(B0, sdesc_mn128(base + ST_G + k * 2048, 16384), sdesc_mn128(base + ST_H1 + k * 2048, 16384),
-               ID_DW2, k != 0 ? 1u : 0u);
-    mma_commit(saddr(&b_t0));
-    for (int c = 0; c < 2; ++c) {
-      wait(&b_c[c], 0, 36);
-      mbar_expect_tx(saddr(&b_r[c]), MLP_H * 128);
-      bulk_load(base + ST_W + c * 32768, a.wt + (2 + c) * WT_CHUNK, MLP_H * 128, saddr(&b_r[c]));
-    }
-    for (int c = 0; c < 2; ++c) {
-      wait(&b_r[c], 0, 37);
-      dh1_chunk(2 + c);
-    }
-    mma_commit(saddr(&b_mma));
-  }
-  __syncwarp();
-  wait(&b_t0, 0, 38);
-  __syncwarp();
-  fence_after();
-  add_dw2(tl + 256, 0);
-  wait_mma(39);
-  mask(tl, ST_H1, ST_W);
-  publish();
-  if (tid == 0) {
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-      mma_bf16(A0, sdesc_mn128(base + ST_G + 32768 + k * 2048, 16384),
-               sdesc_mn128(base + ST_H1 + k * 2048, 16384), ID_DW2, k != 0 ? 1u : 0u);
-#pragma unroll
-    for (int m = 0; m < 2; ++m)
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const uint32_t xt = base + ST_XT + (k >> 2) * 6144 + (k & 3) * 32;
-        mma_bf16(B0 + 48 * m, sdesc_mn128(base + ST_W + m * 32768 + k * 2048, 16384), sdesc_sw128(xt), ID_DW1,
-                 k != 0 ? 1u : 0u);
-        mma_bf16(B0 + 96 + 16 * m, sdesc_mn128(base + ST_G + m * 32768 + k * 2048, 16384),
-                 sdesc_sw128(xt + 4096), ID_DW3, k != 0 ? 1u : 0u);
+        for (int i = 0; i < 8; ++i)
+          sts16(base + ST_XT + (uint32_t)((xr >> 6) * 6144 + (8 * part + i) * 128 +
+                                          ((((xr & 63) >> 3) ^ i) << 4) + (xr & 7) * 2),
+                __float2bfloat16_rn(v[i]));
       }
-    mma_commit(saddr(&b_mma));
-  }
-  wait_mma(40);
-  if (*((volatile int*)&s_fail) == 0) {
-    const int o = 128 * half + r;
-    uint32_t v[32], s[8];
-    tmem_ld32(tl + 256 + 48 * half, v);
+      {
+        // W3 twice, the biases (read past L1: the last step's optimiser ran
+        // on other SMs too)
+        const int c = tid >> 7, copy = (tid >> 6) & 1, n = (tid >> 3) & 7, j = tid & 7;
+        const uint4 w = __ldcg(reinterpret_cast<const uint4*>(a.adam.w3 + n * MLP_H + 64 * c + 8 * j));
+        sts128(base + ST_W3 + (uint32_t)(c * 2048 + copy * 1024 + n * 128 + ((j ^ n) << 4)), w.x, w.y, w.z,
+               w.w);
+        const float b = __ldcg(par + (tid < MLP_H ? OFF_B1 + tid : OFF_B2 + tid - MLP_H));
+        asm volatile("st.shared.f32 [%0], %1;" ::"r"(base + ST_B1 + 4 * tid), "f"(b) : "memory");
+        if (tid < MLP_OUT) s_b3[tid] = __ldcg(par + OFF_B3 + tid);
+      }
+      // target qt of row r
+      const float tv = live ? __ldg(a.t + source_row(row0 + r) * MLP_NQ + qt) : 0.0f;
+      publish();
+
+      // ---- forward
+      if (tid == 0) {
+        wait(&b_w1, ph_t, 30);
+        fence_after();
 #pragma unroll
-    for (int j = 0; j < 32; j += 4) red_add4(a.g_W1 + (size_t)o * MLP_IN + j, v + j);
-    tmem_ld8(tl + 256 + 48 * half + 32, s);
-    atomicAdd(a.g_b1 + o, __uint_as_float(s[0]));
-    tmem_ld8(tl + 256 + 96 + 16 * half, s);
-    atomicAdd(a.g_b2 + o, __uint_as_float(s[0]));
+        for (int k = 0; k < 2; ++k)
+          mma_bf16(A0, sdesc_sw64(base + ST_X + 32 * k), sdesc_sw64(base + ST_W1 + 32 * k), ID_FWD,
+                   k != 0 ? 1u : 0u);
+        mma_commit(saddr(&b_mma));
+      }
+      wait_mma(31);
+      activate(tl, ST_H1, ST_B1, live);
+      publish();
+      if (tid == 0) {
+        for (int c = 0; c < 4; ++c) {
+          wait(&b_w2[c], ph_t, 32);
+          const uint32_t w = base + (c < 2 ? ST_W + c * 32768 : ST_G + (c - 2) * 32768);
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            mma_bf16(B0, sdesc_sw128(base + ST_H1 + c * 16384 + 32 * k), sdesc_sw128(w + 32 * k), ID_FWD,
+                     (c | k) != 0 ? 1u : 0u);
+        }
+        mma_commit(saddr(&b_mma));
+      }
+      wait_mma(33);
+      activate(tl + 256, ST_G, ST_B2, live);
+      publish();
+      if (tid == 0) {
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            mma_bf16(A0, sdesc_sw128(base + ST_G + c * 16384 + 32 * k),
+                     sdesc_sw128(base + ST_W3 + c * 2048 + 32 * k), ID_RAW, (c | k) != 0 ? 1u : 0u);
+        mma_commit(saddr(&b_mma));
+      }
+      wait_mma(34);
+
+      // ---- loss and the outputs' gradient: a thread a row and output pair
+      // (mean qt, log standard deviation qt)
+      {
+        uint32_t raw[8];
+        tmem_ld8(tl, raw);
+        const float inv_m = 1.0f / (float)a.M;
+        const float rm = __uint_as_float(qt == 0 ? raw[0] : qt == 1 ? raw[1] : qt == 2 ? raw[2] : raw[3]);
+        const float rs = __uint_as_float(qt == 0 ? raw[4] : qt == 1 ? raw[5] : qt == 2 ? raw[6] : raw[7]);
+        const float mu = tanhf(rm + s_b3[qt]);
+        const float lr = rs + s_b3[MLP_NQ + qt];
+        const bool clamped = lr < MLP_LOGSTD_MIN || lr > MLP_LOGSTD_MAX;
+        const float ls = fminf(fmaxf(lr, MLP_LOGSTD_MIN), MLP_LOGSTD_MAX);
+        const float is = expf(-ls);
+        const float z = (tv - mu) * is;
+        float sum[3] = {live ? ls + 0.5f * z * z : 0.0f,
+                        live ? -z * is * (1.0f - mu * mu) * inv_m : 0.0f,
+                        live && !clamped ? (1.0f - z * z) * inv_m : 0.0f};
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const int n = qt + MLP_NQ * i;
+          const float d = sum[1 + i];
+          // three BF16 parts of the value: rounding, then what is left, twice
+          const __nv_bfloat16 p0 = __float2bfloat16_rn(d);
+          const float r1 = d - __bfloat162float(p0);
+          const __nv_bfloat16 p1 = __float2bfloat16_rn(r1);
+          const __nv_bfloat16 p2 = __float2bfloat16_rn(r1 - __bfloat162float(p1));
+          sts16(base + ST_DT + (uint32_t)((r >> 6) * 2048 + n * 128 + ((((r & 63) >> 3) ^ n) << 4) +
+                                          (r & 7) * 2),
+                p0);
+          const uint32_t da = base + ST_DA + (uint32_t)(r * 64 + 2 * n), sw = (uint32_t)((r >> 1) & 3);
+          sts16(da + ((0u ^ sw) << 4), p0);
+          sts16(da + ((1u ^ sw) << 4), p1);
+          sts16(da + ((2u ^ sw) << 4), p2);
+          sts16(da + ((3u ^ sw) << 4), __float2bfloat16_rn(0.0f));
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+          for (int i = 0; i < 3; ++i) sum[i] += __shfl_xor_sync(0xffffffffu, sum[i], o);
+        if (lane == 0)
+#pragma unroll
+          for (int i = 0; i < 3; ++i) s_red[q][qt][i] = sum[i];
+      }
+      publish();
+
+      // ---- backward
+      if (tid == 0) {
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+            mma_bf16(A0 + 16 + 16 * m, sdesc_mn128(base + ST_G + m * 32768 + k * 2048, 16384),
+                     sdesc_sw128(base + ST_DT + (k >> 2) * 2048 + (k & 3) * 32), ID_DW3, k != 0 ? 1u : 0u);
+#pragma unroll
+        for (int k = 0; k < 2; ++k)  // both K groups of W3's tile hold W3: parts 0 and 1, then 2 and zeros
+          mma_bf16(B0, sdesc_sw64(base + ST_DA + 32 * k), sdesc_mn128(base + ST_W3, 2048), ID_DH2,
+                   k != 0 ? 1u : 0u);
+        mma_commit(saddr(&b_mma));
+      }
+      if (tid >= 64 && tid < 64 + MLP_OUT + 1) {  // db3 and the loss from the warps' sums
+        const int n = tid - 64;
+        float sum = 0.0f;
+        for (int w = 0; w < 4; ++w) {
+          if (n < MLP_OUT) {
+            sum += s_red[w][n & 3][1 + (n >> 2)];
+          } else {
+            for (int i = 0; i < MLP_NQ; ++i) sum += s_red[w][i][0];
+          }
+        }
+        slot_put(g + (n < MLP_OUT ? OFF_B3 + n : N_PARAMS), n < MLP_OUT ? sum : sum / (float)a.M, add);
+      }
+      wait_mma(35);
+      mask(tl + 256, ST_G, ST_G);
+      if (qt < 2) {
+        uint32_t v[8];
+        tmem_ld8(tl + 16 + 16 * qt, v);
+#pragma unroll
+        for (int n = 0; n < MLP_OUT; ++n)
+          slot_put(g + OFF_W3 + n * MLP_H + 128 * qt + r, __uint_as_float(v[n]), add);
+      }
+      publish();
+      if (tid == 0) {
+        auto dh1_half = [&](int c) {  // 128 columns: two chunks of W2
+#pragma unroll
+          for (int k = 0; k < 16; ++k)
+            mma_bf16(A0 + 128 * c, sdesc_sw128(base + ST_G + (k >> 2) * 16384 + (k & 3) * 32),
+                     sdesc_mn128(base + ST_W + k * 2048, 32768), ID_DH1, k != 0 ? 1u : 0u);
+        };
+        dh1_half(0);
+        mma_commit(saddr(&b_c));
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          mma_bf16(B0, sdesc_mn128(base + ST_G + k * 2048, 16384),
+                   sdesc_mn128(base + ST_H1 + k * 2048, 16384), ID_DW2, k != 0 ? 1u : 0u);
+        wait(&b_c, ph_t, 36);
+        mbar_expect_tx(saddr(&b_r), 2 * MLP_H * 128);
+        for (int c = 0; c < 2; ++c)
+          bulk_load(base + ST_W + c * 32768, a.adam.wt + (2 + c) * WT_CHUNK, MLP_H * 128, saddr(&b_r));
+        wait(&b_r, ph_t, 37);
+        dh1_half(1);
+        mma_commit(saddr(&b_mma));
+      }
+      wait_mma(39);
+      mask(tl, ST_H1, ST_W);
+      publish();
+      if (tid == 0) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          mma_bf16(A0, sdesc_mn128(base + ST_G + 32768 + k * 2048, 16384),
+                   sdesc_mn128(base + ST_H1 + k * 2048, 16384), ID_DW2, k != 0 ? 1u : 0u);
+        mma_commit(saddr(&b_t0));
+      }
+      __syncwarp();
+      put_dw2(tl + 256, 0, add);  // beside the second half's products
+      publish();
+      if (tid == 0) {
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            const uint32_t xt = base + ST_XT + (k >> 2) * 6144 + (k & 3) * 32;
+            mma_bf16(B0 + 48 * m, sdesc_mn128(base + ST_W + m * 32768 + k * 2048, 16384), sdesc_sw128(xt),
+                     ID_DW1, k != 0 ? 1u : 0u);
+            mma_bf16(B0 + 96 + 16 * m, sdesc_mn128(base + ST_G + m * 32768 + k * 2048, 16384),
+                     sdesc_sw128(xt + 4096), ID_DW3, k != 0 ? 1u : 0u);
+          }
+        mma_commit(saddr(&b_mma));
+      }
+      __syncwarp();
+      wait(&b_t0, ph_t, 38);
+      __syncwarp();
+      fence_after();
+      put_dw2(tl, 1, add);
+      wait_mma(40);
+      {
+        const int o = 128 * (qt & 1) + r;
+        uint32_t v[8];
+        if (qt < 2) {
+#pragma unroll
+          for (int j = 0; j < 8; j += 2) {
+            tmem_ld8(tl + 256 + 48 * qt + (uint32_t)(4 * j), v);
+            slot_put4(g + 4 * slot_group_w1(qt, q, j, lane), v, add);
+            slot_put4(g + 4 * slot_group_w1(qt, q, j + 1, lane), v + 4, add);
+          }
+          tmem_ld8(tl + 256 + 48 * qt + 32, v);
+          slot_put(g + OFF_B1 + o, __uint_as_float(v[0]), add);
+        } else {
+          tmem_ld8(tl + 256 + 96 + 16 * (qt - 2), v);
+          slot_put(g + OFF_B2 + o, __uint_as_float(v[0]), add);
+        }
+      }
+      fence_before();
+      __syncthreads();
+      fence_after();
+    }
+    if (!a.epoch) break;
+    // ---- optimiser: every tile's gradient is in; this CTA's share of the
+    // parameters; then the next mini-batch may read them
+    __syncthreads();
+    arrivals += gridDim.x;
+    if (tid == 0 && (failed1() || !grid_arrive_wait(a.bar, arrivals, a.err, a.wait_ns))) {
+      if (!failed1()) s_fail = 50;
+      atomicExch(a.err, 100 + s_fail);  // the other CTAs' barrier waits see it
+    }
+    __syncthreads();
+    if (failed()) break;
+    float c1, c2;
+    adam_corrections((int)(a.step0 + s + 1), &c1, &c2);
+    // groups of four parameters, the loss after them; a warp's groups are
+    // consecutive, the warps of all CTAs take turns
+    for (int i = ((int)blockIdx.x + (int)gridDim.x * warp) * 32 + lane; i <= N_PARAMS / 4;
+         i += (int)gridDim.x * ST_THREADS) {
+      if (i < N_PARAMS / 4)
+        adam_update(a.adam, i, c1, c2);
+      else
+        *a.loss_sum += slot_sum(a.adam.slots, a.adam.n_slots, i).x;
+    }
+    asm volatile("fence.proxy.async;" ::: "memory");  // the BF16 copies are read by bulk copies
+    __syncthreads();
+    arrivals += gridDim.x;
+    if (tid == 0 && !grid_arrive_wait(a.bar, arrivals, a.err, a.wait_ns)) {
+      s_fail = 51;
+      atomicExch(a.err, 100 + s_fail);
+    }
+    __syncthreads();
+    if (failed()) break;
   }
-  add_dw2(tl, 128);
   fence_before();
   __syncthreads();
   if (warp == 0) {
@@ -929,9 +1116,9 @@ __global__ void __launch_bounds__(ST_THREADS, 1) kp_mlp_step_kernel(StepArgs a) 
   }
   if (tid == 0 && s_fail) {
     // a wait gave up: copies may be in flight, wait for them once more
-    mbar_wait(saddr(&b_w1), 0, a.wait_ns);
-    for (int c = 0; c < 4; ++c) mbar_wait(saddr(&b_w2[c]), 0, a.wait_ns);
-    for (int c = 0; c < 2; ++c) mbar_wait(saddr(&b_r[c]), 0, a.wait_ns);
+    mbar_wait(saddr(&b_w1), ph_t, a.wait_ns);
+    for (int c = 0; c < 4; ++c) mbar_wait(saddr(&b_w2[c]), ph_t, a.wait_ns);
+    mbar_wait(saddr(&b_r), ph_t, a.wait_ns);
     atomicExch(a.err, 100 + s_fail);
   }
 }
