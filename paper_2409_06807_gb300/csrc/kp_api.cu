@@ -253,6 +253,7 @@ struct kp_ctx {
   kp_goal goal;
   uint64_t seed;
   bool have_tree;
+  bool tree_outside;  // an imported tree has states outside the state box
   bool poisoned;
   bool log_on;
   KLog log;
@@ -347,6 +348,7 @@ KParams params_now(kp_ctx* c) {
   P.seed_hi = (uint32_t)(c->seed >> 32);
   P.log = c->log_on ? c->log : KLog{};
   P.wait_ns = c->wait_ns;
+  if (c->tree_outside) P.state_inside = P.small_angles = 0;
   return P;
 }
 
@@ -554,6 +556,8 @@ size_t build_blob(unsigned char* blob, const float* boxes, int nb, const kp_work
     P.bp_scale[a] = scale[a];
     P.bp_last[a] = (float)(g[a] - 1);
   }
+  P.bp_gxy = g[0] * g[1];
+  P.bp_bias = bp_bias_of(P.bp_g);
   P.bp_start_off = (int32_t)start_off;
   P.bp_ids_off = (int32_t)ids_off;
   return bytes;
@@ -793,10 +797,40 @@ kp_status enqueue_reset(kp_ctx* ctx, const float* x_init) {
     if (std::isnan(x_init[i])) return fail(ctx, KP_ERR_ARG, "NaN in x_init");
   RootState root{};
   for (int i = 0; i < ctx->dims.D; ++i) root.x[i] = x_init[i];
+  ctx->tree_outside = false;
   KParams P = params_now(ctx);
   KP_CUDA(launch_reset(ctx, P, root));
   ctx->have_tree = true;
   return KP_OK;
+}
+
+// Whether at every stage of an integrator step from the state box the
+// quadrotor's roll and pitch stay in (-3, 3): bounds of the angles and rates after each stage, in
+// the stages' order (the margin to pi is far above the FP32 rounding of the
+// stages).
+bool angles_small(const kp_system* sys) {
+  const double h = sys->dt, lim = 3.0;
+  auto mag = [&](int i) { return std::max(std::fabs((double)sys->x_lo[i]), std::fabs((double)sys->x_hi[i])); };
+  double u = 0.0;
+  for (int i = 0; i < 4; ++i)
+    u = std::max(u, std::max(std::fabs((double)sys->u_lo[i]), std::fabs((double)sys->u_hi[i])));
+  if (sys->id != KP_QUADROTOR_12D) return false;
+  // roll' = p + tan(pitch) (..), |..| <= 2 w; pitch' at most 2 w; omega' =
+  // (tau - omega x I omega) / I
+  const double a0 = std::max(mag(3), mag(4)), w0 = std::max(mag(9), std::max(mag(10), mag(11)));
+  const double tau = std::max(2.0 * std::fabs((double)sys->phys[2]), 4.0 * std::fabs((double)sys->phys[3])) * u;
+  const double imin = std::min({(double)sys->phys[4], (double)sys->phys[5], (double)sys->phys[6]});
+  const double imax = std::max({(double)sys->phys[4], (double)sys->phys[5], (double)sys->phys[6]});
+  double a = a0, w = w0;
+  for (int stage = 0; stage < 3; ++stage) {
+    if (!(a < 1.5) || !(w < 1e6)) return false;  // tan below 15
+    const double c = stage < 2 ? 0.5 * h : h;
+    const double da = w + 2.0 * w * std::max(1.0, std::tan(a));
+    const double dw = (tau + 2.0 * imax * w * w) / imin;
+    a = a0 + c * da;
+    w = w0 + c * dw;
+  }
+  return a < lim;
 }
 
 // Launch constants and arena slices of a validated problem.
@@ -859,6 +893,13 @@ void fill_params(KParams& P, const Dims& d, const Layout& lay, const kp_system* 
   P.delta = prm->delta;
   P.eps = prm->eps;
   P.vol = vol;
+  P.state_inside = 1;
+  for (int a = 0; a < 3; ++a)
+    if (!(sys->x_lo[a] >= ws->lo[a] && sys->x_hi[a] <= ws->hi[a])) P.state_inside = 0;
+  P.small_angles = angles_small(sys) ? 1 : 0;
+  P.state_symmetric = 1;
+  for (int i = 3; i < (d.sys == KP_SYS_DUBINS ? 5 : d.D); ++i)
+    if (sys->x_lo[i] != -sys->x_hi[i]) P.state_symmetric = 0;
   P.fso = d.fso;
   P.kd_smem_off = -1;
   P.bp_clear_off = -1;
@@ -1067,6 +1108,7 @@ kp_status kp_plan_async(kp_ctx* ctx, const float* x_init, const kp_goal* goal,
   ctx->goal = *goal;
   RootState root{};
   for (int i = 0; i < ctx->dims.D; ++i) root.x[i] = x_init[i];
+  ctx->tree_outside = false;
   KParams P = params_now(ctx);
   const uint64_t max_ns = budget->max_ms > 0.0 ? (uint64_t)(budget->max_ms * 1e6) : 0ull;
   // one launch: initialisation, the passes, the chain
@@ -1228,7 +1270,12 @@ kp_status kp_import_tree(kp_ctx* ctx, const kp_tree_view* v) {
   const Layout& L = ctx->lay;
   std::vector<float> st((size_t)D * n), ct((size_t)N * n);
   std::vector<uint8_t> steps(n), inve(n);
+  bool outside = false;
   for (int u = 0; u < n; ++u) {
+    for (int i = 0; i < D; ++i) {
+      const float x = v->state[(size_t)u * 12 + i];
+      outside = outside || !(ctx->sys.x_lo[i] <= x && x <= ctx->sys.x_hi[i]);
+    }
     for (int i = 0; i < D; ++i) st[(size_t)i * n + u] = v->state[(size_t)u * 12 + i];
     for (int i = 0; i < N; ++i) ct[(size_t)i * n + u] = v->ctrl[(size_t)u * 4 + i];
     steps[u] = (uint8_t)v->steps[u];
@@ -1252,6 +1299,7 @@ kp_status kp_import_tree(kp_ctx* ctx, const kp_tree_view* v) {
   if ((s = h2d(L.thr, v->thr, (size_t)R * 8)) != KP_OK) return s;
   if ((s = h2d(L.visited, v->visited, ctx->dims.n_sub)) != KP_OK) return s;
   KP_CUDA(cudaMemsetAsync(ctx->arena + L.claim, 0xff, ctx->dims.n_sub * 4, ctx->stream));
+  ctx->tree_outside = outside;
   KParams P = params_now(ctx);
   kp_import_regions_kernel<<<(R + 255) / 256 < 1024 ? (R + 255) / 256 : 1024, 256, 0, ctx->stream>>>(P);
   KP_CUDA(cudaGetLastError());
@@ -1352,6 +1400,8 @@ kp_status kp_grow(kp_ctx* ctx, void* dev_arena, size_t arena_bytes, int32_t t_e)
   P.bp_n_ids = old.bp_n_ids;
   for (int a = 0; a < 3; ++a) P.bp_scale[a] = old.bp_scale[a];
   for (int a = 0; a < 3; ++a) P.bp_last[a] = old.bp_last[a];
+  P.bp_gxy = old.bp_gxy;
+  P.bp_bias = old.bp_bias;
   P.nch = old.nch;
   P.sd_bytes = old.sd_bytes;
   P.extract_cap = old.extract_cap;
@@ -1854,6 +1904,8 @@ extern "C" kp_status kp_plan_static(const kp_system* sys, const kp_workspace* ws
         P.bp_scale[a] = sc[a];
         P.bp_last[a] = (float)(gc - 1);
       }
+      P.bp_gxy = gc * gc;
+      P.bp_bias = bp_bias_of(P.bp_g);
       P.bp_start_off = pad * 32;
       P.bp_ids_off = P.bp_start_off + (int32_t)round16((cells3 + 1) * 2);
       P.bp_clear_off = P.bp_ids_off + (int32_t)round16((size_t)entries * 2);

@@ -223,6 +223,17 @@ __device__ __forceinline__ void sincos_reduced(float x, float* s, float* c) {
   __sincosf(r, s, c);
 }
 
+// Sine and cosine of an angle known to lie in (-3, 3) when SMALL: the
+// reduction above leaves such an angle as it is (k = 0), but for a -0, which
+// it makes +0 as the addition here does.  One instruction instead of four.
+template <bool SMALL>
+__device__ __forceinline__ void sincos_bounded(float x, float* s, float* c) {
+  if (SMALL)
+    __sincosf(__fadd_rn(x, 0.0f), s, c);
+  else
+    sincos_reduced(x, s, c);
+}
+
 // ---------------------------------------------------------------------------
 // systems (Sec. II, Eq. 1-2), FP32 in registers
 //
@@ -239,6 +250,7 @@ struct System;
 // 6D double integrator: p' = v, v' = u; explicit Euler.
 template <>
 struct System<KP_SYS_DI> {
+  static constexpr int SYM0 = 3, SYM1 = 6;
   static constexpr int D = 6, N = 3;
   // finished lanes a warp waits for before it finalises and refills them
   // (measured on the GB300: cheap steps favour large refill groups; for
@@ -274,10 +286,55 @@ struct System<KP_SYS_DI> {
 // one stage derivative is live at a time (the register budget of the loop
 // kernel holds no four of them for the 12D system).  F(t, k) evaluates the
 // field at t into k.
+// Two FP32 fused multiply-adds (additions) in one instruction, each correctly
+// rounded as the single ones.
+__device__ __forceinline__ void fma2(float s, const float* a, const float* b, float* r) {
+  asm("{\n .reg .b64 p, q, t;\n mov.b64 p, {%2, %2};\n mov.b64 q, {%3, %4};\n mov.b64 t, {%5, %6};\n"
+      " fma.rn.f32x2 t, p, q, t;\n mov.b64 {%0, %1}, t;\n}"
+      : "=f"(r[0]), "=f"(r[1])
+      : "f"(s), "f"(a[0]), "f"(a[1]), "f"(b[0]), "f"(b[1]));
+}
+
+__device__ __forceinline__ void add2(const float* a, const float* b, float* r) {
+  asm("{\n .reg .b64 q, t;\n mov.b64 q, {%2, %3};\n mov.b64 t, {%4, %5};\n"
+      " add.rn.f32x2 t, q, t;\n mov.b64 {%0, %1}, t;\n}"
+      : "=f"(r[0]), "=f"(r[1])
+      : "f"(a[0]), "f"(a[1]), "f"(b[0]), "f"(b[1]));
+}
+
 template <int D, class F>
 __device__ __forceinline__ void rk4_step(float* x, float h, float h6, F field) {
   float acc[D], k[D], t[D];
   const float hh = __fmul_rn(0.5f, h);
+  if (D == 12) {
+    // the quadrotor's stage points and combination two dimensions at a time
+    field(x, k);
+#pragma unroll
+    for (int i = 0; i < D; i += 2) {
+      acc[i] = k[i];
+      acc[i + 1] = k[i + 1];
+      fma2(hh, k + i, x + i, t + i);
+    }
+    field(t, k);
+#pragma unroll
+    for (int i = 0; i < D; i += 2) {
+      fma2(2.0f, k + i, acc + i, acc + i);
+      fma2(hh, k + i, x + i, t + i);
+    }
+    field(t, k);
+#pragma unroll
+    for (int i = 0; i < D; i += 2) {
+      fma2(2.0f, k + i, acc + i, acc + i);
+      fma2(h, k + i, x + i, t + i);
+    }
+    field(t, k);
+#pragma unroll
+    for (int i = 0; i < D; i += 2) {
+      add2(acc + i, k + i, acc + i);
+      fma2(h6, acc + i, x + i, x + i);
+    }
+    return;
+  }
   field(x, k);
 #pragma unroll
   for (int i = 0; i < D; ++i) {
@@ -304,6 +361,7 @@ __device__ __forceinline__ void rk4_step(float* x, float h, float h6, F field) {
 // 6D Dubins airplane (Chitsaz & LaValle 2007); classic RK4.
 template <>
 struct System<KP_SYS_DUBINS> {
+  static constexpr int SYM0 = 3, SYM1 = 5;
   static constexpr int D = 6, N = 3;
   static constexpr int REFILL_MIN = 16;
   static constexpr int FIRST_BATCH_MIN = 16;
@@ -330,18 +388,20 @@ struct System<KP_SYS_DUBINS> {
 // x = (p, phi theta psi, v_world, omega_body); u = rotor thrusts T1..T4.
 template <>
 struct System<KP_SYS_QUAD> {
+  static constexpr int SYM0 = 3, SYM1 = 12;
   static constexpr int D = 12, N = 4;
   static constexpr int REFILL_MIN = 12;
   static constexpr int FIRST_BATCH_MIN = 16;
   static constexpr int GUIDED_DIV = 4;
+  template <bool SMALL>
   __device__ __forceinline__ static void f(const float* x, const float* u, const KParams& P,
                                            float* dx) {
     // phys: m g l c Ixx Iyy Izz; recip: 1/m 1/Ixx 1/Iyy 1/Izz
     const float g = P.phys[1], l = P.phys[2], c = P.phys[3];
     const float Ix = P.phys[4], Iy = P.phys[5], Iz = P.phys[6];
     float sphi, cphi, sth, cth, sps, cps;
-    sincos_reduced(x[3], &sphi, &cphi);
-    sincos_reduced(x[4], &sth, &cth);
+    sincos_bounded<SMALL>(x[3], &sphi, &cphi);
+    sincos_bounded<SMALL>(x[4], &sth, &cth);
     sincos_reduced(x[5], &sps, &cps);
     const float sec = __frcp_rn(cth);
     const float tth = __fmul_rn(sth, sec);
@@ -371,7 +431,10 @@ struct System<KP_SYS_QUAD> {
   }
   __device__ __forceinline__ static void step(float* x, const float* u, float h,
                                               const KParams& P) {
-    rk4_step<12>(x, h, P.dt_sixth, [&](const float* y, float* dy) { f(y, u, P, dy); });
+    if (P.small_angles)
+      rk4_step<12>(x, h, P.dt_sixth, [&](const float* y, float* dy) { f<true>(y, u, P, dy); });
+    else
+      rk4_step<12>(x, h, P.dt_sixth, [&](const float* y, float* dy) { f<false>(y, u, P, dy); });
   }
   __device__ __forceinline__ static float speed(const float* x) {
     return sqrtf(__fmaf_rn(x[8], x[8], __fmaf_rn(x[7], x[7], __fmul_rn(x[6], x[6]))));
@@ -470,11 +533,22 @@ __device__ __forceinline__ void bin_state(const float* x, const KParams& P, int*
 // validity (Sec. II valid set): state box and segment hull vs closed boxes
 // ---------------------------------------------------------------------------
 
-template <int D>
+// Dimensions SYM0 .. SYM1 - 1 of a system usually have bounds of one size on
+// both sides (state_symmetric, from the host): one comparison of the magnitude
+// then does for two (compares issue at half the rate of FP32 arithmetic).
+template <class Sys>
 __device__ __forceinline__ bool in_state_box(const float* x, const KParams& P) {
   bool ok = true;
 #pragma unroll
-  for (int i = 0; i < D; ++i) ok &= (P.x_lo[i] <= x[i]) & (x[i] <= P.x_hi[i]);
+  for (int i = 0; i < Sys::D; ++i)
+    if (i < Sys::SYM0 || i >= Sys::SYM1) ok &= (P.x_lo[i] <= x[i]) & (x[i] <= P.x_hi[i]);
+  if (P.state_symmetric) {
+#pragma unroll
+    for (int i = Sys::SYM0; i < Sys::SYM1; ++i) ok &= fabsf(x[i]) <= P.x_hi[i];
+    return ok;
+  }
+#pragma unroll
+  for (int i = Sys::SYM0; i < Sys::SYM1; ++i) ok &= (P.x_lo[i] <= x[i]) & (x[i] <= P.x_hi[i]);
   return ok;
 }
 
@@ -509,48 +583,78 @@ __device__ __forceinline__ float byte_as_float(uint32_t q) {
   return __fsub_rn(__int_as_float(0x4B000000 | q), 8388608.0f);
 }
 
-// Exact coarse-then-fine collision test of a step hull (the paper's coarse
-// phase, Sec. III-B).  First the clearance of the cell holding the hull's
-// low corner: a hull inside that cell grown by its clearance on every side
-// meets no box (the clearance is a lower bound on the L-infinity gap, per
-// axis in cell units, from the cell to every box; the host subtracts a
-// margin far above the FP32 rounding of the cell coordinates).  Otherwise
-// only the boxes listed in the uniform-grid cells the hull touches are
-// tested: a box meeting the hull shares a point with it, that point's cell
-// lies in both cell ranges (the cell map is monotone), so the box is in
-// one of the visited lists.  Either way the verdict equals testing every
-// box.  'tests' counts the box tests made.
+// Whether the hull (low and high corners tl, th in cell units) lies in the cell
+// of its low corner grown by that cell's clearance: it then meets no box.  The
+// clearance q / 16 is a lower bound on the L-infinity gap, per axis in cell
+// units, from the cell to every box (the host subtracts a margin far above the
+// FP32 rounding of the cell coordinates).  INSIDE: the hull's low corner lies
+// in the workspace, so it is in its cell and only the high corner can leave
+// the grown cell; otherwise both sides are checked and the cell is clamped.
+// The one comparison is d <= 1 + q / 16 for the largest distance d of the hull
+// from the cell's low corner (or, outside, of the cell's low corner from it
+// plus 1), taken as an integer: 16 d - 16 rounded up against q.  Minimum,
+// maximum, compare and logic instructions issue at half the rate of FP32
+// additions and products on this GPU, so the test is written with few of them.
+template <bool INSIDE>
+__device__ __forceinline__ bool hull_clear(const KParams& P, const uint8_t* __restrict__ sclear,
+                                           const float* tl, const float* th) {
+  float d[3];
+  int v[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const float c = fminf(INSIDE ? tl[a] : fmaxf(tl[a], 0.0f), P.bp_last[a]);
+    const float f2 = __fadd_rd(c, 8388608.0f);
+    const float f = __fsub_rn(f2, 8388608.0f);
+    v[a] = __float_as_int(f2);
+    d[a] = __fsub_rn(th[a], f);
+    if (!INSIDE) d[a] = fmaxf(d[a], __fadd_rn(__fsub_rn(f, tl[a]), 1.0f));
+  }
+  const int c = KP_IDX(P, v[0] + P.bp_g[0] * v[1] + P.bp_gxy * v[2] - P.bp_bias,
+                       P.bp_g[0] * P.bp_g[1] * P.bp_g[2], 60);
+  const int q = sclear[c];
+  const int e = __float_as_int(__fmaf_ru(fmaxf(fmaxf(d[0], d[1]), d[2]), 16.0f, 8388592.0f));
+  return q != 0 && e - 0x4B000000 <= q;
+}
+
+// Exact coarse-then-fine collision test of the hull of a step from p to x (the
+// paper's coarse phase, Sec. III-B).  First the clearance of the cell holding
+// the hull's low corner (hull_clear).  Otherwise only the boxes listed in the
+// uniform-grid cells the hull touches are tested: a box meeting the hull
+// shares a point with it, that point's cell lies in both cell ranges (the cell
+// map is monotone), so the box is in one of the visited lists.  Either way the
+// verdict equals testing every box.  'tests' counts the box tests made.
 __device__ __forceinline__ bool hull_hits_grid(const KParams& P, const float4* __restrict__ sbox,
                                                const uint16_t* __restrict__ sstart,
                                                const uint16_t* __restrict__ sids,
-                                               const uint8_t* __restrict__ sclear, float lx,
-                                               float ly, float lz, float hx, float hy, float hz,
-                                               uint32_t* tests) {
-  const int gx = P.bp_g[0], gy = P.bp_g[1], gz = P.bp_g[2];
-  const float tlx = __fmul_rn(__fsub_rn(lx, P.ws_lo[0]), P.bp_scale[0]);
-  const float thx = __fmul_rn(__fsub_rn(hx, P.ws_lo[0]), P.bp_scale[0]);
-  const float tly = __fmul_rn(__fsub_rn(ly, P.ws_lo[1]), P.bp_scale[1]);
-  const float thy = __fmul_rn(__fsub_rn(hy, P.ws_lo[1]), P.bp_scale[1]);
-  const float tlz = __fmul_rn(__fsub_rn(lz, P.ws_lo[2]), P.bp_scale[2]);
-  const float thz = __fmul_rn(__fsub_rn(hz, P.ws_lo[2]), P.bp_scale[2]);
-  float fx, fy, fz, dummy;
-  const int x0 = bp_cell_of(tlx, P.bp_last[0], &fx), x1 = bp_cell_of(thx, P.bp_last[0], &dummy);
-  const int y0 = bp_cell_of(tly, P.bp_last[1], &fy), y1 = bp_cell_of(thy, P.bp_last[1], &dummy);
-  const int z0 = bp_cell_of(tlz, P.bp_last[2], &fz), z1 = bp_cell_of(thz, P.bp_last[2], &dummy);
-  if (sclear != nullptr) {
-    const float r =
-        __fmul_rn(byte_as_float(sclear[KP_IDX(P, x0 + gx * (y0 + gy * z0), gx * gy * gz, 60)]),
-                  0.0625f);
-    if (r > 0.0f && tlx >= fx - r && thx <= fx + 1.0f + r && tly >= fy - r &&
-        thy <= fy + 1.0f + r && tlz >= fz - r && thz <= fz + 1.0f + r)
-      return false;
+                                               const uint8_t* __restrict__ sclear, const float* p,
+                                               const float* x, uint32_t* tests) {
+  // corners in cell units (the map is monotone, so the corners' cells come
+  // from the smaller and the larger end)
+  float tl[3], th[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const float t0 = __fmul_rn(__fsub_rn(p[a], P.ws_lo[a]), P.bp_scale[a]);
+    const float t1 = __fmul_rn(__fsub_rn(x[a], P.ws_lo[a]), P.bp_scale[a]);
+    tl[a] = fminf(t0, t1);
+    th[a] = fmaxf(t0, t1);
   }
+  if (sclear != nullptr &&
+      (P.state_inside ? hull_clear<true>(P, sclear, tl, th) : hull_clear<false>(P, sclear, tl, th)))
+    return false;
+  const int gx = P.bp_g[0], gy = P.bp_g[1];
+  float dummy;
+  const int x0 = bp_cell_of(tl[0], P.bp_last[0], &dummy), x1 = bp_cell_of(th[0], P.bp_last[0], &dummy);
+  const int y0 = bp_cell_of(tl[1], P.bp_last[1], &dummy), y1 = bp_cell_of(th[1], P.bp_last[1], &dummy);
+  const int z0 = bp_cell_of(tl[2], P.bp_last[2], &dummy), z1 = bp_cell_of(th[2], P.bp_last[2], &dummy);
+  // + 0.0f turns a -0 into +0 for the box test
+  const float lx = fminf(p[0], x[0]) + 0.0f, ly = fminf(p[1], x[1]) + 0.0f, lz = fminf(p[2], x[2]) + 0.0f;
+  const float hx = fmaxf(p[0], x[0]) + 0.0f, hy = fmaxf(p[1], x[1]) + 0.0f, hz = fmaxf(p[2], x[2]) + 0.0f;
   uint32_t n = 0;
   bool hit = false;
   for (int cz = z0; cz <= z1 && !hit; ++cz)
     for (int cy = y0; cy <= y1 && !hit; ++cy)
       for (int cx = x0; cx <= x1 && !hit; ++cx) {
-        const int c = KP_IDX(P, cx + gx * (cy + gy * cz), gx * gy * gz, 61);
+        const int c = KP_IDX(P, cx + gx * (cy + gy * cz), gx * gy * P.bp_g[2], 61);
         const int e = sstart[c + 1];
         for (int q = sstart[c]; q < e; ++q) {
           const int b = KP_IDX(P, sids[KP_IDX(P, q, P.bp_n_ids, 62)], P.n_boxes_pad, 63);

@@ -46,6 +46,13 @@ constexpr int KP_FSO_MAX_LEAVES = 16384; // regions of a kd-tree decomposition
 __host__ __device__ constexpr int kp_xs_stride(int D) { return D <= 8 ? 8 : 16; }
 constexpr int KP_FSO_MAX_DEPTH = 64;     // its deepest leaf
 
+// Cell indices come from the low mantissa bits of 2^23 + cell, that is with
+// 0x4B000000 added: the sum x + gx y + gx gy z of three such indices is off by
+// this much (modulo 2^32).
+inline int32_t bp_bias_of(const int32_t g[3]) {
+  return (int32_t)(0x4B000000u * (1u + (uint32_t)g[0] + (uint32_t)g[0] * (uint32_t)g[1]));
+}
+
 // Device control block (one per context, in the arena).
 struct KCtl {
   // loop state, persistent across launches
@@ -183,6 +190,15 @@ struct KParams {
   int32_t bp_n_ids;      // (cell, box) entries of the grid
   float bp_scale[3];     // cells per unit length, per axis
   float bp_last[3];      // bp_g - 1 per axis, as a float
+  int32_t bp_gxy;        // cells of a z layer
+  int32_t bp_bias;       // what the biased cell indices add up to (bp_bias_of)
+  // state_inside: every state of the tree lies in the state box, and the box's
+  // positions in the workspace.  small_angles: besides, at no stage of a step
+  // from the state box does the quadrotor's roll or pitch leave (-3, 3).
+  // state_symmetric: x_lo = -x_hi in the system's dimensions SYM0 .. SYM1 - 1.
+  int32_t state_inside;
+  int32_t small_angles;
+  int32_t state_symmetric;
   // tree, SoA over t_e nodes
   float* st;          // [D][t_e]
   int32_t* parent;

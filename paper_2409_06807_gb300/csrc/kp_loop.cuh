@@ -339,12 +339,35 @@ __device__ __forceinline__ void box_muller4(uint4 w, float* z) {
 // The expand phase and the node-set phase (which appends accepted samples
 // by their keys) both draw through this function, so both see the same
 // numbers.
+// Division of a sample key by the pass's lambda (at most 1024) by a
+// multiplication: for lam in [2^s, 2^(s+1)) and mul = ceil(2^(31+s) / lam), key
+// / lam = (key mul) >> (31 + s) for every key below 2^30 (the product exceeds
+// the quotient's by key (mul lam - 2^(31+s)) / lam < key, less than the 2^(31+s)
+// / lam that is left).  Two 32-bit divisions a pass and thread instead of one a
+// sample: mul's quotient in two steps, 2^31 = a lam + b, 2^s b = c lam + d.
+struct KeyDiv {
+  int lam, shift;
+  uint32_t mul;
+  __device__ __forceinline__ explicit KeyDiv(int l) : lam(l), shift(0), mul(0) {
+    if (l > 0) {
+      const uint32_t u = (uint32_t)l;
+      shift = 31 - __clz(l);
+      const uint32_t a = 0x80000000u / u, b = 0x80000000u - a * u;
+      const uint32_t c = (b << shift) / u, d = (b << shift) - c * u;
+      mul = (a << shift) + c + (d != 0u ? 1u : 0u);
+    }
+  }
+  __device__ __forceinline__ int quot(int key) const {
+    return (int)(__umulhi((uint32_t)key << 1, mul) >> shift);
+  }
+};
+
 template <int SYS>
-__device__ __forceinline__ int draw_controls(const KParams& P, uint32_t it, int key, int lam,
+__device__ __forceinline__ int draw_controls(const KParams& P, uint32_t it, int key, const KeyDiv& kd,
                                              float* u, int* k, uint32_t* wacc, uint32_t* wr) {
   constexpr int N = System<SYS>::N;
-  const int p = key / lam;
-  const int j = key - p * lam;
+  const int p = kd.quot(key);
+  const int j = key - p * kd.lam;
   const int v = KP_IDX(P, P.ve[KP_IDX(P, p, P.t_e, 5)], P.t_e, 6);
   const uint4 w0 = philox4x32_10(make_uint4(it, (uint32_t)v, (uint32_t)j, 0u), P.seed_lo, P.seed_hi);
   const uint4 w1 = philox4x32_10(make_uint4(it, (uint32_t)v, (uint32_t)j, 1u), P.seed_lo, P.seed_hi);
@@ -371,10 +394,10 @@ __device__ __forceinline__ int draw_controls(const KParams& P, uint32_t it, int 
 // The draw of sample 'key' and its parent's state (the start of the
 // segment).
 template <int SYS>
-__device__ __forceinline__ int draw_sample(const KParams& P, uint32_t it, int key, int lam, float* x,
+__device__ __forceinline__ int draw_sample(const KParams& P, uint32_t it, int key, const KeyDiv& kd, float* x,
                                            float* u, int* k, uint32_t* wacc, uint32_t* wr) {
   constexpr int D = System<SYS>::D;
-  const int v = draw_controls<SYS>(P, it, key, lam, u, k, wacc, wr);
+  const int v = draw_controls<SYS>(P, it, key, kd, u, k, wacc, wr);
 #pragma unroll
   for (int d = 0; d < D; ++d) x[d] = P.st[(size_t)d * P.t_e + v];
   return v;
@@ -394,7 +417,7 @@ constexpr int KP_KEY_BATCH = 128; // keys a warp takes from the grid counter
 
 template <int SYS, bool LOG>
 __device__ __forceinline__ void phase_expand(const KParams& P, const Team& T,
-                                             const unsigned char* sblob, uint32_t it, int lam,
+                                             const unsigned char* sblob, uint32_t it, const KeyDiv& kd,
                                              int S, LoopShared& sh) {
   using Sys = System<SYS>;
   constexpr int D = Sys::D, N = Sys::N;
@@ -548,7 +571,7 @@ __device__ __forceinline__ void phase_expand(const KParams& P, const Team& T,
           key = pool_next + rank;
           n_refill += ran ? 1u : 0u;
           ran = true;
-          v = draw_sample<SYS>(P, it, key, lam, x, u, &k, &wacc, wr);
+          v = draw_sample<SYS>(P, it, key, kd, x, u, &k, &wacc, wr);
           i = 0;
           fail = 0;
           done = false;
@@ -564,14 +587,11 @@ __device__ __forceinline__ void phase_expand(const KParams& P, const Team& T,
       const float px = x[0], py = x[1], pz = x[2];
       Sys::step(x, u, P.dt, P);
       ++i;
-      const bool inbox = in_state_box<D>(x, P);
+      const bool inbox = in_state_box<Sys>(x, P);
       bool ok = inbox;
       if (inbox) {
-        // hull of the step; + 0.0f turns a -0 into +0 for the box test
-        ok = !hull_hits_grid(P, sbox, sstart, sids, sclear, fminf(px, x[0]) + 0.0f,
-                             fminf(py, x[1]) + 0.0f, fminf(pz, x[2]) + 0.0f,
-                             fmaxf(px, x[0]) + 0.0f, fmaxf(py, x[1]) + 0.0f,
-                             fmaxf(pz, x[2]) + 0.0f, &n_box);
+        const float p0[3] = {px, py, pz};
+        ok = !hull_hits_grid(P, sbox, sstart, sids, sclear, p0, x, &n_box);
       }
       if (!ok) {
         done = true;
@@ -827,7 +847,7 @@ __device__ __forceinline__ void phase_thresholds(const KParams& P, const Team& T
 // integrator steps, explicitly rounded, so the same numbers) and must match
 // the kept and the logged state bit for bit.
 template <int SYS, bool LOG>
-__device__ __forceinline__ void materialise(const KParams& P, uint32_t it, int id0, int lam,
+__device__ __forceinline__ void materialise(const KParams& P, uint32_t it, int id0, const KeyDiv& kd,
                                             const LoopShared& sh, const unsigned char* sblob) {
   using Sys = System<SYS>;
   constexpr int D = Sys::D, N = Sys::N;
@@ -842,7 +862,7 @@ __device__ __forceinline__ void materialise(const KParams& P, uint32_t it, int i
     float x[D], u[N];
     int k;
     uint32_t wacc, wr[4];
-    const int v = draw_controls<SYS>(P, it, key, lam, u, &k, &wacc, wr);
+    const int v = draw_controls<SYS>(P, it, key, kd, u, &k, &wacc, wr);
     {
       const float4* row = reinterpret_cast<const float4*>(P.xs + (size_t)key * kp_xs_stride(D));
 #pragma unroll
@@ -877,7 +897,7 @@ __device__ __forceinline__ void materialise(const KParams& P, uint32_t it, int i
       const uint32_t h = atomicAdd(P.hv_count, 1u);
       if (h < (uint32_t)P.hv_cap) {
         const __nv_bfloat16* fr =
-            reinterpret_cast<const __nv_bfloat16*>(P.feat) + (size_t)(key / lam) * 32;
+            reinterpret_cast<const __nv_bfloat16*>(P.feat) + (size_t)kd.quot(key) * 32;
         for (int c = 0; c < 32; ++c) P.hv_feat[(size_t)h * 32 + c] = __bfloat162float(fr[c]);
 #pragma unroll
         for (int d = 0; d < 3; ++d)
@@ -914,7 +934,7 @@ __device__ __forceinline__ void materialise(const KParams& P, uint32_t it, int i
 // reading their sets.
 template <int SYS, bool LOG>
 __device__ __forceinline__ void phase_nodesets(const KParams& P, const Team& T, uint32_t it,
-                                               int t_old, int lam, LoopShared& sh, int* n_new,
+                                               int t_old, const KeyDiv& kd, LoopShared& sh, int* n_new,
                                                const unsigned char* sblob, double* sd) {
   const int nch = P.nch;
   if (threadIdx.x < 32 && T.b < nch) {
@@ -927,7 +947,7 @@ __device__ __forceinline__ void phase_nodesets(const KParams& P, const Team& T, 
   block_prefix(T, P.blk_a, sh, &acc_before, &acc_total);
   *n_new = (int)acc_total;
   const int t_new = t_old + (int)acc_total;
-  materialise<SYS, LOG>(P, it, t_old + (int)acc_before, lam, sh, sblob);
+  materialise<SYS, LOG>(P, it, t_old + (int)acc_before, kd, sh, sblob);
   if (threadIdx.x == 0) {
     const uint64_t t0 = global_ns();
     uint32_t spins = 0;
@@ -1043,7 +1063,8 @@ __device__ __forceinline__ bool run_loop(const KParams& P, const Team& T, unsign
       phase_ns[3] = phase_ns[6] = 0;
     }
     const int S = n_ve > 0 ? n_ve * lam : 0;
-    phase_expand<SYS, LOG>(P, T, smem, it, lam, S, sh);
+    const KeyDiv kd(lam);
+    phase_expand<SYS, LOG>(P, T, smem, it, kd, S, sh);
     stamp(0);
     if (!team_sync(T, ctl, P.wait_ns, 20)) return false;
     stamp(1);
@@ -1054,7 +1075,7 @@ __device__ __forceinline__ bool run_loop(const KParams& P, const Team& T, unsign
     if (timer) phase_ns[5] = phase_ns[7] = 0;
     const int t_old = n_tree;
     int n_acc;
-    phase_nodesets<SYS, LOG>(P, T, it, t_old, lam, sh, &n_acc, smem, sd);
+    phase_nodesets<SYS, LOG>(P, T, it, t_old, kd, sh, &n_acc, smem, sd);
     n_tree = t_old + n_acc;
     stamp(8);
     if (!team_sync(T, ctl, P.wait_ns, 23)) return false;
@@ -1247,7 +1268,7 @@ __device__ void init_root(const KParams& P, const RootState& root, bool box_free
   KCtl* ctl = P.ctl;
   float x[D];
   for (int i = 0; i < D; ++i) x[i] = root.x[i];
-  bool ok = in_state_box<D>(x, P) && box_free;
+  bool ok = in_state_box<Sys>(x, P) && box_free;
   ctl->n_run = 0;
   ctl->stop = 0;
   ctl->it_valid = 0;

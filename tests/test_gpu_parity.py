@@ -102,6 +102,52 @@ def test_lockstep_tiny(P, system, seed):
     assert exact >= min(ran, 3)
 
 
+@pytest.mark.parametrize("system", [W.DI, W.DUBINS, W.QUAD])
+@pytest.mark.parametrize("case", ["small_workspace", "lopsided", "wide_angles"])
+def test_lockstep_general_step_forms(P, system, case):
+    """The forms of a step that the usual workloads do not take: positions
+    outside the workspace (cells clamped, both sides of the clearance checked),
+    state bounds of different size on both sides, and roll and pitch bounds
+    that need the argument reduction."""
+    w = W.tiny(system, seed=4, t_e=2000, lambda_max=8)
+    if case == "small_workspace":
+        w = w.with_(ws_lo=np.float32([0.15, 0.15, 0.4]), ws_hi=np.float32([0.85, 0.9, 0.95]))
+    x_lo, x_hi = w.x_lo.copy(), w.x_hi.copy()
+    if case == "lopsided":
+        x_lo[3 if system == W.DI else 4] *= np.float32(0.75)
+    if case == "wide_angles":
+        if system != W.QUAD:
+            pytest.skip("the quadrotor's roll and pitch")
+        x_lo[3:5], x_hi[3:5] = -1.5, 1.5
+    exact, ran, flips, n, _ = lockstep(P, w.with_(x_lo=x_lo, x_hi=x_hi), 12)
+    assert exact >= min(ran, 3)
+
+
+@pytest.mark.parametrize("system", [W.DUBINS, W.QUAD])
+def test_imported_state_outside_the_box(P, system):
+    """An imported tree with a state outside the state box (and outside the
+    workspace): its samples take the general step forms, and the pass agrees
+    with the oracle's."""
+    w = W.tiny(system, seed=5, t_e=2000, lambda_max=8)
+    g = P.Planner(w)
+    g.reset()
+    g.expand_step(2)
+    t = g.export_tree()
+    t["state"] = t["state"].copy()
+    t["state"][-1, :3] = (-0.4, 1.3, 0.5)
+    t["in_ve"][:] = 1
+    g.import_tree(t)
+    g.enable_log(w.t_e)
+    o = Oracle(w)
+    o.set_work_grid(g.info()["bp_grid"])
+    o.import_(_as_input(t))
+    _, ost, orec = o.iterate(records=True)
+    gst = g.expand_step(1)[0]
+    flips = compare_pass(w, ost, orec, gst, g.read_log(ost["n_samples"]))
+    if flips == 0:
+        compare_trees(w, g.export_tree(), o.export())
+
+
 @pytest.mark.parametrize("seed", [0, 1, 2, 3])
 def test_lockstep_c1(P, seed):
     """Double integrator, 16 boxes, 8^3 x 4^3 decomposition, lambda 32,
