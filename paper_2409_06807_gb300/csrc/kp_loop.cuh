@@ -28,6 +28,7 @@
 // it on every V_E node.
 #pragma once
 
+#include <cstddef>
 #include <cstdint>
 
 #include "kp_device.cuh"
@@ -38,11 +39,15 @@ namespace kp {
 constexpr int KP_WARPS = KP_BLOCK / 32;
 
 struct LoopShared {
-  ScanSmem scan;
-  unsigned long long red[64];
+  // one value a warp: the expand phase's five counters, the counts a block
+  // prefix adds up, the warps' tile counts (two tiles in turn)
+  unsigned long long cnt[5][KP_WARPS];
+  uint32_t pre[KP_WARPS], tot[KP_WARPS];
+  uint32_t tile[2][KP_WARPS];
   uint64_t mbar;
   int flag;
   int bcast[2];
+  int goal, err;         // the pass's goal node and error word, read in phase L
   int32_t phase_ns[12];  // per-pass phase timers (block 0, thread 0)
   // accepted samples of this block, from the accept phase to the node-set
   // phase: warp w compacted acc_n[w] keys at acc_key[acc_a[w]...], which
@@ -127,47 +132,47 @@ __device__ __forceinline__ void chunk_of(const Team& T, int n, int* c0, int* c1)
   *c1 = (int)(a + per < n ? a + per : n);
 }
 
-// Sum of blk[0..G) and of blk[0..blockIdx.x), by one warp (no block sync).
-__device__ __forceinline__ void warp_prefix(const Team& T, const uint32_t* blk,
-                                            unsigned long long* before,
-                                            unsigned long long* total) {
-  unsigned long long pre = 0, tot = 0;
-  for (int i = (int)(threadIdx.x & 31u); i < T.nb; i += 32) {
-    const unsigned long long c = __ldcg(blk + i);
+// Sum of blk[0..nb) and of blk[0..b) (counts of at most 2^28 in all): a
+// reduction per warp, one block barrier, then every thread adds the warps'
+// sums.  The shared values are free again after the block's next barrier.
+__device__ __forceinline__ void block_prefix(const Team& T, const uint32_t* blk, LoopShared& sh,
+                                             uint32_t* before, uint32_t* total) {
+  uint32_t pre = 0, tot = 0;
+  for (int i = threadIdx.x; i < T.nb; i += blockDim.x) {
+    const uint32_t c = __ldcg(blk + i);
     tot += c;
     if (i < T.b) pre += c;
   }
+  pre = __reduce_add_sync(0xffffffffu, pre);
+  tot = __reduce_add_sync(0xffffffffu, tot);
+  if ((threadIdx.x & 31u) == 0) {
+    sh.pre[threadIdx.x >> 5] = pre;
+    sh.tot[threadIdx.x >> 5] = tot;
+  }
+  __syncthreads();
+  pre = tot = 0;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    pre += __shfl_xor_sync(0xffffffffu, pre, o);
-    tot += __shfl_xor_sync(0xffffffffu, tot, o);
+  for (int w = 0; w < KP_WARPS; ++w) {
+    pre += sh.pre[w];
+    tot += sh.tot[w];
   }
   *before = pre;
   *total = tot;
-}
-
-// Sum of blk[0..G) and of blk[0..blockIdx.x).
-__device__ __forceinline__ void block_prefix(const Team& T, const uint32_t* blk, LoopShared& sh,
-                                             unsigned long long* before,
-                                             unsigned long long* total) {
-  unsigned long long pre = 0, tot = 0;
-  for (int i = threadIdx.x; i < T.nb; i += blockDim.x) {
-    const unsigned long long c = __ldcg(blk + i);
-    tot += c;
-    if (i < T.b) pre += c;
-  }
-  block_sum2(pre, tot, sh.red, before, total);
 }
 
 // Nodes of a block's chunk are visited in tiles of blockDim.x: node v0 +
 // tile * blockDim.x + threadIdx.x, so that a warp's loads and stores of the
 // per-node arrays are coalesced.
 
-// Block sum of one int per thread (every thread gets it).
-__device__ __forceinline__ int block_sum(int c, LoopShared& sh) {
-  unsigned long long a, dummy;
-  block_sum2((unsigned long long)c, 0, sh.red, &a, &dummy);
-  return (int)a;
+// Block sum of one count per thread (at most 2^31 in all), for thread 0.
+__device__ __forceinline__ uint32_t block_sum(uint32_t c, LoopShared& sh) {
+  c = __reduce_add_sync(0xffffffffu, c);
+  if ((threadIdx.x & 31u) == 0) sh.pre[threadIdx.x >> 5] = c;
+  __syncthreads();
+  uint32_t s = 0;
+#pragma unroll
+  for (int w = 0; w < KP_WARPS; ++w) s += sh.pre[w];
+  return s;
 }
 
 // Phase N': count V_E members of this block's node chunk (no draws) and
@@ -178,8 +183,8 @@ __device__ __forceinline__ void count_ve(const KParams& P, const Team& T, int n,
   int c = 0;
   for (int v = v0 + (int)threadIdx.x; v < v1; v += (int)blockDim.x)
     c += P.in_ve[KP_IDX(P, v, P.t_e, 1)] ? 1 : 0;
-  const int tot = block_sum(c, sh);
-  if (threadIdx.x == 0) P.blk_b[KP_IDX(P, T.b, KP_MAX_GRID, 2)] = (uint32_t)tot;
+  const uint32_t tot = block_sum((uint32_t)c, sh);
+  if (threadIdx.x == 0) P.blk_b[KP_IDX(P, T.b, KP_MAX_GRID, 2)] = tot;
 }
 
 // Phase L: write the V_E list (ascending node id) from the per-block counts:
@@ -189,26 +194,26 @@ __device__ __forceinline__ void count_ve(const KParams& P, const Team& T, int n,
 __device__ __forceinline__ int write_ve(const KParams& P, const Team& T, int n, LoopShared& sh) {
   int v0, v1;
   chunk_of(T, n, &v0, &v1);
-  unsigned long long off, total;
+  uint32_t off, total;
   block_prefix(T, P.blk_b, sh, &off, &total);
   const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5;
-  const int nw = (int)(blockDim.x >> 5);
-  int base = (int)off;
-  for (int t0 = v0; t0 < v1; t0 += (int)blockDim.x) {
+  int base = (int)off, buf = 0;
+  for (int t0 = v0; t0 < v1; t0 += (int)blockDim.x, buf ^= 1) {
     const int v = t0 + (int)threadIdx.x;
     const bool m = v < v1 && P.in_ve[KP_IDX(P, v, P.t_e, 3)];
     const uint32_t bal = __ballot_sync(0xffffffffu, m);
-    if (lane == 0) sh.scan.warp[w] = __popc(bal);
+    // the other buffer's readers are past this barrier before it is written
+    if (lane == 0) sh.tile[buf][w] = (uint32_t)__popc(bal);
     __syncthreads();
     int before = 0, tile = 0;
-    for (int q = 0; q < nw; ++q) {
-      const int cq = sh.scan.warp[q];
+#pragma unroll
+    for (int q = 0; q < KP_WARPS; ++q) {
+      const int cq = (int)sh.tile[buf][q];
       before += q < (int)w ? cq : 0;
       tile += cq;
     }
     if (m) P.ve[KP_IDX(P, base + before + __popc(bal & ((1u << lane) - 1u)), P.t_e, 4)] = v;
     base += tile;
-    __syncthreads();
   }
   return (int)total;
 }
@@ -601,16 +606,20 @@ __device__ __forceinline__ void phase_expand(const KParams& P, const Team& T,
       }
     }
   }
-  unsigned long long bs, bh, bb, brf, bbt, dummy;
-  block_sum2((unsigned long long)n_steps, (unsigned long long)n_hull, sh.red, &bs, &bh);
-  block_sum2((unsigned long long)n_box, (unsigned long long)n_refill, sh.red, &bb, &brf);
-  block_sum2((unsigned long long)n_batch, 0, sh.red, &bbt, &dummy);
-  if (threadIdx.x == 0 && bs) {
-    atomicAdd(&P.ctl->tot_steps, bs);
-    atomicAdd(&P.ctl->tot_hull, bh);
-    atomicAdd(&P.ctl->tot_box_tests, bb);
-    if (brf) atomicAdd(&P.ctl->tot_refills, brf);
-    if (bbt) atomicAdd(&P.ctl->tot_batches, bbt);
+  // a sum per warp, then one thread a counter adds the warps' sums (the team
+  // barrier that follows frees the shared values)
+  const uint32_t mine[5] = {n_steps, n_hull, n_box, n_batch, n_refill};
+#pragma unroll
+  for (int c = 0; c < 5; ++c) {
+    const unsigned long long s = warp_sum_wide(mine[c]);
+    if (lane == 0) sh.cnt[c][threadIdx.x >> 5] = s;
+  }
+  __syncthreads();
+  if (threadIdx.x < 5) {
+    unsigned long long s = 0;
+    for (int w = 0; w < KP_WARPS; ++w) s += sh.cnt[threadIdx.x][w];
+    static_assert(offsetof(KCtl, tot_refills) == offsetof(KCtl, tot_steps) + 32, "counters in order");
+    if (s) atomicAdd(&P.ctl->tot_steps + threadIdx.x, s);
   }
 }
 
@@ -641,11 +650,12 @@ __device__ __forceinline__ void warp_range(int c0, int c1, int* a, int* b) {
 constexpr int KP_ACC_KPL = 8;
 
 __device__ __forceinline__ void phase_scores(const KParams& P, const Team& T, int nch, double* sd);
+__device__ __forceinline__ void phase_score_sum(const KParams& P, const Team& T, int nch, double* sd);
 
 template <bool LOG>
 __device__ __forceinline__ void phase_accept(const KParams& P, const Team& T, int S, int nch,
                                              double* sd, LoopShared& sh) {
-  if (threadIdx.x < 32) phase_scores(P, T, nch, sd);
+  phase_scores(P, T, nch, sd);
   const uint32_t FULL = 0xffffffffu;
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t lt = (1u << lane) - 1u;
@@ -689,11 +699,16 @@ __device__ __forceinline__ void phase_accept(const KParams& P, const Team& T, in
   }
   // warp counts -> offsets in key order (warps own ascending ranges)
   const int w = (int)(threadIdx.x >> 5);
-  if (lane == 0) sh.scan.warp[w] = n_acc;
+  n_valid = __reduce_add_sync(FULL, n_valid);
+  if (lane == 0) {
+    sh.pre[w] = (uint32_t)n_acc;
+    sh.tot[w] = n_valid;
+  }
   __syncthreads();
   int off = 0, block_acc = 0;
-  for (int q = 0; q < (int)(blockDim.x >> 5); ++q) {
-    const int cq = sh.scan.warp[q];
+#pragma unroll
+  for (int q = 0; q < KP_WARPS; ++q) {
+    const int cq = (int)sh.pre[q];
     off += q < w ? cq : 0;
     block_acc += cq;
   }
@@ -702,14 +717,16 @@ __device__ __forceinline__ void phase_accept(const KParams& P, const Team& T, in
     sh.acc_n[w] = n_acc;
     sh.acc_off[w] = off;
   }
-  if (threadIdx.x == 0) sh.acc_tot = block_acc;
-  unsigned long long bv, dummy;
-  block_sum2((unsigned long long)n_valid, 0, sh.red, &bv, &dummy);
   if (threadIdx.x == 0) {
+    sh.acc_tot = block_acc;
+    uint32_t bv = 0;
+    for (int q = 0; q < KP_WARPS; ++q) bv += sh.tot[q];
     if (T.b == 0) P.ctl->work_next = 0;  // the expand phase is over
     P.blk_a[KP_IDX(P, T.b, KP_MAX_GRID, 15)] = (uint32_t)block_acc;
-    if (bv) atomicAdd(&P.ctl->it_valid, (uint32_t)bv);
+    if (bv) atomicAdd(&P.ctl->it_valid, bv);
   }
+  // the chunk's partial sum, once every warp's scores are there
+  if (threadIdx.x < 32) phase_score_sum(P, T, nch, sd);
 }
 
 // Pairwise sum of buf[0..n), n a power of two, by one warp (bottom-up
@@ -756,19 +773,19 @@ __device__ __forceinline__ double warp_tree_sum(int n, L load) {
   return __shfl_sync(0xffffffffu, sum, 0);
 }
 
-// Phase S (warp 0): Eq. 3-4 for this block's region chunk and its pairwise
-// partial sum (published before the grid barrier that ends the phase).
-// Every operation is an explicitly rounded IEEE double operation in the
-// order
+// Phase S: Eq. 3-4 for this block's region chunk, 32 regions a warp in turn
+// (the FP64 unit makes about two operations a clock and SM, and a division is
+// a chain of a dozen: one warp that took all of a 512-region chunk, as the
+// server's small teams have, held the pass up by 16 chains).  Every operation
+// is an explicitly rounded IEEE double operation in the order
 // FreeVol = ((delta + nv) vol) / ((delta + nv) + ni),
 // f4 = (FreeVol FreeVol)(FreeVol FreeVol),
 // Score = f4 / ((1 + Cov)(1 + (nv + ni)(nv + ni))).
 __device__ __forceinline__ void phase_scores(const KParams& P, const Team& T, int nch, double* sd) {
   if (T.b >= nch) return;
-  const int lane = (int)(threadIdx.x & 31u);
   const int ch = P.R_pad / nch;
   const int r0 = T.b * ch;
-  for (int i = lane; i < ch; i += 32) {
+  for (int i = (int)threadIdx.x; i < ch; i += (int)blockDim.x) {
     const int r = r0 + i;
     double sc = 0.0;
     if (r < P.R && P.avail[r]) {
@@ -786,25 +803,39 @@ __device__ __forceinline__ void phase_scores(const KParams& P, const Team& T, in
     if (r < P.R) P.score[r] = sc;
     sd[i] = sc;
   }
+}
+
+// The chunk's pairwise partial sum (warp 0, after a block barrier that follows
+// phase_scores; published before the grid barrier that ends the phase).
+__device__ __forceinline__ void phase_score_sum(const KParams& P, const Team& T, int nch, double* sd) {
+  if (T.b >= nch) return;
+  const int lane = (int)(threadIdx.x & 31u);
+  const int ch = P.R_pad / nch;
   double part;
   if (ch <= 32 * KP_TREE_PER_LANE) {
-    __syncwarp();
     part = warp_tree_sum(ch, [&](int i) { return sd[i]; });
   } else {
     warp_pairwise(sd, ch);
     part = sd[0];
   }
   if (lane == 0) P.chunk_sum[KP_IDX(P, T.b, KP_MAX_GRID, 16)] = part;
-  __syncwarp();
 }
 
-// Phase T (warp 0 of the node-set phase): the sum of Eq. 5 from the chunks'
-// partial sums (every chunk's warp reduces them itself, in the same
-// pairwise tree, so all get the same value), then P_accept and the integer
-// threshold of this block's region chunk.
-__device__ __forceinline__ void phase_thresholds(const KParams& P, const Team& T, int nch,
+// Warps of a region-chunk block that write thresholds: one for 32 regions (one
+// in all where the chunk sums are added up in the shared scratch).
+__device__ __forceinline__ int threshold_warps(const KParams& P, int nch) {
+  if (nch > 32 * KP_TREE_PER_LANE) return 1;
+  const int w = (P.R_pad / nch + 31) >> 5;
+  return w < KP_WARPS ? w : KP_WARPS;
+}
+
+// Phase T (the first 'warps' warps of a chunk block in the node-set phase):
+// the sum of Eq. 5 from the chunks' partial sums (each of these warps reduces
+// them itself, in the same pairwise tree, so all get the same value; in
+// registers up to 256 chunks, else by the one warp in the scratch), then
+// P_accept and the integer threshold of the warp's regions.
+__device__ __forceinline__ void phase_thresholds(const KParams& P, const Team& T, int nch, int warps,
                                                  double* sd) {
-  if (T.b >= nch) return;
   const int lane = (int)(threadIdx.x & 31u);
   double sum;
   if (nch <= 32 * KP_TREE_PER_LANE) {
@@ -814,10 +845,10 @@ __device__ __forceinline__ void phase_thresholds(const KParams& P, const Team& T
     warp_pairwise(sd, nch);
     sum = sd[0];
   }
-  if (T.b == 0 && lane == 0) P.ctl->score_sum = sum;
+  if (T.b == 0 && threadIdx.x == 0) P.ctl->score_sum = sum;
   const int ch = P.R_pad / nch;
   const int r0 = T.b * ch;
-  for (int i = (int)(threadIdx.x & 31u); i < ch; i += 32) {
+  for (int i = (int)threadIdx.x; i < ch; i += 32 * warps) {
     const int r = r0 + i;
     if (r >= P.R) break;
     uint64_t thr = 1ull << 32;  // P_accept = 1 outside R_avail
@@ -926,8 +957,9 @@ __device__ __forceinline__ void materialise(const KParams& P, uint32_t it, int i
 // purpose 2) against the threshold of its region; new nodes are in V_E.
 // Publishes the block chunk's V_E count; returns in *n_new the number of
 // accepted samples of the pass (the new nodes).
-// Order inside the phase: warp 0 of every region-chunk block first writes
-// its chunk's thresholds (phase T) and counts itself done; every block then
+// Order inside the phase: the first warps of every region-chunk block write
+// its chunk's thresholds (phase T, 32 regions a warp in turn) and count
+// themselves done; every block
 // appends its own accepted samples (ids from t_old, in key order), which
 // needs no threshold; then it waits (bounded) until every chunk is done and
 // makes the node-set draws.  New nodes are counted as V_E members without
@@ -936,24 +968,25 @@ template <int SYS, bool LOG>
 __device__ __forceinline__ void phase_nodesets(const KParams& P, const Team& T, uint32_t it,
                                                int t_old, const KeyDiv& kd, LoopShared& sh, int* n_new,
                                                const unsigned char* sblob, double* sd) {
-  const int nch = P.nch;
-  if (threadIdx.x < 32 && T.b < nch) {
-    phase_thresholds(P, T, nch, sd);
+  const int nch = P.nch, warps = threshold_warps(P, nch);
+  uint32_t acc_before, acc_total;
+  block_prefix(T, P.blk_a, sh, &acc_before, &acc_total);
+  if (T.b < nch && (int)(threadIdx.x >> 5) < warps) {
+    phase_thresholds(P, T, nch, warps, sd);
     __threadfence();
     __syncwarp();
-    if (threadIdx.x == 0) atomicAdd(&P.ctl->t_done, 1u);
+    if ((threadIdx.x & 31u) == 0) atomicAdd(&P.ctl->t_done, 1u);
   }
-  unsigned long long acc_before, acc_total;
-  block_prefix(T, P.blk_a, sh, &acc_before, &acc_total);
   *n_new = (int)acc_total;
   const int t_new = t_old + (int)acc_total;
   materialise<SYS, LOG>(P, it, t_old + (int)acc_before, kd, sh, sblob);
   if (threadIdx.x == 0) {
-    const uint64_t t0 = global_ns();
+    uint64_t t0 = 0;
     uint32_t spins = 0;
-    while (ld_acquire(&P.ctl->t_done) < (uint32_t)nch) {
+    while (ld_acquire(&P.ctl->t_done) < (uint32_t)(nch * warps)) {
       if ((++spins & 63u) == 0) {
         if (*((volatile int*)&P.ctl->err) != 0) break;
+        if (t0 == 0) t0 = global_ns();
         if (global_ns() - t0 > P.wait_ns) {
           raise_error(P.ctl, KP_DEV_ERR_TIMEOUT, 25);
           break;
@@ -994,8 +1027,8 @@ __device__ __forceinline__ void phase_nodesets(const KParams& P, const Team& T, 
   // new nodes are V_E members (their flags are set by the blocks that
   // appended them, so they are counted, not read)
   const int new0 = v0 > t_old ? v0 : t_old;
-  const int tot = block_sum(c, sh) + (v1 > new0 ? v1 - new0 : 0);
-  if (threadIdx.x == 0) P.blk_b[KP_IDX(P, T.b, KP_MAX_GRID, 24)] = (uint32_t)tot;
+  const uint32_t tot = block_sum((uint32_t)c, sh) + (uint32_t)(v1 > new0 ? v1 - new0 : 0);
+  if (threadIdx.x == 0) P.blk_b[KP_IDX(P, T.b, KP_MAX_GRID, 24)] = tot;
 }
 
 // The loop of one query (Algorithm 1 body, repeated) run by a team of
@@ -1081,13 +1114,21 @@ __device__ __forceinline__ bool run_loop(const KParams& P, const Team& T, unsign
     if (!team_sync(T, ctl, P.wait_ns, 23)) return false;
     stamp(9);
     const int ve_prev = n_ve, lam_prev = lam;
+    // the pass's goal node and any error raised before the barrier above:
+    // every block reads the same words, beside the counts of the V_E list
+    if (threadIdx.x == 0) {
+      sh.goal = *((volatile int*)&ctl->goal_node);
+      sh.err = *((volatile int*)&ctl->err);
+    }
     n_ve = write_ve(P, T, n_tree, sh);
     lam = eq6_lambda(P.t_e, n_tree, n_ve, P.lambda_max);
     ++run;
+    const int goal = sh.goal;
+    if (sh.err != 0) return false;
+    const bool solved = goal != KP_NO_GOAL;
+    const bool full = n_ve > 0 && lam == 0;
+    int stop = solved || full || run >= max_iters ? 1 : 0;
     if (T.b == 0 && threadIdx.x == 0) {
-      const int goal = *((volatile int*)&ctl->goal_node);
-      const bool solved = goal != KP_NO_GOAL;
-      const bool full = n_ve > 0 && lam == 0;
       if (run <= P.stats_cap && P.stats) {
         KStats s;
         s.iteration = (int)it;
@@ -1106,14 +1147,13 @@ __device__ __forceinline__ bool run_loop(const KParams& P, const Team& T, unsign
       ctl->it_valid = 0;
       ctl->t_done = 0;  // every block is past its threshold wait
       ctl->tot_samples += (unsigned long long)S;
-      const bool out_of_time = max_ns > 0 && global_ns() - t_start >= max_ns;
       ctl->state = solved ? KP_DEV_SOLVED : (full ? KP_DEV_FULL : KP_DEV_RUNNING);
-      ctl->stop = (solved || full || run >= max_iters || out_of_time) ? 1 : 0;
+      // a time limit ends the loop by block 0's clock
+      if (max_ns > 0) ctl->stop = stop || global_ns() - t_start >= max_ns ? 1 : 0;
     }
     ++it;
     const uint64_t t_l = timer ? global_ns() : 0;
-    int stop;
-    if (!team_sync(T, ctl, P.wait_ns, 24, &ctl->stop, &stop)) return false;
+    if (!team_sync(T, ctl, P.wait_ns, 24, max_ns > 0 ? &ctl->stop : nullptr, &stop)) return false;
     if (timer) {
       t_mark = global_ns();
       prev_wait = (int32_t)(t_mark - t_l);  // reported with the next pass
