@@ -488,7 +488,7 @@ kp_status kp_set_harvest(kp_ctx *ctx, float *dev_feat, float *dev_target,
  * leave; the server launches again when work arrives.  All device memory
  * comes from the caller's pool (kp_server_required_bytes for the control
  * area plus the query arenas); host memory holds the rings and results.
- * Per query: at most 1,500 obstacle boxes (blob of 48 KB) and
+ * Per query: at most 1,440 obstacle boxes (their slots and ids in 48 KB) and
  * kp_required_bytes regions up to 1024 * team_blocks in the padded count;
  * no sample log, learned proposal or harvest. */
 typedef struct kp_server kp_server;

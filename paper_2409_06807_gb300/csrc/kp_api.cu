@@ -2187,7 +2187,9 @@ bool try_admit(kp_server* s, PendingQuery& q) {
   // no cell clearances: the host would spend milliseconds per query on them
   const size_t blob_bytes = build_blob(s->blob.data(), q.boxes.empty() ? nullptr : q.boxes.data(),
                                        (int)(q.boxes.size() / 6), q.ws, P, KS_BLOB_MAX, false);
-  if (blob_bytes > (size_t)KS_BLOB_MAX || d.R_pad / nch > KS_SD_DOUBLES) {
+  const size_t least = (size_t)P.n_boxes_pad * 32 + round16(4) + round16((q.boxes.size() / 6) * 2);
+  if (least > (size_t)KS_BLOB_MIN || blob_bytes > (size_t)KS_BLOB_MAX ||
+      d.R_pad / nch > KS_SD_DOUBLES) {
     pool_free(s, off, lay.total);
     finish_now(s, q.id, KP_ERR_ARG, q.t_submit);
     return true;

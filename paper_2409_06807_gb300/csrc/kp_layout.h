@@ -260,7 +260,12 @@ constexpr int KS_MAX_TEAMS = 1024;
 constexpr int KS_RING = 4096;          // submission / completion ring entries
 constexpr uint32_t KS_EXIT = 0xffffffffu;
 constexpr int KS_SD_DOUBLES = 1024;    // score scratch of a server block
-constexpr int KS_BLOB_MAX = 49152;     // obstacle blob of a server query (bytes)
+// Obstacle blob of a server query (bytes): its boxes, one cell and its list
+// must fit KS_BLOB_MIN (1,440 boxes do), and the grid is the finest whose blob
+// fits KS_BLOB_MAX.  With 48 KB for both, 900 forest boxes fell back from 64 x 64
+// cells of one or two boxes to 4^3 cells of 60, and a pass of 1,200 samples took
+// 100 us instead of 30; 64 KB hold 1,100 of them and keep two blocks an SM.
+constexpr int KS_BLOB_MIN = 49152, KS_BLOB_MAX = 65536;
 
 // One admitted query, written by the host into its descriptor slot.
 struct KQuery {

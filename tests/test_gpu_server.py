@@ -134,3 +134,28 @@ def test_serving_run_reports_latency(S):
     summ = serve.summarize(recs, time.perf_counter() - t0)
     assert summ["queries"] == 48 and summ["p99_ms"] >= summ["p50_ms"] > 0
     srv.close()
+
+
+def test_box_count_limit(S):
+    """1,440 boxes are the most whose slots, one cell and its list fit 48 KB:
+    accepted; the next multiple of eight is refused as before the grid's own
+    room grew, and a forest of 1,000 keeps its 4,096-cell grid's result."""
+    P, serve = S
+    srv = serve.Server(pool_bytes=1 << 30, team_blocks=16, max_slots=8)
+    side = (0.002, 0.004)
+    for n, ok in ((1440, True), (1448, False)):
+        w = W.c1(2, t_e=4096).with_(boxes=W.random_boxes(2, n, side=side, keep_clear=[
+            ((0.1, 0.1, 0.1), 0.02)]))
+        q = srv.submit(w, max_iters=3)
+        d = [x for x in srv.drain() if x["id"] == q][0]
+        assert (d["status"] != P.ERR_ARG) == ok
+        srv.result(q)
+    w = W.c2(7, t_e=60000, lambda_max=32)
+    w = w.with_(boxes=W.forest_boxes(7, 1000, width=(0.01, 0.015), keep_clear=[
+        (tuple(w.x_init[:3]), 0.03), (tuple(w.goal_c), float(w.goal_r))]))
+    st, ref = P.Planner(w).plan(max_iters=60)
+    q = srv.submit(w, max_iters=60)
+    srv.drain()
+    st2, got = srv.result(q)
+    assert st2 == st and _same(got, ref)
+    srv.close()
