@@ -98,6 +98,8 @@ namespace {
 
 constexpr int kStatsCap = 4096;
 constexpr int kFirstRows = 256;  // trajectory rows read with the header
+constexpr int kChainRoom = 1024;          // bytes behind the blob for chain ids at the least
+constexpr size_t kStaticRoom = 1024 + 2048;  // the loop kernel's static and reserved shared memory
 
 struct Dims {
   int sys, D, N, R, R_pad, n_sub_per, t_e, boxes_pad;
@@ -261,6 +263,7 @@ struct kp_ctx {
   int grid[2];
   int grid_limit;  // 0: the resident maximum; else at most this many blocks
   size_t smem;
+  size_t smem_max;  // shared memory a block may have
   int blob_base;  // blob bytes without the kd-tree copy
   int blob_kd;    // blob bytes with it (0: no tree)
   std::string err;
@@ -673,13 +676,13 @@ int build_kd(unsigned char* host, const float* fb, int nb, const kp_workspace& w
 
 kp_status configure_launch(kp_ctx* ctx);
 
-// Region chunks of the Score sums (Eq. 5): a power of two, at most one per
-// block, chunks of at least 32 regions (one per lane of the warp that
-// scores them), at most 1024 chunks.  Any power of two gives the same
-// pairwise tree.
-int region_chunks(int blocks, int R_pad) {
+// Region chunks of the Score sums (Eq. 5): a power of two, chunks of at least
+// 32 regions (one per lane of the warp that scores them), at most 256 chunks
+// (one tree in a warp's registers).  Any power of two gives the same pairwise
+// tree.
+int region_chunks(int R_pad) {
   int nch = 1;
-  while (nch * 2 <= blocks && nch * 2 * 32 <= R_pad && nch * 2 <= 1024) nch *= 2;
+  while (nch * 2 * 32 <= R_pad && nch * 2 <= 256) nch *= 2;
   return nch;
 }
 
@@ -740,53 +743,45 @@ kp_status upload_boxes(kp_ctx* ctx, const kp_obstacles* obs) {
 
 kp_status configure_launch(kp_ctx* ctx) {
   const Dims& d = ctx->dims;
-  ctx->P.blob_bytes = ctx->blob_base;
-  ctx->P.kd_smem_off = -1;
-  // shared memory: boxes + the double scratch of the region-score sums (a
-  // chunk's scores, then the chunk sums) + the network tile (learned form)
-  auto grids = [&](int sd) -> kp_status {
-    ctx->P.sd_bytes = sd * 8;
-    ctx->smem = (size_t)ctx->P.blob_bytes + (size_t)sd * 8 +
-                (ctx->P.features_on ? (size_t)MLP_LOOP_TILE_SMEM : 0);
+  KParams& P = ctx->P;
+  P.nch = region_chunks(d.R_pad);
+  P.sd_bytes = kChainRoom;
+  // shared memory: the obstacles, room for chain ids, the network tiles (a tile
+  // for each group of threads, fewer when the obstacles leave no room for all)
+  P.threads = ctx->grid_limit > 0 ? KP_LIMITED_THREADS : kp_loop_threads(d.sys);
+  P.mlp_groups = P.threads / KP_MLP_GROUP;
+  auto bytes = [&](int blob) {
+    return (size_t)blob + (size_t)P.sd_bytes +
+           (P.features_on ? (size_t)MLP_LOOP_TILE_SMEM * P.mlp_groups : 0);
+  };
+  while (P.features_on && P.mlp_groups > 1 && bytes(ctx->blob_base) + kStaticRoom > ctx->smem_max)
+    --P.mlp_groups;
+  // the kd-tree goes into shared memory with the blob (it is read at every
+  // binning) when that keeps the resident blocks
+  auto shape = [&](size_t smem, int* grid) -> kp_status {
     for (int log = 0; log < 2; ++log) {
-      int bps = 0;
-      KP_CUDA(occupancy(d.sys, log != 0, ctx->smem, &bps));
+      int bps = P.threads;
+      KP_CUDA(occupancy(d.sys, log != 0, smem, &bps));
       if (bps < 1) return fail(ctx, KP_ERR_ARG, "loop kernel cannot be resident");
       int g = bps * ctx->num_sms;
       if (g > KP_MAX_GRID) g = KP_MAX_GRID;
       if (ctx->grid_limit > 0 && g > ctx->grid_limit) g = ctx->grid_limit;
-      ctx->grid[log] = g;
+      grid[log] = g;
     }
     return KP_OK;
   };
-  // first with room for any chunking (chunks of at least R_pad / 1024
-  // regions, at most 1024 chunk sums) ...
-  const int min_ch = d.R_pad / (d.R_pad < 1024 ? d.R_pad : 1024);
-  kp_status s = grids(min_ch > 1024 ? min_ch : 1024);
+  P.blob_bytes = ctx->blob_base;
+  P.kd_smem_off = -1;
+  ctx->smem = bytes(ctx->blob_base);
+  kp_status s = shape(ctx->smem, ctx->grid);
+  if (s != KP_OK || ctx->blob_kd == 0 || bytes(ctx->blob_kd) + kStaticRoom > ctx->smem_max) return s;
+  int with_kd[2];
+  s = shape(bytes(ctx->blob_kd), with_kd);
   if (s != KP_OK) return s;
-  // region chunks: a power of two <= the smaller grid, <= R_pad, <= 1024
-  const int gmin = ctx->grid[0] < ctx->grid[1] ? ctx->grid[0] : ctx->grid[1];
-  const int nch = region_chunks(gmin, d.R_pad);
-  ctx->P.nch = nch;
-  // ... then with the scratch this chunking needs (smaller shared memory
-  // never lowers the grid, so nch stays at most the grid)
-  const int need = d.R_pad / nch > nch ? d.R_pad / nch : nch;
-  s = grids(need);
-  if (s != KP_OK || ctx->blob_kd == 0) return s;
-  // the kd-tree goes into shared memory with the blob when that keeps the
-  // resident blocks (it is read at every binning)
-  const size_t smem_kd = ctx->smem + (size_t)(ctx->blob_kd - ctx->blob_base);
-  for (int log = 0; log < 2; ++log) {
-    int bps = 0;
-    KP_CUDA(occupancy(d.sys, log != 0, smem_kd, &bps));
-    int g = bps * ctx->num_sms;
-    if (g > KP_MAX_GRID) g = KP_MAX_GRID;
-    if (ctx->grid_limit > 0 && g > ctx->grid_limit) g = ctx->grid_limit;
-    if (g < ctx->grid[log]) return KP_OK;
-  }
-  ctx->P.blob_bytes = ctx->blob_kd;
-  ctx->P.kd_smem_off = (int)round16((size_t)ctx->blob_base);
-  ctx->smem = smem_kd;
+  if (with_kd[0] < ctx->grid[0] || with_kd[1] < ctx->grid[1]) return KP_OK;
+  P.blob_bytes = ctx->blob_kd;
+  P.kd_smem_off = (int)round16((size_t)ctx->blob_base);
+  ctx->smem = bytes(ctx->blob_kd);
   return KP_OK;
 }
 
@@ -1005,14 +1000,17 @@ kp_status kp_create(const kp_system* sys, const kp_workspace* ws, const kp_obsta
   ctx->goal = kp_goal{{0, 0, 0}, 0};
   kp_status s = KP_OK;
   {
-    int dev = 0;
+    int dev = 0, smem_max = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev != ctx->device ||
         cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, dev) !=
+            cudaSuccess ||
+        cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
             cudaSuccess) {
       cudaGetLastError();
       delete ctx;
       return KP_ERR_CUDA;
     }
+    ctx->smem_max = (size_t)smem_max;
   }
 
   fill_params(ctx->P, d, lay, sys, ws, prm, ctx->arena);
@@ -1402,8 +1400,6 @@ kp_status kp_grow(kp_ctx* ctx, void* dev_arena, size_t arena_bytes, int32_t t_e)
   for (int a = 0; a < 3; ++a) P.bp_last[a] = old.bp_last[a];
   P.bp_gxy = old.bp_gxy;
   P.bp_bias = old.bp_bias;
-  P.nch = old.nch;
-  P.sd_bytes = old.sd_bytes;
   P.extract_cap = old.extract_cap;
   P.mlp_W1 = old.mlp_W1;
   P.mlp_b1 = old.mlp_b1;
@@ -1922,33 +1918,22 @@ extern "C" kp_status kp_plan_static(const kp_system* sys, const kp_workspace* ws
   P.wait_ns = 2000000000ull;
 
   // launch shape, as for a context with this obstacle count
-  int num_sms = 0, bps = 0;
+  P.threads = kp_loop_threads(d.sys);
+  int num_sms = 0, bps = P.threads;
   if (cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
     cudaGetLastError();
     return KP_ERR_CUDA;
   }
-  // as configure_launch: the grid with room for any chunking, the chunks
-  // of that grid, then the score scratch those chunks need
-  int grid = 0;
-  auto shape = [&](int sd) -> kp_status {
-    const size_t smem = (size_t)P.blob_bytes + (size_t)sd * 8;
-    if (occupancy(d.sys, false, smem, &bps) != cudaSuccess) {
-      cudaGetLastError();
-      return KP_ERR_CUDA;
-    }
-    if (bps < 1) return KP_ERR_ARG;  // no block of this shape can be resident
-    grid = bps * num_sms;
-    if (grid > KP_MAX_GRID) grid = KP_MAX_GRID;
-    P.sd_bytes = sd * 8;
-    return KP_OK;
-  };
-  const int min_ch = d.R_pad / (d.R_pad < 1024 ? d.R_pad : 1024);
-  kp_status ss = shape(min_ch > 1024 ? min_ch : 1024);
-  if (ss != KP_OK) return ss;
-  P.nch = region_chunks(grid, d.R_pad);
-  ss = shape(d.R_pad / P.nch > P.nch ? d.R_pad / P.nch : P.nch);
-  if (ss != KP_OK) return ss;
+  P.nch = region_chunks(d.R_pad);
+  P.sd_bytes = kChainRoom;
   const size_t smem = (size_t)P.blob_bytes + (size_t)P.sd_bytes;
+  if (occupancy(d.sys, false, smem, &bps) != cudaSuccess) {
+    cudaGetLastError();
+    return KP_ERR_CUDA;
+  }
+  if (bps < 1) return KP_ERR_ARG;  // no block of this shape can be resident
+  int grid = bps * num_sms;
+  if (grid > KP_MAX_GRID) grid = KP_MAX_GRID;
 
   cudaError_t e = cudaSuccess;
   auto ok = [&](cudaError_t r) {
@@ -2181,15 +2166,17 @@ bool try_admit(kp_server* s, PendingQuery& q) {
   P.seed_lo = (uint32_t)(q.prm.seed & 0xffffffffu);
   P.seed_hi = (uint32_t)(q.prm.seed >> 32);
   P.wait_ns = 2000000000ull;
-  const int nch = region_chunks(s->team_blocks, d.R_pad);
-  P.nch = nch;
-  P.sd_bytes = KS_SD_DOUBLES * 8;
+  P.nch = region_chunks(d.R_pad);
+  P.sd_bytes = kChainRoom;
+  // regions (padded) to one of the team's blocks, a power of two of them
+  int shares = 1;
+  while (shares * 2 <= s->team_blocks && shares * 2 * 32 <= d.R_pad && shares * 2 <= 1024) shares *= 2;
   // no cell clearances: the host would spend milliseconds per query on them
   const size_t blob_bytes = build_blob(s->blob.data(), q.boxes.empty() ? nullptr : q.boxes.data(),
                                        (int)(q.boxes.size() / 6), q.ws, P, KS_BLOB_MAX, false);
   const size_t least = (size_t)P.n_boxes_pad * 32 + round16(4) + round16((q.boxes.size() / 6) * 2);
   if (least > (size_t)KS_BLOB_MIN || blob_bytes > (size_t)KS_BLOB_MAX ||
-      d.R_pad / nch > KS_SD_DOUBLES) {
+      d.R_pad / shares > KS_MAX_SHARE) {
     pool_free(s, off, lay.total);
     finish_now(s, q.id, KP_ERR_ARG, q.t_submit);
     return true;
@@ -2366,7 +2353,7 @@ kp_status kp_server_create(const kp_server_config* cfg, void* dev_pool, size_t p
       cudaDeviceGetAttribute(&s->num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return bad(KP_ERR_CUDA);
   s->smem = ((sizeof(KParams) + 127) & ~(size_t)127) + (size_t)KS_BLOB_MAX +
-            (size_t)KS_SD_DOUBLES * 8;
+            (size_t)kChainRoom;
   if (server_occupancy(s->smem, &bps) != cudaSuccess || bps < 1) return bad(KP_ERR_CUDA);
   const int resident = bps * s->num_sms;
   s->n_teams = resident / s->team_blocks;

@@ -12,12 +12,14 @@
 
 namespace kp {
 
+// *blocks_per_sm: the threads of a block on entry, the resident blocks on return.
 cudaError_t KP_CAT(loop_occupancy_, KP_SYS_NAME)(bool log, size_t smem, int* blocks_per_sm) {
+  const int threads = *blocks_per_sm;
   const void* f = log ? (const void*)kp_loop_kernel<KP_SYS, true>
                       : (const void*)kp_loop_kernel<KP_SYS, false>;
   cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, f, KP_BLOCK, smem);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, f, threads, smem);
 }
 
 cudaError_t KP_CAT(launch_loop_, KP_SYS_NAME)(const KParams& P, int grid, size_t smem,
@@ -32,7 +34,7 @@ cudaError_t KP_CAT(launch_loop_, KP_SYS_NAME)(const KParams& P, int grid, size_t
   void* args[] = {&p, &mi, &mn, &rs, &md};
   const void* f = log ? (const void*)kp_loop_kernel<KP_SYS, true>
                       : (const void*)kp_loop_kernel<KP_SYS, false>;
-  return cudaLaunchCooperativeKernel(f, dim3(grid), dim3(KP_BLOCK), args, smem, stream);
+  return cudaLaunchCooperativeKernel(f, dim3(grid), dim3(P.threads), args, smem, stream);
 }
 
 cudaError_t KP_CAT(launch_reset_, KP_SYS_NAME)(const KParams& P, const RootState& root,

@@ -28,7 +28,21 @@ enum {
   KP_F_GOAL = 32
 };
 
-constexpr int KP_BLOCK = 256;          // threads per block of the loop kernel
+// Threads per block of a system's loop kernel: one block an SM, of as many warps
+// as the kernel's registers allow (128 a thread for the double integrator, 80
+// for the others).  Blocks of 256, two or three an SM, made every grid barrier
+// wait for 304 or 456 arrivals instead of 152 (3,300 against 2,500 clocks),
+// every block prefix add up as many counts and every SM hold the obstacles two
+// or three times.  Loop launches, 256 against these: double integrator 216 ->
+// 214 us, Dubins forest 1067 -> 1044, ragged state grid 1181 -> 1100, kd-tree
+// 966 -> 953, large frontier 5144 -> 5094, quadrotor 17.7 -> 17.2 ms; 384 (two an
+// SM) lay between, or 0.4 % ahead on the kd-tree.
+constexpr int kp_loop_threads(int sys) { return sys == KP_SYS_DI ? 512 : 768; }
+// A launch whose blocks the caller limits has blocks of 256: a few lanes that
+// each run many keys are what the limit is for.
+constexpr int KP_LIMITED_THREADS = 256;
+constexpr int KP_SERVER_THREADS = 256;  // of a block of the server's kernel
+constexpr int KP_MLP_GROUP = 256;       // threads that work on one network tile
 constexpr int KP_MAX_GRID = 8192;      // upper bound on loop-kernel blocks
 constexpr int KP_NO_GOAL = 0x7fffffff; // goal_node sentinel on the device
 constexpr int KP_TRAJ_ROWS = 16384;    // longest root-to-goal chain returned
@@ -181,7 +195,7 @@ struct KParams {
   const float* boxes;
   int32_t n_boxes_pad;
   int32_t blob_bytes;
-  int32_t sd_bytes;      // score scratch after the blob; the network tile follows
+  int32_t sd_bytes;      // room for chain ids after the blob; the network tiles follow
   int32_t extract_cap;   // chain ids kept in shared memory at most (0: room only)
   int32_t bp_g[3];       // broad-phase cells along x, y, z (1 1 1: every box in one cell)
   int32_t bp_start_off;  // byte offsets inside the blob
@@ -243,6 +257,8 @@ struct KParams {
   const float* mlp_b3;
   uint32_t mix_thr;        // learned draw iff selector word < mix_thr (0: off)
   int32_t features_on;     // node features computed each pass
+  int32_t mlp_groups;      // groups of threads with room for a network tile
+  int32_t threads;         // of a block of the loop launch
   uint16_t* feat;          // bf16 [t_e][32]: features of the V_E positions
   float* net_raw;          // [t_e][8]: network outputs of the V_E positions
   float feat_scale[6];     // 2 / (hi - lo) of a bounded state entry, 0 if unbounded
@@ -259,7 +275,7 @@ struct KParams {
 constexpr int KS_MAX_TEAMS = 1024;
 constexpr int KS_RING = 4096;          // submission / completion ring entries
 constexpr uint32_t KS_EXIT = 0xffffffffu;
-constexpr int KS_SD_DOUBLES = 1024;    // score scratch of a server block
+constexpr int KS_MAX_SHARE = 1024;     // most regions to one block of a server team
 // Obstacle blob of a server query (bytes): its boxes, one cell and its list
 // must fit KS_BLOB_MIN (1,440 boxes do), and the grid is the finest whose blob
 // fits KS_BLOB_MAX.  With 48 KB for both, 900 forest boxes fell back from 64 x 64

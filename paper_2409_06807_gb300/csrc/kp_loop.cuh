@@ -12,7 +12,8 @@
 //      reached sub-regions (smallest sample key wins), keep the end state
 //      of a sample that may still be accepted.
 //   A  accept decisions (representative or P_accept draw), accepted keys
-//      compacted per warp in key order; alongside, on warp 0:
+//      compacted per warp in key order; before it, on the warps with a region
+//      chunk (a block's first, which takes no keys):
 //   S  Score per region (Eq. 3-4, FP64, rounded exactly as written) and
 //      the pairwise partial sum of each aligned region chunk (Eq. 5's sum).
 //   N  first, on warp 0 of each region-chunk block, T: the sum of Eq. 5
@@ -34,26 +35,37 @@
 #include "kp_device.cuh"
 #include "kp_mlp.cuh"
 
+#ifndef KP_MIN_BLOCKS
+#define KP_MIN_BLOCKS 1
+#endif
+
 namespace kp {
 
+// (KP_BLOCK, the most threads of a block, is set by the including file)
 constexpr int KP_WARPS = KP_BLOCK / 32;
+static_assert(KP_WARPS <= 32 && KP_BLOCK % KP_MLP_GROUP == 0, "warps fit a lane each, groups are whole");
 
 struct LoopShared {
-  // one value a warp: the expand phase's five counters, the counts a block
-  // prefix adds up, the warps' tile counts (two tiles in turn)
-  unsigned long long cnt[5][KP_WARPS];
-  uint32_t pre[KP_WARPS], tot[KP_WARPS];
-  uint32_t tile[2][KP_WARPS];
+  union {
+    // the expand phase's five counters, a value a warp
+    unsigned long long cnt[5][KP_WARPS];
+    struct {
+      // a value a warp: the counts a block prefix adds up, the tile counts of
+      // the V_E list (two tiles in turn)
+      uint32_t pre[KP_WARPS], tot[KP_WARPS];
+      uint32_t tile[2][KP_WARPS];
+      // accepted samples of this block, from the accept phase to the node-set
+      // phase: warp w compacted acc_n[w] keys at acc_key[acc_a[w]...], which
+      // are the block's accepted samples acc_off[w] .. acc_off[w] + acc_n[w] - 1
+      int acc_a[KP_WARPS], acc_n[KP_WARPS], acc_off[KP_WARPS];
+      int acc_tot;
+    };
+  };
   uint64_t mbar;
   int flag;
   int bcast[2];
   int goal, err;         // the pass's goal node and error word, read in phase L
   int32_t phase_ns[12];  // per-pass phase timers (block 0, thread 0)
-  // accepted samples of this block, from the accept phase to the node-set
-  // phase: warp w compacted acc_n[w] keys at acc_key[acc_a[w]...], which
-  // are the block's accepted samples acc_off[w] .. acc_off[w] + acc_n[w] - 1
-  int acc_a[KP_WARPS], acc_n[KP_WARPS], acc_off[KP_WARPS];
-  int acc_tot;
 };
 
 // Stage the obstacle blob (boxes and broad-phase grid) into shared memory
@@ -132,6 +144,18 @@ __device__ __forceinline__ void chunk_of(const Team& T, int n, int* c0, int* c1)
   *c1 = (int)(a + per < n ? a + per : n);
 }
 
+// Sum of one value per warp of the block, by every warp (a lane a value).
+__device__ __forceinline__ uint32_t warp_total(const uint32_t* v) {
+  const uint32_t lane = threadIdx.x & 31u;
+  return __reduce_add_sync(0xffffffffu, lane < (blockDim.x >> 5) ? v[lane] : 0u);
+}
+
+// The same over the warps before this one.
+__device__ __forceinline__ uint32_t warp_before(const uint32_t* v) {
+  const uint32_t lane = threadIdx.x & 31u;
+  return __reduce_add_sync(0xffffffffu, lane < (threadIdx.x >> 5) ? v[lane] : 0u);
+}
+
 // Sum of blk[0..nb) and of blk[0..b) (counts of at most 2^28 in all): a
 // reduction per warp, one block barrier, then every thread adds the warps'
 // sums.  The shared values are free again after the block's next barrier.
@@ -150,14 +174,8 @@ __device__ __forceinline__ void block_prefix(const Team& T, const uint32_t* blk,
     sh.tot[threadIdx.x >> 5] = tot;
   }
   __syncthreads();
-  pre = tot = 0;
-#pragma unroll
-  for (int w = 0; w < KP_WARPS; ++w) {
-    pre += sh.pre[w];
-    tot += sh.tot[w];
-  }
-  *before = pre;
-  *total = tot;
+  *before = warp_total(sh.pre);
+  *total = warp_total(sh.tot);
 }
 
 // Nodes of a block's chunk are visited in tiles of blockDim.x: node v0 +
@@ -169,10 +187,7 @@ __device__ __forceinline__ uint32_t block_sum(uint32_t c, LoopShared& sh) {
   c = __reduce_add_sync(0xffffffffu, c);
   if ((threadIdx.x & 31u) == 0) sh.pre[threadIdx.x >> 5] = c;
   __syncthreads();
-  uint32_t s = 0;
-#pragma unroll
-  for (int w = 0; w < KP_WARPS; ++w) s += sh.pre[w];
-  return s;
+  return warp_total(sh.pre);
 }
 
 // Phase N': count V_E members of this block's node chunk (no draws) and
@@ -205,13 +220,7 @@ __device__ __forceinline__ int write_ve(const KParams& P, const Team& T, int n, 
     // the other buffer's readers are past this barrier before it is written
     if (lane == 0) sh.tile[buf][w] = (uint32_t)__popc(bal);
     __syncthreads();
-    int before = 0, tile = 0;
-#pragma unroll
-    for (int q = 0; q < KP_WARPS; ++q) {
-      const int cq = (int)sh.tile[buf][q];
-      before += q < (int)w ? cq : 0;
-      tile += cq;
-    }
+    const int before = (int)warp_before(sh.tile[buf]), tile = (int)warp_total(sh.tile[buf]);
     if (m) P.ve[KP_IDX(P, base + before + __popc(bal & ((1u << lane) - 1u)), P.t_e, 4)] = v;
     base += tile;
   }
@@ -282,13 +291,16 @@ __device__ __forceinline__ void node_feature_pair(const KParams& P, int v, int q
 }
 
 // Phase F: features of every V_E position (kept for the harvest) and, with
-// a network attached, its outputs, in tiles of 32 positions per block; 16
-// threads share the features of one position.  Not inlined: it runs once
+// a network attached, its outputs, in tiles of 32 positions per group of 256
+// threads; 16 threads share the features of one position.  Not inlined: it runs once
 // per pass, and as a call it gets the register budget of the loop kernel
 // to itself instead of sharing it with the loop state live around it.
 static __device__ __noinline__ void phase_features(const KParams& P, const Team& T, int n_ve,
                                                    unsigned char* mtile) {
-  __nv_bfloat16* sX = reinterpret_cast<__nv_bfloat16*>(mtile);
+  const int group = (int)threadIdx.x / KP_MLP_GROUP, groups = P.mlp_groups;
+  if (group >= groups) return;  // (no room for their tiles)
+  const int tid = (int)threadIdx.x % KP_MLP_GROUP;
+  __nv_bfloat16* sX = reinterpret_cast<__nv_bfloat16*>(mtile + group * MLP_LOOP_TILE_SMEM);
   __nv_bfloat16* sH = sX + MLP_LOOP_TILE * MLP_XS;
   MlpWeights w;
   w.W1 = reinterpret_cast<const __nv_bfloat16*>(P.mlp_W1);
@@ -298,23 +310,23 @@ static __device__ __noinline__ void phase_features(const KParams& P, const Team&
   w.W3 = reinterpret_cast<const __nv_bfloat16*>(P.mlp_W3);
   w.b3 = P.mlp_b3;
   const int n_tiles = (n_ve + MLP_LOOP_TILE - 1) / MLP_LOOP_TILE;
-  const int q = threadIdx.x & 15;  // 16 rows x 16 feature pairs per round
-  for (int tile = T.b; tile < n_tiles; tile += T.nb) {
+  const int q = tid & 15;  // 16 rows x 16 feature pairs per round
+  for (int tile = T.b + T.nb * group; tile < n_tiles; tile += T.nb * groups) {
     const int p0 = tile * MLP_LOOP_TILE;
     const int rows = n_ve - p0 < MLP_LOOP_TILE ? n_ve - p0 : MLP_LOOP_TILE;
 #pragma unroll
     for (int rr = 0; rr < MLP_LOOP_TILE; rr += 16) {
-      const int row = rr + (threadIdx.x >> 4);
+      const int row = rr + (tid >> 4);
       float f2[2] = {0.0f, 0.0f};
       if (row < rows) node_feature_pair(P, P.ve[p0 + row], q, f2);
       const uint32_t v2 = pack_bf16(f2[0], f2[1]);
       *reinterpret_cast<uint32_t*>(sX + row * MLP_XS + 2 * q) = v2;
       if (row < rows) *reinterpret_cast<uint32_t*>(P.feat + (size_t)(p0 + row) * 32 + 2 * q) = v2;
     }
-    __syncthreads();
+    mlp_group_sync();
     if (P.mix_thr)
       mlp_tile_forward<MLP_LOOP_TILE / 16>(w, sX, sH, P.net_raw, p0, rows);
-    __syncthreads();
+    mlp_group_sync();
   }
 }
 
@@ -617,7 +629,8 @@ __device__ __forceinline__ void phase_expand(const KParams& P, const Team& T,
   __syncthreads();
   if (threadIdx.x < 5) {
     unsigned long long s = 0;
-    for (int w = 0; w < KP_WARPS; ++w) s += sh.cnt[threadIdx.x][w];
+#pragma unroll 4
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += sh.cnt[threadIdx.x][w];
     static_assert(offsetof(KCtl, tot_refills) == offsetof(KCtl, tot_steps) + 32, "counters in order");
     if (s) atomicAdd(&P.ctl->tot_steps + threadIdx.x, s);
   }
@@ -649,13 +662,12 @@ __device__ __forceinline__ void warp_range(int c0, int c1, int* a, int* b) {
 // offsets among the block's, in shared memory for the node-set phase.
 constexpr int KP_ACC_KPL = 8;
 
-__device__ __forceinline__ void phase_scores(const KParams& P, const Team& T, int nch, double* sd);
-__device__ __forceinline__ void phase_score_sum(const KParams& P, const Team& T, int nch, double* sd);
+__device__ __forceinline__ void phase_scores(const KParams& P, const Team& T, int nch);
 
 template <bool LOG>
 __device__ __forceinline__ void phase_accept(const KParams& P, const Team& T, int S, int nch,
-                                             double* sd, LoopShared& sh) {
-  phase_scores(P, T, nch, sd);
+                                             LoopShared& sh) {
+  phase_scores(P, T, nch);
   const uint32_t FULL = 0xffffffffu;
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t lt = (1u << lane) - 1u;
@@ -705,13 +717,8 @@ __device__ __forceinline__ void phase_accept(const KParams& P, const Team& T, in
     sh.tot[w] = n_valid;
   }
   __syncthreads();
-  int off = 0, block_acc = 0;
-#pragma unroll
-  for (int q = 0; q < KP_WARPS; ++q) {
-    const int cq = (int)sh.pre[q];
-    off += q < w ? cq : 0;
-    block_acc += cq;
-  }
+  const int off = (int)warp_before(sh.pre), block_acc = (int)warp_total(sh.pre);
+  const uint32_t bv = warp_total(sh.tot);
   if (lane == 0) {
     sh.acc_a[w] = a;
     sh.acc_n[w] = n_acc;
@@ -719,35 +726,29 @@ __device__ __forceinline__ void phase_accept(const KParams& P, const Team& T, in
   }
   if (threadIdx.x == 0) {
     sh.acc_tot = block_acc;
-    uint32_t bv = 0;
-    for (int q = 0; q < KP_WARPS; ++q) bv += sh.tot[q];
     if (T.b == 0) P.ctl->work_next = 0;  // the expand phase is over
     P.blk_a[KP_IDX(P, T.b, KP_MAX_GRID, 15)] = (uint32_t)block_acc;
     if (bv) atomicAdd(&P.ctl->it_valid, bv);
   }
-  // the chunk's partial sum, once every warp's scores are there
-  if (threadIdx.x < 32) phase_score_sum(P, T, nch, sd);
 }
 
-// Pairwise sum of buf[0..n), n a power of two, by one warp (bottom-up
-// tree, the same tree as recursive halving); result in buf[0].
-__device__ __forceinline__ void warp_pairwise(double* buf, int n) {
-  const int lane = (int)(threadIdx.x & 31u);
-  for (int stride = 1; stride < n; stride <<= 1) {
-    __syncwarp();
-    for (int i = lane * 2 * stride; i < n; i += 64 * stride)
-      buf[i] = __dadd_rn(buf[i], buf[i + stride]);
-  }
-  __syncwarp();
-}
-
-// The same tree for n <= 32 KP_TREE_PER_LANE, in registers: lane l loads
-// the m = max(n / 32, 1) values l m .. l m + m - 1 through load(i), adds
+// Pairwise (bottom-up, the same tree as recursive halving) sum of n values, n a
+// power of two at most 32 KP_TREE_PER_LANE, by one warp in registers: lane l
+// loads the m = max(n / 32, 1) values l m .. l m + m - 1 through load(i), adds
 // the tree's levels of stride below m in place, and the levels of stride m,
-// 2m, ... across lanes by shuffles (left operand the lower index, as in
-// the shared-memory tree).  Every lane gets the sum.  No shared memory and
-// no warp barrier per level.
+// 2m, ... across lanes by shuffles (left operand the lower index).  Every lane
+// gets the sum.
 constexpr int KP_TREE_PER_LANE = 8;
+
+// The levels across the first 'lanes' lanes (a power of two).
+__device__ __forceinline__ double warp_tree_lanes(double sum, int lanes) {
+  const int lane = (int)(threadIdx.x & 31u);
+  for (int d = 1; d < lanes; d <<= 1) {
+    const double o = __shfl_down_sync(0xffffffffu, sum, d);
+    if ((lane & (2 * d - 1)) == 0) sum = __dadd_rn(sum, o);
+  }
+  return __shfl_sync(0xffffffffu, sum, 0);
+}
 
 template <class L>
 __device__ __forceinline__ double warp_tree_sum(int n, L load) {
@@ -764,106 +765,95 @@ __device__ __forceinline__ double warp_tree_sum(int n, L load) {
 #pragma unroll
     for (int q = 0; q + st < KP_TREE_PER_LANE; q += 2 * st)
       if (st < m) v[q] = __dadd_rn(v[q], v[q + st]);
-  double sum = v[0];
-  const int lanes = n / m;
-  for (int d = 1; d < lanes; d <<= 1) {
-    const double o = __shfl_down_sync(0xffffffffu, sum, d);
-    if ((lane & (2 * d - 1)) == 0) sum = __dadd_rn(sum, o);
-  }
-  return __shfl_sync(0xffffffffu, sum, 0);
+  return warp_tree_lanes(v[0], n / m);
 }
 
-// Phase S: Eq. 3-4 for this block's region chunk, 32 regions a warp in turn
-// (the FP64 unit makes about two operations a clock and SM, and a division is
-// a chain of a dozen: one warp that took all of a 512-region chunk, as the
-// server's small teams have, held the pass up by 16 chains).  Every operation
-// is an explicitly rounded IEEE double operation in the order
+// Region chunks of the score sums: nch of them (a power of two, at most 256),
+// chunk c the work of warp c / blocks of block c % blocks (then of the same
+// warp again, were there more chunks than warps).
+template <class F>
+__device__ __forceinline__ void for_own_chunks(const Team& T, int nch, F body) {
+  for (int c = T.b + T.nb * (int)(threadIdx.x >> 5); c < nch; c += T.nb * (int)(blockDim.x >> 5)) body(c);
+}
+
+// Phase S: Eq. 3-4 for a warp's region chunk and the chunk's pairwise partial
+// sum (published by the grid barrier that ends the phase).  Lane l takes the
+// chunk's m = max(ch / 32, 1) regions from l m on and adds their scores up as
+// they come: level k of the tree waits in left[k] for its right half.  Most
+// decompositions have chunks of 32 (a region a lane): FP64 divisions are long
+// chains here (about two FP64 operations a clock and SM), and one warp that
+// took all of a 512-region chunk, as a small team has, held the pass up by 16
+// of them.  Every operation is an explicitly rounded IEEE double operation in
+// the order
 // FreeVol = ((delta + nv) vol) / ((delta + nv) + ni),
 // f4 = (FreeVol FreeVol)(FreeVol FreeVol),
 // Score = f4 / ((1 + Cov)(1 + (nv + ni)(nv + ni))).
-__device__ __forceinline__ void phase_scores(const KParams& P, const Team& T, int nch, double* sd) {
-  if (T.b >= nch) return;
+__device__ __forceinline__ void phase_scores(const KParams& P, const Team& T, int nch) {
+  const int lane = (int)(threadIdx.x & 31u);
   const int ch = P.R_pad / nch;
-  const int r0 = T.b * ch;
-  for (int i = (int)threadIdx.x; i < ch; i += (int)blockDim.x) {
-    const int r = r0 + i;
-    double sc = 0.0;
-    if (r < P.R && P.avail[r]) {
-      const double nv = (double)P.n_valid[r], ni = (double)P.n_invalid[r];
-      const double dn = __dadd_rn(P.delta, nv);
-      const double vol = P.region_vol ? P.region_vol[r] : P.vol;
-      const double fv = __ddiv_rn(__dmul_rn(dn, vol), __dadd_rn(dn, ni));
-      const double f2 = __dmul_rn(fv, fv);
-      const double f4 = __dmul_rn(f2, f2);
-      const double na = __dadd_rn(nv, ni);
-      const double den =
-          __dmul_rn(__dadd_rn(1.0, (double)P.cov[r]), __dadd_rn(1.0, __dmul_rn(na, na)));
-      sc = __ddiv_rn(f4, den);
+  const int m = ch >= 32 ? ch >> 5 : 1;  // below 2^12: R is at most 2^24
+  for_own_chunks(T, nch, [&](int c) {
+    double left[12], sum = 0.0;
+#pragma unroll 1
+    for (int q = 0; q < m; ++q) {
+      const int r = c * ch + lane * m + q;
+      double sc = 0.0;
+      if (lane < ch && r < P.R) {
+        if (P.avail[r]) {
+          const double nv = (double)P.n_valid[r], ni = (double)P.n_invalid[r];
+          const double dn = __dadd_rn(P.delta, nv);
+          const double vol = P.region_vol ? P.region_vol[r] : P.vol;
+          const double fv = __ddiv_rn(__dmul_rn(dn, vol), __dadd_rn(dn, ni));
+          const double f2 = __dmul_rn(fv, fv);
+          const double f4 = __dmul_rn(f2, f2);
+          const double na = __dadd_rn(nv, ni);
+          const double den =
+              __dmul_rn(__dadd_rn(1.0, (double)P.cov[r]), __dadd_rn(1.0, __dmul_rn(na, na)));
+          sc = __ddiv_rn(f4, den);
+        }
+        P.score[r] = sc;
+      }
+      int k = 0;
+      for (; (q >> k) & 1; ++k) sc = __dadd_rn(left[k], sc);
+      if (k < 12) left[k] = sc;
+      sum = sc;
     }
-    if (r < P.R) P.score[r] = sc;
-    sd[i] = sc;
-  }
+    const double part = warp_tree_lanes(sum, ch < 32 ? ch : 32);
+    if (lane == 0) P.chunk_sum[KP_IDX(P, c, KP_MAX_GRID, 16)] = part;
+  });
 }
 
-// The chunk's pairwise partial sum (warp 0, after a block barrier that follows
-// phase_scores; published before the grid barrier that ends the phase).
-__device__ __forceinline__ void phase_score_sum(const KParams& P, const Team& T, int nch, double* sd) {
-  if (T.b >= nch) return;
+// Phase T (the chunks' warps in the node-set phase): the sum of Eq. 5 from the
+// chunks' partial sums (each of these warps reduces them itself, in the same
+// pairwise tree, so all get the same value), then P_accept and the integer
+// threshold of the chunk's regions; each chunk done is counted in t_done.
+__device__ __forceinline__ void phase_thresholds(const KParams& P, const Team& T, int nch) {
   const int lane = (int)(threadIdx.x & 31u);
-  const int ch = P.R_pad / nch;
-  double part;
-  if (ch <= 32 * KP_TREE_PER_LANE) {
-    part = warp_tree_sum(ch, [&](int i) { return sd[i]; });
-  } else {
-    warp_pairwise(sd, ch);
-    part = sd[0];
-  }
-  if (lane == 0) P.chunk_sum[KP_IDX(P, T.b, KP_MAX_GRID, 16)] = part;
-}
-
-// Warps of a region-chunk block that write thresholds: one for 32 regions (one
-// in all where the chunk sums are added up in the shared scratch).
-__device__ __forceinline__ int threshold_warps(const KParams& P, int nch) {
-  if (nch > 32 * KP_TREE_PER_LANE) return 1;
-  const int w = (P.R_pad / nch + 31) >> 5;
-  return w < KP_WARPS ? w : KP_WARPS;
-}
-
-// Phase T (the first 'warps' warps of a chunk block in the node-set phase):
-// the sum of Eq. 5 from the chunks' partial sums (each of these warps reduces
-// them itself, in the same pairwise tree, so all get the same value; in
-// registers up to 256 chunks, else by the one warp in the scratch), then
-// P_accept and the integer threshold of the warp's regions.
-__device__ __forceinline__ void phase_thresholds(const KParams& P, const Team& T, int nch, int warps,
-                                                 double* sd) {
-  const int lane = (int)(threadIdx.x & 31u);
-  double sum;
-  if (nch <= 32 * KP_TREE_PER_LANE) {
-    sum = warp_tree_sum(nch, [&](int i) { return __ldcg(P.chunk_sum + i); });
-  } else {
-    for (int i = lane; i < nch; i += 32) sd[i] = __ldcg(P.chunk_sum + i);
-    warp_pairwise(sd, nch);
-    sum = sd[0];
-  }
+  if (T.b + T.nb * (int)(threadIdx.x >> 5) >= nch) return;
+  const double sum = warp_tree_sum(nch, [&](int i) { return __ldcg(P.chunk_sum + i); });
   if (T.b == 0 && threadIdx.x == 0) P.ctl->score_sum = sum;
   const int ch = P.R_pad / nch;
-  const int r0 = T.b * ch;
-  for (int i = (int)threadIdx.x; i < ch; i += 32 * warps) {
-    const int r = r0 + i;
-    if (r >= P.R) break;
-    uint64_t thr = 1ull << 32;  // P_accept = 1 outside R_avail
-    if (P.avail[r]) {
-      double p;
-      if (sum > 0.0) {
-        p = __dadd_rn(__ddiv_rn(P.score[r], sum), P.eps);
-        if (p > 1.0) p = 1.0;
-      } else {
-        p = P.eps < 1.0 ? P.eps : 1.0;
+  for_own_chunks(T, nch, [&](int c) {
+    for (int i = lane; i < ch; i += 32) {
+      const int r = c * ch + i;
+      if (r >= P.R) break;
+      uint64_t thr = 1ull << 32;  // P_accept = 1 outside R_avail
+      if (P.avail[r]) {
+        double p;
+        if (sum > 0.0) {
+          p = __dadd_rn(__ddiv_rn(P.score[r], sum), P.eps);
+          if (p > 1.0) p = 1.0;
+        } else {
+          p = P.eps < 1.0 ? P.eps : 1.0;
+        }
+        if (p < 1.0) thr = (uint64_t)floor(__dmul_rn(p, 4294967296.0));
       }
-      if (p < 1.0) thr = (uint64_t)floor(__dmul_rn(p, 4294967296.0));
+      P.thr[r] = thr;
     }
-    P.thr[r] = thr;
-  }
+    __threadfence();
+    __syncwarp();
+    if (lane == 0) atomicAdd(&P.ctl->t_done, 1u);
+  });
 }
 
 // Materialises this block's accepted samples as the nodes id0 .. id0 +
@@ -883,10 +873,12 @@ __device__ __forceinline__ void materialise(const KParams& P, uint32_t it, int i
   using Sys = System<SYS>;
   constexpr int D = Sys::D, N = Sys::N;
   for (int j = (int)threadIdx.x; j < sh.acc_tot; j += (int)blockDim.x) {
+    // the warp that holds it: the last one whose offset is at most j (warps
+    // without samples have their successor's offset)
     int w = 0;
 #pragma unroll
-    for (int q = 0; q < KP_WARPS; ++q)
-      if (j >= sh.acc_off[q] && j < sh.acc_off[q] + sh.acc_n[q]) w = q;
+    for (int s = 16; s > 0; s >>= 1)
+      if (w + s < (int)(blockDim.x >> 5) && sh.acc_off[w + s] <= j) w += s;
     const uint32_t e = P.acc_key[KP_IDX(P, sh.acc_a[w] + (j - sh.acc_off[w]), P.t_e, 17)];
     const int key = KP_IDX(P, (int)(e & 0x7fffffffu), P.t_e, 18);
     const int id = KP_IDX(P, id0 + j, P.t_e, 19);
@@ -957,9 +949,8 @@ __device__ __forceinline__ void materialise(const KParams& P, uint32_t it, int i
 // purpose 2) against the threshold of its region; new nodes are in V_E.
 // Publishes the block chunk's V_E count; returns in *n_new the number of
 // accepted samples of the pass (the new nodes).
-// Order inside the phase: the first warps of every region-chunk block write
-// its chunk's thresholds (phase T, 32 regions a warp in turn) and count
-// themselves done; every block
+// Order inside the phase: the warps with a region chunk write its thresholds
+// (phase T) and count it done; every block then
 // appends its own accepted samples (ids from t_old, in key order), which
 // needs no threshold; then it waits (bounded) until every chunk is done and
 // makes the node-set draws.  New nodes are counted as V_E members without
@@ -967,23 +958,18 @@ __device__ __forceinline__ void materialise(const KParams& P, uint32_t it, int i
 template <int SYS, bool LOG>
 __device__ __forceinline__ void phase_nodesets(const KParams& P, const Team& T, uint32_t it,
                                                int t_old, const KeyDiv& kd, LoopShared& sh, int* n_new,
-                                               const unsigned char* sblob, double* sd) {
-  const int nch = P.nch, warps = threshold_warps(P, nch);
+                                               const unsigned char* sblob) {
+  const int nch = P.nch;
   uint32_t acc_before, acc_total;
   block_prefix(T, P.blk_a, sh, &acc_before, &acc_total);
-  if (T.b < nch && (int)(threadIdx.x >> 5) < warps) {
-    phase_thresholds(P, T, nch, warps, sd);
-    __threadfence();
-    __syncwarp();
-    if ((threadIdx.x & 31u) == 0) atomicAdd(&P.ctl->t_done, 1u);
-  }
+  phase_thresholds(P, T, nch);
   *n_new = (int)acc_total;
   const int t_new = t_old + (int)acc_total;
   materialise<SYS, LOG>(P, it, t_old + (int)acc_before, kd, sh, sblob);
   if (threadIdx.x == 0) {
     uint64_t t0 = 0;
     uint32_t spins = 0;
-    while (ld_acquire(&P.ctl->t_done) < (uint32_t)(nch * warps)) {
+    while (ld_acquire(&P.ctl->t_done) < (uint32_t)nch) {
       if ((++spins & 63u) == 0) {
         if (*((volatile int*)&P.ctl->err) != 0) break;
         if (t0 == 0) t0 = global_ns();
@@ -1038,7 +1024,6 @@ __device__ __forceinline__ void phase_nodesets(const KParams& P, const Team& T, 
 template <int SYS, bool LOG>
 __device__ __forceinline__ bool run_loop(const KParams& P, const Team& T, unsigned char* smem,
                                          LoopShared& sh, int max_iters, uint64_t max_ns) {
-  double* sd = reinterpret_cast<double*>(smem + (size_t)P.blob_bytes);
   KCtl* ctl = P.ctl;
   const uint64_t t_start = global_ns();
   if (T.b == 0 && threadIdx.x == 0) {
@@ -1101,14 +1086,14 @@ __device__ __forceinline__ bool run_loop(const KParams& P, const Team& T, unsign
     stamp(0);
     if (!team_sync(T, ctl, P.wait_ns, 20)) return false;
     stamp(1);
-    phase_accept<LOG>(P, T, S, nch, sd, sh);
+    phase_accept<LOG>(P, T, S, nch, sh);
     stamp(2);
     if (!team_sync(T, ctl, P.wait_ns, 21)) return false;
     stamp(4);
     if (timer) phase_ns[5] = phase_ns[7] = 0;
     const int t_old = n_tree;
     int n_acc;
-    phase_nodesets<SYS, LOG>(P, T, it, t_old, kd, sh, &n_acc, smem, sd);
+    phase_nodesets<SYS, LOG>(P, T, it, t_old, kd, sh, &n_acc, smem);
     n_tree = t_old + n_acc;
     stamp(8);
     if (!team_sync(T, ctl, P.wait_ns, 23)) return false;
@@ -1268,9 +1253,6 @@ __device__ void extract_chain_block(const KParams& P, int* ids, int cap) {
   }
 }
 
-#ifndef KP_MIN_BLOCKS
-#define KP_MIN_BLOCKS 1
-#endif
 // Single-query launch: the whole grid is one team.  mode: KP_LOOP_RESET
 // runs Algorithm 1's initialisation from 'root' first, KP_LOOP_EXTRACT
 // writes the root-to-goal chain after the passes (block 0, the ids kept in

@@ -22,6 +22,14 @@ constexpr float MLP_LOGSTD_MIN = -4.0f, MLP_LOGSTD_MAX = 1.0f;
 // shared memory of one loop tile: input rows + hidden rows (bf16)
 constexpr int MLP_LOOP_TILE_SMEM = MLP_LOOP_TILE * MLP_XS * 2 + MLP_LOOP_TILE * MLP_HS * 2;
 
+// The 256 threads that share a network tile: their warp's number in the group,
+// and a barrier among them (named barriers 1, 2, .. of the block).
+__device__ __forceinline__ int mlp_warp() { return (int)(threadIdx.x & 255u) >> 5; }
+
+__device__ __forceinline__ void mlp_group_sync() {
+  asm volatile("bar.sync %0, 256;" ::"r"(1 + (int)(threadIdx.x >> 8)) : "memory");
+}
+
 struct MlpWeights {         // weights in fragment order
   const __nv_bfloat16* W1;  // [256][32]
   const float* b1;
@@ -92,7 +100,7 @@ __host__ __device__ __forceinline__ int frag_index_out(int n, int k) {
 // hidden layer's weights in fragment order.
 __device__ __forceinline__ void frag_b4_ordered(const __nv_bfloat16* Wf, int K, int s,
                                                 uint32_t b[4][2]) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = mlp_warp(), lane = threadIdx.x & 31;
   const uint4* q = reinterpret_cast<const uint4*>(Wf) + (((warp * (K >> 4) + s) * 32 + lane) * 2);
   const uint4 u0 = __ldg(q), u1 = __ldg(q + 1);
   b[0][0] = u0.x; b[0][1] = u0.y; b[1][0] = u0.z; b[1][1] = u0.w;
@@ -107,7 +115,7 @@ template <int K, int MI>
 __device__ __forceinline__ void layer_relu(const __nv_bfloat16* in, int ld_in,
                                            const __nv_bfloat16* W, const float* bias,
                                            float acc[MI][4][4]) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, t = lane & 3;
+  const int warp = mlp_warp(), lane = threadIdx.x & 31, t = lane & 3;
   const int n_base = warp * 32;
 #pragma unroll
   for (int mi = 0; mi < MI; ++mi)
@@ -141,7 +149,7 @@ __device__ __forceinline__ void layer_relu(const __nv_bfloat16* in, int ld_in,
 // Writes a layer's register results as bf16 into a smem tile.
 template <int MI>
 __device__ __forceinline__ void store_hidden(const float acc[MI][4][4], __nv_bfloat16* s) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gi = lane >> 2, t = lane & 3;
+  const int warp = mlp_warp(), lane = threadIdx.x & 31, gi = lane >> 2, t = lane & 3;
 #pragma unroll
   for (int mi = 0; mi < MI; ++mi)
 #pragma unroll
@@ -157,7 +165,7 @@ __device__ __forceinline__ void store_hidden(const float acc[MI][4][4], __nv_bfl
 
 // Forward pass of one tile of 16*MI rows.  sX holds the bf16 inputs (row
 // stride MLP_XS), sH is scratch (16*MI x MLP_HS bf16).  Writes the 8 raw
-// outputs of valid rows to raw[(row0 + r) * 8 ..].  Every thread of the block
+// outputs of valid rows to raw[(row0 + r) * 8 ..].  Every thread of the group
 // (256) must call it.
 //
 // The output layer (K = 256, 8 columns) is split over K: warp w multiplies
@@ -172,12 +180,12 @@ __device__ __forceinline__ void mlp_tile_forward(const MlpWeights& w, const __nv
   float acc[MI][4][4];
   layer_relu<MLP_IN, MI>(sX, MLP_XS, w.W1, w.b1, acc);
   store_hidden<MI>(acc, sH);
-  __syncthreads();
+  mlp_group_sync();
   layer_relu<MLP_H, MI>(sH, MLP_HS, w.W2, w.b2, acc);
-  __syncthreads();  // every warp has read h1
+  mlp_group_sync();  // every warp has read h1
   store_hidden<MI>(acc, sH);
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gi = lane >> 2, t = lane & 3;
+  mlp_group_sync();
+  const int warp = mlp_warp(), lane = threadIdx.x & 31, gi = lane >> 2, t = lane & 3;
   float d[MI][4];
   uint32_t b[2][2];
   {
@@ -194,7 +202,7 @@ __device__ __forceinline__ void mlp_tile_forward(const MlpWeights& w, const __nv
       mma_bf16_16816(d[mi], a, b[ks]);
     }
   }
-  __syncthreads();  // every warp has read h2: sH now holds the partials
+  mlp_group_sync();  // every warp has read h2: sH now holds the partials
   float* part = reinterpret_cast<float*>(sH);  // [8 warps][16*MI rows][8]
 #pragma unroll
   for (int mi = 0; mi < MI; ++mi)
@@ -204,15 +212,15 @@ __device__ __forceinline__ void mlp_tile_forward(const MlpWeights& w, const __nv
       part[(warp * 16 * MI + r) * MLP_OUT + 2 * t] = d[mi][2 * h];
       part[(warp * 16 * MI + r) * MLP_OUT + 2 * t + 1] = d[mi][2 * h + 1];
     }
-  __syncthreads();
-  for (int e = threadIdx.x; e < 16 * MI * MLP_OUT; e += blockDim.x) {
+  mlp_group_sync();
+  for (int e = threadIdx.x & 255; e < 16 * MI * MLP_OUT; e += 256) {
     const int r = e / MLP_OUT, c = e % MLP_OUT;
     float s = w.b3[c];
 #pragma unroll
     for (int q = 0; q < 8; ++q) s += part[(q * 16 * MI + r) * MLP_OUT + c];
     if (r < rows_valid) raw[(size_t)(row0 + r) * MLP_OUT + c] = s;
   }
-  __syncthreads();
+  mlp_group_sync();
 }
 
 // Heads of one output row: mean = tanh, log_std clamped.
