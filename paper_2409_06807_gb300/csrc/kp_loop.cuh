@@ -159,8 +159,14 @@ __device__ __forceinline__ uint32_t warp_before(const uint32_t* v) {
 // Sum of blk[0..nb) and of blk[0..b) (counts of at most 2^28 in all): a
 // reduction per warp, one block barrier, then every thread adds the warps'
 // sums.  The shared values are free again after the block's next barrier.
+// 'publish' runs before the barrier: what it writes is read after it.
+struct Nothing {
+  __device__ __forceinline__ void operator()() const {}
+};
+
+template <class F = Nothing>
 __device__ __forceinline__ void block_prefix(const Team& T, const uint32_t* blk, LoopShared& sh,
-                                             uint32_t* before, uint32_t* total) {
+                                             uint32_t* before, uint32_t* total, F publish = F()) {
   uint32_t pre = 0, tot = 0;
   for (int i = threadIdx.x; i < T.nb; i += blockDim.x) {
     const uint32_t c = __ldcg(blk + i);
@@ -173,6 +179,7 @@ __device__ __forceinline__ void block_prefix(const Team& T, const uint32_t* blk,
     sh.pre[threadIdx.x >> 5] = pre;
     sh.tot[threadIdx.x >> 5] = tot;
   }
+  publish();
   __syncthreads();
   *before = warp_total(sh.pre);
   *total = warp_total(sh.tot);
@@ -206,16 +213,26 @@ __device__ __forceinline__ void count_ve(const KParams& P, const Team& T, int n,
 // the block's offset is the sum of the counts before it; inside the chunk
 // each tile is compacted in node order (warp ballots, then the warps'
 // counts in order).  Returns |V_E|.
-__device__ __forceinline__ int write_ve(const KParams& P, const Team& T, int n, LoopShared& sh) {
+// goal_now, err_now: thread 0's reads of those words, for the block (sh.goal,
+// sh.err); they and the first tile's flags are fetched beside the counts.
+__device__ __forceinline__ int write_ve(const KParams& P, const Team& T, int n, LoopShared& sh,
+                                        int goal_now = 0, int err_now = 0) {
   int v0, v1;
   chunk_of(T, n, &v0, &v1);
+  auto member = [&](int v) { return v < v1 && P.in_ve[KP_IDX(P, v, P.t_e, 3)]; };
+  bool first = member(v0 + (int)threadIdx.x);
   uint32_t off, total;
-  block_prefix(T, P.blk_b, sh, &off, &total);
+  block_prefix(T, P.blk_b, sh, &off, &total, [&]() {
+    if (threadIdx.x == 0) {
+      sh.goal = goal_now;
+      sh.err = err_now;
+    }
+  });
   const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5;
   int base = (int)off, buf = 0;
   for (int t0 = v0; t0 < v1; t0 += (int)blockDim.x, buf ^= 1) {
     const int v = t0 + (int)threadIdx.x;
-    const bool m = v < v1 && P.in_ve[KP_IDX(P, v, P.t_e, 3)];
+    const bool m = t0 == v0 ? first : member(v);
     const uint32_t bal = __ballot_sync(0xffffffffu, m);
     // the other buffer's readers are past this barrier before it is written
     if (lane == 0) sh.tile[buf][w] = (uint32_t)__popc(bal);
@@ -799,17 +816,19 @@ __device__ __forceinline__ void phase_scores(const KParams& P, const Team& T, in
       const int r = c * ch + lane * m + q;
       double sc = 0.0;
       if (lane < ch && r < P.R) {
-        if (P.avail[r]) {
-          const double nv = (double)P.n_valid[r], ni = (double)P.n_invalid[r];
+        // every input is loaded at once; the counts' sum is exact as an
+        // integer, so its conversion is the double sum
+        const uint32_t cv = P.n_valid[r], ci = P.n_invalid[r], cc = P.cov[r];
+        const bool avail = P.avail[r] != 0;
+        const double vol = P.region_vol ? P.region_vol[r] : P.vol;
+        if (avail) {
+          const double nv = (double)cv, ni = (double)ci;
+          const double na = (double)((unsigned long long)cv + ci);
           const double dn = __dadd_rn(P.delta, nv);
-          const double vol = P.region_vol ? P.region_vol[r] : P.vol;
+          const double den = __dmul_rn(__dadd_rn(1.0, (double)cc), __dadd_rn(1.0, __dmul_rn(na, na)));
           const double fv = __ddiv_rn(__dmul_rn(dn, vol), __dadd_rn(dn, ni));
           const double f2 = __dmul_rn(fv, fv);
-          const double f4 = __dmul_rn(f2, f2);
-          const double na = __dadd_rn(nv, ni);
-          const double den =
-              __dmul_rn(__dadd_rn(1.0, (double)P.cov[r]), __dadd_rn(1.0, __dmul_rn(na, na)));
-          sc = __ddiv_rn(f4, den);
+          sc = __ddiv_rn(__dmul_rn(f2, f2), den);
         }
         P.score[r] = sc;
       }
@@ -823,6 +842,18 @@ __device__ __forceinline__ void phase_scores(const KParams& P, const Team& T, in
   });
 }
 
+// floor(min(p, 1) 2^32) of a positive p, from its bits: the mantissa shifted
+// down by as much as its last place lies below 2^-32 (an FP64 instruction
+// takes 64 clocks here, and this was four of them).
+__device__ __forceinline__ uint64_t threshold_of(double p) {
+  const uint64_t bits = (uint64_t)__double_as_longlong(p);
+  const int e = (int)(bits >> 52) - 1023;  // p in [2^e, 2^(e+1))
+  if (e >= 0) return 1ull << 32;           // infinities too
+  const uint64_t mant = (bits & 0xfffffffffffffull) | (1ull << 52);
+  const int down = 20 - e;                 // 52 - 32 - e
+  return down < 64 ? mant >> down : 0ull;
+}
+
 // Phase T (the chunks' warps in the node-set phase): the sum of Eq. 5 from the
 // chunks' partial sums (each of these warps reduces them itself, in the same
 // pairwise tree, so all get the same value), then P_accept and the integer
@@ -830,23 +861,26 @@ __device__ __forceinline__ void phase_scores(const KParams& P, const Team& T, in
 __device__ __forceinline__ void phase_thresholds(const KParams& P, const Team& T, int nch) {
   const int lane = (int)(threadIdx.x & 31u);
   if (T.b + T.nb * (int)(threadIdx.x >> 5) >= nch) return;
+  const int ch = P.R_pad / nch;
+  // the first regions' scores are fetched beside the chunk sums
+  int r = (T.b + T.nb * (int)(threadIdx.x >> 5)) * ch + lane;
+  bool avail = lane < ch && r < P.R && P.avail[r] != 0;
+  double score = avail ? P.score[r] : 0.0;
   const double sum = warp_tree_sum(nch, [&](int i) { return __ldcg(P.chunk_sum + i); });
   if (T.b == 0 && threadIdx.x == 0) P.ctl->score_sum = sum;
-  const int ch = P.R_pad / nch;
   for_own_chunks(T, nch, [&](int c) {
     for (int i = lane; i < ch; i += 32) {
-      const int r = c * ch + i;
+      if (c * ch + i != r) {
+        r = c * ch + i;
+        avail = r < P.R && P.avail[r] != 0;
+        score = avail ? P.score[r] : 0.0;
+      }
       if (r >= P.R) break;
       uint64_t thr = 1ull << 32;  // P_accept = 1 outside R_avail
-      if (P.avail[r]) {
-        double p;
-        if (sum > 0.0) {
-          p = __dadd_rn(__ddiv_rn(P.score[r], sum), P.eps);
-          if (p > 1.0) p = 1.0;
-        } else {
-          p = P.eps < 1.0 ? P.eps : 1.0;
-        }
-        if (p < 1.0) thr = (uint64_t)floor(__dmul_rn(p, 4294967296.0));
+      if (avail) {
+        double p = P.eps;  // below 1
+        if (sum > 0.0) p = __dadd_rn(__ddiv_rn(score, sum), P.eps);
+        thr = threshold_of(p);
       }
       P.thr[r] = thr;
     }
@@ -856,6 +890,17 @@ __device__ __forceinline__ void phase_thresholds(const KParams& P, const Team& T
   });
 }
 
+// Accepted sample j of this block: its key, bit 31 set for a claim winner.  The
+// warp that holds it is the last one whose offset is at most j (warps without
+// samples have their successor's offset).
+__device__ __forceinline__ uint32_t accepted_key(const KParams& P, const LoopShared& sh, int j) {
+  int w = 0;
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1)
+    if (w + s < (int)(blockDim.x >> 5) && sh.acc_off[w + s] <= j) w += s;
+  return P.acc_key[KP_IDX(P, sh.acc_a[w] + (j - sh.acc_off[w]), P.t_e, 17)];
+}
+
 // Materialises this block's accepted samples as the nodes id0 .. id0 +
 // acc_tot - 1 (id0 = t_old + the accepted samples of the blocks before it:
 // node ids follow the sample keys).  Every accepted sample takes the end
@@ -863,23 +908,19 @@ __device__ __forceinline__ void phase_thresholds(const KParams& P, const Team& T
 // from its key (the same draw), and its region and sub-region; visited and
 // the goal test (closed ball on position; the smallest new goal node wins)
 // follow.  Thread j of the block takes the block's samples j, j +
-// blockDim.x, ...; consecutive threads write consecutive nodes.  With the
-// sample log on, the sample is also re-derived from its key (the same
-// integrator steps, explicitly rounded, so the same numbers) and must match
-// the kept and the logged state bit for bit.
+// blockDim.x, ... (e: sample threadIdx.x's accepted_key, fetched by the
+// caller beside its own loads); consecutive threads write consecutive nodes.
+// With the sample log on, the sample is also re-derived from its key (the
+// same integrator steps, explicitly rounded, so the same numbers) and must
+// match the kept and the logged state bit for bit.
 template <int SYS, bool LOG>
 __device__ __forceinline__ void materialise(const KParams& P, uint32_t it, int id0, const KeyDiv& kd,
-                                            const LoopShared& sh, const unsigned char* sblob) {
+                                            const LoopShared& sh, const unsigned char* sblob,
+                                            uint32_t e) {
   using Sys = System<SYS>;
   constexpr int D = Sys::D, N = Sys::N;
   for (int j = (int)threadIdx.x; j < sh.acc_tot; j += (int)blockDim.x) {
-    // the warp that holds it: the last one whose offset is at most j (warps
-    // without samples have their successor's offset)
-    int w = 0;
-#pragma unroll
-    for (int s = 16; s > 0; s >>= 1)
-      if (w + s < (int)(blockDim.x >> 5) && sh.acc_off[w + s] <= j) w += s;
-    const uint32_t e = P.acc_key[KP_IDX(P, sh.acc_a[w] + (j - sh.acc_off[w]), P.t_e, 17)];
+    if (j != (int)threadIdx.x) e = accepted_key(P, sh, j);
     const int key = KP_IDX(P, (int)(e & 0x7fffffffu), P.t_e, 18);
     const int id = KP_IDX(P, id0 + j, P.t_e, 19);
     float x[D], u[N];
@@ -961,11 +1002,28 @@ __device__ __forceinline__ void phase_nodesets(const KParams& P, const Team& T, 
                                                const unsigned char* sblob) {
   const int nch = P.nch;
   uint32_t acc_before, acc_total;
+  const uint32_t e0 = (int)threadIdx.x < sh.acc_tot ? accepted_key(P, sh, (int)threadIdx.x) : 0u;
   block_prefix(T, P.blk_a, sh, &acc_before, &acc_total);
   phase_thresholds(P, T, nch);
   *n_new = (int)acc_total;
   const int t_new = t_old + (int)acc_total;
-  materialise<SYS, LOG>(P, it, t_old + (int)acc_before, kd, sh, sblob);
+  materialise<SYS, LOG>(P, it, t_old + (int)acc_before, kd, sh, sblob, e0);
+  // old nodes of the chunk: four tiles at a time, their region and
+  // threshold loads issued together (the first four tiles' regions before the
+  // wait for the thresholds)
+  int v0, v1;
+  chunk_of(T, t_new, &v0, &v1);
+  const int o1 = v1 < t_old ? v1 : t_old;
+  const int stride = (int)blockDim.x;
+  int rq[4];
+  auto regions = [&](int t0) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int v = t0 + q * stride + (int)threadIdx.x;
+      rq[q] = v < o1 ? KP_IDX(P, __ldcg(P.region + KP_IDX(P, v, P.t_e, 22)), P.R, 23) : 0;
+    }
+  };
+  regions(v0);
   if (threadIdx.x == 0) {
     uint64_t t0 = 0;
     uint32_t spins = 0;
@@ -982,30 +1040,20 @@ __device__ __forceinline__ void phase_nodesets(const KParams& P, const Team& T, 
     __threadfence();
   }
   __syncthreads();
-  int v0, v1;
-  chunk_of(T, t_new, &v0, &v1);
-  // old nodes of the chunk: four tiles at a time, their region and
-  // threshold loads issued together
-  const int o1 = v1 < t_old ? v1 : t_old;
-  const int stride = (int)blockDim.x;
   int c = 0;
   for (int t0 = v0; t0 < o1; t0 += 4 * stride) {
-    int vq[4], rq[4];
     uint64_t tq[4];
+    if (t0 != v0) regions(t0);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      tq[q] = t0 + q * stride + (int)threadIdx.x < o1 ? __ldcg(P.thr + rq[q]) : 0ull;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      vq[q] = t0 + q * stride + (int)threadIdx.x;
-      rq[q] = vq[q] < o1 ? KP_IDX(P, __ldcg(P.region + KP_IDX(P, vq[q], P.t_e, 22)), P.R, 23) : 0;
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) tq[q] = vq[q] < o1 ? __ldcg(P.thr + rq[q]) : 0ull;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if (vq[q] < o1) {
-        const uint4 w =
-            philox4x32_10(make_uint4(it, (uint32_t)vq[q], 0u, 2u), P.seed_lo, P.seed_hi);
+      const int v = t0 + q * stride + (int)threadIdx.x;
+      if (v < o1) {
+        const uint4 w = philox4x32_10(make_uint4(it, (uint32_t)v, 0u, 2u), P.seed_lo, P.seed_hi);
         const int e = (uint64_t)w.x < tq[q] ? 1 : 0;
-        P.in_ve[vq[q]] = (uint8_t)e;
+        P.in_ve[v] = (uint8_t)e;
         c += e;
       }
     }
@@ -1101,11 +1149,12 @@ __device__ __forceinline__ bool run_loop(const KParams& P, const Team& T, unsign
     const int ve_prev = n_ve, lam_prev = lam;
     // the pass's goal node and any error raised before the barrier above:
     // every block reads the same words, beside the counts of the V_E list
+    int goal_now = 0, err_now = 0;
     if (threadIdx.x == 0) {
-      sh.goal = *((volatile int*)&ctl->goal_node);
-      sh.err = *((volatile int*)&ctl->err);
+      goal_now = *((volatile int*)&ctl->goal_node);
+      err_now = *((volatile int*)&ctl->err);
     }
-    n_ve = write_ve(P, T, n_tree, sh);
+    n_ve = write_ve(P, T, n_tree, sh, goal_now, err_now);
     lam = eq6_lambda(P.t_e, n_tree, n_ve, P.lambda_max);
     ++run;
     const int goal = sh.goal;

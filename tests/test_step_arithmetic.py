@@ -49,3 +49,26 @@ def test_clearance_comparison_in_integers():
                   np.nextafter(edge, np.float32(0)), np.nextafter(edge, np.float32(9)), np.float32(300.0)):
             up = int(np.ceil(float(d) * 16.0 - 16.0))  # fused, rounded up to the integers' spacing
             assert (up <= q) == (float(d) <= 1.0 + q / 16.0)
+
+
+def threshold_of(p):
+    bits = int(np.float64(p).view(np.uint64))
+    e = (bits >> 52) - 1023
+    if e >= 0:
+        return 1 << 32
+    mant = (bits & ((1 << 52) - 1)) | (1 << 52)
+    return mant >> (20 - e) if 20 - e < 64 else 0
+
+
+def test_threshold_from_the_bits():
+    """floor(min(p, 1) 2^32): every binary exponent, the neighbours of whole
+    thresholds, 1 and above, infinity and NaN (neither compares below 1)."""
+    rng = np.random.default_rng(1)
+    p = [2.0 ** e * m for e in range(-80, 3) for m in (1.0, 1.0 + 2.0**-52, 1.5, 2.0 - 2.0**-52)]
+    for k in [1, 2, 3, 2**31, 2**32 - 1, 2**32, *rng.integers(1, 2**32, 200).tolist()]:
+        p += [k / 2.0**32, np.nextafter(k / 2.0**32, 0.0), np.nextafter(k / 2.0**32, 9.0)]
+    p += [5e-324, 1e300]
+    for v in p:
+        assert threshold_of(v) == int(np.floor(min(v, 1.0) * 2.0**32)), v
+    for v in (np.inf, np.nan, -np.nan):
+        assert threshold_of(v) == 1 << 32
