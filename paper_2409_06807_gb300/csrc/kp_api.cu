@@ -114,7 +114,7 @@ struct Dims {
 struct Layout {
   size_t ctl, boxes, st, parent, ctrl, steps, region, sub, in_ve, cs, xs, flags, acc_key,
       n_valid, n_invalid, cov, avail, visited, claim, score, thr, ve, blk_a, blk_b, chunk_sum,
-      stats, traj, feat, net_raw, kd_node, kd_split, leaf_box, region_vol, total;
+      stats, traj, feat, net_heads, kd_node, kd_split, leaf_box, region_vol, total;
 };
 
 // Bytes of the kd-tree slices (nodes, splits, leaf boxes, leaf volumes);
@@ -162,7 +162,7 @@ Layout make_layout(const Dims& d) {
   L.stats = take((size_t)kStatsCap * sizeof(KStats));
   L.traj = take((size_t)KP_TRAJ_ROWS * 17 * 4);
   L.feat = take(te * 32 * 2);     // bf16 node features of the V_E positions
-  L.net_raw = take(te * 8 * 4);   // network outputs of the V_E positions
+  L.net_heads = take(te * 8 * 4); // network heads of the V_E positions
   if (d.fso) {
     L.kd_node = take(kKdNodes * 4);
     L.kd_split = take(kKdNodes * 4);
@@ -756,8 +756,6 @@ kp_status configure_launch(kp_ctx* ctx) {
   };
   while (P.features_on && P.mlp_groups > 1 && bytes(ctx->blob_base) + kStaticRoom > ctx->smem_max)
     --P.mlp_groups;
-  // the kd-tree goes into shared memory with the blob (it is read at every
-  // binning) when that keeps the resident blocks
   auto shape = [&](size_t smem, int* grid) -> kp_status {
     for (int log = 0; log < 2; ++log) {
       int bps = P.threads;
@@ -773,16 +771,37 @@ kp_status configure_launch(kp_ctx* ctx) {
   P.blob_bytes = ctx->blob_base;
   P.kd_smem_off = -1;
   ctx->smem = bytes(ctx->blob_base);
+  P.mlp_w2_off = 0;
   kp_status s = shape(ctx->smem, ctx->grid);
-  if (s != KP_OK || ctx->blob_kd == 0 || bytes(ctx->blob_kd) + kStaticRoom > ctx->smem_max) return s;
-  int with_kd[2];
-  s = shape(bytes(ctx->blob_kd), with_kd);
-  if (s != KP_OK) return s;
-  if (with_kd[0] < ctx->grid[0] || with_kd[1] < ctx->grid[1]) return KP_OK;
-  P.blob_bytes = ctx->blob_kd;
-  P.kd_smem_off = (int)round16((size_t)ctx->blob_base);
-  ctx->smem = bytes(ctx->blob_kd);
-  return KP_OK;
+  // more goes into shared memory when that keeps the resident blocks
+  auto room_for = [&](size_t smem, bool* fits) -> kp_status {
+    *fits = false;
+    if (smem + kStaticRoom > ctx->smem_max) return KP_OK;
+    int with[2];
+    const kp_status st = shape(smem, with);
+    *fits = st == KP_OK && with[0] >= ctx->grid[0] && with[1] >= ctx->grid[1];
+    return st;
+  };
+  bool fits = false;
+  // the kd-tree, with the blob (it is read at every binning)
+  if (s == KP_OK && ctx->blob_kd != 0) {
+    s = room_for(bytes(ctx->blob_kd), &fits);
+    if (fits) {
+      P.blob_bytes = ctx->blob_kd;
+      P.kd_smem_off = (int)round16((size_t)ctx->blob_base);
+      ctx->smem = bytes(ctx->blob_kd);
+    }
+  }
+  // the network's second layer, behind the tiles
+  if (s == KP_OK && P.mix_thr != 0) {
+    const size_t off = round16(ctx->smem);
+    s = room_for(off + MLP_W2_SMEM, &fits);
+    if (fits) {
+      P.mlp_w2_off = (int)off;
+      ctx->smem = off + MLP_W2_SMEM;
+    }
+  }
+  return s;
 }
 
 // Algorithm 1's initialisation: one launch clears the tables and writes
@@ -933,7 +952,7 @@ void fill_params(KParams& P, const Dims& d, const Layout& lay, const kp_system* 
   P.stats_cap = kStatsCap;
   P.traj = reinterpret_cast<float*>(A + lay.traj);
   P.feat = reinterpret_cast<uint16_t*>(A + lay.feat);
-  P.net_raw = reinterpret_cast<float*>(A + lay.net_raw);
+  P.net_heads = reinterpret_cast<float*>(A + lay.net_heads);
   for (int i = 0; i < 6; ++i) {
     const float lo = i < d.D ? sys->x_lo[i] : 0.0f, hi = i < d.D ? sys->x_hi[i] : 0.0f;
     P.feat_scale[i] =

@@ -258,9 +258,10 @@ struct KParams {
   uint32_t mix_thr;        // learned draw iff selector word < mix_thr (0: off)
   int32_t features_on;     // node features computed each pass
   int32_t mlp_groups;      // groups of threads with room for a network tile
+  int32_t mlp_w2_off;      // shared-memory offset of the second layer's staged weights, 0: not staged
   int32_t threads;         // of a block of the loop launch
   uint16_t* feat;          // bf16 [t_e][32]: features of the V_E positions
-  float* net_raw;          // [t_e][8]: network outputs of the V_E positions
+  float* net_heads;        // [t_e][8]: Gaussian means and deviations of the V_E positions
   float feat_scale[6];     // 2 / (hi - lo) of a bounded state entry, 0 if unbounded
   float* hv_feat;          // harvest: [hv_cap][32]
   float* hv_target;        // [hv_cap][4]

@@ -262,88 +262,127 @@ __device__ __forceinline__ float state_feature(const KParams& P, int i, float x)
   return y * 0.318309886183790672f;
 }
 
-__device__ __forceinline__ float neighbour_accept(const KParams& P, int r, int k) {
-  const int gx = P.grid[0], gy = P.grid[1], gz = P.grid[2];
-  const int cx = r % gx, cy = (r / gx) % gy, cz = (r / (gx * gy)) % gz, sb = r / (gx * gy * gz);
-  const int nx = cx + (k == 0 ? -1 : k == 1 ? 1 : 0);
-  const int ny = cy + (k == 2 ? -1 : k == 3 ? 1 : 0);
-  const int nz = cz + (k == 4 ? -1 : k == 5 ? 1 : 0);
-  if (nx < 0 || nx >= gx || ny < 0 || ny >= gy || nz < 0 || nz >= gz) return 0.0f;
-  return (float)P.thr[nx + gx * (ny + gy * (nz + gz * sb))] * 2.3283064365386963e-10f;
+// What a feature pair is computed from.  Fetched without branches, every lane
+// the same fields (the sixteen lanes of a node read the same addresses but for
+// states and thresholds): behind a branch a pair's loads would wait for the
+// ones before it.
+struct FeatureInput {
+  float s0, s1;           // state entries
+  uint32_t nv, ni, cov;   // region counts
+  uint64_t t0, t1;        // thresholds, 0 outside the grid
+};
+
+__device__ __forceinline__ FeatureInput feature_input(const KParams& P, int v, int q) {
+  FeatureInput in;
+  const int r = P.region[v];
+  // q < 3: entries 2q, 2q + 1; q = 3: 0, 1; q = 4: 2
+  const int d0 = q < 3 ? 2 * q : q == 3 ? 0 : 2, d1 = q < 3 ? 2 * q + 1 : 1;
+  in.s0 = P.st[(size_t)d0 * P.t_e + v];
+  in.s1 = P.st[(size_t)d1 * P.t_e + v];
+  in.nv = P.n_valid[r];
+  in.ni = P.n_invalid[r];
+  in.cov = P.cov[r];
+  // q = 6: the region's threshold second; q = 7, 8, 9: those of its
+  // neighbours along axis q - 7 (none for kd-tree regions)
+  const bool axis = q >= 7 && q < 10 && !P.fso;
+  const int g = q == 7 ? P.grid[0] : q == 8 ? P.grid[1] : P.grid[2];
+  const int stride = q == 7 ? 1 : q == 8 ? P.grid[0] : P.grid[0] * P.grid[1];
+  const int c = (r / stride) % g;
+  const bool has0 = axis && c > 0, has1 = (axis && c < g - 1) || q == 6;
+  const uint64_t t0 = P.thr[has0 ? r - stride : r], t1 = P.thr[has1 && axis ? r + stride : r];
+  in.t0 = has0 ? t0 : 0ull;
+  in.t1 = has1 ? t1 : 0ull;
+  return in;
 }
 
-__device__ __forceinline__ void node_feature_pair(const KParams& P, int v, int q, float* f2) {
-  f2[0] = f2[1] = 0.0f;
+__device__ __forceinline__ void node_feature_pair(const KParams& P, int q, const FeatureInput& in,
+                                                  float* f2) {
+  const float nv = (float)in.nv, ni = (float)in.ni, dl = (float)P.delta;
+  // thresholds first; zeros where a pair has none
+  f2[0] = (float)in.t0 * 2.3283064365386963e-10f;
+  f2[1] = (float)in.t1 * 2.3283064365386963e-10f;
   if (q < 3) {
-    f2[0] = state_feature(P, 2 * q, P.st[(size_t)(2 * q) * P.t_e + v]);
-    f2[1] = state_feature(P, 2 * q + 1, P.st[(size_t)(2 * q + 1) * P.t_e + v]);
-    return;
+    f2[0] = state_feature(P, 2 * q, in.s0);
+    f2[1] = state_feature(P, 2 * q + 1, in.s1);
+  } else if (q == 3) {
+    f2[0] = P.goal_c[0] - in.s0;
+    f2[1] = P.goal_c[1] - in.s1;
+  } else if (q < 7) {
+    const float ratio = (q == 4 ? (float)in.cov : dl + nv) / (q == 4 ? (float)P.n_sub_per : dl + nv + ni);
+    const float lg = log1pf(q == 5 ? nv : ni);
+    f2[0] = q == 4 ? P.goal_c[2] - in.s0 : q == 5 ? ratio : lg;
+    if (q < 6) f2[1] = q == 4 ? ratio : lg;
   }
-  if (q == 3) {
-    f2[0] = P.goal_c[0] - P.st[v];
-    f2[1] = P.goal_c[1] - P.st[(size_t)P.t_e + v];
-    return;
-  }
-  if (q >= 10) return;
-  const int r = P.region[v];
-  const float nv = (float)P.n_valid[r], ni = (float)P.n_invalid[r], dl = (float)P.delta;
-  switch (q) {
-    case 4:
-      f2[0] = P.goal_c[2] - P.st[(size_t)2 * P.t_e + v];
-      f2[1] = (float)P.cov[r] / (float)P.n_sub_per;
-      break;
-    case 5:
-      f2[0] = (dl + nv) / (dl + nv + ni);
-      f2[1] = log1pf(nv);
-      break;
-    case 6:
-      f2[0] = log1pf(ni);
-      f2[1] = (float)P.thr[r] * 2.3283064365386963e-10f;
-      break;
-    default:  // q = 7, 8, 9: neighbours 2(q-7) and 2(q-7)+1 (none for kd-tree regions)
-      if (P.fso) break;
-      f2[0] = neighbour_accept(P, r, 2 * (q - 7));
-      f2[1] = neighbour_accept(P, r, 2 * (q - 7) + 1);
-  }
+}
+
+// One network tile.  Not inlined: it runs a few times per pass, and as a call
+// it gets the register budget of the loop kernel to itself instead of sharing
+// it with the loop state live around it.  What it needs is passed by value: a
+// field read through a reference to the kernel's parameters is a load from
+// memory here, not from the constant bank.
+template <bool STAGED>
+static __device__ __noinline__ void network_tile(MlpWeights w, const uint4* W2,
+                                                 const __nv_bfloat16* sX, __nv_bfloat16* sH,
+                                                 float* heads, int row0, int rows) {
+  mlp_tile_forward<MLP_LOOP_TILE / 16, STAGED>(w, W2, sX, sH, heads, row0, rows);
 }
 
 // Phase F: features of every V_E position (kept for the harvest) and, with
 // a network attached, its outputs, in tiles of 32 positions per group of 256
-// threads; 16 threads share the features of one position.  Not inlined: it runs once
-// per pass, and as a call it gets the register budget of the loop kernel
-// to itself instead of sharing it with the loop state live around it.
-static __device__ __noinline__ void phase_features(const KParams& P, const Team& T, int n_ve,
-                                                   unsigned char* mtile) {
+// threads; 16 threads share the features of one position.  The chain of loads
+// bounds it: a pass has at most a few tiles a group.  The second layer's weights
+// (128 KB, which every tile reads) are staged in shared memory where they
+// fit.  Measured at the last pass of a 200-box forest query (35,000 positions,
+// three tiles a group): 45 us with a branch a feature pair, parameters read
+// through a reference and the weights fetched from L2, 26 us as it is; one tile
+// 18,000 and 11,700 clocks (features 8,700 -> 5,000, second layer 5,200 ->
+// 2,900; with three groups an SM, mma.sync's rate bounds that layer at 2,000).
+// Fetching the next tile's lines into L1 ahead made a launch 2 % slower.
+__device__ __forceinline__ void phase_features(const KParams& P, const Team& T, int n_ve,
+                                               unsigned char* mtile, const uint4* staged) {
   const int group = (int)threadIdx.x / KP_MLP_GROUP, groups = P.mlp_groups;
   if (group >= groups) return;  // (no room for their tiles)
   const int tid = (int)threadIdx.x % KP_MLP_GROUP;
   __nv_bfloat16* sX = reinterpret_cast<__nv_bfloat16*>(mtile + group * MLP_LOOP_TILE_SMEM);
   __nv_bfloat16* sH = sX + MLP_LOOP_TILE * MLP_XS;
-  MlpWeights w;
-  w.W1 = reinterpret_cast<const __nv_bfloat16*>(P.mlp_W1);
-  w.b1 = P.mlp_b1;
-  w.W2 = reinterpret_cast<const __nv_bfloat16*>(P.mlp_W2);
-  w.b2 = P.mlp_b2;
-  w.W3 = reinterpret_cast<const __nv_bfloat16*>(P.mlp_W3);
-  w.b3 = P.mlp_b3;
   const int n_tiles = (n_ve + MLP_LOOP_TILE - 1) / MLP_LOOP_TILE;
-  const int q = tid & 15;  // 16 rows x 16 feature pairs per round
+  constexpr int ROUNDS = MLP_LOOP_TILE / 16;  // 16 rows x 16 feature pairs per round
+  const int q = tid & 15;
   for (int tile = T.b + T.nb * group; tile < n_tiles; tile += T.nb * groups) {
     const int p0 = tile * MLP_LOOP_TILE;
     const int rows = n_ve - p0 < MLP_LOOP_TILE ? n_ve - p0 : MLP_LOOP_TILE;
+    FeatureInput in[ROUNDS];
+    int v[ROUNDS];
 #pragma unroll
-    for (int rr = 0; rr < MLP_LOOP_TILE; rr += 16) {
-      const int row = rr + (tid >> 4);
-      float f2[2] = {0.0f, 0.0f};
-      if (row < rows) node_feature_pair(P, P.ve[p0 + row], q, f2);
-      const uint32_t v2 = pack_bf16(f2[0], f2[1]);
+    for (int rr = 0; rr < ROUNDS; ++rr) {
+      const int row = rr * 16 + (tid >> 4);
+      v[rr] = P.ve[p0 + (row < rows ? row : 0)];
+    }
+#pragma unroll
+    for (int rr = 0; rr < ROUNDS; ++rr) in[rr] = feature_input(P, v[rr], q);
+#pragma unroll
+    for (int rr = 0; rr < ROUNDS; ++rr) {
+      const int row = rr * 16 + (tid >> 4);
+      float f2[2];
+      node_feature_pair(P, q, in[rr], f2);
+      const uint32_t v2 = row < rows ? pack_bf16(f2[0], f2[1]) : 0u;
       *reinterpret_cast<uint32_t*>(sX + row * MLP_XS + 2 * q) = v2;
       if (row < rows) *reinterpret_cast<uint32_t*>(P.feat + (size_t)(p0 + row) * 32 + 2 * q) = v2;
     }
-    mlp_group_sync();
-    if (P.mix_thr)
-      mlp_tile_forward<MLP_LOOP_TILE / 16>(w, sX, sH, P.net_raw, p0, rows);
-    mlp_group_sync();
+    // the next tile's inputs and hidden rows are written after this tile's last
+    // and the next one's first barrier: every thread is past its reads by then
+    if (P.mix_thr) {
+      MlpWeights w;
+      w.W1 = reinterpret_cast<const __nv_bfloat16*>(P.mlp_W1);
+      w.b1 = P.mlp_b1;
+      w.b2 = P.mlp_b2;
+      w.W3 = reinterpret_cast<const __nv_bfloat16*>(P.mlp_W3);
+      w.b3 = P.mlp_b3;
+      if (P.mlp_w2_off > 0)
+        network_tile<true>(w, staged, sX, sH, P.net_heads, p0, rows);
+      else
+        network_tile<false>(w, reinterpret_cast<const uint4*>(P.mlp_W2), sX, sH, P.net_heads, p0, rows);
+    }
   }
 }
 
@@ -412,11 +451,13 @@ __device__ __forceinline__ int draw_controls(const KParams& P, uint32_t it, int 
   if (w1.z < P.mix_thr) {
     // learned draw from the node's Gaussian (normals: purpose 3)
     const uint4 w3 = philox4x32_10(make_uint4(it, (uint32_t)v, (uint32_t)j, 3u), P.seed_lo, P.seed_hi);
-    float z[4], mean[MLP_NQ], ls[MLP_NQ], q[4];
+    const float4* heads = reinterpret_cast<const float4*>(P.net_heads + (size_t)p * MLP_OUT);
+    const float4 m4 = heads[0], s4 = heads[1];
+    const float mean[4] = {m4.x, m4.y, m4.z, m4.w}, sd[4] = {s4.x, s4.y, s4.z, s4.w};
+    float z[4], q[4];
     box_muller4(w3, z);
-    mlp_heads(P.net_raw + (size_t)p * MLP_OUT, mean, ls);
 #pragma unroll
-    for (int d = 0; d < N; ++d) q[d] = fminf(fmaxf(__fmaf_rn(expf(ls[d]), z[d], mean[d]), -1.0f), 1.0f);
+    for (int d = 0; d < N; ++d) q[d] = fminf(fmaxf(__fmaf_rn(sd[d], z[d], mean[d]), -1.0f), 1.0f);
 #pragma unroll
     for (int d = 0; d < N; ++d)
       u[d] = __fmaf_rn(P.u_scale[d], __fmul_rn(__fadd_rn(q[d], 1.0f), 0.5f), P.u_lo[d]);
@@ -1082,6 +1123,11 @@ __device__ __forceinline__ bool run_loop(const KParams& P, const Team& T, unsign
     ctl->t_done = 0;
   }
   // the loop state, read once per block
+  // the second layer's weights of an attached network, for every pass
+  uint4* staged = reinterpret_cast<uint4*>(smem + P.mlp_w2_off);
+  if (P.mlp_w2_off > 0)
+    for (int i = (int)threadIdx.x; i < MLP_W2_SMEM / 16; i += (int)blockDim.x)
+      staged[staged_index(i)] = __ldg(reinterpret_cast<const uint4*>(P.mlp_W2) + i);
   if (threadIdx.x == 0) {
     sh.bcast[0] = ctl->n_nodes;
     sh.bcast[1] = ctl->iteration;
@@ -1121,7 +1167,7 @@ __device__ __forceinline__ bool run_loop(const KParams& P, const Team& T, unsign
   unsigned char* mtile = smem + P.blob_bytes + P.sd_bytes;
   for (;;) {
     if (P.features_on) {
-      phase_features(P, T, n_ve, mtile);
+      phase_features(P, T, n_ve, mtile, staged);
       stamp(3);
       if (!team_sync(T, ctl, P.wait_ns, 19)) return false;
       stamp(6);

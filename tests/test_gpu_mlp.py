@@ -362,3 +362,29 @@ def test_learned_gain_and_its_break_even(M):
     print(f"learned: {gain:+.3f} new sub-regions per sample, {(n1 / k1) / (n0 / k0) - 1:+.3f} per "
           f"integrator step; network phase / expand = {break_even:.3f}")
     assert gain > 0.01, gain
+
+
+@pytest.mark.parametrize("extra,limit", [(400, 0), (900, 0), (3800, 0), (0, 60)])
+def test_learned_plan_with_less_shared_memory(M, extra, limit):
+    """The second layer's weights are staged in shared memory beside the
+    obstacles where they fit: with boxes added inside an obstacle (which changes
+    no verdict) there is no room for them, and a capped launch has blocks of one
+    group of threads.  The result is the same bytes."""
+    mlp, P = M
+    net = mlp.Mlp(mlp.init_params(4), max_batch=64)
+    w = W.c2(3, lambda_max=32)
+    boxes = np.asarray(w.boxes, dtype=np.float32)
+    lo, hi = boxes[0, :3], boxes[0, 3:]
+    mid = np.concatenate([lo + 0.4 * (hi - lo), lo + 0.6 * (hi - lo)])
+    out = []
+    for n, lim in ((0, 0), (extra, limit)):
+        g = P.Planner(w.with_(boxes=np.concatenate([boxes, np.tile(mid, (n, 1))]).astype(np.float32)))
+        g.attach_mlp(net, 0.5)
+        g.set_grid_limit(lim)
+        st, traj = g.plan(max_iters=12)
+        i = g.info()
+        out.append((st, traj, [i[k] for k in ("n_nodes", "n_ve", "n_samples", "n_steps", "goal_node")]))
+    (s0, t0, i0), (s1, t1, i1) = out
+    assert s0 == s1 and i0 == i1 and i0[0] > 1000
+    for k in t0 or {}:
+        assert np.array_equal(t0[k], t1[k])
