@@ -402,16 +402,6 @@ __device__ __forceinline__ void box_muller4(uint4 w, float* z) {
   }
 }
 
-// The draw of sample key (V_E position p = key / lam, j = key - p lam) in
-// pass it (Algorithm 2: random control in U, random duration): returns the
-// parent's node id.  Counter (it, node, j, purpose): purpose 0 the control
-// words (kept in wr), purpose 1 (duration, accept word, selector); with a
-// network attached and the selector below the mix threshold, the control
-// comes from the node's Gaussian with normals from purpose 3 (the duration
-// keeps the uniform draw).
-// The expand phase and the node-set phase (which appends accepted samples
-// by their keys) both draw through this function, so both see the same
-// numbers.
 // Division of a sample key by the pass's lambda (at most 1024) by a
 // multiplication: for lam in [2^s, 2^(s+1)) and mul = ceil(2^(31+s) / lam), key
 // / lam = (key mul) >> (31 + s) for every key below 2^30 (the product exceeds
@@ -435,13 +425,22 @@ struct KeyDiv {
   }
 };
 
+// The draw of sample key (V_E position p = key / lam of node v, j = key - p
+// lam) in pass it (Algorithm 2: random control in U, random duration).
+// Counter (it, node, j, purpose): purpose 0 the control words (kept in wr),
+// purpose 1 (duration, accept word, selector); with a network attached and the
+// selector below the mix threshold, the control comes from the node's Gaussian
+// with normals from purpose 3 (the duration keeps the uniform draw).
+// The expand phase and the node-set phase (which appends accepted samples
+// by their keys) both draw through this function, so both see the same
+// numbers.
 template <int SYS>
-__device__ __forceinline__ int draw_controls(const KParams& P, uint32_t it, int key, const KeyDiv& kd,
-                                             float* u, int* k, uint32_t* wacc, uint32_t* wr) {
+__device__ __forceinline__ void draw_controls(const KParams& P, uint32_t it, int key, int v,
+                                              const KeyDiv& kd, float* u, int* k, uint32_t* wacc,
+                                              uint32_t* wr) {
   constexpr int N = System<SYS>::N;
   const int p = kd.quot(key);
   const int j = key - p * kd.lam;
-  const int v = KP_IDX(P, P.ve[KP_IDX(P, p, P.t_e, 5)], P.t_e, 6);
   const uint4 w0 = philox4x32_10(make_uint4(it, (uint32_t)v, (uint32_t)j, 0u), P.seed_lo, P.seed_hi);
   const uint4 w1 = philox4x32_10(make_uint4(it, (uint32_t)v, (uint32_t)j, 1u), P.seed_lo, P.seed_hi);
   wr[0] = w0.x; wr[1] = w0.y; wr[2] = w0.z; wr[3] = w0.w;
@@ -463,19 +462,18 @@ __device__ __forceinline__ int draw_controls(const KParams& P, uint32_t it, int 
       u[d] = __fmaf_rn(P.u_scale[d], __fmul_rn(__fadd_rn(q[d], 1.0f), 0.5f), P.u_lo[d]);
   }
   *wacc = w1.y;
-  return v;
 }
 
 // The draw of sample 'key' and its parent's state (the start of the
 // segment).
 template <int SYS>
-__device__ __forceinline__ int draw_sample(const KParams& P, uint32_t it, int key, const KeyDiv& kd, float* x,
-                                           float* u, int* k, uint32_t* wacc, uint32_t* wr) {
+__device__ __forceinline__ void draw_sample(const KParams& P, uint32_t it, int key, int v,
+                                            const KeyDiv& kd, float* x, float* u, int* k,
+                                            uint32_t* wacc, uint32_t* wr) {
   constexpr int D = System<SYS>::D;
-  const int v = draw_controls<SYS>(P, it, key, kd, u, k, wacc, wr);
 #pragma unroll
   for (int d = 0; d < D; ++d) x[d] = P.st[(size_t)d * P.t_e + v];
-  return v;
+  draw_controls<SYS>(P, it, key, v, kd, u, k, wacc, wr);
 }
 
 // Phase E: Algorithm 2 for every sample key in [0, S).
@@ -488,7 +486,9 @@ __device__ __forceinline__ int draw_sample(const KParams& P, uint32_t it, int ke
 // start-up work is shared by many lanes and no lane idles while a long
 // sample runs next to it.  Every sample's arithmetic depends on its key
 // alone, so the result does not depend on which lane ran it.
-constexpr int KP_KEY_BATCH = 128; // keys a warp takes from the grid counter
+// keys a warp takes from the grid counter at most (256: 0.5 % of a launch with a
+// large frontier faster than 128, 64 1.5 % slower)
+constexpr int KP_KEY_BATCH = 256;
 
 template <int SYS, bool LOG>
 __device__ __forceinline__ void phase_expand(const KParams& P, const Team& T,
@@ -545,57 +545,96 @@ __device__ __forceinline__ void phase_expand(const KParams& P, const Team& T,
         if (lane == 0) raise_error(P.ctl, KP_DEV_ERR_TIMEOUT, 30);
         break;
       }
-      // ---- finalise the lanes that finished -------------------------------
-      if (key >= 0 && done) {
+      // Finalise and refill together: what each needs from memory is issued
+      // side by side, two round trips to L2 in a row (three when the warp
+      // needs a batch of keys) where one after the other took four to six
+      // (0.5 to 1 % of a launch: the other warps hide most of a round trip).
+      // ---- first round trip -----------------------------------------------
+      // the pool's keys for the free lanes (and their nodes), and, when it
+      // holds too few, the counter's value
+      const bool fin = key >= 0 && done;
+      const int rank = __popc(m_free & lt), avail = pool_end - pool_next;
+      const int short_by = __popc(m_free) - avail;
+      const bool take = !exhausted && short_by > 0;
+      int next = -1, next_v = 0, cur = 0;
+      if ((key < 0 || done) && rank < avail) {
+        next = pool_next + rank;
+        next_v = P.ve[KP_IDX(P, kd.quot(next), P.t_e, 5)];
+      }
+      pool_next = short_by > 0 ? pool_end : pool_next + __popc(m_free);
+      if (take && lane == 0 && static_end < S) cur = *((volatile int*)&P.ctl->work_next);
+      // the finished lanes' bins: whether the sub-region was visited, its
+      // claim so far, the region's threshold
+      int r = 0, s = 0;
+      uint32_t claimed = 0;
+      uint64_t thr = 0;
+      bool cont = false;
+      const bool valid = fin && fail == 0;
+      if (fin) {
         // steps run, and hull tests (every step but one that left the
         // state box)
         n_steps += (uint32_t)i;
         n_hull += (uint32_t)(fail < 0 ? i - 1 : i);
-        int r, s;
         bin_state<SYS>(x, P, &r, &s, sblob);
-        const bool valid = fail == 0;
-        uint32_t f = 0;
         if (valid) {
           r = KP_IDX(P, r, P.R, 7);
           s = KP_IDX(P, s, (long long)P.R * P.n_sub_per, 8);
           key = KP_IDX(P, key, P.t_e, 9);
-          atomicAdd(&P.n_valid[r], 1u);
-          f = KP_F_VALID;
-          const bool cont = P.visited[s] == 0;
-          const bool bern = (uint64_t)wacc < P.thr[r];
-          bool may_win = false;
-          if (cont) {
-            f |= KP_F_CONTENDER;
-            // the first claimant of a sub-region knows it is newly reached:
-            // it will get exactly one representative in region r; a
-            // claimant that finds a smaller key there has already lost
-            const uint32_t prev = atomicMin(&P.claim[s], (uint32_t)key);
-            if (prev == 0xffffffffu) {
-              atomicAdd(&P.cov[r], 1u);
-              P.avail[r] = 1;
-            }
-            may_win = prev > (uint32_t)key;
-          }
-          if (bern) {
-            f |= KP_F_BERN;
-            P.avail[r] = 1;
-          }
-          // a sample that may still be accepted (a contender not yet beaten,
-          // or past its draw) keeps its end state for the append, and a
-          // contender its sub-region for the claim check
-          if (cont) P.cs[key] = s;
-          if (may_win || bern) {
-            float4* row = reinterpret_cast<float4*>(P.xs + (size_t)key * kp_xs_stride(D));
-#pragma unroll
-            for (int q = 0; q < kp_xs_stride(D) / 4; ++q)
-              row[q] = make_float4(4 * q < D ? x[4 * q] : 0.0f, 4 * q + 1 < D ? x[4 * q + 1] : 0.0f,
-                                   4 * q + 2 < D ? x[4 * q + 2] : 0.0f,
-                                   4 * q + 3 < D ? x[4 * q + 3] : 0.0f);
-          }
-        } else {
-          atomicAdd(&P.n_invalid[KP_IDX(P, r, P.R, 10)], 1u);
+          cont = P.visited[s] == 0;
+          claimed = __ldcg(P.claim + s);
+          thr = P.thr[r];
         }
-        P.flags[KP_IDX(P, key, P.t_e, 11)] = (uint8_t)f;
+      }
+      // ---- second round trip ----------------------------------------------
+      // the claim, unless a smaller key is there already (it is lost then)
+      const bool bern = valid && (uint64_t)wacc < thr;
+      const bool may_win = cont && claimed > (uint32_t)key;
+      uint32_t prev = 0;
+      if (may_win) prev = atomicMin(&P.claim[s], (uint32_t)key);
+      // the first claimant of a sub-region knows it is newly reached: it will
+      // get exactly one representative in region r (before the draw where its
+      // twelve states leave no registers to keep the answer: 0.5 % of a
+      // quadrotor query; after it 0.8 % of a Dubins one)
+      auto new_region = [&]() {
+        if (prev == 0xffffffffu) {
+          atomicAdd(&P.cov[r], 1u);
+          P.avail[r] = 1;
+        }
+      };
+      // batches shrink towards the end of the pass so that warps run out of
+      // work together
+      // (at the very end a warp takes only what its idle lanes can start
+      // now, so no warp is left with a second round of samples)
+      // (the batch is sized from the counter's current value: a warp that
+      // last took keys long ago must not size it from a stale position and
+      // leave with a large batch just before the end)
+      int base = S;
+      if (take && lane == 0 && static_end < S) {
+        int want = (S - static_end - cur) / (Sys::GUIDED_DIV * n_warps);
+        want = want < short_by ? short_by : (want > KP_KEY_BATCH ? KP_KEY_BATCH : want);
+        base = static_end + atomicAdd(&P.ctl->work_next, want);
+        base = base < S ? base : S;
+        n_batch += base < S ? 1u : 0u;
+        pool_end = base + want < S ? base + want : S;
+      }
+      if (fin) {
+        atomicAdd((valid ? P.n_valid : P.n_invalid) + KP_IDX(P, r, P.R, 10), 1u);
+        // a sample that may still be accepted (a contender not yet beaten,
+        // or past its draw) keeps its end state for the append, and a
+        // contender its sub-region for the claim check
+        if (cont) P.cs[key] = s;
+        if (may_win || bern) {
+          float4* row = reinterpret_cast<float4*>(P.xs + (size_t)key * kp_xs_stride(D));
+#pragma unroll
+          for (int q = 0; q < kp_xs_stride(D) / 4; ++q)
+            row[q] = make_float4(4 * q < D ? x[4 * q] : 0.0f, 4 * q + 1 < D ? x[4 * q + 1] : 0.0f,
+                                 4 * q + 2 < D ? x[4 * q + 2] : 0.0f,
+                                 4 * q + 3 < D ? x[4 * q + 3] : 0.0f);
+        }
+        if (bern) P.avail[r] = 1;
+        P.flags[KP_IDX(P, key, P.t_e, 11)] = (uint8_t)(valid ? KP_F_VALID | (cont ? KP_F_CONTENDER : 0u) |
+                                                                   (bern ? KP_F_BERN : 0u)
+                                                             : 0u);
         if (LOG && key < P.log.capacity) {
           P.log.node[key] = v;
           P.log.k[key] = k;
@@ -609,52 +648,34 @@ __device__ __forceinline__ void phase_expand(const KParams& P, const Team& T,
         }
         key = -1;
       }
-      // ---- hand new keys to the free lanes --------------------------------
-      uint32_t m_idle = __ballot_sync(FULL, key < 0);
-      while (m_idle && !exhausted) {
-        if (pool_next >= pool_end) {
-          // batches shrink towards the end of the pass so that warps run
-          // out of work together
-          // (at the very end a warp takes only what its idle lanes can
-          // start now, so no warp is left with a second round of samples)
-          // (the batch is sized from the counter's current value: a warp
-          // that last took keys long ago must not size it from a stale
-          // position and leave with a large batch just before the end)
-          const int n_idle_now = __popc(m_idle);
-          int base = S;
-          if (lane == 0 && static_end < S) {
-            const int cur = static_end + *((volatile int*)&P.ctl->work_next);
-            int want = (S - cur) / (Sys::GUIDED_DIV * n_warps);
-            want = want < n_idle_now ? n_idle_now : (want > KP_KEY_BATCH ? KP_KEY_BATCH : want);
-            base = static_end + atomicAdd(&P.ctl->work_next, want);
-            base = base < S ? base : S;
-            n_batch += base < S ? 1u : 0u;
-            pool_end = base + want < S ? base + want : S;
-          }
-          base = __shfl_sync(FULL, base, 0);
-          const int end_now = __shfl_sync(FULL, pool_end, 0);
-          if (base >= S) {
-            exhausted = true;
-            break;
-          }
-          pool_next = base;
-          pool_end = end_now;
+      if (take) {
+        base = __shfl_sync(FULL, base, 0);
+        pool_end = __shfl_sync(FULL, pool_end, 0);
+        pool_next = base;
+        if (key < 0 && rank >= avail && rank - avail < pool_end - base) {
+          next = base + rank - avail;
+          next_v = P.ve[KP_IDX(P, kd.quot(next), P.t_e, 5)];
         }
-        const int avail = pool_end - pool_next;
-        const int rank = __popc(m_idle & lt);
-        if (key < 0 && rank < avail) {
-          key = pool_next + rank;
-          n_refill += ran ? 1u : 0u;
-          ran = true;
-          v = draw_sample<SYS>(P, it, key, kd, x, u, &k, &wacc, wr);
-          i = 0;
-          fail = 0;
-          done = false;
+        // (a batch covers the free lanes unless the keys end)
+        if (pool_end - base >= short_by) {
+          pool_next = base + short_by;
+        } else {
+          pool_next = pool_end = S;
+          exhausted = true;
         }
-        const int n_idle = __popc(m_idle);
-        pool_next += n_idle < avail ? n_idle : avail;
-        m_idle = __ballot_sync(FULL, key < 0);
       }
+      if (D == 12) new_region();
+      if (next >= 0) {
+        key = next;
+        n_refill += ran ? 1u : 0u;
+        ran = true;
+        v = KP_IDX(P, next_v, P.t_e, 6);
+        draw_sample<SYS>(P, it, key, v, kd, x, u, &k, &wacc, wr);
+        i = 0;
+        fail = 0;
+        done = false;
+      }
+      if (D != 12) new_region();
       if (__ballot_sync(FULL, key >= 0) == 0) break;
     }
     // ---- one integrator step (PropagateODE) and its validity check --------
@@ -967,7 +988,8 @@ __device__ __forceinline__ void materialise(const KParams& P, uint32_t it, int i
     float x[D], u[N];
     int k;
     uint32_t wacc, wr[4];
-    const int v = draw_controls<SYS>(P, it, key, kd, u, &k, &wacc, wr);
+    const int v = KP_IDX(P, P.ve[KP_IDX(P, kd.quot(key), P.t_e, 5)], P.t_e, 6);
+    draw_controls<SYS>(P, it, key, v, kd, u, &k, &wacc, wr);
     {
       const float4* row = reinterpret_cast<const float4*>(P.xs + (size_t)key * kp_xs_stride(D));
 #pragma unroll
