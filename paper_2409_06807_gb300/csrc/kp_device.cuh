@@ -226,15 +226,10 @@ struct System<KP_SYS_DI> {
   }
 };
 
-// One classic RK4 step x <- x + h/6 (k1 + 2 k2 + 2 k3 + k4), stage points
-// x + h/2 k1, x + h/2 k2, x + h k3; h6 = h / 6, rounded as an FP32 division
-// (KParams::dt_sixth).  The combination is accumulated as each
-// stage is evaluated, in the fixed order ((k1 + 2 k2) + 2 k3) + k4, so only
-// one stage derivative is live at a time (the register budget of the loop
-// kernel holds no four of them for the 12D system).  F(t, k) evaluates the
-// field at t into k.
-// Two FP32 fused multiply-adds (additions) in one instruction, each correctly
-// rounded as the single ones.
+// Two FP32 fused multiply-adds (additions, products) in one instruction, each
+// correctly rounded as the single ones.  A product of mul2 must not enter add2
+// or fma2: the assembler was seen to fuse packed products into packed sums,
+// which it never does to the scalar ones.
 __device__ __forceinline__ void fma2(float s, const float* a, const float* b, float* r) {
   asm("{\n .reg .b64 p, q, t;\n mov.b64 p, {%2, %2};\n mov.b64 q, {%3, %4};\n mov.b64 t, {%5, %6};\n"
       " fma.rn.f32x2 t, p, q, t;\n mov.b64 {%0, %1}, t;\n}"
@@ -249,84 +244,95 @@ __device__ __forceinline__ void add2(const float* a, const float* b, float* r) {
       : "f"(a[0]), "f"(a[1]), "f"(b[0]), "f"(b[1]));
 }
 
+__device__ __forceinline__ void mul2(float s, const float* a, float* r) {
+  asm("{\n .reg .b64 p, q, t;\n mov.b64 p, {%2, %2};\n mov.b64 q, {%3, %4};\n"
+      " mul.rn.f32x2 t, p, q;\n mov.b64 {%0, %1}, t;\n}"
+      : "=f"(r[0]), "=f"(r[1])
+      : "f"(s), "f"(a[0]), "f"(a[1]));
+}
+// One classic RK4 step x <- x + h/6 (k1 + 2 k2 + 2 k3 + k4), stage points
+// x + h/2 k1, x + h/2 k2, x + h k3; h6 = h / 6, rounded as an FP32 division
+// (KParams::dt_sixth).  The combination is accumulated as each
+// stage is evaluated, in the fixed order ((k1 + 2 k2) + 2 k3) + k4, so only
+// one stage derivative is live at a time (the register budget of the loop
+// kernel holds no four of them for the 12D system), two dimensions at a time.
+// F(t, k) evaluates the field at t into k, by scalar operations (see mul2).
 template <int D, class F>
 __device__ __forceinline__ void rk4_step(float* x, float h, float h6, F field) {
+  static_assert(D % 2 == 0, "dimensions in pairs");
   float acc[D], k[D], t[D];
   const float hh = __fmul_rn(0.5f, h);
-  if (D == 12) {
-    // the quadrotor's stage points and combination two dimensions at a time
-    field(x, k);
-#pragma unroll
-    for (int i = 0; i < D; i += 2) {
-      acc[i] = k[i];
-      acc[i + 1] = k[i + 1];
-      fma2(hh, k + i, x + i, t + i);
-    }
-    field(t, k);
-#pragma unroll
-    for (int i = 0; i < D; i += 2) {
-      fma2(2.0f, k + i, acc + i, acc + i);
-      fma2(hh, k + i, x + i, t + i);
-    }
-    field(t, k);
-#pragma unroll
-    for (int i = 0; i < D; i += 2) {
-      fma2(2.0f, k + i, acc + i, acc + i);
-      fma2(h, k + i, x + i, t + i);
-    }
-    field(t, k);
-#pragma unroll
-    for (int i = 0; i < D; i += 2) {
-      add2(acc + i, k + i, acc + i);
-      fma2(h6, acc + i, x + i, x + i);
-    }
-    return;
-  }
   field(x, k);
 #pragma unroll
-  for (int i = 0; i < D; ++i) {
+  for (int i = 0; i < D; i += 2) {
     acc[i] = k[i];
-    t[i] = __fmaf_rn(hh, k[i], x[i]);
+    acc[i + 1] = k[i + 1];
+    fma2(hh, k + i, x + i, t + i);
   }
   field(t, k);
 #pragma unroll
-  for (int i = 0; i < D; ++i) {
-    acc[i] = __fmaf_rn(2.0f, k[i], acc[i]);
-    t[i] = __fmaf_rn(hh, k[i], x[i]);
+  for (int i = 0; i < D; i += 2) {
+    fma2(2.0f, k + i, acc + i, acc + i);
+    fma2(hh, k + i, x + i, t + i);
   }
   field(t, k);
 #pragma unroll
-  for (int i = 0; i < D; ++i) {
-    acc[i] = __fmaf_rn(2.0f, k[i], acc[i]);
-    t[i] = __fmaf_rn(h, k[i], x[i]);
+  for (int i = 0; i < D; i += 2) {
+    fma2(2.0f, k + i, acc + i, acc + i);
+    fma2(h, k + i, x + i, t + i);
   }
   field(t, k);
 #pragma unroll
-  for (int i = 0; i < D; ++i) x[i] = __fmaf_rn(h6, __fadd_rn(acc[i], k[i]), x[i]);
+  for (int i = 0; i < D; i += 2) {
+    add2(acc + i, k + i, acc + i);
+    fma2(h6, acc + i, x + i, x + i);
+  }
 }
 
-// 6D Dubins airplane (Chitsaz & LaValle 2007); classic RK4.
+// 6D Dubins airplane (Chitsaz & LaValle 2007): p' = v (cos a cos b, sin a cos
+// b, sin b), heading a, pitch b and speed v with the controls as constant
+// rates.  Classic RK4 (rk4_step's operations in its order): the second and
+// third stages have the same angles and speed, so they are evaluated once.
+// Issue slots bound the expand phase (78 % of them taken); the packed
+// reduction and products took 1.5 % off a launch, packing the combination or the
+// stage angles too cost 1 to 2 % (register pairs, moves).
 template <>
 struct System<KP_SYS_DUBINS> {
   static constexpr int SYM0 = 3, SYM1 = 5;
   static constexpr int D = 6, N = 3;
-  static constexpr int REFILL_MIN = 16;
+  // (16 lanes 0.4 to 0.9 % slower, 24 1 to 2 %)
+  static constexpr int REFILL_MIN = 20;
   static constexpr int FIRST_BATCH_MIN = 16;
   static constexpr int GUIDED_DIV = 2;
-  __device__ __forceinline__ static void f(const float* x, const float* u, float* dx) {
-    float sp, cp, st, ct;
-    sincos_reduced(x[3], &sp, &cp);
-    sincos_reduced(x[4], &st, &ct);
-    dx[0] = __fmul_rn(__fmul_rn(x[5], cp), ct);
-    dx[1] = __fmul_rn(__fmul_rn(x[5], sp), ct);
-    dx[2] = __fmul_rn(x[5], st);
-    dx[3] = u[0];
-    dx[4] = u[1];
-    dx[5] = u[2];
-  }
   __device__ __forceinline__ static void step(float* x, const float* u, float h,
                                               const KParams& P) {
-    rk4_step<6>(x, h, P.dt_sixth, [&](const float* y, float* dy) { f(y, u, dy); });
+    const float hh = __fmul_rn(0.5f, h), h6 = P.dt_sixth;
+    float ka[3], kb[3], kc[3];
+    // p' at heading a, pitch b and speed v: the two angles' reduction
+    // (sincos_reduced) and the two horizontal products in pairs
+    auto field = [](float a, float b, float v, float* k) {
+      const float ab[2] = {a, b}, t0[2] = {12582912.0f, 12582912.0f}, t1[2] = {-12582912.0f, -12582912.0f};
+      float q[2], r[2], cs[2], st, ct;
+      fma2(0.159154943091895336f, ab, t0, q);
+      add2(q, t1, q);
+      fma2(-6.28318548202514648f, q, ab, r);
+      fma2(1.74845560007448838e-07f, q, r, r);
+      __sincosf(r[0], &cs[1], &cs[0]);
+      __sincosf(r[1], &st, &ct);
+      mul2(v, cs, k);
+      mul2(ct, k, k);
+      k[2] = __fmul_rn(v, st);
+    };
+    field(x[3], x[4], x[5], ka);
+    field(__fmaf_rn(hh, u[0], x[3]), __fmaf_rn(hh, u[1], x[4]), __fmaf_rn(hh, u[2], x[5]), kb);
+    field(__fmaf_rn(h, u[0], x[3]), __fmaf_rn(h, u[1], x[4]), __fmaf_rn(h, u[2], x[5]), kc);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const float a = __fmaf_rn(2.0f, kb[i], __fmaf_rn(2.0f, kb[i], ka[i]));
+      x[i] = __fmaf_rn(h6, __fadd_rn(a, kc[i]), x[i]);
+      const float c = __fmaf_rn(2.0f, u[i], __fmaf_rn(2.0f, u[i], u[i]));
+      x[3 + i] = __fmaf_rn(h6, __fadd_rn(c, u[i]), x[3 + i]);
+    }
   }
   __device__ __forceinline__ static float speed(const float* x) { return fabsf(x[5]); }
 };
@@ -580,10 +586,12 @@ __device__ __forceinline__ bool hull_hits_grid(const KParams& P, const float4* _
   float tl[3], th[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    const float t0 = __fmul_rn(__fsub_rn(p[a], P.ws_lo[a]), P.bp_scale[a]);
-    const float t1 = __fmul_rn(__fsub_rn(x[a], P.ws_lo[a]), P.bp_scale[a]);
-    tl[a] = fminf(t0, t1);
-    th[a] = fmaxf(t0, t1);
+    const float px[2] = {p[a], x[a]}, m[2] = {-P.ws_lo[a], -P.ws_lo[a]};
+    float t[2];
+    add2(px, m, t);
+    mul2(P.bp_scale[a], t, t);
+    tl[a] = fminf(t[0], t[1]);
+    th[a] = fmaxf(t[0], t[1]);
   }
   if (sclear != nullptr &&
       (P.state_inside ? hull_clear<true>(P, sclear, tl, th) : hull_clear<false>(P, sclear, tl, th)))
