@@ -1674,8 +1674,8 @@ __device__ __forceinline__ bool static_listed(const StaticGrid& G, const float* 
   for (int a = 0; a < 3; ++a) {
     const float tl = __fmul_rn(__fsub_rn(lo[a], G.lo[a]), G.scale[a]);
     const float th = __fmul_rn(__fsub_rn(hi[a], G.lo[a]), G.scale[a]);
-    float f;
-    in = in && cc[a] >= bp_cell_of(tl, last, &f) && cc[a] <= bp_cell_of(th, last, &f);
+    const int c = cc[a] + 0x4B000000;  // with bp_cell_of's bits
+    in = in && c >= bp_cell_of(tl, last) && c <= bp_cell_of(th, last);
     m = fmaxf(m, fmaxf(tl - (float)(cc[a] + 1), (float)cc[a] - th));
   }
   *gap = m;

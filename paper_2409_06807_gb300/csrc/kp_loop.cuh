@@ -512,7 +512,7 @@ __device__ __forceinline__ void phase_expand(const KParams& P, const Team& T,
   bool ran = false;
   // lane state: the sample being integrated
   int key = -1, v = 0, k = 0, i = 0, fail = 0;
-  bool done = false;
+  bool busy = false;  // a sample in flight (a finished one keeps its key)
   float x[D], u[N];
   uint32_t wacc = 0, wr[4] = {0, 0, 0, 0};
   // warp state (uniform): the current batch of keys.  The first batch of
@@ -528,6 +528,7 @@ __device__ __forceinline__ void phase_expand(const KParams& P, const Team& T,
   int pool_next = gw * b0 < S ? gw * b0 : S;
   int pool_end = pool_next + b0 < S ? pool_next + b0 : S;
   bool exhausted = S <= 0;
+  int refill_at = exhausted ? 32 : Sys::REFILL_MIN;
   // bound on the phase's device time, checked warp-uniformly at every
   // refill (a sample runs at most 255 steps, so refills are at most 255
   // iterations apart)
@@ -538,8 +539,8 @@ __device__ __forceinline__ void phase_expand(const KParams& P, const Team& T,
     // remain (they are refilled at once), and once the pass's keys are all
     // handed out, only when every lane has finished, so that the warp's
     // last samples cost one finalise instead of one per finishing step
-    const uint32_t m_free = __ballot_sync(FULL, key < 0 || done);
-    if (exhausted ? m_free == FULL : __popc(m_free) >= Sys::REFILL_MIN) {
+    const uint32_t m_free = __ballot_sync(FULL, !busy);
+    if (__popc(m_free) >= refill_at) {
       const uint64_t now = __shfl_sync(FULL, global_ns(), 0);
       if (now - t_phase > P.wait_ns) {
         if (lane == 0) raise_error(P.ctl, KP_DEV_ERR_TIMEOUT, 30);
@@ -552,12 +553,12 @@ __device__ __forceinline__ void phase_expand(const KParams& P, const Team& T,
       // ---- first round trip -----------------------------------------------
       // the pool's keys for the free lanes (and their nodes), and, when it
       // holds too few, the counter's value
-      const bool fin = key >= 0 && done;
+      const bool fin = key >= 0 && !busy;
       const int rank = __popc(m_free & lt), avail = pool_end - pool_next;
       const int short_by = __popc(m_free) - avail;
       const bool take = !exhausted && short_by > 0;
       int next = -1, next_v = 0, cur = 0;
-      if ((key < 0 || done) && rank < avail) {
+      if (!busy && rank < avail) {
         next = pool_next + rank;
         next_v = P.ve[KP_IDX(P, kd.quot(next), P.t_e, 5)];
       }
@@ -662,6 +663,7 @@ __device__ __forceinline__ void phase_expand(const KParams& P, const Team& T,
         } else {
           pool_next = pool_end = S;
           exhausted = true;
+          refill_at = 32;
         }
       }
       if (D == 12) new_region();
@@ -673,27 +675,25 @@ __device__ __forceinline__ void phase_expand(const KParams& P, const Team& T,
         draw_sample<SYS>(P, it, key, v, kd, x, u, &k, &wacc, wr);
         i = 0;
         fail = 0;
-        done = false;
+        busy = true;
       }
       if (D != 12) new_region();
-      if (__ballot_sync(FULL, key >= 0) == 0) break;
+      if (!__any_sync(FULL, busy)) break;
     }
     // ---- one integrator step (PropagateODE) and its validity check --------
-    if (key >= 0 && !done) {
+    if (busy) {
       const float px = x[0], py = x[1], pz = x[2];
       Sys::step(x, u, P.dt, P);
       ++i;
       const bool inbox = in_state_box<Sys>(x, P);
-      bool ok = inbox;
+      busy = inbox && i < k;
+      fail = inbox ? 0 : -i;  // negative: the end state left the state box
       if (inbox) {
         const float p0[3] = {px, py, pz};
-        ok = !hull_hits_grid(P, sbox, sstart, sids, sclear, p0, x, &n_box);
-      }
-      if (!ok) {
-        done = true;
-        fail = inbox ? i : -i;  // negative: the end state left the state box
-      } else if (i >= k) {
-        done = true;
+        if (hull_hits_grid(P, sbox, sstart, sids, sclear, p0, x, &n_box)) {
+          fail = i;
+          busy = false;
+        }
       }
     }
   }
