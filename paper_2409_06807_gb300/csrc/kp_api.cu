@@ -889,6 +889,7 @@ void fill_params(KParams& P, const Dims& d, const Layout& lay, const kp_system* 
   for (int dd = 0; dd < 12; ++dd) {
     const int n = dd >= 3 && dd < d.D && ws->state_grid[dd] > 1 ? ws->state_grid[dd] : 1;
     P.state_grid[dd] = n;
+    P.state_dims += n > 1 ? 1 : 0;
     P.state_scale[dd] = 0.0f;
     if (n > 1) {
       const bool bounded = std::isfinite(sys->x_lo[dd]) && std::isfinite(sys->x_hi[dd]);

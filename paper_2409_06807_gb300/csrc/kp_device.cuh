@@ -343,7 +343,7 @@ template <>
 struct System<KP_SYS_QUAD> {
   static constexpr int SYM0 = 3, SYM1 = 12;
   static constexpr int D = 12, N = 4;
-  static constexpr int REFILL_MIN = 12;
+  static constexpr int REFILL_MIN = 10;
   static constexpr int FIRST_BATCH_MIN = 16;
   static constexpr int GUIDED_DIV = 4;
   template <bool SMALL>
@@ -455,23 +455,27 @@ __device__ __forceinline__ void bin_state(const float* x, const KParams& P, int*
   int sb = 0;
   if (P.speed_bins > 1)
     sb = fine_cell(__fmul_rn(System<SYS>::speed(x), P.speed_scale), P.speed_bins);
-  // further state dimensions (a grid over the state space), slowest
+  // further state dimensions (a grid over the state space), slowest; looked at
+  // one by one only if any is decomposed (nine comparisons and branches a sample
+  // were 2.4 % of a quadrotor query)
   int e = 0, stride = 1;
+  if (P.state_dims != 0) {
 #pragma unroll
-  for (int dd = 3; dd < System<SYS>::D; ++dd) {
-    const int n = P.state_grid[dd];
-    if (n > 1) {
-      float t;
-      if (P.state_wrap[dd]) {
-        const float pi = 3.14159265358979324f;
-        const float turns = floorf(__fmul_rn(__fadd_rn(x[dd], pi), 0.159154943091895336f));
-        const float y = __fsub_rn(x[dd], __fmul_rn(turns, 6.28318530717958648f));
-        t = __fmul_rn(__fadd_rn(y, pi), P.state_scale[dd]);
-      } else {
-        t = __fmul_rn(__fsub_rn(x[dd], P.x_lo[dd]), P.state_scale[dd]);
+    for (int dd = 3; dd < System<SYS>::D; ++dd) {
+      const int n = P.state_grid[dd];
+      if (n > 1) {
+        float t;
+        if (P.state_wrap[dd]) {
+          const float pi = 3.14159265358979324f;
+          const float turns = floorf(__fmul_rn(__fadd_rn(x[dd], pi), 0.159154943091895336f));
+          const float y = __fsub_rn(x[dd], __fmul_rn(turns, 6.28318530717958648f));
+          t = __fmul_rn(__fadd_rn(y, pi), P.state_scale[dd]);
+        } else {
+          t = __fmul_rn(__fsub_rn(x[dd], P.x_lo[dd]), P.state_scale[dd]);
+        }
+        e += stride * fine_cell(t, n);
+        stride *= n;
       }
-      e += stride * fine_cell(t, n);
-      stride *= n;
     }
   }
   const int nsb = P.speed_bins > 1 ? P.speed_bins : 1;

@@ -160,6 +160,7 @@ struct KParams {
   int32_t speed_bins;
   float speed_scale;    // speed_bins / speed_hi
   int32_t state_grid[12];  // cells over state dimension d (1: not decomposed)
+  int32_t state_dims;      // state dimensions that are decomposed
   float state_scale[12];   // cells per unit of that dimension
   int32_t state_wrap[12];  // 1: an angle, wrapped to [-pi, pi) before binning
   // free-space-obeying decomposition (fso = 1): a kd-tree over position;
