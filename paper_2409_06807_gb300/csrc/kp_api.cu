@@ -363,7 +363,10 @@ kp_status check_ctx(kp_ctx* c) {
 
 kp_status ensure_pinned(kp_ctx* ctx, size_t bytes) {
   if (ctx->pinned_bytes >= bytes) return KP_OK;
-  if (ctx->pinned) cudaFreeHost(ctx->pinned);
+  if (ctx->pinned) {
+    KP_CUDA(cudaStreamSynchronize(ctx->stream));  // no copy is in flight
+    cudaFreeHost(ctx->pinned);
+  }
   ctx->pinned = nullptr;
   ctx->pinned_bytes = 0;
   KP_CUDA(cudaHostAlloc(&ctx->pinned, bytes, cudaHostAllocDefault));
@@ -391,24 +394,54 @@ int host_bp_cell(float v, float lo, float scale, int g) {
   return t >= 0.0f ? (t < (float)g ? (int)t : g - 1) : 0;
 }
 
-// Cell ranges of every padded box on the grid g (cells per axis), with the
-// grid's scale; returns the (cell, box) entry count.
-long long bp_ranges(const float* fb, int nb, const kp_workspace& ws, const int g[3],
-                    float scale[3], std::vector<int>& lo3, std::vector<int>& hi3) {
-  for (int a = 0; a < 3; ++a) scale[a] = (float)((double)g[a] / ((double)ws.hi[a] - (double)ws.lo[a]));
-  lo3.resize((size_t)nb * 3);
-  hi3.resize((size_t)nb * 3);
-  long long entries = 0;
+// Grid cells per axis of the shapes below; cell ranges [lo, hi] of the boxes on
+// an axis cut into g cells, and the axis's cells per unit.
+constexpr int kAxisCells[5] = {1, 4, 16, 32, 64};
+
+float bp_axis_scale(const kp_workspace& ws, int a, int g) {
+  return (float)((double)g / ((double)ws.hi[a] - (double)ws.lo[a]));
+}
+
+void bp_axis_ranges(const float* fb, int nb, const kp_workspace& ws, int a, int g, uint8_t* lo,
+                    uint8_t* hi) {
+  const float scale = bp_axis_scale(ws, a, g);
   for (int b = 0; b < nb; ++b) {
-    long long cells = 1;
-    for (int a = 0; a < 3; ++a) {
-      lo3[(size_t)b * 3 + a] = host_bp_cell(fb[b * 8 + a], ws.lo[a], scale[a], g[a]);
-      hi3[(size_t)b * 3 + a] = host_bp_cell(fb[b * 8 + 4 + a], ws.lo[a], scale[a], g[a]);
-      cells *= hi3[(size_t)b * 3 + a] - lo3[(size_t)b * 3 + a] + 1;
-    }
-    entries += cells;
+    lo[b] = (uint8_t)host_bp_cell(fb[b * 8 + a], ws.lo[a], scale, g);
+    hi[b] = (uint8_t)host_bp_cell(fb[b * 8 + 4 + a], ws.lo[a], scale, g);
   }
-  return entries;
+}
+
+// The boxes' cell ranges on a grid: one pair of arrays an axis.
+struct BpRanges {
+  const uint8_t *lo[3], *hi[3];
+  long long entries(int nb) const {
+    long long n = 0;
+    for (int b = 0; b < nb; ++b)
+      n += (long long)(hi[0][b] - lo[0][b] + 1) * (hi[1][b] - lo[1][b] + 1) * (hi[2][b] - lo[2][b] + 1);
+    return n;
+  }
+  // f(first cell of a row, cells of the row) for every row of cells of box b
+  template <class F>
+  void rows(int b, const int g[3], F f) const {
+    for (int z = lo[2][b]; z <= hi[2][b]; ++z)
+      for (int y = lo[1][b]; y <= hi[1][b]; ++y)
+        f(lo[0][b] + g[0] * (y + g[1] * z), hi[0][b] - lo[0][b] + 1);
+  }
+};
+
+// min(d, max(q, m)) on 16 bytes (one vector instruction each)
+inline void min_of_max16(uint8_t* __restrict__ d, const uint8_t* __restrict__ q, uint8_t m) {
+  for (int j = 0; j < 16; ++j) {
+    const uint8_t v = q[j] > m ? q[j] : m;
+    d[j] = d[j] < v ? d[j] : v;
+  }
+}
+
+// Clearance of a gap in cells, less the margin, in sixteenths rounded down
+// (255 at most, 0 below one); it grows with the gap.
+uint8_t bp_clear_of(double gap) {
+  const double v = (gap - KP_BP_CLEAR_MARGIN) * 16.0;
+  return v >= 1.0 ? (uint8_t)(v < 255.0 ? (int)v : 255) : 0;
 }
 
 // Writes the obstacle blob (padded boxes, then the broad-phase grid: cell
@@ -460,37 +493,72 @@ size_t build_blob(unsigned char* blob, const float* boxes, int nb, const kp_work
                                     {32, 32, 4},  {32, 4, 32}, {4, 32, 32}};
   static_assert(KP_BP_MAX_G * KP_BP_MAX_G * KP_BP_MAX_G == 4096, "grid shapes hold 4096 cells");
   int g[3] = {1, 1, 1};
-  float scale[3];
-  std::vector<int> lo3, hi3;
+  // every axis's ranges on every cut of it (all 0 on one cell)
+  const size_t cut = (size_t)nb;
+  std::vector<uint8_t> range(3 * 5 * 2 * cut, 0);
+  auto ranges_of = [&](const int s[3]) {
+    BpRanges r;
+    for (int a = 0; a < 3; ++a) {
+      int i = 0;
+      while (kAxisCells[i] != s[a]) ++i;
+      r.lo[a] = range.data() + (size_t)(a * 5 + i) * 2 * cut;
+      r.hi[a] = r.lo[a] + cut;
+    }
+    return r;
+  };
+  BpRanges R = ranges_of(g);
+  std::vector<uint16_t> count(4096, 0), best_count(4096, 0);
   if (nb > 0) {
+    for (int a = 0; a < 3; ++a)
+      for (int i = 1; i < 5; ++i) {
+        uint8_t* lo = range.data() + (size_t)(a * 5 + i) * 2 * cut;
+        bp_axis_ranges(fb, nb, ws, a, kAxisCells[i], lo, lo + cut);
+      }
     long long best = -1;
-    std::vector<int> count(4096);
     for (const auto& s : kShapes) {
-      const long long entries = bp_ranges(fb, nb, ws, s, scale, lo3, hi3);
+      const BpRanges r = ranges_of(s);
+      const long long entries = r.entries(nb);
       if (!fits(s, entries)) continue;
-      std::fill(count.begin(), count.end(), 0);
-      for (int b = 0; b < nb; ++b)
-        for (int z = lo3[(size_t)b * 3 + 2]; z <= hi3[(size_t)b * 3 + 2]; ++z)
-          for (int y = lo3[(size_t)b * 3 + 1]; y <= hi3[(size_t)b * 3 + 1]; ++y)
-            for (int x = lo3[(size_t)b * 3]; x <= hi3[(size_t)b * 3]; ++x)
-              count[(size_t)x + (size_t)s[0] * ((size_t)y + (size_t)s[1] * z)] += 1;
+      // (the sum of squares is at least the sum)
+      if (best >= 0 && entries >= best) continue;
+      // the sum of squares as the counts grow; no use once it has reached the best
+      std::fill(count.begin(), count.end(), (uint16_t)0);
       long long sq = 0;
-      for (int c : count) sq += (long long)c * c;
+      for (int b = 0; b < nb && (best < 0 || sq < best); ++b)
+        r.rows(b, s, [&](int c, int n) {
+          for (int x = 0; x < n; ++x) sq += 2 * count[(size_t)(c + x)]++ + 1;
+        });
       if (best < 0 || sq < best) {
         best = sq;
+        std::swap(count, best_count);
         for (int a = 0; a < 3; ++a) g[a] = s[a];
       }
     }
-    if (best < 0)
+    if (best >= 0) {
+      R = ranges_of(g);
+    } else {
+      // (the cut of one cell is all zeros: its place holds the coarse cubes')
       for (int gi = KP_BP_MAX_G / 2; gi >= 1; gi /= 2) {
         const int s[3] = {gi, gi, gi};
-        if (fits(s, bp_ranges(fb, nb, ws, s, scale, lo3, hi3)) || gi == 1) {
+        for (int a = 0; a < 3; ++a) {
+          uint8_t* lo = range.data() + (size_t)(a * 5) * 2 * cut;
+          bp_axis_ranges(fb, nb, ws, a, gi, lo, lo + cut);
+          R.lo[a] = lo;
+          R.hi[a] = lo + cut;
+        }
+        if (fits(s, R.entries(nb)) || gi == 1) {
           for (int a = 0; a < 3; ++a) g[a] = gi;
           break;
         }
       }
+      for (int b = 0; b < nb; ++b)
+        R.rows(b, g, [&](int c, int n) {
+          for (int x = 0; x < n; ++x) ++best_count[(size_t)(c + x)];
+        });
+    }
   }
-  bp_ranges(fb, nb, ws, g, scale, lo3, hi3);
+  float scale[3];
+  for (int a = 0; a < 3; ++a) scale[a] = bp_axis_scale(ws, a, g[a]);
   const int C = g[0] * g[1] * g[2];
   const size_t start_off = (size_t)pad * 32;
   const size_t ids_off = start_off + round16((size_t)(C + 1) * 2);
@@ -498,61 +566,61 @@ size_t build_blob(unsigned char* blob, const float* boxes, int nb, const kp_work
   // box count for the single-cell grid
   uint16_t* start16 = reinterpret_cast<uint16_t*>(blob + start_off);
   uint16_t* ids = reinterpret_cast<uint16_t*>(blob + ids_off);
-  auto cell = [&](int x, int y, int z) { return x + g[0] * (y + g[1] * z); };
-  std::vector<int> start((size_t)C + 1, 0);
+  std::vector<int> cursor((size_t)C);
+  int n_ids = 0;
+  for (int c = 0; c < C; ++c) {
+    cursor[c] = n_ids;
+    start16[c] = (uint16_t)n_ids;
+    n_ids += best_count[c];
+  }
+  start16[C] = (uint16_t)n_ids;
   for (int b = 0; b < nb; ++b)
-    for (int z = lo3[(size_t)b * 3 + 2]; z <= hi3[(size_t)b * 3 + 2]; ++z)
-      for (int y = lo3[(size_t)b * 3 + 1]; y <= hi3[(size_t)b * 3 + 1]; ++y)
-        for (int x = lo3[(size_t)b * 3]; x <= hi3[(size_t)b * 3]; ++x) start[cell(x, y, z) + 1] += 1;
-  for (int c = 0; c < C; ++c) start[c + 1] += start[c];
-  for (int c = 0; c <= C; ++c) start16[c] = (uint16_t)start[c];
-  std::vector<int> cursor(start.begin(), start.begin() + C);
-  for (int b = 0; b < nb; ++b)
-    for (int z = lo3[(size_t)b * 3 + 2]; z <= hi3[(size_t)b * 3 + 2]; ++z)
-      for (int y = lo3[(size_t)b * 3 + 1]; y <= hi3[(size_t)b * 3 + 1]; ++y)
-        for (int x = lo3[(size_t)b * 3]; x <= hi3[(size_t)b * 3]; ++x)
-          ids[cursor[cell(x, y, z)]++] = (uint16_t)b;
-  size_t bytes = ids_off + round16((size_t)start[C] * 2);
+    R.rows(b, g, [&](int c, int n) {
+      for (int x = 0; x < n; ++x) ids[cursor[c + x]++] = (uint16_t)b;
+    });
+  size_t bytes = ids_off + round16((size_t)n_ids * 2);
   P.bp_clear_off = -1;
   if (clearance && bytes + round16((size_t)C) <= max_bytes) {
-    // every box lowers the clearance of the cells within the cap of it
-    std::vector<double> rc((size_t)C, (double)KP_BP_CLEAR_CAP);
+    // Every box lowers the clearance of the cells within the cap of it.  A cell's
+    // gap to a box is the largest of its three axes' gaps, and a clearance byte
+    // grows with the gap, so the axes' gaps are made bytes first and a row of
+    // cells is a minimum of maxima of bytes, 16 at a time.
+    uint8_t* q = blob + bytes;
+    std::memset(q, 0, round16((size_t)C));
+    std::memset(q, bp_clear_of((double)KP_BP_CLEAR_CAP), (size_t)C);
+    // rows along the axis whose cells follow each other: x, or y where x is not cut
+    const int in = g[0] > 1 ? 0 : 1, mid = 1 - in, len = g[in];
     double sc[3];
     for (int a = 0; a < 3; ++a) sc[a] = (double)g[a] / ((double)ws.hi[a] - (double)ws.lo[a]);
+    alignas(16) uint8_t qa[3][64];
     for (int b = 0; b < nb; ++b) {
-      double bl[3], bh[3];
       int c0[3], c1[3];
       for (int a = 0; a < 3; ++a) {
-        bl[a] = ((double)fb[b * 8 + a] - (double)ws.lo[a]) * sc[a];
-        bh[a] = ((double)fb[b * 8 + 4 + a] - (double)ws.lo[a]) * sc[a];
-        const double f0 = std::floor(bl[a]) - KP_BP_CLEAR_CAP, f1 = std::floor(bh[a]) + KP_BP_CLEAR_CAP;
+        const double bl = ((double)fb[b * 8 + a] - (double)ws.lo[a]) * sc[a];
+        const double bh = ((double)fb[b * 8 + 4 + a] - (double)ws.lo[a]) * sc[a];
+        const double f0 = std::floor(bl) - KP_BP_CLEAR_CAP, f1 = std::floor(bh) + KP_BP_CLEAR_CAP;
         c0[a] = f0 < 0.0 ? 0 : (f0 > g[a] - 1 ? g[a] - 1 : (int)f0);
         c1[a] = f1 < 0.0 ? 0 : (f1 > g[a] - 1 ? g[a] - 1 : (int)f1);
+        if (a == in) std::memset(qa[a], 255, (size_t)len);
+        for (int c = c0[a]; c <= c1[a]; ++c)
+          qa[a][c] = bp_clear_of(std::max(0.0, std::max(bl - (double)(c + 1), (double)c - bh)));
       }
       for (int z = c0[2]; z <= c1[2]; ++z)
-        for (int y = c0[1]; y <= c1[1]; ++y)
-          for (int x = c0[0]; x <= c1[0]; ++x) {
-            const int cc[3] = {x, y, z};
-            double gap = 0.0;
-            for (int a = 0; a < 3; ++a) {
-              const double ga = std::max(bl[a] - (double)(cc[a] + 1), (double)cc[a] - bh[a]);
-              gap = std::max(gap, ga);
-            }
-            double& r = rc[(size_t)cell(x, y, z)];
-            r = std::min(r, gap);
-          }
+        for (int y = c0[mid]; y <= c1[mid]; ++y) {
+          const uint8_t m = std::max(qa[2][z], qa[mid][y]);
+          uint8_t* row = q + (size_t)len * (y + g[mid] * z);
+          if (len % 16 == 0)
+            for (int x = c0[in] & ~15; x <= c1[in]; x += 16) min_of_max16(row + x, qa[in] + x, m);
+          else
+            for (int x = c0[in]; x <= c1[in]; ++x)
+              row[x] = std::min(row[x], std::max(m, qa[in][x]));
+        }
     }
-    unsigned char* q = blob + bytes;
-    for (int c = 0; c < C; ++c) {
-      const double v = (rc[c] - KP_BP_CLEAR_MARGIN) * 16.0;
-      q[c] = v >= 1.0 ? (unsigned char)std::min(255.0, std::floor(v)) : 0;
-    }
-    std::memset(q + C, 0, round16((size_t)C) - (size_t)C);
     P.bp_clear_off = (int32_t)bytes;
     bytes += round16((size_t)C);
   }
   P.n_boxes_pad = pad;
-  P.bp_n_ids = start[C];
+  P.bp_n_ids = n_ids;
   P.blob_bytes = (int32_t)bytes;
   for (int a = 0; a < 3; ++a) {
     P.bp_g[a] = g[a];
@@ -722,7 +790,8 @@ kp_status upload_boxes(kp_ctx* ctx, const kp_obstacles* obs) {
   if (ctx->dims.fso)
     KP_CUDA(cudaMemcpyAsync(ctx->arena + L.kd_node, kd, kd_bytes, cudaMemcpyHostToDevice,
                             ctx->stream));
-  KP_CUDA(cudaStreamSynchronize(ctx->stream));
+  // (what reads the copy is queued behind it, and whoever writes the staging
+  // buffer next waits for the stream first)
   ctx->P = Pn;
   ctx->blob_base = (int)bytes;
   ctx->blob_kd = blob_kd;
@@ -1044,6 +1113,7 @@ kp_status kp_create(const kp_system* sys, const kp_workspace* ws, const kp_obsta
   }
   if (s == KP_OK) s = upload_boxes(ctx, obs);
   if (s != KP_OK) {
+    cudaStreamSynchronize(ctx->stream);  // (the obstacles' copy may be in flight)
     if (ctx->pinned) cudaFreeHost(ctx->pinned);
     if (ctx->ev_loop0) cudaEventDestroy(ctx->ev_loop0);
     if (ctx->ev_loop1) cudaEventDestroy(ctx->ev_loop1);
@@ -1332,6 +1402,7 @@ kp_status kp_import_tree(kp_ctx* ctx, const kp_tree_view* v) {
   // the barrier word starts at 0 (no launch is in flight)
   kp_status rs = ensure_pinned(ctx, sizeof(KCtl));
   if (rs != KP_OK) return rs;
+  KP_CUDA(cudaStreamSynchronize(ctx->stream));  // the staging buffer is free
   std::memcpy(ctx->pinned, &h, sizeof(KCtl));
   KP_CUDA(cudaMemcpyAsync(ctx->arena + L.ctl, ctx->pinned, sizeof(KCtl), cudaMemcpyHostToDevice,
                           ctx->stream));

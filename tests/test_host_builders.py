@@ -208,6 +208,56 @@ def test_cell_clearance_never_hides_a_box(H, name):
     np.testing.assert_array_equal(o.work_clearance(), bp["clear"].astype(np.int32))
 
 
+@pytest.mark.parametrize("name", list(layouts()) + ["one box", "infinite boxes"])
+def test_grid_is_the_rule_computed_plainly(H, name):
+    """Shape (smallest sum of squared counts, the first on a tie), cell lists in
+    box order and clearance bytes against the rule written out in FP64."""
+    inf = np.inf
+    boxes = {"one box": [[.3, .3, .3, .4, .6, .3]],
+             "infinite boxes": [[-inf, .2, .2, inf, .3, .3], [.5, -inf, .9, .5, .1, inf],
+                                [inf] * 6, [-inf] * 6]}.get(name)
+    boxes = np.asarray(layouts()[name] if boxes is None else boxes, np.float32)
+    shapes = [(16, 16, 16), (64, 64, 1), (64, 1, 64), (1, 64, 64), (32, 32, 4), (32, 4, 32), (4, 32, 32)]
+
+    def cells(v, a, g):
+        with np.errstate(over="ignore", invalid="ignore"):
+            t = (v - LO[a]) * np.float32(np.float64(g) / (np.float64(HI[a]) - np.float64(LO[a])))
+            return np.where(t >= 0, np.where(t < g, np.clip(t, 0, g).astype(np.int64), g - 1), 0)
+
+    best = None
+    for s in shapes:
+        r = [(cells(boxes[:, a], a, s[a]), cells(boxes[:, 3 + a], a, s[a])) for a in range(3)]
+        n = sum(int(np.prod([r[a][1][b] - r[a][0][b] + 1 for a in range(3)])) for b in range(len(boxes)))
+        if n > 32768:
+            continue
+        c = np.zeros(s[::-1], np.int64)
+        for b in range(len(boxes)):
+            c[tuple(slice(r[a][0][b], r[a][1][b] + 1) for a in (2, 1, 0))] += 1
+        if best is None or (c ** 2).sum() < best[0]:
+            best = ((c ** 2).sum(), s, r, c)
+    bp = blob(H, boxes)
+    if best is None:
+        assert np.prod(bp["g"]) < 4096
+        return
+    _, s, r, c = best
+    assert bp["g"] == list(s) and np.array_equal(np.diff(bp["start"]), c.ravel())
+    want = [[] for _ in range(4096)]
+    gap = np.full(s[::-1], 4.0)
+    for b in range(len(boxes)):
+        box = tuple(slice(r[a][0][b], r[a][1][b] + 1) for a in (2, 1, 0))
+        for k in np.arange(4096).reshape(s[::-1])[box].ravel():
+            want[k].append(b)
+        g = []
+        for a in range(3):
+            sc = np.float64(s[a]) / (np.float64(HI[a]) - np.float64(LO[a]))
+            l, h = ((np.float64(boxes[b, 3 * e + a]) - np.float64(LO[a])) * sc for e in (0, 1))
+            k = np.arange(s[a], dtype=np.float64)
+            g.append(np.maximum(0.0, np.maximum(l - (k + 1), k - h)))
+        gap = np.minimum(gap, np.maximum(np.maximum(g[2][:, None, None], g[1][None, :, None]), g[0]))
+    assert bp["ids"].tolist() == [b for k in want for b in k]
+    assert np.array_equal(bp["clear"], np.floor(np.maximum((gap - 1e-3) * 16, 0)).astype(np.uint8).ravel())
+
+
 def test_grid_respects_the_byte_budget(H):
     """A query whose blob must fit a small budget (a server slot) gets a
     coarser grid, never a larger blob."""
