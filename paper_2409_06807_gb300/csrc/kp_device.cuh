@@ -209,7 +209,7 @@ struct System<KP_SYS_DI> {
   static constexpr int FIRST_BATCH_MIN = 32;
   // later key batches are the keys left over GUIDED_DIV x the warps (at
   // most KP_KEY_BATCH): larger divisors hand out smaller batches towards
-  // the end of a pass (measured: 4 helps the quadrotor's long samples)
+  // the end of a pass (measured: 3 helps the quadrotor's long samples)
   static constexpr int GUIDED_DIV = 2;
   __device__ __forceinline__ static void step(float* x, const float* u, float h,
                                               const KParams&) {
@@ -345,7 +345,7 @@ struct System<KP_SYS_QUAD> {
   static constexpr int D = 12, N = 4;
   static constexpr int REFILL_MIN = 10;
   static constexpr int FIRST_BATCH_MIN = 16;
-  static constexpr int GUIDED_DIV = 4;
+  static constexpr int GUIDED_DIV = 3;
   template <bool SMALL>
   __device__ __forceinline__ static void f(const float* x, const float* u, const KParams& P,
                                            float* dx) {

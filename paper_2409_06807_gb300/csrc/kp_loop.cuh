@@ -64,6 +64,10 @@ struct LoopShared {
   uint64_t mbar;
   int flag;
   int bcast[2];
+  // of the pass's scores, see accept_threshold and draw_accepted
+  double score_sum, score_inv;
+  float inv_m, eps32;
+  int inv_e;
   int goal, err;         // the pass's goal node and error word, read in phase L
   int32_t phase_ns[12];  // per-pass phase timers (block 0, thread 0)
 };
@@ -892,7 +896,7 @@ __device__ __forceinline__ void phase_scores(const KParams& P, const Team& T, in
           const double f2 = __dmul_rn(fv, fv);
           sc = __ddiv_rn(__dmul_rn(f2, f2), den);
         }
-        P.score[r] = sc;
+        P.score[r] = avail ? sc : -1.0;  // no score: P_accept = 1
       }
       int k = 0;
       for (; (q >> k) & 1; ++k) sc = __dadd_rn(left[k], sc);
@@ -916,39 +920,73 @@ __device__ __forceinline__ uint64_t threshold_of(double p) {
   return down < 64 ? mant >> down : 0ull;
 }
 
-// Phase T (the chunks' warps in the node-set phase): the sum of Eq. 5 from the
-// chunks' partial sums (each of these warps reduces them itself, in the same
-// pairwise tree, so all get the same value), then P_accept and the integer
-// threshold of the chunk's regions; each chunk done is counted in t_done.
-__device__ __forceinline__ void phase_thresholds(const KParams& P, const Team& T, int nch) {
-  const int lane = (int)(threadIdx.x & 31u);
-  if (T.b + T.nb * (int)(threadIdx.x >> 5) >= nch) return;
-  const int ch = P.R_pad / nch;
-  // the first regions' scores are fetched beside the chunk sums
-  int r = (T.b + T.nb * (int)(threadIdx.x >> 5)) * ch + lane;
-  bool avail = lane < ch && r < P.R && P.avail[r] != 0;
-  double score = avail ? P.score[r] : 0.0;
+// The acceptance threshold of a region with this score (negative: outside
+// R_avail, P_accept = 1): threshold_of(score / sum + eps), eps below 1, or
+// threshold_of(eps) when the sum is not positive.  inv = 1 / sum gives it without
+// the division (573 clocks and about ten FP64 operations, of which an SM does
+// two a clock): score inv + eps in one rounding is within 4 units in the last
+// place of the value it stands for (half from inv, half each from the two
+// roundings there and one here, at most doubled by a binade), so where 16 units
+// more or less make no difference to the threshold it is the same one.  inv =
+// 0: always by the division (a sum that is not a number between 2^-900 and
+// 2^900).
+__device__ __forceinline__ uint64_t accept_threshold(double score, double sum, double inv, double eps) {
+  if (__double2hiint(score) < 0) return 1ull << 32;
+  if (__double2hiint(inv) != 0) {
+    const long long near = __double_as_longlong(__fma_rn(score, inv, eps));
+    const uint64_t lo = threshold_of(__longlong_as_double(near - 16));
+    if (lo == threshold_of(__longlong_as_double(near + 16))) return lo;
+  }
+  return threshold_of(sum > 0.0 ? __dadd_rn(__ddiv_rn(score, sum), eps) : eps);
+}
+
+// Whether the draw w of a node is below its region's accept_threshold.  Decided
+// in FP32 (an FP64 operation a node was 0.6 % of a query that ends with a
+// million nodes): w < floor(t), t = (score / sum + eps) 2^32, is w + 1 <= t, and
+// t from 24 bits of score and 1 / sum is off by less than 2^-21 of it (2^-23
+// from cutting the score, 2^-24 from each of 1 / sum, eps, w + 1 and three
+// roundings), so a difference above 2^-18 of the larger side has the right sign.
+// The rest, one draw in some 100,000, takes the threshold itself.
+__device__ __forceinline__ bool draw_accepted(uint32_t w, double score, const LoopShared& sh, double eps) {
+  const int hi = __double2hiint(score);
+  if (hi < 0) return true;
+  // score inv_m 2^inv_e in two factors: the mantissas' product, a power of two
+  const int e = (hi >> 20) - 1023 + sh.inv_e;  // at most 1: a score is a part of the sum
+  const float m = __int_as_float(0x3f800000 | (int)(__funnelshift_l((uint32_t)__double2loint(score),
+                                                                    (uint32_t)hi, 3) & 0x7fffffu));
+  const float scale = __int_as_float((e < -126 ? 0 : e + 127) << 23);
+  const float t = __fmul_rn(__fmaf_rn(__fmul_rn(m, sh.inv_m), scale, sh.eps32), 4294967296.0f);
+  const float w1 = __fadd_rn((float)w, 1.0f);
+  if (e < 64 && fabsf(t - w1) > fmaxf(t, w1) * 3.814697265625e-06f) return w1 < t;
+  return (uint64_t)w < accept_threshold(score, sh.score_sum, sh.score_inv, eps);
+}
+
+// The sum of Eq. 5 from the chunks' partial sums, by the calling warp, for the
+// block: sh.score_sum and sh.score_inv (accept_threshold's inv).
+__device__ __forceinline__ void sum_scores(const KParams& P, const Team& T, int nch, LoopShared& sh) {
   const double sum = warp_tree_sum(nch, [&](int i) { return __ldcg(P.chunk_sum + i); });
-  if (T.b == 0 && threadIdx.x == 0) P.ctl->score_sum = sum;
+  if ((threadIdx.x & 31u) == 0) {
+    const int e = (__double2hiint(sum) >> 20) - 1023;  // of a positive number
+    sh.score_sum = sum;
+    const double inv = e >= -900 && e <= 900 ? __ddiv_rn(1.0, sum) : 0.0;
+    sh.score_inv = inv;
+    // (draw_accepted takes the threshold itself where there is no inverse)
+    sh.inv_e = inv > 0.0 ? (__double2hiint(inv) >> 20) - 1023 : 1 << 16;
+    sh.inv_m = inv > 0.0 ? (float)__longlong_as_double((__double_as_longlong(inv) & 0xfffffffffffffll) |
+                                                      0x3ff0000000000000ll)
+                         : 1.0f;
+    sh.eps32 = (float)P.eps;
+    if (T.b == 0) P.ctl->score_sum = sum;
+  }
+}
+
+// Phase T: the thresholds of the warp's region chunks, for the next expand phase.
+__device__ __forceinline__ void phase_thresholds(const KParams& P, const Team& T, int nch,
+                                                 const LoopShared& sh) {
+  const int ch = P.R_pad / nch;
   for_own_chunks(T, nch, [&](int c) {
-    for (int i = lane; i < ch; i += 32) {
-      if (c * ch + i != r) {
-        r = c * ch + i;
-        avail = r < P.R && P.avail[r] != 0;
-        score = avail ? P.score[r] : 0.0;
-      }
-      if (r >= P.R) break;
-      uint64_t thr = 1ull << 32;  // P_accept = 1 outside R_avail
-      if (avail) {
-        double p = P.eps;  // below 1
-        if (sum > 0.0) p = __dadd_rn(__ddiv_rn(score, sum), P.eps);
-        thr = threshold_of(p);
-      }
-      P.thr[r] = thr;
-    }
-    __threadfence();
-    __syncwarp();
-    if (lane == 0) atomicAdd(&P.ctl->t_done, 1u);
+    for (int r = c * ch + (int)(threadIdx.x & 31u); r < (c + 1) * ch && r < P.R; r += 32)
+      P.thr[r] = accept_threshold(P.score[r], sh.score_sum, sh.score_inv, P.eps);
   });
 }
 
@@ -1053,12 +1091,13 @@ __device__ __forceinline__ void materialise(const KParams& P, uint32_t it, int i
 // purpose 2) against the threshold of its region; new nodes are in V_E.
 // Publishes the block chunk's V_E count; returns in *n_new the number of
 // accepted samples of the pass (the new nodes).
-// Order inside the phase: the warps with a region chunk write its thresholds
-// (phase T) and count it done; every block then
-// appends its own accepted samples (ids from t_old, in key order), which
-// needs no threshold; then it waits (bounded) until every chunk is done and
-// makes the node-set draws.  New nodes are counted as V_E members without
-// reading their sets.
+// Order inside the phase: a warp sums the scores while the others append the
+// block's accepted samples (ids from t_old, in key order); then the block makes
+// its draws, each with the threshold of its node's region worked out from the
+// region's score, and last the warps with a region chunk write its thresholds
+// for the next pass.  (With the table written first, every block waited for the
+// chunks' sums, divisions and a count of the chunks done: 3,900 to 6,100 clocks and
+// 1,500 more.)  New nodes are counted as V_E members without reading their sets.
 template <int SYS, bool LOG>
 __device__ __forceinline__ void phase_nodesets(const KParams& P, const Team& T, uint32_t it,
                                                int t_old, const KeyDiv& kd, LoopShared& sh, int* n_new,
@@ -1067,60 +1106,45 @@ __device__ __forceinline__ void phase_nodesets(const KParams& P, const Team& T, 
   uint32_t acc_before, acc_total;
   const uint32_t e0 = (int)threadIdx.x < sh.acc_tot ? accepted_key(P, sh, (int)threadIdx.x) : 0u;
   block_prefix(T, P.blk_a, sh, &acc_before, &acc_total);
-  phase_thresholds(P, T, nch);
+  if ((threadIdx.x >> 5) == (blockDim.x >> 5) - 1) sum_scores(P, T, nch, sh);
   *n_new = (int)acc_total;
   const int t_new = t_old + (int)acc_total;
   materialise<SYS, LOG>(P, it, t_old + (int)acc_before, kd, sh, sblob, e0);
-  // old nodes of the chunk: four tiles at a time, their region and
-  // threshold loads issued together (the first four tiles' regions before the
-  // wait for the thresholds)
+  // old nodes of the chunk: four tiles at a time, their region and score loads
+  // issued together (the first four tiles' before the wait for the sum)
   int v0, v1;
   chunk_of(T, t_new, &v0, &v1);
   const int o1 = v1 < t_old ? v1 : t_old;
   const int stride = (int)blockDim.x;
-  int rq[4];
-  auto regions = [&](int t0) {
+  double sq[2];
+  auto scores = [&](int t0) {
+    int rq[2];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < 2; ++q) {
       const int v = t0 + q * stride + (int)threadIdx.x;
       rq[q] = v < o1 ? KP_IDX(P, __ldcg(P.region + KP_IDX(P, v, P.t_e, 22)), P.R, 23) : 0;
     }
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+      sq[q] = t0 + q * stride + (int)threadIdx.x < o1 ? __ldcg(P.score + rq[q]) : 0.0;
   };
-  regions(v0);
-  if (threadIdx.x == 0) {
-    uint64_t t0 = 0;
-    uint32_t spins = 0;
-    while (ld_acquire(&P.ctl->t_done) < (uint32_t)nch) {
-      if ((++spins & 63u) == 0) {
-        if (*((volatile int*)&P.ctl->err) != 0) break;
-        if (t0 == 0) t0 = global_ns();
-        if (global_ns() - t0 > P.wait_ns) {
-          raise_error(P.ctl, KP_DEV_ERR_TIMEOUT, 25);
-          break;
-        }
-      }
-    }
-    __threadfence();
-  }
+  scores(v0);
   __syncthreads();
   int c = 0;
-  for (int t0 = v0; t0 < o1; t0 += 4 * stride) {
-    uint64_t tq[4];
-    if (t0 != v0) regions(t0);
+  for (int t0 = v0; t0 < o1; t0 += 2 * stride) {
+    if (t0 != v0) scores(t0);
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-      tq[q] = t0 + q * stride + (int)threadIdx.x < o1 ? __ldcg(P.thr + rq[q]) : 0ull;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < 2; ++q) {
       const int v = t0 + q * stride + (int)threadIdx.x;
       if (v < o1) {
         const uint4 w = philox4x32_10(make_uint4(it, (uint32_t)v, 0u, 2u), P.seed_lo, P.seed_hi);
-        const int e = (uint64_t)w.x < tq[q] ? 1 : 0;
+        const int e = draw_accepted(w.x, sq[q], sh, P.eps) ? 1 : 0;
         P.in_ve[v] = (uint8_t)e;
         c += e;
       }
     }
   }
+  phase_thresholds(P, T, nch, sh);
   // new nodes are V_E members (their flags are set by the blocks that
   // appended them, so they are counted, not read)
   const int new0 = v0 > t_old ? v0 : t_old;
@@ -1142,7 +1166,6 @@ __device__ __forceinline__ bool run_loop(const KParams& P, const Team& T, unsign
     ctl->stop = 0;
     ctl->n_run = 0;
     ctl->work_next = 0;
-    ctl->t_done = 0;
   }
   // the loop state, read once per block
   // the second layer's weights of an attached network, for every pass
@@ -1247,7 +1270,6 @@ __device__ __forceinline__ bool run_loop(const KParams& P, const Team& T, unsign
         P.stats[run - 1] = s;
       }
       ctl->it_valid = 0;
-      ctl->t_done = 0;  // every block is past its threshold wait
       ctl->tot_samples += (unsigned long long)S;
       ctl->state = solved ? KP_DEV_SOLVED : (full ? KP_DEV_FULL : KP_DEV_RUNNING);
       // a time limit ends the loop by block 0's clock

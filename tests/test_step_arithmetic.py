@@ -72,3 +72,56 @@ def test_threshold_from_the_bits():
         assert threshold_of(v) == int(np.floor(min(v, 1.0) * 2.0**32)), v
     for v in (np.inf, np.nan, -np.nan):
         assert threshold_of(v) == 1 << 32
+
+
+def exact_threshold(score, total, eps):
+    return threshold_of(score / total + eps if total > 0 else eps)
+
+
+def fast_threshold(score, inv, eps):
+    """accept_threshold's answer without the division, None where it divides."""
+    near = int(np.float64(np.longdouble(score) * np.longdouble(inv) + np.longdouble(eps)).view(np.int64))
+    lo, hi = (threshold_of(np.int64(near + d).view(np.float64)) for d in (-16, 16))
+    return lo if lo == hi else None
+
+
+def fast_draw(w, score, inv, eps):
+    """draw_accepted's answer in FP32, None where it takes the threshold."""
+    f = np.float32
+    m, e = np.frexp(score)
+    im, ie = np.frexp(inv)
+    e = int(e) - 1 + int(ie) - 1 if score > 0 else -2000
+    m = f(np.floor(m * 2.0**24) / 2.0**23) if score > 0 else f(1.0)
+    scale = f(0.0) if e < -126 else f(2.0) ** f(e)
+    r = f(np.float64(f(m * f(im * 2.0))) * np.float64(scale) + np.float64(f(eps)))
+    t, w1 = f(r * f(4294967296.0)), f(f(w) + f(1.0))
+    if abs(f(t - w1)) > f(max(t, w1) * f(2.0**-18)):
+        return bool(w1 < t)
+    return None
+
+
+def test_acceptance_without_the_division():
+    """Scores over 40 binary orders, the draws on, next to and around the
+    threshold, eps from 1e-300 to 0.9: what is decided without the division is
+    decided as with it, and few random draws need it."""
+    rng = np.random.default_rng(2)
+    undecided = draws = 0
+    for _ in range(300):
+        n = int(rng.integers(1, 50))
+        s = np.exp2(rng.uniform(-40, 0, n) - rng.integers(0, 600)) * (rng.random(n) > 0.1)
+        total, eps = s.sum(), float(rng.choice([1e-300, 1e-12, 1e-4, 0.01, 0.5, 0.9]))
+        if not total > 0:
+            continue
+        inv = 1.0 / total
+        for score in s[:6]:
+            thr = exact_threshold(score, total, eps)
+            fast = fast_threshold(score, inv, eps)
+            assert fast is None or fast == thr
+            for w in {0, 1, thr - 2, thr - 1, thr, thr + 1, 2**32 - 1, *rng.integers(0, 2**32, 4).tolist()}:
+                if 0 <= w < 2**32:
+                    d = fast_draw(w, score, inv, eps)
+                    assert d is None or d == (w < thr)
+            for w in rng.integers(0, 2**32, 4).tolist():
+                draws += 1
+                undecided += fast_draw(w, score, inv, eps) is None
+    assert undecided < 0.01 * draws
