@@ -677,6 +677,7 @@ __device__ __forceinline__ void phase_expand(const KParams& P, const Team& T,
         ran = true;
         v = KP_IDX(P, next_v, P.t_e, 6);
         draw_sample<SYS>(P, it, key, v, kd, x, u, &k, &wacc, wr);
+        Sys::prepare(u, P);
         i = 0;
         fail = 0;
         busy = true;
@@ -1076,6 +1077,7 @@ __device__ __forceinline__ void materialise(const KParams& P, uint32_t it, int i
       float y[D];
 #pragma unroll
       for (int d = 0; d < D; ++d) y[d] = P.st[(size_t)d * P.t_e + v];
+      Sys::prepare(u, P);  // (the node's controls are written above)
       for (int st = 0; st < k; ++st) Sys::step(y, u, P.dt, P);
       bool same = P.log.region[key] == r && P.log.sub[key] == s;
 #pragma unroll
