@@ -16,13 +16,13 @@
 //      chunk (a block's first, which takes no keys):
 //   S  Score per region (Eq. 3-4, FP64, rounded exactly as written) and
 //      the pairwise partial sum of each aligned region chunk (Eq. 5's sum).
-//   N  first, on warp 0 of each region-chunk block, T: the sum of Eq. 5
-//      from the partial sums and P_accept with its integer accept threshold
-//      per region; each block appends its own accepted samples (Algorithm
-//      4, to T and V_E) at their key-order node ids, from the kept end
-//      states, with the goal test; then one selection draw per old node
-//      against its region's new threshold (Algorithm 4, V_E <-> V_O) and
-//      per-block V_E counts.
+//   N  a warp of each block takes the sum of Eq. 5 from the partial sums while
+//      the block appends its own accepted samples (Algorithm 4, to T and V_E)
+//      at their key-order node ids, from the kept end states, with the goal
+//      test; then one selection draw per old node against P_accept of its
+//      region, from the region's score (Algorithm 4, V_E <-> V_O), per-block
+//      V_E counts, and on the warps with a region chunk, T: the integer
+//      accept threshold per region, for the next pass.
 //   L  V_E list in ascending node id, lambda for the next pass (Eq. 6),
 //      stop decision.
 // With a network attached (learned proposal) a phase F before E evaluates
@@ -740,10 +740,10 @@ __device__ __forceinline__ void warp_range(int c0, int c1, int* a, int* b) {
 // takes keys t0 + 32q + l: every load is coalesced), with the loads of a
 // tile's flags, contenders' sub-regions and their claims issued together,
 // and compacts its accepted keys (claim winners marked in bit 31) in key
-// order at the start of its range in acc_key.  Phase S (warp 0) runs
-// alongside.  Publishes the block's accepted count, adds the valid count to
-// the pass, and leaves where each warp's accepted keys are, and their
-// offsets among the block's, in shared memory for the node-set phase.
+// order at the start of its range in acc_key.  Phase S comes before it, on the
+// warps with a region chunk.  Publishes the block's accepted count, adds the
+// valid count to the pass, and leaves where each warp's accepted keys are, and
+// their offsets among the block's, in shared memory for the node-set phase.
 constexpr int KP_ACC_KPL = 8;
 
 __device__ __forceinline__ void phase_scores(const KParams& P, const Team& T, int nch);
