@@ -17,7 +17,7 @@ cudaError_t KP_CAT(loop_occupancy_, KP_SYS_NAME)(bool log, size_t smem, int* blo
   const int threads = *blocks_per_sm;
   const void* f = log ? (const void*)kp_loop_kernel<KP_SYS, true>
                       : (const void*)kp_loop_kernel<KP_SYS, false>;
-  cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = raise_shared_limit(f, smem);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, f, threads, smem);
 }

@@ -41,6 +41,21 @@
 
 namespace kp {
 
+// Sets a kernel's limit of dynamic shared memory to what the device has beside
+// the kernel's static shared memory, whatever this context or server needs of
+// it: the limit is one for all of them, and the one configured last must not
+// lower it below what another one's launch takes.
+inline cudaError_t raise_shared_limit(const void* kernel, size_t smem) {
+  constexpr int kStaticShared = 1280;  // LoopShared and the barrier's words fit it
+  int dev = 0, most = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e != cudaSuccess) return e;
+  most -= kStaticShared;
+  if (smem > (size_t)most) most = (int)smem;  // refused by the next call if it is too much
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 // (KP_BLOCK, the most threads of a block, is set by the including file)
 constexpr int KP_WARPS = KP_BLOCK / 32;
 static_assert(KP_WARPS <= 32 && KP_BLOCK % KP_MLP_GROUP == 0, "warps fit a lane each, groups are whole");
@@ -71,6 +86,7 @@ struct LoopShared {
   int goal, err;         // the pass's goal node and error word, read in phase L
   int32_t phase_ns[12];  // per-pass phase timers (block 0, thread 0)
 };
+static_assert(sizeof(LoopShared) <= 1200, "see raise_shared_limit");
 
 // Stage the obstacle blob (boxes and broad-phase grid) into shared memory
 // with bulk asynchronous copies (TMA engine) completing on one mbarrier.

@@ -163,8 +163,7 @@ __global__ void __launch_bounds__(KP_BLOCK, KP_MIN_BLOCKS) kp_server_kernel(KSer
 }
 
 cudaError_t server_occupancy(size_t smem, int* blocks_per_sm) {
-  cudaError_t e = cudaFuncSetAttribute(kp_server_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  cudaError_t e = raise_shared_limit((const void*)kp_server_kernel, smem);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kp_server_kernel, KP_BLOCK,
                                                        smem);

@@ -388,3 +388,25 @@ def test_learned_plan_with_less_shared_memory(M, extra, limit):
     assert s0 == s1 and i0 == i1 and i0[0] > 1000
     for k in t0 or {}:
         assert np.array_equal(t0[k], t1[k])
+
+
+def test_contexts_of_different_shared_memory(M):
+    """A context's launch does not depend on which context was configured last:
+    one with the network's weights staged, one with many obstacles, one plain."""
+    mlp, P = M
+    net = mlp.Mlp(mlp.init_params(4), max_batch=64)
+    w = W.c2(3, lambda_max=32)
+    boxes = np.asarray(w.boxes, dtype=np.float32)
+    many = np.concatenate([boxes, np.tile(boxes[:1], (2000, 1))]).astype(np.float32)
+    a, b, c = P.Planner(w), P.Planner(w.with_(boxes=many)), P.Planner(w)
+    a.attach_mlp(net, 0.5)
+    b.attach_mlp(net, 0.5)
+    first = [g.plan(max_iters=6) for g in (a, b, c)]
+    for order in ((0, 1, 2), (2, 1, 0), (1, 2, 0)):
+        gs = (a, b, c)
+        for k in order:
+            gs[k].set_obstacles(many if k == 1 else boxes)
+        for k in (0, 1, 2):
+            st, t = gs[k].plan(max_iters=6)
+            assert st == first[k][0] and np.array_equal(t["steps"], first[k][1]["steps"])
+    assert first[0][0] == first[1][0]
