@@ -541,7 +541,10 @@ __device__ __forceinline__ void phase_expand(const KParams& P, const Team& T,
   // queues on the counter to start; later batches come from the counter,
   // offset past the statically handed-out keys.
   const int n_warps = T.nb * (int)(blockDim.x >> 5);
-  const int gw = T.b * (int)(blockDim.x >> 5) + (int)(threadIdx.x >> 5);
+  // The warps are numbered across the blocks first, so that a pass of fewer
+  // batches than warps spreads over all SMs (block by block, a small pass filled
+  // some SMs and left the others idle: 0.9 to 1.7 % of a launch).
+  const int gw = T.b + T.nb * (int)(threadIdx.x >> 5);
   int b0 = S / (2 * n_warps);
   b0 = b0 < Sys::FIRST_BATCH_MIN ? Sys::FIRST_BATCH_MIN : (b0 > KP_KEY_BATCH ? KP_KEY_BATCH : b0);
   const int static_end = n_warps * b0 < S ? n_warps * b0 : S;
