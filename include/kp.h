@@ -328,8 +328,9 @@ kp_status kp_resume(kp_ctx *ctx, const kp_budget *budget, kp_traj *traj);
 kp_status kp_set_sample_log(kp_ctx *ctx, const kp_sample_log *log);
 
 /* Upper bound, in nanoseconds, of every device-side wait (grid barrier,
- * bulk-copy completion).  On expiry the launch stops, the call returns
- * KP_ERR_TIMEOUT and the context is poisoned.  Default 2e9 (2 s). */
+ * bulk-copy completion) and of a pass's expand phase.  On expiry the launch
+ * stops, the call returns KP_ERR_TIMEOUT and the context is poisoned.
+ * Default 2e9 (2 s). */
 kp_status kp_set_wait_limit(kp_ctx *ctx, uint64_t ns);
 
 /* Launch shape of the persistent loop (no counterpart in the paper: a
@@ -360,9 +361,9 @@ kp_status kp_set_extract_ids(kp_ctx *ctx, int32_t max_ids);
  * sample keys, regions, sub-regions, V_E positions, accepted-sample slots,
  * block slots, broad-phase cells, box lists and box ids) against its
  * array: an index out of range records the site, is replaced by 0 so that
- * no access leaves its array (nothing traps), and the launch stops at its
- * next barrier; the call then returns KP_ERR_CUDA with the site in
- * kp_last_error and the context is poisoned.  kp_bounds_checked returns 1
+ * no access leaves its array (nothing traps), and the launch stops at the
+ * end of the pass at the latest; the call then returns KP_ERR_CUDA with the
+ * site in kp_last_error and the context is poisoned.  kp_bounds_checked returns 1
  * in that build, 0 otherwise.  kp_selftest_bounds looks up an index one
  * past the tree through the checked path and returns what the launch
  * reports (KP_ERR_CUDA, site 97, in the checked build); in the normal build

@@ -36,9 +36,9 @@ __device__ __forceinline__ void raise_error(KCtl* ctl, int code, int where) {
 
 // Array indices of the loop kernel.  In the bounds-checked build (KP_CHECK
 // defined) an index outside [0, n) records KP_DEV_ERR_BOUNDS with its site
-// and 0 is used in its place, so that no access leaves its array, nothing
-// traps, and every block stops at its next barrier; the host reports the
-// site.  Otherwise the index is used as it is.
+// and 0 is used in its place, so that no access leaves its array and nothing
+// traps; every block stops at the end of the pass at the latest (team_sync) and
+// the host reports the site.  Otherwise the index is used as it is.
 #ifdef KP_CHECK
 __device__ __forceinline__ long long kp_checked(KCtl* ctl, long long i, long long n, int site) {
   if (i >= 0 && i < n) return i;
@@ -70,13 +70,15 @@ struct Team {
 // load that sees the flip synchronises with every block's fence, and the
 // closing __syncthreads carries that to the block's other threads (a fence
 // after the wait measured slower and adds nothing).  Every wait is bounded by 'limit_ns'
-// of device time; on expiry the block records KP_ERR_TIMEOUT and all blocks
-// leave at their next wait (the word is then left mid-phase: a launch that
-// timed out poisons its context).  Returns false when the launch must stop:
-// the wait expired, or it was long and saw an error (an error that stops no
-// block's arrival is found by the loop's own look at the error word, once a
-// pass).  Reading the error word after every barrier cost a round trip to L2:
-// a barrier of 456 blocks took 3,650 clocks with it, 3,300 without.  With
+// of device time; on expiry the block records KP_ERR_TIMEOUT and leaves, and the
+// others leave at the next barrier, which it does not reach (the word is then
+// left mid-phase: a launch that timed out poisons its context).  Returns false
+// when the launch must stop: the wait expired, or it was long and saw an error.
+// True does not say that there is none: an error that stops no block's arrival is
+// found by the loop's look at the error word at the end of the pass, so what the
+// phases up to there read must be defined all the same (give_up_keys).  Reading
+// the error word after every barrier cost a round trip to L2: a barrier of 456
+// blocks took 3,650 clocks with it, 3,300 without.  With
 // 'watch' given, thread 0 also reads that word after the barrier and the block
 // gets its value in *watched.  With check_err false the wait ignores the
 // control block's error word (the barriers around a launch's own

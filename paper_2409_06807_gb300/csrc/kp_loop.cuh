@@ -510,6 +510,25 @@ __device__ __forceinline__ void draw_sample(const KParams& P, uint32_t it, int k
 // large frontier faster than 128, 64 1.5 % slower)
 constexpr int KP_KEY_BATCH = 256;
 
+// A warp whose time ran out gives up its lanes' samples, the keys it has taken
+// and those that no warp has taken (whoever asks for more finds none): their
+// flags say that nothing came of them.  The accept phase reads every key's flags,
+// and the barrier before it stops only blocks that wait for long.  (Every warp
+// looking at the error word there cost a pass 0.1 to 0.6 us, a call of 20 passes
+// 1.1 %; this costs 0 to 0.3 %, a call, so that the loop's registers stay.)
+static __device__ __noinline__ void give_up_keys(const KParams& P, int key, int pool_next, int pool_end,
+                                             int static_end, int S) {
+  const int lane = (int)(threadIdx.x & 31u);
+  auto clear = [&](int q) { P.flags[KP_IDX(P, q, P.t_e, 11)] = 0; };
+  if (key >= 0) clear(key);
+  for (int q = pool_next + lane; q < pool_end; q += 32) clear(q);
+  int rest = S;
+  if (lane == 0 && static_end < S)
+    rest = static_end + atomicMax(&P.ctl->work_next, S - static_end);
+  rest = __shfl_sync(0xffffffffu, rest, 0);
+  for (int q = rest + lane; q < S; q += 32) clear(q);
+}
+
 template <int SYS, bool LOG>
 __device__ __forceinline__ void phase_expand(const KParams& P, const Team& T,
                                              const unsigned char* sblob, uint32_t it, const KeyDiv& kd,
@@ -567,6 +586,7 @@ __device__ __forceinline__ void phase_expand(const KParams& P, const Team& T,
       const uint64_t now = __shfl_sync(FULL, global_ns(), 0);
       if (now - t_phase > P.wait_ns) {
         if (lane == 0) raise_error(P.ctl, KP_DEV_ERR_TIMEOUT, 30);
+        give_up_keys(P, key, pool_next, pool_end, static_end, S);
         break;
       }
       // Finalise and refill together: what each needs from memory is issued

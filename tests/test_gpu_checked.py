@@ -59,3 +59,17 @@ def test_lockstep_suites_on_the_bounds_checked_build():
     tail = (r.stdout + r.stderr)[-3000:]
     assert r.returncode == 0, tail
     assert " passed" in r.stdout and "failed" not in r.stdout, tail
+
+
+def test_expand_phase_past_its_wait_limit_on_the_bounds_checked_build():
+    """The pass that gives up leaves records unwritten; on this build an index
+    read from them could not leave its array, whatever the accept phase does."""
+    env = dict(os.environ, KP_TEST_BOUNDS_CHECKED="1")
+    r = subprocess.run([sys.executable, "-m", "pytest", os.path.join(ROOT, "tests",
+                                                                     "test_gpu_parity.py"),
+                        "-m", "gpu", "-q", "-x", "-p", "no:cacheprovider", "-k",
+                        "past_its_wait_limit"],
+                       capture_output=True, text=True, env=env, cwd=ROOT, timeout=900)
+    tail = (r.stdout + r.stderr)[-3000:]
+    assert r.returncode == 0, tail
+    assert "3 passed" in r.stdout, tail

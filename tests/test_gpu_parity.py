@@ -483,6 +483,43 @@ def test_bounded_wait_reports_timeout(P):
     assert h.reset() == P.OK
 
 
+@pytest.mark.parametrize("system", [W.DI, W.DUBINS, W.QUAD])
+def test_expand_phase_past_its_wait_limit(P, system):
+    """A pass whose expand phase outlasts the wait limit: warps give up with
+    samples in flight and keys not handed out, so these have no records but
+    what the arena held before (here words that are no index and, as flags,
+    say that the sample is a contender).  The call ends with KP_ERR_TIMEOUT
+    from that phase (site 30) and nothing is read through those records."""
+    import torch
+    w = {W.DI: W.c1, W.DUBINS: W.c2, W.QUAD: W.c3}[system](0)
+    w = w.with_(t_e=1 << 23, lambda_max=128, goal_c=np.full(3, 9.0, np.float32),
+                goal_r=np.float32(0.0))
+    probe = P.Planner(w)
+    nbytes = probe.arena_bytes
+    probe.close()
+    del probe
+    torch.full((nbytes,), 0xff, dtype=torch.uint8, device="cuda")  # the arena's memory, from the cache
+    g = P.Planner(w)
+    assert g.reset() == P.OK
+    for _ in range(40):
+        if g.info()["n_nodes"] >= 20000:
+            break
+        g.expand_step(1)
+    t = g.export_tree()
+    assert t["n_nodes"] >= 20000
+    t["in_ve"][:] = 1  # a pass of 2.5 million samples and more
+    g.import_tree(t)
+    g.set_wait_limit(60_000)  # 60 us: the pass takes several times as long
+    with pytest.raises(P.KpError) as e:
+        g.expand_step(1)
+    assert e.value.status == P.ERR_TIMEOUT and "site 30)" in str(e.value)
+    with pytest.raises(P.KpError) as e:
+        g.reset()
+    assert e.value.status == P.ERR_STATE  # poisoned
+    g.close()
+    assert P.Planner(W.tiny(system)).reset() == P.OK
+
+
 def test_broad_phase_coarsens_for_large_boxes(P):
     """Many boxes spanning most of the workspace overflow the finest
     broad-phase grid; the planner coarsens it and the verdicts still match
