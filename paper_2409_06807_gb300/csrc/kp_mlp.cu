@@ -122,18 +122,14 @@ MlpLayout mlp_layout(int B) {
     }                                             \
   } while (0)
 
-
-// Raises the dynamic shared memory limit of the tensor-core kernels (once,
-// outside any stream capture).
+// Raises the dynamic shared memory limit of the tensor-core kernels on the
+// current device (outside any stream capture): with every network, since the
+// limit is a device's own and a process may have networks on several.
 kp_status tc_configure() {
-  static bool done = false;
-  if (!done) {
-    MLP_CUDA(cudaFuncSetAttribute(tc::kp_mlp_forward_tc_kernel,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, tc::FT_SMEM));
-    MLP_CUDA(cudaFuncSetAttribute(tc::kp_mlp_train_kernel,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, tc::ST_SMEM));
-    done = true;
-  }
+  MLP_CUDA(cudaFuncSetAttribute(tc::kp_mlp_forward_tc_kernel,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, tc::FT_SMEM));
+  MLP_CUDA(cudaFuncSetAttribute(tc::kp_mlp_train_kernel,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, tc::ST_SMEM));
   return KP_OK;
 }
 
