@@ -437,7 +437,10 @@ kp_status kp_mlp_create(void *dev_arena, size_t arena_bytes, int32_t max_batch,
 kp_status kp_mlp_set_params(kp_mlp *mlp, const float *host_params);
 kp_status kp_mlp_get_params(kp_mlp *mlp, float *host_params);
 /* dev_x: device [M][32] FP32 inputs; dev_out: device [M][8] FP32 (mean[4],
- * log_std[4]).  Enqueued only. */
+ * log_std[4]).  Enqueued only.  Rows for which a bounded wait of the kernel
+ * (2 s) expired are NaN in all eight outputs; the network's next call that
+ * reports such a wait (gradients, training) then returns KP_ERR_TIMEOUT, until
+ * its parameters are set again. */
 kp_status kp_mlp_forward(kp_mlp *mlp, const float *dev_x, int32_t M,
                          float *dev_out);
 /* Gradient of the batch-mean Gaussian negative log-likelihood of the device
@@ -460,6 +463,10 @@ kp_status kp_mlp_train_step(kp_mlp *mlp, const float *dev_x,
 kp_status kp_mlp_train_epoch(kp_mlp *mlp, const float *dev_x, const float *dev_t,
                              const int32_t *dev_perm, int64_t rows, float lr,
                              float *host_loss);
+/* Test hook for the bounded waits: with limit_ns > 0 (2 s at most) the
+ * network's inference launches hold their first product back, so that the
+ * waits for it expire after limit_ns; 0 ends this.  KP_ERR_ARG past 2 s. */
+kp_status kp_mlp_selftest_hold(kp_mlp *mlp, uint64_t limit_ns);
 void kp_mlp_destroy(kp_mlp *mlp);
 /* Planner use of a network (6D systems): each pass evaluates the network on
  * the features of every V_E node; a sample whose selector draw falls below

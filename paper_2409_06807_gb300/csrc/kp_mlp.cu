@@ -74,6 +74,8 @@ struct kp_mlp {
   bf16* wf;     // W1 | W2 | W3 in BF16, fragment order (planner loop)
   bf16* wt;     // W2 | W1 in BF16, tensor-core operand order
   int* err;     // nonzero: a tensor-core kernel's bounded wait expired
+  unsigned long long wait_ns;  // limit of those waits
+  int hold;                    // test hook: launches hold their products back
 };
 
 namespace {
@@ -172,7 +174,7 @@ tc::StepArgs step_args(const kp_mlp* n, const float* x, const float* t, int M, f
   a.adam = adam_args(n, M, lr);
   a.slots = n->slots;
   a.err = n->err;
-  a.wait_ns = kWaitNs;
+  a.wait_ns = n->wait_ns;
   return a;
 }
 
@@ -206,6 +208,8 @@ kp_status kp_mlp_create(void* dev_arena, size_t arena_bytes, int32_t max_batch,
   n->bytes = arena_bytes;
   n->stream = static_cast<cudaStream_t>(cuda_stream);
   n->max_batch = max_batch;
+  n->wait_ns = kWaitNs;
+  n->hold = 0;
   char* A = n->arena;
   n->p = reinterpret_cast<float*>(A + L.p);
   n->m = reinterpret_cast<float*>(A + L.m);
@@ -262,6 +266,13 @@ kp_status kp_mlp_get_params(kp_mlp* n, float* host_params) {
 
 int32_t kp_mlp_num_params(void) { return N_PARAMS; }
 
+kp_status kp_mlp_selftest_hold(kp_mlp* n, uint64_t limit_ns) {
+  if (!n || limit_ns > kWaitNs) return KP_ERR_ARG;
+  n->hold = limit_ns > 0 ? 1 : 0;
+  n->wait_ns = limit_ns > 0 ? limit_ns : kWaitNs;
+  return KP_OK;
+}
+
 kp_status kp_mlp_forward(kp_mlp* n, const float* dev_x, int32_t M, float* dev_out) {
   if (!n || !dev_x || !dev_out || M < 0 || M > n->max_batch) return KP_ERR_ARG;
   if (M == 0) return KP_OK;
@@ -276,7 +287,8 @@ kp_status kp_mlp_forward(kp_mlp* n, const float* dev_x, int32_t M, float* dev_ou
   a.M = M;
   a.vec = ((uintptr_t)dev_x & 15u) == 0 && ((uintptr_t)dev_out & 7u) == 0;
   a.err = n->err;
-  a.wait_ns = kWaitNs;
+  a.wait_ns = n->wait_ns;
+  a.hold = n->hold;
   const int tiles = (M + tc::FT_ROWS - 1) / tc::FT_ROWS;
   tc::kp_mlp_forward_tc_kernel<<<tiles < n->num_sms ? tiles : n->num_sms, tc::FT_THREADS,
                                  tc::FT_SMEM, n->stream>>>(a);

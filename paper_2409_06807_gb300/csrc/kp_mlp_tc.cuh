@@ -163,6 +163,7 @@ struct FtArgs {
   int M, vec;               // vec: x and out allow 16- and 8-byte accesses
   int* err;
   unsigned long long wait_ns;
+  int hold;                 // test hook: no product is issued
 };
 
 // Inputs 16 part .. 16 part + 15 of a row (zeros past the last row).
@@ -256,7 +257,9 @@ __global__ void __launch_bounds__(FT_THREADS, 1) kp_mlp_forward_tc_kernel(FtArgs
     if (lane == 0) mbar_arrive(saddr(bar));
   };
   // After a wait that gave up the epilogues run on to their end (the waits
-  // left return at once) without storing.
+  // left return at once), and the rows that are still to come are NaN: the
+  // caller has no status to ask, and must not take what the output held before
+  // for a result.
   auto wait = [&](uint64_t* bar, uint32_t parity, int site) {
     const bool ok = mbar_wait_or(saddr(bar), parity, a.wait_ns, &s_fail, site);
     __syncwarp(__activemask());
@@ -275,6 +278,7 @@ __global__ void __launch_bounds__(FT_THREADS, 1) kp_mlp_forward_tc_kernel(FtArgs
         mma_commit(saddr(&b_d1));
       };
       bool ok = wait(&b_w1, 0, 10) && wait(&b_x, 0, 11);
+      if (a.hold) ok = wait(&b_d2, 0, 16);  // (nothing is committed to it)
       if (ok) layer1();
       uint32_t ph = 0;
       for (int t = blockIdx.x; ok && t < n_tiles; t += stride, ph ^= 1u) {
@@ -425,7 +429,8 @@ __global__ void __launch_bounds__(FT_THREADS, 1) kp_mlp_forward_tc_kernel(FtArgs
           v1 = fminf(fmaxf(v1, MLP_LOGSTD_MIN), MLP_LOGSTD_MAX);
         }
         const int row = t * FT_ROWS + rl;
-        if (row < a.M && *((volatile int*)&s_fail) == 0) {
+        if (*((volatile int*)&s_fail) != 0) v0 = v1 = __int_as_float(0x7fffffff);
+        if (row < a.M) {
           float* dst = a.out + (size_t)row * MLP_OUT + 2 * tq;
           if (a.vec) {
             *reinterpret_cast<float2*>(dst) = make_float2(v0, v1);

@@ -94,7 +94,8 @@ class Mlp:
                   "kp_mlp_set_params")
 
     def forward(self, x):
-        """x: CUDA float32 [M, 32] -> CUDA float32 [M, 8] (mean[4], log_std[4])."""
+        """x: CUDA float32 [M, 32] -> CUDA float32 [M, 8] (mean[4], log_std[4]);
+        NaN in rows for which a bounded wait on the device expired."""
         import torch
         x = x.contiguous()
         out = torch.empty((x.shape[0], N_OUT), dtype=torch.float32, device=x.device)
@@ -129,6 +130,9 @@ class Mlp:
                                           float(lr), C.byref(loss) if want_loss else None),
                   "kp_mlp_train_step")
         return loss.value if want_loss else None
+
+    def selftest_hold(self, ns):
+        self._chk(lib().kp_mlp_selftest_hold(self._ctx, int(ns)), "kp_mlp_selftest_hold")
 
 
 def harvest(make_workload, seeds, n_pairs, max_iters=400, planner=None, per_query_cap=1 << 18,

@@ -143,6 +143,7 @@ SIGNATURES = {
     "kp_mlp_train_step": (C.c_int, [_vp, _vp, _vp, C.c_int32, C.c_float, C.POINTER(C.c_float)]),
     "kp_mlp_train_epoch": (C.c_int, [_vp, _vp, _vp, _vp, C.c_int64, C.c_float,
                                      C.POINTER(C.c_float)]),
+    "kp_mlp_selftest_hold": (C.c_int, [_vp, C.c_uint64]),
     "kp_mlp_destroy": (None, [_vp]),
     "kp_attach_mlp": (C.c_int, [_vp, _vp, C.c_float]),
     "kp_set_harvest": (C.c_int, [_vp, _vp, _vp, C.c_int32, _vp]),

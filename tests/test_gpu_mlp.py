@@ -410,3 +410,33 @@ def test_contexts_of_different_shared_memory(M):
             st, t = gs[k].plan(max_iters=6)
             assert st == first[k][0] and np.array_equal(t["steps"], first[k][1]["steps"])
     assert first[0][0] == first[1][0]
+
+
+@pytest.mark.parametrize("n", [1, 129, 2 * 152 * 128 + 5])
+def test_inference_that_gives_up_says_so(M, n):
+    """Inference whose products never come (the test hook) ends after the wait
+    limit: every row is NaN, not what the output held before, the next call
+    that reports says KP_ERR_TIMEOUT, and setting the parameters clears it."""
+    import time
+
+    import torch
+    mlp, planner = M
+    p = mlp.init_params(3)
+    net = mlp.Mlp(p, max_batch=n)
+    x, t = [torch.from_numpy(v).cuda() for v in _data(n, n)]
+    want = net.forward(x)
+    out = torch.full((n, 8), 0.25, device="cuda")
+    net.selftest_hold(50_000_000)  # 50 ms
+    torch.cuda.synchronize()
+    t0 = time.perf_counter()
+    assert planner.lib().kp_mlp_forward(net._ctx, x.data_ptr(), n, out.data_ptr()) == 0
+    torch.cuda.synchronize()
+    assert 0.04 < time.perf_counter() - t0 < 0.15
+    net.selftest_hold(0)
+    assert bool(torch.isnan(out).all())
+    with pytest.raises(planner.KpError) as e:
+        net.gradients(x, t)
+    assert e.value.status == planner.ERR_TIMEOUT
+    net.set_params(p)
+    assert torch.equal(net.forward(x), want)
+    net.gradients(x, t)
