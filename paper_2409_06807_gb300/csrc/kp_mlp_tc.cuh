@@ -163,7 +163,7 @@ struct FtArgs {
   int M, vec;               // vec: x and out allow 16- and 8-byte accesses
   int* err;
   unsigned long long wait_ns;
-  int hold;                 // test hook: no product is issued
+  int hold;                 // test hook: no product after the first ones is issued
 };
 
 // Inputs 16 part .. 16 part + 15 of a row (zeros past the last row).
@@ -214,7 +214,7 @@ __device__ __forceinline__ void ft_load_x(const FtArgs& a, int row, int part, fl
 // shared memory (51 us).
 __global__ void __launch_bounds__(FT_THREADS, 1) kp_mlp_forward_tc_kernel(FtArgs a) {
   extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t b_w1, b_w2[4], b_x, b_d1, b_h[4], b_d2, b_e2;
+  __shared__ __align__(8) uint64_t b_w1, b_w2[4], b_x, b_d1, b_h[4], b_d2, b_e2, b_end;
   __shared__ __align__(8) float s_part[2][FT_ROWS][MLP_OUT];
   __shared__ uint32_t tmem_slot;
   __shared__ int s_fail;
@@ -232,6 +232,7 @@ __global__ void __launch_bounds__(FT_THREADS, 1) kp_mlp_forward_tc_kernel(FtArgs
     }
     mbar_init(saddr(&b_d2), 1);
     mbar_init(saddr(&b_e2), FT_G2);
+    mbar_init(saddr(&b_end), 1);
     s_fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async();
@@ -278,8 +279,8 @@ __global__ void __launch_bounds__(FT_THREADS, 1) kp_mlp_forward_tc_kernel(FtArgs
         mma_commit(saddr(&b_d1));
       };
       bool ok = wait(&b_w1, 0, 10) && wait(&b_x, 0, 11);
-      if (a.hold) ok = wait(&b_d2, 0, 16);  // (nothing is committed to it)
       if (ok) layer1();
+      if (a.hold) ok = wait(&b_d2, 0, 16);  // (nothing is committed to it)
       uint32_t ph = 0;
       for (int t = blockIdx.x; ok && t < n_tiles; t += stride, ph ^= 1u) {
         const bool first = t == (int)blockIdx.x, more = t + stride < n_tiles;
@@ -299,8 +300,6 @@ __global__ void __launch_bounds__(FT_THREADS, 1) kp_mlp_forward_tc_kernel(FtArgs
           if (ok) layer1();
         }
       }
-      // the weights' copies have landed before the block's memory goes
-      for (int c = 0; c < 4; ++c) mbar_wait(saddr(&b_w2[c]), 0, a.wait_ns);
     }
     __syncwarp();
   } else if (warp < FT_G1) {
@@ -445,6 +444,15 @@ __global__ void __launch_bounds__(FT_THREADS, 1) kp_mlp_forward_tc_kernel(FtArgs
   fence_before();
   __syncthreads();
   if (warp == FT_G1 + FT_G2) {
+    if (lane == 0 && s_fail) {
+      // a wait gave up: products and the weights' copies may be in flight, and
+      // they end before the block's memories go
+      mma_commit(saddr(&b_end));
+      mbar_wait(saddr(&b_end), 0, a.wait_ns);
+      mbar_wait(saddr(&b_w1), 0, a.wait_ns);
+      for (int c = 0; c < 4; ++c) mbar_wait(saddr(&b_w2[c]), 0, a.wait_ns);
+    }
+    __syncwarp();
     fence_after();
     tmem_dealloc(tmem, 512);
   }
