@@ -463,9 +463,10 @@ kp_status kp_mlp_train_step(kp_mlp *mlp, const float *dev_x,
 kp_status kp_mlp_train_epoch(kp_mlp *mlp, const float *dev_x, const float *dev_t,
                              const int32_t *dev_perm, int64_t rows, float lr,
                              float *host_loss);
-/* Test hook for the bounded waits: with limit_ns > 0 (2 s at most) the
- * network's inference launches hold their second layer's products back, so
- * that the waits for them expire after limit_ns; 0 ends this.  KP_ERR_ARG past 2 s. */
+/* Test hook for the bounded waits: with limit_ns > 0 (2 s at most) a wait in
+ * each of the network's launches (inference: for the second layer's products,
+ * training: for a copy that has not been asked for) expires after limit_ns; 0
+ * ends this.  KP_ERR_ARG past 2 s. */
 kp_status kp_mlp_selftest_hold(kp_mlp *mlp, uint64_t limit_ns);
 void kp_mlp_destroy(kp_mlp *mlp);
 /* Planner use of a network (6D systems): each pass evaluates the network on

@@ -175,6 +175,7 @@ tc::StepArgs step_args(const kp_mlp* n, const float* x, const float* t, int M, f
   a.slots = n->slots;
   a.err = n->err;
   a.wait_ns = n->wait_ns;
+  a.hold = n->hold;
   return a;
 }
 

@@ -606,6 +606,7 @@ struct StepArgs {
   uint32_t* bar;           // epoch: grid barrier word, 0 at launch
   int* err;
   unsigned long long wait_ns;
+  int hold;                // test hook: a wait for what is not yet asked for
 };
 
 // kind::f16 descriptor with the operands' majors (1: M or N contiguous).
@@ -714,7 +715,7 @@ __device__ __forceinline__ bool grid_arrive_wait(uint32_t* bar, uint32_t n, cons
 // us).
 __global__ void __launch_bounds__(ST_THREADS, 1) kp_mlp_train_kernel(StepArgs a) {
   extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t b_w1, b_w2[4], b_mma, b_c, b_t0, b_r;
+  __shared__ __align__(8) uint64_t b_w1, b_w2[4], b_mma, b_c, b_t0, b_r, b_end;
   __shared__ float s_red[4][MLP_NQ][3];  // sums over a warp's rows: loss, both gradients
   __shared__ float s_b3[MLP_OUT];
   __shared__ uint32_t tmem_slot;
@@ -729,6 +730,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) kp_mlp_train_kernel(StepArgs a)
     mbar_init(saddr(&b_c), 1);
     mbar_init(saddr(&b_r), 1);
     mbar_init(saddr(&b_t0), 1);
+    mbar_init(saddr(&b_end), 1);
     s_fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -835,6 +837,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) kp_mlp_train_kernel(StepArgs a)
 
   const int n_tiles = (a.M + 127) / 128;
   uint32_t arrivals = 0;
+  bool in_tile = false;  // a wait of the last tile gave up
   for (int64_t s = 0; s < a.steps; ++s) {
     for (int tile = blockIdx.x; tile < n_tiles; tile += (int)gridDim.x, ph_t ^= 1u) {
       const int row0 = tile * 128;
@@ -899,6 +902,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) kp_mlp_train_kernel(StepArgs a)
 
       // ---- forward
       if (tid == 0) {
+        if (a.hold) wait(&b_r, ph_t, 41);  // (W2's second copy starts below)
         wait(&b_w1, ph_t, 30);
         fence_after();
 #pragma unroll
@@ -1088,6 +1092,11 @@ __global__ void __launch_bounds__(ST_THREADS, 1) kp_mlp_train_kernel(StepArgs a)
       fence_before();
       __syncthreads();
       fence_after();
+      // a wait gave up: no further tile, and the barriers stay at this tile's
+      // phases (every thread sees the flag: the next one to set it would wait
+      // behind the next tile's first __syncthreads)
+      in_tile = failed();
+      if (in_tile) break;
     }
     if (!a.epoch) break;
     // ---- optimiser: every tile's gradient is in; this CTA's share of the
@@ -1124,15 +1133,22 @@ __global__ void __launch_bounds__(ST_THREADS, 1) kp_mlp_train_kernel(StepArgs a)
   fence_before();
   __syncthreads();
   if (warp == 0) {
+    if (lane == 0 && s_fail) {
+      if (in_tile) {
+        // the tile's products and copies may be in flight, and they end before
+        // the block's memories go (a block whose grid barrier gave up, or that
+        // had no tile, has none)
+        mma_commit(saddr(&b_end));
+        mbar_wait(saddr(&b_end), 0, a.wait_ns);
+        mbar_wait(saddr(&b_w1), ph_t, a.wait_ns);
+        for (int c = 0; c < 4; ++c) mbar_wait(saddr(&b_w2[c]), ph_t, a.wait_ns);
+        mbar_wait(saddr(&b_r), ph_t, a.wait_ns);
+      }
+      atomicExch(a.err, 100 + s_fail);
+    }
+    __syncwarp();
     fence_after();
     tmem_dealloc(tmem, 512);
-  }
-  if (tid == 0 && s_fail) {
-    // a wait gave up: copies may be in flight, wait for them once more
-    mbar_wait(saddr(&b_w1), ph_t, a.wait_ns);
-    for (int c = 0; c < 4; ++c) mbar_wait(saddr(&b_w2[c]), ph_t, a.wait_ns);
-    mbar_wait(saddr(&b_r), ph_t, a.wait_ns);
-    atomicExch(a.err, 100 + s_fail);
   }
 }
 

@@ -440,3 +440,38 @@ def test_inference_that_gives_up_says_so(M, n):
     net.set_params(p)
     assert torch.equal(net.forward(x), want)
     net.gradients(x, t)
+
+
+@pytest.mark.parametrize("n", [1, 129, 152 * 128 + 5])
+@pytest.mark.parametrize("form", ["gradients", "epoch"])
+def test_training_that_gives_up_ends_at_once(M, n, form):
+    """A training launch whose wait expires (the test hook) ends with
+    KP_ERR_TIMEOUT after one wait limit: blocks wait for what they have in
+    flight and for nothing else, those without a tile and those of one that had
+    finished its tiles included.  Setting the parameters clears the error."""
+    import time
+
+    import torch
+    mlp, planner = M
+    p = mlp.init_params(3)
+    net = mlp.Mlp(p, max_batch=n)
+    x, t = [torch.from_numpy(v).cuda() for v in _data(2 * n, n)]
+    perm = torch.arange(2 * n, dtype=torch.int32, device="cuda")
+    call = (lambda: net.gradients(x[:n], t[:n])) if form == "gradients" else \
+        (lambda: net.train_epoch(x, t, perm))
+    want = call()
+    net.set_params(p)
+    net.selftest_hold(100_000_000)  # 100 ms
+    torch.cuda.synchronize()
+    t0 = time.perf_counter()
+    with pytest.raises(planner.KpError) as e:
+        call()
+    took = time.perf_counter() - t0
+    assert e.value.status == planner.ERR_TIMEOUT and 0.09 < took < 0.2
+    net.selftest_hold(0)
+    net.set_params(p)
+    got = call()
+    if form == "gradients":
+        assert np.array_equal(got[0], want[0]) and got[1] == want[1]
+    else:
+        assert got == want
