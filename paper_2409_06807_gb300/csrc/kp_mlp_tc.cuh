@@ -960,13 +960,18 @@ __global__ void __launch_bounds__(ST_THREADS, 1) kp_mlp_train_kernel(StepArgs a)
           const int n = qt + MLP_NQ * i;
           const float d = sum[1 + i];
           // three BF16 parts of the value: rounding, then what is left, twice
-          const __nv_bfloat16 p0 = __float2bfloat16_rn(d);
-          const float r1 = d - __bfloat162float(p0);
+          // (nothing of an infinite one: infinity minus infinity would be NaN;
+          // what would round to infinity, only for the first part's weight, is
+          // cut to BF16's largest number)
+          const __nv_bfloat16 pd = __float2bfloat16_rn(d);
+          const bool over = __hisinf(pd) != 0;
+          const __nv_bfloat16 p0 = over ? __float2bfloat16_rz(d) : pd;
+          const float r1 = over && isinf(d) ? 0.0f : d - __bfloat162float(p0);
           const __nv_bfloat16 p1 = __float2bfloat16_rn(r1);
           const __nv_bfloat16 p2 = __float2bfloat16_rn(r1 - __bfloat162float(p1));
           sts16(base + ST_DT + (uint32_t)((r >> 6) * 2048 + n * 128 + ((((r & 63) >> 3) ^ n) << 4) +
                                           (r & 7) * 2),
-                p0);
+                pd);
           const uint32_t da = base + ST_DA + (uint32_t)(r * 64 + 2 * n), sw = (uint32_t)((r >> 1) & 3);
           sts16(da + ((0u ^ sw) << 4), p0);
           sts16(da + ((1u ^ sw) << 4), p1);

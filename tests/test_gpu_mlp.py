@@ -475,3 +475,44 @@ def test_training_that_gives_up_ends_at_once(M, n, form):
         assert np.array_equal(got[0], want[0]) and got[1] == want[1]
     else:
         assert got == want
+
+
+@pytest.mark.parametrize("n", [40, 300])
+def test_gradients_of_an_infinite_output_gradient(M, n):
+    """A target so far off that the squared deviation overflows FP32: the
+    gradient of that output is -inf, and what follows from it is infinite or NaN
+    where FP32 arithmetic makes it so (every infinity in the second layer's
+    gradient with its weight's sign), not NaN throughout."""
+    import torch
+    mlp, _ = M
+    p = mlp.init_params(5)
+    net = mlp.Mlp(p, max_batch=n)
+    x, t = [torch.from_numpy(v).cuda() for v in _data(n, n)]
+    t[7, 2] = 1e25
+    g, loss = net.gradients(x, t)
+    assert loss == np.inf
+
+    def rnd(v):
+        return v.to(torch.float32).to(torch.bfloat16).double()
+
+    W1, b1, W2, b2, W3, b3 = [torch.from_numpy(v.copy()).cuda() for v in mlp.split(p)]
+    W1, W2, W3, xb = rnd(W1), rnd(W2), rnd(W3), rnd(x)
+    h1 = rnd((xb @ W1.T + b1.double()).clamp(min=0))
+    h2 = rnd((h1 @ W2.T + b2.double()).clamp(min=0))
+    o = (h2 @ W3.T + b3.double()).float()
+    mu, ls = torch.tanh(o[:, :4]), o[:, 4:]
+    assert float(ls.abs().max()) < 1
+    z = (t - mu) * torch.exp(-ls)
+    d = (torch.cat([-z * torch.exp(-ls) * (1 - mu * mu), 1 - z * z], 1) / n).double()
+    assert int(torch.isinf(d).sum()) == 1
+    # (no matrix product here: it may split the sums)
+    d2 = torch.where(h2 > 0, (d[:, :, None] * W3[None]).sum(1), 0.0).float().to(torch.bfloat16).double()
+    ref = dict(W2=(d2[:, :, None] * h1[:, None, :]).sum(0), b2=d2.sum(0),
+               W3=(d[:, :, None] * h2[:, None, :]).sum(0), b3=d.sum(0))
+    got = dict(zip(("W1", "b1", "W2", "b2", "W3", "b3"), mlp.split(g)))
+    for k, want in ref.items():
+        want = want.cpu().numpy()
+        assert np.isinf(want).any(), k
+        assert np.array_equal(np.isnan(got[k]), np.isnan(want)), k
+        assert np.array_equal(np.isposinf(got[k]), np.isposinf(want)), k
+        assert np.array_equal(np.isneginf(got[k]), np.isneginf(want)), k
