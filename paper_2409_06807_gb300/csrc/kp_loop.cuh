@@ -899,6 +899,12 @@ __device__ __forceinline__ void for_own_chunks(const Team& T, int nch, F body) {
   for (int c = T.b + T.nb * (int)(threadIdx.x >> 5); c < nch; c += T.nb * (int)(blockDim.x >> 5)) body(c);
 }
 
+// The score that stands for none (outside R_avail), told from all others by its
+// high word: a score is not negative, but one that is not a number (an infinite
+// delta) has the sign bit set.
+constexpr double KP_NO_SCORE = -1.0;
+__device__ __forceinline__ bool no_score(int score_hi) { return score_hi == (int)0xbff00000; }
+
 // Phase S: Eq. 3-4 for a warp's region chunk and the chunk's pairwise partial
 // sum (published by the grid barrier that ends the phase).  Lane l takes the
 // chunk's m = max(ch / 32, 1) regions from l m on and adds their scores up as
@@ -936,7 +942,7 @@ __device__ __forceinline__ void phase_scores(const KParams& P, const Team& T, in
           const double f2 = __dmul_rn(fv, fv);
           sc = __ddiv_rn(__dmul_rn(f2, f2), den);
         }
-        P.score[r] = avail ? sc : -1.0;  // no score: P_accept = 1
+        P.score[r] = avail ? sc : KP_NO_SCORE;  // P_accept = 1
       }
       int k = 0;
       for (; (q >> k) & 1; ++k) sc = __dadd_rn(left[k], sc);
@@ -960,8 +966,8 @@ __device__ __forceinline__ uint64_t threshold_of(double p) {
   return down < 64 ? mant >> down : 0ull;
 }
 
-// The acceptance threshold of a region with this score (negative: outside
-// R_avail, P_accept = 1): threshold_of(score / sum + eps), eps below 1, or
+// The acceptance threshold of a region with this score (none: outside R_avail,
+// P_accept = 1): threshold_of(score / sum + eps), eps below 1, or
 // threshold_of(eps) when the sum is not positive.  inv = 1 / sum gives it without
 // the division (573 clocks and about ten FP64 operations, of which an SM does
 // two a clock): score inv + eps in one rounding is within 4 units in the last
@@ -971,7 +977,7 @@ __device__ __forceinline__ uint64_t threshold_of(double p) {
 // 0: always by the division (a sum that is not a number between 2^-900 and
 // 2^900).
 __device__ __forceinline__ uint64_t accept_threshold(double score, double sum, double inv, double eps) {
-  if (__double2hiint(score) < 0) return 1ull << 32;
+  if (no_score(__double2hiint(score))) return 1ull << 32;
   if (__double2hiint(inv) != 0) {
     const long long near = __double_as_longlong(__fma_rn(score, inv, eps));
     const uint64_t lo = threshold_of(__longlong_as_double(near - 16));
@@ -989,7 +995,7 @@ __device__ __forceinline__ uint64_t accept_threshold(double score, double sum, d
 // The rest, one draw in some 100,000, takes the threshold itself.
 __device__ __forceinline__ bool draw_accepted(uint32_t w, double score, const LoopShared& sh, double eps) {
   const int hi = __double2hiint(score);
-  if (hi < 0) return true;
+  if (no_score(hi)) return true;
   // score inv_m 2^inv_e in two factors: the mantissas' product, a power of two
   const int e = (hi >> 20) - 1023 + sh.inv_e;  // at most 1: a score is a part of the sum
   const float m = __int_as_float(0x3f800000 | (int)(__funnelshift_l((uint32_t)__double2loint(score),

@@ -462,6 +462,29 @@ def test_consecutive_queries_start_clean(P):
         f.close()
 
 
+def test_scores_that_are_no_numbers(P):
+    """An infinite delta makes every score of Eq. 3-4 infinity over infinity:
+    the sum is not positive, so P_accept is eps in R_avail (the form of Eq. 5
+    without a positive sum) and 1 outside, in the table and in the draws."""
+    w = W.tiny(W.DI, seed=2, t_e=40000, lambda_max=32, sub=(8, 8, 8)).with_(
+        delta=float("inf"), eps=0.3, goal_c=np.full(3, 9.0, np.float32), goal_r=np.float32(0.0))
+    g = P.Planner(w)
+    assert g.reset() == P.OK
+    for _ in range(20):
+        if g.info()["n_nodes"] >= 1000:
+            break
+        g.expand_step(1)
+    t = g.export_tree()
+    thr = np.where(t["avail"] != 0, int(0.3 * 2.0**32), 1 << 32)
+    assert t["avail"].any() and np.array_equal(t["thr"], thr.astype(np.uint64))
+    n = t["n_nodes"]
+    old = g.expand_step(1)[0]
+    t = g.export_tree()
+    kept = t["in_ve"][:n].mean()
+    assert n >= 1000 and t["in_ve"][n:].all() and old["n_nodes"] > n
+    assert abs(kept - 0.3) < 5 * np.sqrt(0.3 * 0.7 / n)  # five standard deviations
+
+
 def test_budget_iterations(P):
     w = W.c2(0)
     g = P.Planner(w)
