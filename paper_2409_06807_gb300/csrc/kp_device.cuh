@@ -5,6 +5,7 @@
 
 #include <cstdint>
 
+#include "kp_arith.cuh"
 #include "kp_layout.h"
 
 namespace kp {
@@ -557,7 +558,7 @@ __device__ __forceinline__ int bp_cell_of(float t, float last) {
 // the grown cell; otherwise both sides are checked and the cell is clamped.
 // The one comparison is d <= 1 + q / 16 for the largest distance d of the hull
 // from the cell's low corner (or, outside, of the cell's low corner from it
-// plus 1), taken as an integer: 16 d - 16 rounded up against q.  Minimum,
+// plus 1), taken as an integer (within_clearance).  Minimum,
 // maximum, compare and logic instructions issue at half the rate of FP32
 // additions and products on this GPU, so the test is written with few of them.
 template <bool INSIDE>
@@ -575,9 +576,7 @@ __device__ __forceinline__ bool hull_clear(const KParams& P, const uint8_t* __re
   }
   const int c = KP_IDX(P, v[0] + P.bp_g[0] * v[1] + P.bp_gxy * v[2] - P.bp_bias,
                        P.bp_g[0] * P.bp_g[1] * P.bp_g[2], 60);
-  const int q = sclear[c];
-  const int e = __float_as_int(__fmaf_ru(fmaxf(fmaxf(d[0], d[1]), d[2]), 16.0f, 8388592.0f));
-  return q != 0 && e - 0x4B000000 <= q;
+  return within_clearance(fmaxf(fmaxf(d[0], d[1]), d[2]), sclear[c]);
 }
 
 // Exact coarse-then-fine collision test of the hull of a step from p to x (the

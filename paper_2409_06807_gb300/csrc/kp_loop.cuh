@@ -79,10 +79,7 @@ struct LoopShared {
   uint64_t mbar;
   int flag;
   int bcast[2];
-  // of the pass's scores, see accept_threshold and draw_accepted
-  double score_sum, score_inv;
-  float inv_m, eps32;
-  int inv_e;
+  ScoreSum score;  // of the pass
   int goal, err;         // the pass's goal node and error word, read in phase L
   int32_t phase_ns[12];  // per-pass phase timers (block 0, thread 0)
 };
@@ -421,29 +418,6 @@ __device__ __forceinline__ void box_muller4(uint4 w, float* z) {
     z[2 * pr + 1] = rad * s;
   }
 }
-
-// Division of a sample key by the pass's lambda (at most 1024) by a
-// multiplication: for lam in [2^s, 2^(s+1)) and mul = ceil(2^(31+s) / lam), key
-// / lam = (key mul) >> (31 + s) for every key below 2^30 (the product exceeds
-// the quotient's by key (mul lam - 2^(31+s)) / lam < key, less than the 2^(31+s)
-// / lam that is left).  Two 32-bit divisions a pass and thread instead of one a
-// sample: mul's quotient in two steps, 2^31 = a lam + b, 2^s b = c lam + d.
-struct KeyDiv {
-  int lam, shift;
-  uint32_t mul;
-  __device__ __forceinline__ explicit KeyDiv(int l) : lam(l), shift(0), mul(0) {
-    if (l > 0) {
-      const uint32_t u = (uint32_t)l;
-      shift = 31 - __clz(l);
-      const uint32_t a = 0x80000000u / u, b = 0x80000000u - a * u;
-      const uint32_t c = (b << shift) / u, d = (b << shift) - c * u;
-      mul = (a << shift) + c + (d != 0u ? 1u : 0u);
-    }
-  }
-  __device__ __forceinline__ int quot(int key) const {
-    return (int)(__umulhi((uint32_t)key << 1, mul) >> shift);
-  }
-};
 
 // The draw of sample key (V_E position p = key / lam of node v, j = key - p
 // lam) in pass it (Algorithm 2: random control in U, random duration).
@@ -899,12 +873,6 @@ __device__ __forceinline__ void for_own_chunks(const Team& T, int nch, F body) {
   for (int c = T.b + T.nb * (int)(threadIdx.x >> 5); c < nch; c += T.nb * (int)(blockDim.x >> 5)) body(c);
 }
 
-// The score that stands for none (outside R_avail), told from all others by its
-// high word: a score is not negative, but one that is not a number (an infinite
-// delta) has the sign bit set.
-constexpr double KP_NO_SCORE = -1.0;
-__device__ __forceinline__ bool no_score(int score_hi) { return score_hi == (int)0xbff00000; }
-
 // Phase S: Eq. 3-4 for a warp's region chunk and the chunk's pairwise partial
 // sum (published by the grid barrier that ends the phase).  Lane l takes the
 // chunk's m = max(ch / 32, 1) regions from l m on and adds their scores up as
@@ -954,74 +922,12 @@ __device__ __forceinline__ void phase_scores(const KParams& P, const Team& T, in
   });
 }
 
-// floor(min(p, 1) 2^32) of a positive p, from its bits: the mantissa shifted
-// down by as much as its last place lies below 2^-32 (an FP64 instruction
-// takes 64 clocks here, and this was four of them).
-__device__ __forceinline__ uint64_t threshold_of(double p) {
-  const uint64_t bits = (uint64_t)__double_as_longlong(p);
-  const int e = (int)(bits >> 52) - 1023;  // p in [2^e, 2^(e+1))
-  if (e >= 0) return 1ull << 32;           // infinities too
-  const uint64_t mant = (bits & 0xfffffffffffffull) | (1ull << 52);
-  const int down = 20 - e;                 // 52 - 32 - e
-  return down < 64 ? mant >> down : 0ull;
-}
-
-// The acceptance threshold of a region with this score (none: outside R_avail,
-// P_accept = 1): threshold_of(score / sum + eps), eps below 1, or
-// threshold_of(eps) when the sum is not positive.  inv = 1 / sum gives it without
-// the division (573 clocks and about ten FP64 operations, of which an SM does
-// two a clock): score inv + eps in one rounding is within 4 units in the last
-// place of the value it stands for (half from inv, half each from the two
-// roundings there and one here, at most doubled by a binade), so where 16 units
-// more or less make no difference to the threshold it is the same one.  inv =
-// 0: always by the division (a sum that is not a number between 2^-900 and
-// 2^900).
-__device__ __forceinline__ uint64_t accept_threshold(double score, double sum, double inv, double eps) {
-  if (no_score(__double2hiint(score))) return 1ull << 32;
-  if (__double2hiint(inv) != 0) {
-    const long long near = __double_as_longlong(__fma_rn(score, inv, eps));
-    const uint64_t lo = threshold_of(__longlong_as_double(near - 16));
-    if (lo == threshold_of(__longlong_as_double(near + 16))) return lo;
-  }
-  return threshold_of(sum > 0.0 ? __dadd_rn(__ddiv_rn(score, sum), eps) : eps);
-}
-
-// Whether the draw w of a node is below its region's accept_threshold.  Decided
-// in FP32 (an FP64 operation a node was 0.6 % of a query that ends with a
-// million nodes): w < floor(t), t = (score / sum + eps) 2^32, is w + 1 <= t, and
-// t from 24 bits of score and 1 / sum is off by less than 2^-21 of it (2^-23
-// from cutting the score, 2^-24 from each of 1 / sum, eps, w + 1 and three
-// roundings), so a difference above 2^-18 of the larger side has the right sign.
-// The rest, one draw in some 100,000, takes the threshold itself.
-__device__ __forceinline__ bool draw_accepted(uint32_t w, double score, const LoopShared& sh, double eps) {
-  const int hi = __double2hiint(score);
-  if (no_score(hi)) return true;
-  // score inv_m 2^inv_e in two factors: the mantissas' product, a power of two
-  const int e = (hi >> 20) - 1023 + sh.inv_e;  // at most 1: a score is a part of the sum
-  const float m = __int_as_float(0x3f800000 | (int)(__funnelshift_l((uint32_t)__double2loint(score),
-                                                                    (uint32_t)hi, 3) & 0x7fffffu));
-  const float scale = __int_as_float((e < -126 ? 0 : e + 127) << 23);
-  const float t = __fmul_rn(__fmaf_rn(__fmul_rn(m, sh.inv_m), scale, sh.eps32), 4294967296.0f);
-  const float w1 = __fadd_rn((float)w, 1.0f);
-  if (e < 64 && fabsf(t - w1) > fmaxf(t, w1) * 3.814697265625e-06f) return w1 < t;
-  return (uint64_t)w < accept_threshold(score, sh.score_sum, sh.score_inv, eps);
-}
-
 // The sum of Eq. 5 from the chunks' partial sums, by the calling warp, for the
-// block: sh.score_sum and sh.score_inv (accept_threshold's inv).
+// block: sh.score.
 __device__ __forceinline__ void sum_scores(const KParams& P, const Team& T, int nch, LoopShared& sh) {
   const double sum = warp_tree_sum(nch, [&](int i) { return __ldcg(P.chunk_sum + i); });
   if ((threadIdx.x & 31u) == 0) {
-    const int e = (__double2hiint(sum) >> 20) - 1023;  // of a positive number
-    sh.score_sum = sum;
-    const double inv = e >= -900 && e <= 900 ? __ddiv_rn(1.0, sum) : 0.0;
-    sh.score_inv = inv;
-    // (draw_accepted takes the threshold itself where there is no inverse)
-    sh.inv_e = inv > 0.0 ? (__double2hiint(inv) >> 20) - 1023 : 1 << 16;
-    sh.inv_m = inv > 0.0 ? (float)__longlong_as_double((__double_as_longlong(inv) & 0xfffffffffffffll) |
-                                                      0x3ff0000000000000ll)
-                         : 1.0f;
-    sh.eps32 = (float)P.eps;
+    sh.score = score_sum_of(sum, P.eps);
     if (T.b == 0) P.ctl->score_sum = sum;
   }
 }
@@ -1032,7 +938,7 @@ __device__ __forceinline__ void phase_thresholds(const KParams& P, const Team& T
   const int ch = P.R_pad / nch;
   for_own_chunks(T, nch, [&](int c) {
     for (int r = c * ch + (int)(threadIdx.x & 31u); r < (c + 1) * ch && r < P.R; r += 32)
-      P.thr[r] = accept_threshold(P.score[r], sh.score_sum, sh.score_inv, P.eps);
+      P.thr[r] = accept_threshold(P.score[r], sh.score.sum, sh.score.inv, P.eps);
   });
 }
 
@@ -1185,7 +1091,7 @@ __device__ __forceinline__ void phase_nodesets(const KParams& P, const Team& T, 
       const int v = t0 + q * stride + (int)threadIdx.x;
       if (v < o1) {
         const uint4 w = philox4x32_10(make_uint4(it, (uint32_t)v, 0u, 2u), P.seed_lo, P.seed_hi);
-        const int e = draw_accepted(w.x, sq[q], sh, P.eps) ? 1 : 0;
+        const int e = draw_accepted(w.x, sq[q], sh.score, P.eps) ? 1 : 0;
         P.in_ve[v] = (uint8_t)e;
         c += e;
       }
