@@ -1186,8 +1186,9 @@ kp_status kp_plan_async(kp_ctx* ctx, const float* x_init, const kp_goal* goal,
     return fail(ctx, KP_ERR_ARG, "bad goal");
   const int rows = traj_capacity < KP_TRAJ_ROWS ? traj_capacity : KP_TRAJ_ROWS;
   const size_t traj_bytes = (size_t)rows * 17 * 4;
-  // every copy through the staging buffer completes before its call
-  // returns, so it is free here
+  // the staging buffer is written by the device only, in stream order behind an
+  // obstacle copy out of it that may still be queued; ensure_pinned waits for the
+  // stream before it replaces the buffer
   if (ctx->plan_pending) return fail(ctx, KP_ERR_STATE, "kp_plan_result not called");
   s = ensure_pinned(ctx, sizeof(KCtl) + traj_bytes);
   if (s != KP_OK) return s;
@@ -2262,7 +2263,9 @@ bool try_admit(kp_server* s, PendingQuery& q) {
   // regions (padded) to one of the team's blocks, a power of two of them
   int shares = 1;
   while (shares * 2 <= s->team_blocks && shares * 2 * 32 <= d.R_pad && shares * 2 <= 1024) shares *= 2;
-  // no cell clearances: the host would spend milliseconds per query on them
+  // without cell clearances: they took the host milliseconds a query when this
+  // was chosen (a whole blob of 1,200 boxes takes 0.3 ms now; served queries with
+  // them have not been measured)
   const size_t blob_bytes = build_blob(s->blob.data(), q.boxes.empty() ? nullptr : q.boxes.data(),
                                        (int)(q.boxes.size() / 6), q.ws, P, KS_BLOB_MAX, false);
   const size_t least = (size_t)P.n_boxes_pad * 32 + round16(4) + round16((q.boxes.size() / 6) * 2);

@@ -1063,8 +1063,8 @@ __device__ __forceinline__ void phase_nodesets(const KParams& P, const Team& T, 
   *n_new = (int)acc_total;
   const int t_new = t_old + (int)acc_total;
   materialise<SYS, LOG>(P, it, t_old + (int)acc_before, kd, sh, sblob, e0);
-  // old nodes of the chunk: four tiles at a time, their region and score loads
-  // issued together (the first four tiles' before the wait for the sum)
+  // old nodes of the chunk: two tiles at a time, their region and score loads
+  // issued together (the first two tiles' before the wait for the sum)
   int v0, v1;
   chunk_of(T, t_new, &v0, &v1);
   const int o1 = v1 < t_old ? v1 : t_old;
@@ -1424,8 +1424,8 @@ __device__ void init_root(const KParams& P, const RootState& root, bool box_free
   ctl->state = in_goal ? KP_DEV_SOLVED : KP_DEV_RUNNING;
 }
 
-// Algorithm 1, initialisation, as a launch of its own (kp_reset and the
-// no-allocation entry): every block clears its share of the tables
+// Algorithm 1, initialisation, as a launch of its own (kp_reset; a query does
+// it inside its loop launch): every block clears its share of the tables
 // (clear_tables); the last block to finish (a counter taken after a fence)
 // writes the root, so the root's table entries come after every clear.
 template <int SYS>

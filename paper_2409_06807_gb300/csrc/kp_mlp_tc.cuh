@@ -203,8 +203,8 @@ __device__ __forceinline__ void ft_load_x(const FtArgs& a, int row, int part, fl
 //
 // Measured (GB300): 262,145 rows in 42.5 us (0.93 PFLOP/s, 49 % of the measured
 // bf16 rate) against 326 us for a kernel of one 32-row tile a block on mma.sync,
-// which fetched every weight fragment from L2 for each tile; 33 rows 8.2
-// against 10.3 us a call.  A tile takes about 5,000 clocks where its products
+// which fetched every weight fragment from L2 for each tile; 33 rows 8.2 to 9.8
+// us a call over runs against 10.3 to 10.6.  A tile takes about 5,000 clocks where its products
 // need 2,300: the chain accumulator -> epilogue 1 -> first chunk -> layer 2 is
 // what is left, and layer 2 runs at two thirds of its rate beside the
 // epilogues' shared-memory and tensor-memory traffic.  Arrangements measured
@@ -706,13 +706,14 @@ __device__ __forceinline__ bool grid_arrive_wait(uint32_t* bar, uint32_t n, cons
 // 17,000 of a step's 57,000 clocks (L2 added 120 values a clock), and the
 // result now has the same bits every time.
 //
-// A mini-batch of 4096 is 32 tiles, so a step is one tile's chain of twelve
-// products and epilogues (21,000 clocks), 9,000 for the slot's 305 KB, 5,000
-// for the optimiser's share and 6,000 in the two barriers: 25 us (GB300).
-// Epochs of 16 steps of 4,096 rows: 1,333 us as 15 launches a step (row-major
-// and transposed activations in global memory, split-K products), 561 us as two
-// launches a step with this pass, 465 us now, with the parameter read-back (50
-// us).
+// A mini-batch of 4096 is 32 tiles, so a step is one tile's chain (21,000
+// clocks: nine products, forward and backward, in six rounds, each round behind
+// the epilogue of the one before), 9,000 for the slot's 305 KB, 5,000 for the
+// optimiser's share and 6,000 in the two barriers: 25 us of the launch (GB300).
+// Epochs of 16 steps of 4,096 rows, whole calls with the parameter read-back
+// (50 us): 1,333 us as 15 launches a step (row-major and transposed activations
+// in global memory, split-K products), 561 us as two launches a step with this
+// pass, 460 us now.
 __global__ void __launch_bounds__(ST_THREADS, 1) kp_mlp_train_kernel(StepArgs a) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t b_w1, b_w2[4], b_mma, b_c, b_t0, b_r, b_end;

@@ -261,10 +261,10 @@ def test_learned_plan_revalidated(M):
 
 
 def test_device_epoch_matches_step_loop(M):
-    """One epoch driven on the device (gather + step as one graph launch per
-    mini-batch) against the same mini-batches stepped from the host: equal
-    mean loss and parameters up to the rounding of FP32 atomic sums; the
-    graph is reused by later epochs, which keep lowering the loss."""
+    """One epoch driven on the device (one launch for all its mini-batches)
+    against the same mini-batches stepped from the host: equal mean loss and
+    parameters up to the rounding of FP32 sums; later epochs keep lowering the
+    loss."""
     import torch
     mlp, _ = M
     rng = np.random.default_rng(21)

@@ -62,7 +62,7 @@ def test_server_results_revalidated_and_match_single_launch(S):
     launch on the same inputs returns the same trajectory bit for bit.  Both
     run the same explicitly rounded FP32 arithmetic on the same keys, and
     the obstacle test's verdict is exact whatever the broad-phase grid (the
-    server's blob is built without cell clearances, within its 48 KB room),
+    server's blob is built without cell clearances, within its 64 KB room),
     so status, edge count, states, controls and durations must agree
     exactly."""
     P, serve = S
